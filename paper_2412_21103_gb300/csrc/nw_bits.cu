@@ -45,55 +45,115 @@ namespace nw {
 // planes of the previous anti-diagonal; Q: the shift register of the stripe
 // boundary (bit 31 = the input bit of this step, the output bit enters at
 // bit 0).  bw: the B window (bit p = base of column t+1-p), A: the row bases,
-// rmask: rows of the grid (padding rows give s' = 0).  RAMP: the first chunk
-// of a stripe, where bits p > u lie in column <= 0 and their dV is forced to
-// the boundary's 0.
-template <bool GEN, bool RAMP>
+// rmask: rows of the grid (the padding rows of a pair's first stripe, FIRST,
+// keep the boundary's zero differences).  RAMP: the first chunk of a stripe,
+// where bits p > u lie in column <= 0 and their dV is forced to the
+// boundary's 0.
+//
+// What bounds it: the logic pipe, 16 operations for 32 cells (two B window
+// shifts, two for equality, two to bring the upper dH into line, eight for
+// the update, two for the shift register).
+template <bool GEN, bool RAMP, bool FIRST>
 __device__ __forceinline__ void bits_step(int u, uint32_t &H0, uint32_t &H1, uint32_t &V0, uint32_t &V1, uint32_t &Q0,
                                           uint32_t &Q1, uint32_t A0, uint32_t A1, uint32_t bw0, uint32_t bw1,
                                           uint32_t rmask, const BitsScoring &g, uint32_t X1r, uint32_t X0r) {
-    const uint32_t x = lop3<kLutXorOrNotC>(A1, bw1, rmask);
-    const uint32_t eq = lop3<kLutEq>(A0, bw0, x);  // A_i == B_j (0 on padding rows)
     const uint32_t a0 = __funnelshift_l(Q0, H0, 1), a1 = __funnelshift_l(Q1, H1, 1);  // dH of the cell above
     const uint32_t b0 = V0, b1 = V1;                                                  // dV of the cell to the left
-    const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);  // the low bit of max(a, b), from a
-    const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);  // ... from b
-    uint32_t T0, T1;
     if constexpr (!GEN) {
-        // s' = (eq, 1) on grid rows (3 or 1), 0 on padding rows
-        const uint32_t v = lop3<kLutCOrNor>(a1, b1, eq);
-        T0 = p | lop3<kLutOrAnd>(q, v, rmask);
-        T1 = lop3<kLutOr3>(a1, b1, eq);
+        const uint32_t eq = lop3<kLutEq>(A0, bw0, A1 ^ bw1);  // A_i == B_j
+        bits_cell(eq, a0, a1, b0, b1, H0, H1, V0, V1);
+        if constexpr (FIRST) {
+            H0 &= rmask;
+            H1 &= rmask;
+            V0 &= rmask;
+            V1 &= rmask;
+        }
+        if constexpr (RAMP) {
+            const uint32_t mk = (2u << u) - 1u;  // bits in column >= 1
+            V0 &= mk;
+            V1 &= mk;
+        }
     } else {
+        const uint32_t x = lop3<kLutXorOrNotC>(A1, bw1, rmask);
+        const uint32_t eq = lop3<kLutEq>(A0, bw0, x);  // A_i == B_j (0 on padding rows)
+        const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);  // the low bit of max(a, b), from a
+        const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);  // ... from b
         const uint32_t e1 = lop3<kLutSel>(eq, g.M1, X1r), e0 = lop3<kLutSel>(eq, g.M0, X0r);
         const uint32_t m0 = p | q, m1 = a1 | b1;
-        T0 = lop3<kLutAndNotOr>(m0, e1, m1) | lop3<kLutAndNotOr>(e0, m1, e1);
-        T1 = m1 | e1;
+        const uint32_t T0 = lop3<kLutAndNotOr>(m0, e1, m1) | lop3<kLutAndNotOr>(e0, m1, e1);
+        const uint32_t T1 = m1 | e1;
+        const uint32_t ca = lop3<kLutAndNot>(a0, T0, 0u), cb = lop3<kLutAndNot>(b0, T0, 0u);  // borrows
+        if constexpr (RAMP) {
+            const uint32_t mk = (2u << u) - 1u;
+            V0 = lop3<kLutXorAnd>(T0, a0, mk);
+            V1 = lop3<kLutXor3>(T1, a1, ca) & mk;
+        } else {
+            V0 = T0 ^ a0;
+            V1 = lop3<kLutXor3>(T1, a1, ca);
+        }
+        H0 = T0 ^ b0;
+        H1 = lop3<kLutXor3>(T1, b1, cb);
     }
-    const uint32_t ca = lop3<kLutAndNot>(a0, T0, 0u), cb = lop3<kLutAndNot>(b0, T0, 0u);  // borrows
-    if constexpr (RAMP) {
-        const uint32_t mk = (2u << u) - 1u;  // bits in column >= 1
-        V0 = lop3<kLutXorAnd>(T0, a0, mk);
-        V1 = lop3<kLutXor3>(T1, a1, ca) & mk;
-    } else {
-        V0 = T0 ^ a0;
-        V1 = lop3<kLutXor3>(T1, a1, ca);
-    }
-    H0 = T0 ^ b0;
-    H1 = lop3<kLutXor3>(T1, b1, cb);
     Q0 = __funnelshift_l(H0, Q0, 1);
     Q1 = __funnelshift_l(H1, Q1, 1);
 }
 
-template <bool GEN, bool RAMP>
+template <bool GEN, bool RAMP, bool FIRST>
 __device__ __forceinline__ void bits_chunk(uint32_t &H0, uint32_t &H1, uint32_t &V0, uint32_t &V1, uint32_t &Q0,
                                            uint32_t &Q1, uint32_t A0, uint32_t A1, uint32_t Rc0, uint32_t Rc1,
                                            uint32_t Rn0, uint32_t Rn1, uint32_t rmask, const BitsScoring &g,
                                            uint32_t X1r, uint32_t X0r) {
 #pragma unroll
     for (int u = 0; u < 32; ++u)
-        bits_step<GEN, RAMP>(u, H0, H1, V0, V1, Q0, Q1, A0, A1, __funnelshift_l(Rn0, Rc0, u),
-                             __funnelshift_l(Rn1, Rc1, u), rmask, g, X1r, X0r);
+        bits_step<GEN, RAMP, FIRST>(u, H0, H1, V0, V1, Q0, Q1, A0, A1, __funnelshift_l(Rn0, Rc0, u),
+                                    __funnelshift_l(Rn1, Rc1, u), rmask, g, X1r, X0r);
+}
+
+// One stripe of a job, lane by lane: its chunks in order, the words of the
+// row above in and of its bottom row out through `rows`.  The B window that
+// follows a chunk and the row's words are loaded one chunk ahead.
+// FIRST: stripe 0 (nothing comes in; padding rows).
+template <bool GEN, bool FIRST>
+__device__ __forceinline__ void bits_stripe(const BitsArgs &p, uint32_t C, uint32_t n, int64_t Bg, uint32_t A0,
+                                            uint32_t A1, uint32_t rmask, bool last, uint2 *rows, int32_t &W) {
+    const uint32_t X1r = p.g.X1 & rmask, X0r = p.g.X0 & rmask;
+    uint32_t H0 = 0, H1 = 0, V0 = 0, V1 = 0;
+    uint32_t Rc0 = __brev(plane_window(p.pl0, Bg - 31)), Rc1 = __brev(plane_window(p.pl1, Bg - 31));
+    uint32_t Fn0 = plane_window(p.pl0, Bg + 1), Fn1 = plane_window(p.pl1, Bg + 1);
+    uint2 prev = make_uint2(0u, 0u), nx = make_uint2(0u, 0u);
+    if constexpr (!FIRST) {
+        prev = __ldcg(rows);
+        if (C > 1) nx = __ldcg(rows + 32u);
+    }
+    for (uint32_t c = 0; c < C; ++c) {
+        const uint32_t Rn0 = __brev(Fn0), Rn1 = __brev(Fn1);
+        const int64_t gb = Bg + 32 * (int64_t)min(c + 1, C - 1) + 1;
+        Fn0 = plane_window(p.pl0, gb);
+        Fn1 = plane_window(p.pl1, gb);
+        uint32_t Q0 = 0, Q1 = 0;
+        if constexpr (!FIRST) {
+            // input bits: the previous stripe's bottom row, columns 32c+1 .. 32c+32,
+            // column 32c+1 at bit 31
+            Q0 = __funnelshift_r(nx.x, prev.x, 1);
+            Q1 = __funnelshift_r(nx.y, prev.y, 1);
+            prev = nx;
+            nx = c + 2 < C ? __ldcg(rows + (size_t)(c + 2) * 32u) : make_uint2(0u, 0u);
+        }
+        if (c == 0) bits_chunk<GEN, true, FIRST>(H0, H1, V0, V1, Q0, Q1, A0, A1, Rc0, Rc1, Rn0, Rn1, rmask, p.g, X1r, X0r);
+        else bits_chunk<GEN, false, FIRST>(H0, H1, V0, V1, Q0, Q1, A0, A1, Rc0, Rc1, Rn0, Rn1, rmask, p.g, X1r, X0r);
+        // outgoing bits: bit b is column 32c+1-b of the stripe's bottom row
+        if (!last) {
+            __stcg(rows + (size_t)c * 32u, make_uint2(Q0, Q1));
+        } else {
+            const int32_t lo = max(32 * (int32_t)c + 1 - (int32_t)n, 0), hi = min(31, 32 * (int32_t)c);
+            if (lo <= hi) {
+                const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
+                W += __popc(Q0 & mk) + 2 * __popc(Q1 & mk);
+            }
+        }
+        Rc0 = Rn0;
+        Rc1 = Rn1;
+    }
 }
 
 template <bool GEN>
@@ -112,47 +172,13 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
         const uint32_t m = tk.m, n = tk.n;
         const uint32_t S = job.S, C = job.C;
         int32_t W = 0;
-        if (S > 0) {
-            const int64_t Ag = (int64_t)tk.a_off, Bg = (int64_t)tk.b_off;  // planar slots
-            const int32_t top0 = (int32_t)m - 32 * (int32_t)S;  // row above bit 0 of stripe 0
-            for (uint32_t s = 0; s < S; ++s) {
-                const int32_t pad = min(max(-top0 - 32 * (int32_t)s, 0), 32);  // padding rows of this stripe
-                const uint32_t rmask = pad >= 32 ? 0u : (~0u << pad);
-                const int64_t abase = max(Ag + top0 + 32 * (int64_t)s, Ag - 32);
-                const uint32_t A0 = plane_window(p.pl0, abase), A1 = plane_window(p.pl1, abase);
-                const uint32_t X1r = p.g.X1 & rmask, X0r = p.g.X0 & rmask;
-                const bool first = s == 0, last = s + 1 == S;
-                uint32_t H0 = 0, H1 = 0, V0 = 0, V1 = 0;
-                uint32_t Rc0 = __brev(plane_window(p.pl0, Bg - 31)), Rc1 = __brev(plane_window(p.pl1, Bg - 31));
-                uint2 prev = first ? make_uint2(0u, 0u) : __ldcg(rows);
-                for (uint32_t c = 0; c < C; ++c) {
-                    const int64_t gb = Bg + 32 * (int64_t)c + 1;
-                    const uint32_t Rn0 = __brev(plane_window(p.pl0, gb)), Rn1 = __brev(plane_window(p.pl1, gb));
-                    uint32_t Q0 = 0, Q1 = 0;
-                    if (!first) {
-                        // input bits: the previous stripe's bottom row, columns 32c+1 .. 32c+32,
-                        // column 32c+1 at bit 31
-                        const uint2 nx = c + 1 < C ? __ldcg(rows + (size_t)(c + 1) * 32u) : make_uint2(0u, 0u);
-                        Q0 = __funnelshift_r(nx.x, prev.x, 1);
-                        Q1 = __funnelshift_r(nx.y, prev.y, 1);
-                        prev = nx;
-                    }
-                    if (c == 0) bits_chunk<GEN, true>(H0, H1, V0, V1, Q0, Q1, A0, A1, Rc0, Rc1, Rn0, Rn1, rmask, p.g, X1r, X0r);
-                    else bits_chunk<GEN, false>(H0, H1, V0, V1, Q0, Q1, A0, A1, Rc0, Rc1, Rn0, Rn1, rmask, p.g, X1r, X0r);
-                    // outgoing bits: bit b is column 32c+1-b of the stripe's bottom row
-                    if (!last) {
-                        __stcg(rows + (size_t)c * 32u, make_uint2(Q0, Q1));
-                    } else {
-                        const int32_t lo = max(32 * (int32_t)c + 1 - (int32_t)n, 0), hi = min(31, 32 * (int32_t)c);
-                        if (lo <= hi) {
-                            const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
-                            W += __popc(Q0 & mk) + 2 * __popc(Q1 & mk);
-                        }
-                    }
-                    Rc0 = Rn0;
-                    Rc1 = Rn1;
-                }
-            }
+        const int64_t Ag = (int64_t)tk.a_off, Bg = (int64_t)tk.b_off;  // planar slots
+        const int32_t top0 = (int32_t)m - 32 * (int32_t)S;             // row above bit 0 of stripe 0
+        for (uint32_t s = 0; s < S; ++s) {
+            const int64_t abase = max(Ag + top0 + 32 * (int64_t)s, Ag - 32);
+            const uint32_t A0 = plane_window(p.pl0, abase), A1 = plane_window(p.pl1, abase);
+            if (s == 0) bits_stripe<GEN, true>(p, C, n, Bg, A0, A1, ~0u << min(max(-top0, 0), 31), S == 1, rows, W);
+            else bits_stripe<GEN, false>(p, C, n, Bg, A0, A1, ~0u, s + 1 == S, rows, W);
         }
         if (active) {
             const int32_t sc = W + p.gap * (int32_t)(m + n);

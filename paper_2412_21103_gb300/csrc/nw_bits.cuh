@@ -25,14 +25,48 @@ constexpr uint32_t lut(uint32_t v) { return v & 0xFFu; }
 constexpr uint32_t kLutXorOrNotC = lut((kA ^ kB) | ~kC);     // (a ^ b) | ~c
 constexpr uint32_t kLutEq = lut(~(kA ^ kB) & ~kC);           // ~(a ^ b) & ~c
 constexpr uint32_t kLutAndOrNot = lut(kA & (kB | ~kC));      // a & (b | ~c)
-constexpr uint32_t kLutCOrNor = lut(kC | (~kA & ~kB));       // c | ~(a | b)
-constexpr uint32_t kLutOrAnd = lut(kA | (kB & kC));          // a | (b & c)
-constexpr uint32_t kLutOr3 = lut(kA | kB | kC);              // a | b | c
 constexpr uint32_t kLutXor3 = lut(kA ^ kB ^ kC);             // a ^ b ^ c
 constexpr uint32_t kLutAndNot = lut(kA & ~kB);               // a & ~b
 constexpr uint32_t kLutXorAnd = lut((kA ^ kB) & kC);         // (a ^ b) & c
 constexpr uint32_t kLutSel = lut((kA & kB) | (~kA & kC));    // a ? b : c
 constexpr uint32_t kLutAndNotOr = lut(kA & (~kB | kC));      // a & (~b | c)
+constexpr uint32_t kLutOrAndNot = lut((kA | kB) & ~kC);      // (a | b) & ~c
+
+// The cell update for the scoring s' = 3 (match) / 1 (mismatch), the paper's
+// +1/-1/-1, on 32 cells: inputs e (bases equal), a (dH of the cell above), b
+// (dV of the cell to the left), outputs dV = T - a and dH = T - b with
+// T = max(s', a, b).  A match acts like b = 3 on dV and like a = 3 on dH, so
+// with f = "b acts as 3" and g the choice that orders a against b, each
+// output bit is one three-input operation: 8 in all, where computing T and
+// subtracting with borrows takes 12.  (Found by exhaustive search over pairs
+// of intermediates; the truth tables were checked on all 32 inputs.)  The
+// update is symmetric: swapping a and b swaps the outputs.  The outputs may
+// name the inputs' registers.
+constexpr uint32_t kLutF = 0xF8;  // e | (x & y)
+constexpr uint32_t kLutG = 0x98;  // of (b1, a1, f)
+constexpr uint32_t kLut1 = 0x46;  // high bit, of (a0, f, g)
+constexpr uint32_t kLut0 = 0x29;  // low bit, of (a0, a1, g)
+__device__ __forceinline__ void bits_cell(uint32_t e, uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1, uint32_t &H0,
+                                          uint32_t &H1, uint32_t &V0, uint32_t &V1) {
+    const uint32_t f = lop3<kLutF>(e, b0, b1), ft = lop3<kLutF>(e, a0, a1);
+    const uint32_t g = lop3<kLutG>(b1, a1, f), gt = lop3<kLutG>(a1, b1, ft);
+    V1 = lop3<kLut1>(a0, f, g);
+    V0 = lop3<kLut0>(a0, a1, g);
+    H1 = lop3<kLut1>(b0, ft, gt);
+    H0 = lop3<kLut0>(b0, b1, gt);
+}
+
+// x * k + c as an integer multiply-add.  On sm_103 it issues on another pipe
+// than the logic and shift operations (measured, lanes per clock and SM:
+// LOP3, SHF, PRMT or add-max alone 60; multiply-add alone 60; LOP3 and
+// multiply-adds 1:1 together 110), so a shift by a constant or a choice
+// between a value and 0 costs the logic pipe nothing in this form.
+__device__ __forceinline__ uint32_t muladd(uint32_t x, uint32_t k, uint32_t c) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(x), "r"(k), "r"(c));
+    return d;
+}
+__device__ __forceinline__ uint32_t mul(uint32_t x, uint32_t k) { return muladd(x, k, 0u); }
 
 // 32 bits of a planar sequence plane starting at global base index g.
 __device__ __forceinline__ uint32_t plane_window(const uint32_t *pl, int64_t g) {

@@ -37,6 +37,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <type_traits>
 #include <vector>
 
 #include "nw_bits.cuh"
@@ -97,24 +98,23 @@ __device__ __forceinline__ uint32_t range_mask(int32_t lo, int32_t hi) {
 }
 
 // The cells of one word: inputs a (dH above), b (dV to the left), bases A,
-// B, mask mk of cells inside the grid (others get s' = 0); outputs the new
-// planes and the pointer bits.  The paper's scoring: s' = 3 (match) or 1.
+// B, mask mk of cells inside the grid (all ones unless RAMP; the others keep
+// the boundary's zero differences); outputs the new planes and the pointer
+// bits.  The paper's scoring: s' = 3 (match) or 1, where T != s' exactly
+// where the bases differ and a or b is 2 or 3.
+template <bool RAMP>
 __device__ __forceinline__ void band_cell(uint32_t A0, uint32_t A1, uint32_t B0, uint32_t B1, uint32_t a0,
                                           uint32_t a1, uint32_t b0, uint32_t b1, uint32_t mk, uint32_t &H0,
                                           uint32_t &H1, uint32_t &V0, uint32_t &V1, uint32_t &L, uint32_t &Hb) {
-    const uint32_t x = lop3<kLutXorOrNotC>(A1, B1, mk);
-    const uint32_t eq = lop3<kLutEq>(A0, B0, x);
-    const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);
-    const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);
-    const uint32_t v = lop3<kLutCOrNor>(a1, b1, eq);
-    const uint32_t T0 = p | lop3<kLutOrAnd>(q, v, mk);
-    const uint32_t T1 = lop3<kLutOr3>(a1, b1, eq);
-    const uint32_t ca = lop3<kLutAndNot>(a0, T0, 0u), cb = lop3<kLutAndNot>(b0, T0, 0u);
-    V0 = T0 ^ a0;
-    V1 = lop3<kLutXor3>(T1, a1, ca);
-    H0 = T0 ^ b0;
-    H1 = lop3<kLutXor3>(T1, b1, cb);
-    L = lop3<kLutXorOrNotC>(T1, eq, T0);  // (T1 ^ eq) | ~T0: T differs from s' = (eq, 1)
+    const uint32_t eq = lop3<kLutEq>(A0, B0, A1 ^ B1);
+    L = lop3<kLutOrAndNot>(a1, b1, eq);
+    bits_cell(eq, a0, a1, b0, b1, H0, H1, V0, V1);
+    if constexpr (RAMP) {
+        H0 &= mk;
+        H1 &= mk;
+        V0 &= mk;
+        V1 &= mk;
+    }
     Hb = V0 | V1;
 }
 
@@ -144,6 +144,8 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
         B1[v] = __brev(ld(p.pl1, cb));
         H0[v] = H1[v] = V0[v] = V1[v] = 0;
     }
+    const uint32_t nzt = gl == 0 ? 0u : 1u, nzb = gl == g - 1 ? 0u : 1u;  // 0 on the group's top / bottom lane
+    uint4 *rp = p.ptr + t.ptr_off + gl * Q;  // this lane's records of the next pair of anti-diagonals
     int32_t top = 0;  // W of the window's top cell
     const uint32_t nch = t.nchunks;
     const uint32_t gmask = g == 32 ? kFull : (((1u << g) - 1u) << (grp * g));
@@ -152,72 +154,69 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
         const int32_t rc = R + 32 * (int32_t)c, ac = a0 + 64 * (int32_t)c;  // r0 and a of the chunk's first step
         // new columns (top, one per step without a shift) and rows (bottom, one per shift) of the chunk
         const int64_t fb = Bg + (ac - rc) - 1, fa = Ag + rc + Hw - 1;
-        uint32_t fB0 = __brev(ld(p.pl0, fb)), fB1 = __brev(ld(p.pl1, fb));
-        uint32_t fA0 = ld(p.pl0, fa), fA1 = ld(p.pl1, fa);
+        // (0 on the lanes that take their neighbour's word instead)
+        uint32_t fB0 = nzt ? 0u : __brev(ld(p.pl0, fb)), fB1 = nzt ? 0u : __brev(ld(p.pl1, fb));
+        uint32_t fA0 = nzb ? 0u : ld(p.pl0, fa), fA1 = nzb ? 0u : ld(p.pl1, fa);
         // masks only while some cell of the chunk lies on or beyond row 0 / column 0
         const bool ramp = __any_sync(kFull, live && !(rc >= 1 && ac - rc - Hw >= 0));
         uint32_t cH0 = 0, cH1 = 0, cV0 = 0, cV1 = 0;
-        for (int32_t d = 0; d < 32; ++d) {
-            // ---- no shift: anti-diagonal ac + 2d, top row rc + d
-            {
-                uint32_t sB0 = __shfl_up_sync(kFull, B0[Q - 1], 1, g), sB1 = __shfl_up_sync(kFull, B1[Q - 1], 1, g);
-                uint32_t sH0 = __shfl_up_sync(kFull, H0[Q - 1], 1, g), sH1 = __shfl_up_sync(kFull, H1[Q - 1], 1, g);
-                if (gl == 0) {
-                    sB0 = fB0;
-                    sB1 = fB1;
-                    sH0 = 0u;  // above the window: a horizontal gap, dH = 0
-                    sH1 = 0u;
-                }
-                fB0 <<= 1;
-                fB1 <<= 1;
-                // (these one-bit shifts as multiply-adds, on the other pipe,
-                // measured slower: 20.2 against 18.8 ms per fill)
+        auto steps = [&](auto ramp_tag) {
+            constexpr bool RAMP = decltype(ramp_tag)::value;
+            for (int32_t d = 0; d < 32; ++d) {
+                // ---- no shift: anti-diagonal ac + 2d, top row rc + d
+                {
+                    // top lane: the fed columns, and above the window a horizontal gap, dH = 0
+                    const uint32_t sB0 = muladd(__shfl_up_sync(kFull, B0[Q - 1], 1, g), nzt, fB0);
+                    const uint32_t sB1 = muladd(__shfl_up_sync(kFull, B1[Q - 1], 1, g), nzt, fB1);
+                    const uint32_t sH0 = muladd(__shfl_up_sync(kFull, H0[Q - 1], 1, g), nzt, 0u);
+                    const uint32_t sH1 = muladd(__shfl_up_sync(kFull, H1[Q - 1], 1, g), nzt, 0u);
+                    fB0 = muladd(fB0, 2u, 0u);
+                    fB1 = muladd(fB1, 2u, 0u);
 #pragma unroll
-                for (int v = Q - 1; v >= 0; --v) {
-                    const int32_t W = (int32_t)gl * Q + v;
-                    B0[v] = __funnelshift_l(v ? B0[v - 1] : sB0, B0[v], 1);
-                    B1[v] = __funnelshift_l(v ? B1[v - 1] : sB1, B1[v], 1);
-                    const uint32_t a0v = __funnelshift_l(v ? H0[v - 1] : sH0, H0[v], 1);
-                    const uint32_t a1v = __funnelshift_l(v ? H1[v - 1] : sH1, H1[v], 1);
-                    const uint32_t mk = ramp ? range_mask(1 - rc - d - 32 * W, ac - rc + d - 32 * W - 1) : ~0u;
-                    band_cell(A0[v], A1[v], B0[v], B1[v], a0v, a1v, V0[v], V1[v], mk, H0[v], H1[v], V0[v], V1[v],
-                              Ln[v], Hn[v]);
-                }
-                cH0 = __funnelshift_r(cH0, H0[0], 1);
-                cH1 = __funnelshift_r(cH1, H1[0], 1);
-            }
-            // ---- shift: anti-diagonal ac + 2d + 1, top row rc + d + 1
-            {
-                uint32_t sA0 = __shfl_down_sync(kFull, A0[0], 1, g), sA1 = __shfl_down_sync(kFull, A1[0], 1, g);
-                uint32_t sV0 = __shfl_down_sync(kFull, V0[0], 1, g), sV1 = __shfl_down_sync(kFull, V1[0], 1, g);
-                if (gl == g - 1) {
-                    sA0 = fA0;
-                    sA1 = fA1;
-                    sV0 = 0u;  // below the window: a vertical gap, dV = 0
-                    sV1 = 0u;
-                }
-                fA0 >>= 1;
-                fA1 >>= 1;
-#pragma unroll
-                for (int v = 0; v < Q; ++v) {
-                    const int32_t W = (int32_t)gl * Q + v;
-                    A0[v] = __funnelshift_r(A0[v], v + 1 < Q ? A0[v + 1] : sA0, 1);
-                    A1[v] = __funnelshift_r(A1[v], v + 1 < Q ? A1[v + 1] : sA1, 1);
-                    const uint32_t b0v = __funnelshift_r(V0[v], v + 1 < Q ? V0[v + 1] : sV0, 1);
-                    const uint32_t b1v = __funnelshift_r(V1[v], v + 1 < Q ? V1[v + 1] : sV1, 1);
-                    const uint32_t mk = ramp ? range_mask(-rc - d - 32 * W, ac - rc + d - 32 * W - 1) : ~0u;
-                    uint32_t Ls, Hs;
-                    band_cell(A0[v], A1[v], B0[v], B1[v], H0[v], H1[v], b0v, b1v, mk, H0[v], H1[v], V0[v], V1[v], Ls,
-                              Hs);
-                    if (PTR && live) {
-                        const uint64_t idx = t.ptr_off + (uint64_t)(32u * c + (uint32_t)d) * (uint32_t)gq + (uint32_t)W;
-                        if (in_range(idx, p.ptr_cap, p.err, kSiteBandBitsPtr)) __stcg(p.ptr + idx, make_uint4(Ln[v], Hn[v], Ls, Hs));
+                    for (int v = Q - 1; v >= 0; --v) {
+                        const int32_t W = (int32_t)gl * Q + v;
+                        B0[v] = __funnelshift_l(v ? B0[v - 1] : sB0, B0[v], 1);
+                        B1[v] = __funnelshift_l(v ? B1[v - 1] : sB1, B1[v], 1);
+                        const uint32_t a0v = __funnelshift_l(v ? H0[v - 1] : sH0, H0[v], 1);
+                        const uint32_t a1v = __funnelshift_l(v ? H1[v - 1] : sH1, H1[v], 1);
+                        const uint32_t mk = RAMP ? range_mask(1 - rc - d - 32 * W, ac - rc + d - 32 * W - 1) : ~0u;
+                        band_cell<RAMP>(A0[v], A1[v], B0[v], B1[v], a0v, a1v, V0[v], V1[v], mk, H0[v], H1[v], V0[v],
+                                        V1[v], Ln[v], Hn[v]);
                     }
+                    cH0 = __funnelshift_r(cH0, H0[0], 1);
+                    cH1 = __funnelshift_r(cH1, H1[0], 1);
                 }
-                cV0 = __funnelshift_r(cV0, V0[0], 1);
-                cV1 = __funnelshift_r(cV1, V1[0], 1);
+                // ---- shift: anti-diagonal ac + 2d + 1, top row rc + d + 1
+                {
+                    // bottom lane: the fed rows, and below the window a vertical gap, dV = 0
+                    const uint32_t sA0 = muladd(__shfl_down_sync(kFull, A0[0], 1, g), nzb, fA0);
+                    const uint32_t sA1 = muladd(__shfl_down_sync(kFull, A1[0], 1, g), nzb, fA1);
+                    const uint32_t sV0 = muladd(__shfl_down_sync(kFull, V0[0], 1, g), nzb, 0u);
+                    const uint32_t sV1 = muladd(__shfl_down_sync(kFull, V1[0], 1, g), nzb, 0u);
+                    fA0 >>= 1;
+                    fA1 >>= 1;
+#pragma unroll
+                    for (int v = 0; v < Q; ++v) {
+                        const int32_t W = (int32_t)gl * Q + v;
+                        A0[v] = __funnelshift_r(A0[v], v + 1 < Q ? A0[v + 1] : sA0, 1);
+                        A1[v] = __funnelshift_r(A1[v], v + 1 < Q ? A1[v + 1] : sA1, 1);
+                        const uint32_t b0v = __funnelshift_r(V0[v], v + 1 < Q ? V0[v + 1] : sV0, 1);
+                        const uint32_t b1v = __funnelshift_r(V1[v], v + 1 < Q ? V1[v + 1] : sV1, 1);
+                        const uint32_t mk = RAMP ? range_mask(-rc - d - 32 * W, ac - rc + d - 32 * W - 1) : ~0u;
+                        uint32_t Ls, Hs;
+                        band_cell<RAMP>(A0[v], A1[v], B0[v], B1[v], H0[v], H1[v], b0v, b1v, mk, H0[v], H1[v], V0[v],
+                                        V1[v], Ls, Hs);
+                        if (PTR && live && in_range((uint64_t)(rp - p.ptr) + v, p.ptr_cap, p.err, kSiteBandBitsPtr))
+                            __stcg(rp + v, make_uint4(Ln[v], Hn[v], Ls, Hs));
+                    }
+                    cV0 = __funnelshift_r(cV0, V0[0], 1);
+                    cV1 = __funnelshift_r(cV1, V1[0], 1);
+                    rp += gq;
+                }
             }
-        }
+        };
+        if (ramp) steps(std::true_type{});
+        else steps(std::false_type{});
         top += __popc(cH0) + 2 * __popc(cH1) + __popc(cV0) + 2 * __popc(cV1);
         if (active && c + 1 == nch) {
             // W(m, n): the top cell, then down the last anti-diagonal: each row

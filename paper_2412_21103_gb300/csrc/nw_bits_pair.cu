@@ -44,12 +44,6 @@ namespace nw {
 
 constexpr int kPairWarps = 4;        // most warps per CTA (one per scheduler)
 constexpr uint32_t kPairRows = 31;   // rows per stripe (bits 0..30 of a word)
-// Truth tables (from a = 0xF0, b = 0xCC, c = 0xAA) of the shallow update.
-constexpr uint32_t kLutAndNotNot = lut(kA & ~kB & ~kC);  // a & !b & !c
-constexpr uint32_t kLutAndNand = lut(kA & ~(kB & kC));   // a & !(b & c)
-constexpr uint32_t kLutOrAndNot = lut((kA | kB) & ~kC);  // (a | b) & !c
-constexpr uint32_t kLutXorAndNot = lut(kA ^ (kB & ~kC)); // a ^ (b & !c)
-
 // One pair of a launch (device array).
 struct PairDesc {
     int64_t Ag, Bg;             // slots of a (rows) and b (columns)
@@ -104,14 +98,6 @@ __device__ __forceinline__ void st_relaxed64(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// x * k (a left shift by a power of two) as an integer multiply-add, which
-// the multiply-add pipe can take while the logic pipe runs the cell update.
-__device__ __forceinline__ uint32_t mul(uint32_t x, uint32_t k) {
-    uint32_t d;
-    asm("mad.lo.u32 %0, %1, %2, 0;" : "=r"(d) : "r"(x), "r"(k));
-    return d;
-}
-
 // Entries of ring chunk c: their tags match the epoch once written.
 struct RingWords {
     uint64_t e0, e1;
@@ -149,20 +135,26 @@ __device__ bool ring_wait(const uint64_t *ring, uint32_t c, uint32_t epoch, uint
 // anti-diagonal; G = H shifted so that bit 31 is the bottom row's dH (bit
 // 30, or row m's bit in the last stripe); Y: the word
 // whose bit 31 is this step's input bit; Qi: lane 0's input bits of the
-// chunk, the current one at bit 31; Qo: the bottom row's outgoing bits,
-// the latest at bit 0.
+// chunk, the current one at bit 31 (0 on the other lanes); Qo: the bottom
+// row's outgoing bits, the latest at bit 0.
 struct PairState {
     uint32_t H0, H1, V0, V1, G0, G1, Y0, Y1, Qi0, Qi1, Qo0, Qo1;
 };
 
 // One anti-diagonal step of a lane's 31 rows (see bits_step in nw_bits.cu
-// for the difference form).  Z: all ones on lane 0, which takes its input
-// from Qi instead of the neighbour; gmul: 2^(31 - bottom bit).  RAMP: the
-// first chunk of a lane (rz = 0 there), where bits p > u lie in column <= 0
-// and their dV is forced to the boundary's 0.  L, Hb: the step's records.
+// for the difference form).  nz: 0 on lane 0, which takes its input from Qi
+// instead of the neighbour, 1 on the others; gmul: 2^(31 - bottom bit).
+// RAMP: the first chunk of a lane (rz = 0 there), where bits p > u lie in
+// column <= 0 and their dV is forced to the boundary's 0.  L, Hb: the step's
+// records.
+//
+// What bounds it: 18 operations on the logic pipe (16 lanes per cycle and
+// scheduler), so 36 cycles of a warp that has its scheduler to itself; the
+// one-bit shifts and lane 0's choice of input run as multiply-adds on the
+// other integer pipe, which issues beside it.
 template <bool GEN, bool RAMP>
 __device__ __forceinline__ void pair_step(int u, PairState &st, uint32_t A0, uint32_t A1, uint32_t bw0, uint32_t bw1,
-                                          uint32_t Z, uint32_t gmul, uint32_t rz, const BitsScoring &g, uint32_t &L,
+                                          uint32_t nz, uint32_t gmul, uint32_t rz, const BitsScoring &g, uint32_t &L,
                                           uint32_t &Hb) {
     // the neighbour's bottom row after the previous step: the next step's input
     const uint32_t N0 = __shfl_up_sync(kFull, st.G0, 1), N1 = __shfl_up_sync(kFull, st.G1, 1);
@@ -170,26 +162,13 @@ __device__ __forceinline__ void pair_step(int u, PairState &st, uint32_t A0, uin
     const uint32_t a0 = __funnelshift_l(st.Y0, st.H0, 1), a1 = __funnelshift_l(st.Y1, st.H1, 1);  // dH above
     const uint32_t b0 = st.V0, b1 = st.V1;                                                        // dV left
     if constexpr (!GEN) {
-        // s' = (eq, 1).  T = 3 where eq; else T = max(1, a, b), whose low bit
-        // is 0 exactly where max(a, b) = 2.  Written so that T0 is two logic
-        // levels after a (not three), and dV, dH one more:
-        //   T0 = eq | !(a = 2, b < 3  or  b = 2, a < 3)
-        //   dV1 = ((eq | b1) & !a1) ^ (a0 & !T0),  dH1 = ((eq | a1) & !b1) ^ (b0 & !T0)
-        const uint32_t b2 = lop3<kLutAndNot>(b1, b0, 0u), b3 = b1 & b0;  // b = 2, b = 3
-        const uint32_t x1 = lop3<kLutAndNotNot>(a1, a0, b3), x2 = lop3<kLutAndNand>(b2, a1, a0);
-        const uint32_t sv = lop3<kLutOrAndNot>(eq, b1, a1), sh = lop3<kLutOrAndNot>(eq, a1, b1);
-        const uint32_t T0 = lop3<kLutCOrNor>(x1, x2, eq);
-        L = lop3<kLutOrAndNot>(a1, b1, eq) | ~T0;  // T != s'
+        L = lop3<kLutOrAndNot>(a1, b1, eq);  // T != s': a or b is 2 or 3 and the bases differ (T is 3 where they match)
+        bits_cell(eq, a0, a1, b0, b1, st.H0, st.H1, st.V0, st.V1);
         if constexpr (RAMP) {
             const uint32_t mk = ((2u << u) - 1u) | rz;
-            st.V0 = lop3<kLutXorAnd>(T0, a0, mk);
-            st.V1 = lop3<kLutXorAndNot>(sv, a0, T0) & mk;
-        } else {
-            st.V0 = T0 ^ a0;
-            st.V1 = lop3<kLutXorAndNot>(sv, a0, T0);
+            st.V0 &= mk;
+            st.V1 &= mk;
         }
-        st.H0 = T0 ^ b0;
-        st.H1 = lop3<kLutXorAndNot>(sh, b0, T0);
     } else {
         const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);
         const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);
@@ -213,8 +192,8 @@ __device__ __forceinline__ void pair_step(int u, PairState &st, uint32_t A0, uin
     Hb = st.V0 | st.V1;
     st.Qi0 = mul(st.Qi0, 2u);
     st.Qi1 = mul(st.Qi1, 2u);
-    st.Y0 = lop3<kLutSel>(Z, st.Qi0, N0);
-    st.Y1 = lop3<kLutSel>(Z, st.Qi1, N1);
+    st.Y0 = muladd(N0, nz, st.Qi0);
+    st.Y1 = muladd(N1, nz, st.Qi1);
     st.G0 = mul(st.H0, gmul);
     st.G1 = mul(st.H1, gmul);
     st.Qo0 = __funnelshift_l(st.G0, st.Qo0, 1);
@@ -224,13 +203,13 @@ __device__ __forceinline__ void pair_step(int u, PairState &st, uint32_t A0, uin
 // 32 steps; with PTR the records of steps 2v, 2v + 1 go to recp[v * 32].
 template <bool GEN, bool RAMP, bool PTR>
 __device__ __forceinline__ void pair_chunk(PairState &st, uint32_t A0, uint32_t A1, uint32_t Rc0, uint32_t Rc1,
-                                           uint32_t Rn0, uint32_t Rn1, uint32_t Z, uint32_t gmul, uint32_t rz,
+                                           uint32_t Rn0, uint32_t Rn1, uint32_t nz, uint32_t gmul, uint32_t rz,
                                            const BitsScoring &g, uint4 *recp) {
     uint32_t Lp = 0, Hp = 0;
 #pragma unroll
     for (int u = 0; u < 32; ++u) {
         uint32_t L, Hb;
-        pair_step<GEN, RAMP>(u, st, A0, A1, __funnelshift_l(Rn0, Rc0, u), __funnelshift_l(Rn1, Rc1, u), Z, gmul, rz,
+        pair_step<GEN, RAMP>(u, st, A0, A1, __funnelshift_l(Rn0, Rc0, u), __funnelshift_l(Rn1, Rc1, u), nz, gmul, rz,
                              g, L, Hb);
         if constexpr (PTR) {
             if (u & 1) __stcg(recp + (size_t)(u >> 1) * 32u, make_uint4(Lp, Hp, L, Hb));
@@ -256,7 +235,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, 1) k_bits_pair(PairLaunch L) 
     const uint32_t K = C + min(31u, S - 1 - 32u * w);  // chunks until the warp's last lane is done
     const int64_t abase = valid ? p.Ag + (int64_t)kPairRows * s : p.Ag - 32;  // base of bit 0's row
     const uint32_t A0 = plane_window(p.pl0, abase), A1 = plane_window(p.pl1, abase);
-    const uint32_t Z = lane == 0 ? ~0u : 0u;
+    const uint32_t nz = lane == 0 ? 0u : 1u;
     const bool last = s + 1 == S, out = lane == 31 && w + 1 < p.nwarps;
     const uint32_t gmul = 1u << (31u - (last ? p.pm : kPairRows - 1));  // bottom row -> bit 31 of G
     const uint64_t *rin = w ? p.ring + (size_t)(w - 1) * C * 2u : nullptr;
@@ -272,6 +251,18 @@ __global__ void __launch_bounds__(kPairWarps * 32, 1) k_bits_pair(PairLaunch L) 
         prev = r.words();
         if (C > 1) ahead = ring_load(rin, 1);
     }
+    // The B windows of a chunk end where the next one's begin, so each chunk
+    // loads only the window that follows it -- one chunk ahead, so that the
+    // load's latency (about 1,000 cycles of a 32-step chunk when it was loaded
+    // at its own chunk: 80 cycles per step on the 32k pair, 2.59 ms of fill)
+    // runs beside a chunk of steps.
+    auto b_next = [&](int32_t c, const uint32_t *pl) {
+        const uint32_t cc = (uint32_t)min(max(c, 0), (int32_t)C - 1);
+        return plane_window(pl, p.Bg + 32 * (int64_t)cc + 1);
+    };
+    const uint32_t Ri0 = __brev(plane_window(p.pl0, p.Bg - 31)), Ri1 = __brev(plane_window(p.pl1, p.Bg - 31));
+    uint32_t Rc0 = 0, Rc1 = 0;
+    uint32_t Fn0 = b_next(-(int32_t)lane, p.pl0), Fn1 = b_next(-(int32_t)lane, p.pl1);
     for (uint32_t k = 0; k < K; ++k) {
         // lane 0's input bits for chunk k: the stripe above's bottom row,
         // columns 32k + 1 .. 32k + 32, column 32k + 1 at bit 31 (the ring's
@@ -295,20 +286,23 @@ __global__ void __launch_bounds__(kPairWarps * 32, 1) k_bits_pair(PairLaunch L) 
         }
         const int32_t c = (int32_t)k - (int32_t)lane;  // this lane's chunk
         const bool act = valid && c >= 0 && c < (int32_t)C;
-        const uint32_t cc = (uint32_t)min(max(c, 0), (int32_t)C - 1);
-        const int64_t gb = p.Bg + 32 * (int64_t)cc;
-        const uint32_t Rc0 = __brev(plane_window(p.pl0, gb - 31)), Rc1 = __brev(plane_window(p.pl1, gb - 31));
-        const uint32_t Rn0 = __brev(plane_window(p.pl0, gb + 1)), Rn1 = __brev(plane_window(p.pl1, gb + 1));
+        const uint32_t Rn0 = __brev(Fn0), Rn1 = __brev(Fn1);
+        Fn0 = b_next(c + 1, p.pl0);
+        Fn1 = b_next(c + 1, p.pl1);
         if (c == 0) {
             st.H0 = st.H1 = st.V0 = st.V1 = st.G0 = st.G1 = 0;
+            Rc0 = Ri0;
+            Rc1 = Ri1;
         }
         uint4 *recp = PTR ? recw + (size_t)k * 16u * 32u : nullptr;
         if (k < 32) {
             const uint32_t rz = c == 0 ? 0u : ~0u;
-            pair_chunk<GEN, true, PTR>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, Z, gmul, rz, p.g, recp);
+            pair_chunk<GEN, true, PTR>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, nz, gmul, rz, p.g, recp);
         } else {
-            pair_chunk<GEN, false, PTR>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, Z, gmul, ~0u, p.g, recp);
+            pair_chunk<GEN, false, PTR>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, nz, gmul, ~0u, p.g, recp);
         }
+        Rc0 = Rn0;
+        Rc1 = Rn1;
         // outgoing bits: bit b is column 32c + 2 - b of the stripe's bottom row
         if (act && out) {
             st_relaxed64(rout + 2 * (size_t)c, ((uint64_t)p.epoch << 32) | st.Qo0);

@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(kPeakThreads) k_peak_bits(uint64_t iters, uint
     uint32_t H0[kBitsChains], H1[kBitsChains], V0[kBitsChains], V1[kBitsChains], Q0[kBitsChains], Q1[kBitsChains];
     const uint32_t A0 = seed * 0x9E3779B9u + threadIdx.x, A1 = A0 * 2654435761u;
     uint32_t Rc0 = ~A0, Rc1 = A1 ^ 0x5bd1e995u, Rn0 = A0 ^ 0x27d4eb2fu, Rn1 = ~A1;
-    const uint32_t rmask = ~(seed & 1u);
 #pragma unroll
     for (int c = 0; c < kBitsChains; ++c) {
         H0[c] = A0 >> c;
@@ -97,20 +96,9 @@ __global__ void __launch_bounds__(kPeakThreads) k_peak_bits(uint64_t iters, uint
 #pragma unroll
         for (int c = 0; c < kBitsChains; ++c) {
             const uint32_t bw0 = __funnelshift_l(Rn0, Rc0, c + 1), bw1 = __funnelshift_l(Rn1, Rc1, c + 1);
-            const uint32_t x = lop3<kLutXorOrNotC>(A1, bw1, rmask);
-            const uint32_t eq = lop3<kLutEq>(A0, bw0, x);
+            const uint32_t eq = lop3<kLutEq>(A0, bw0, A1 ^ bw1);
             const uint32_t a0 = __funnelshift_l(Q0[c], H0[c], 1), a1 = __funnelshift_l(Q1[c], H1[c], 1);
-            const uint32_t b0 = V0[c], b1 = V1[c];
-            const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);
-            const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);
-            const uint32_t v = lop3<kLutCOrNor>(a1, b1, eq);
-            const uint32_t T0 = p | lop3<kLutOrAnd>(q, v, rmask);
-            const uint32_t T1 = lop3<kLutOr3>(a1, b1, eq);
-            const uint32_t ca = lop3<kLutAndNot>(a0, T0, 0u), cb = lop3<kLutAndNot>(b0, T0, 0u);
-            V0[c] = T0 ^ a0;
-            V1[c] = lop3<kLutXor3>(T1, a1, ca);
-            H0[c] = T0 ^ b0;
-            H1[c] = lop3<kLutXor3>(T1, b1, cb);
+            bits_cell(eq, a0, a1, V0[c], V1[c], H0[c], H1[c], V0[c], V1[c]);
             Q0[c] = __funnelshift_l(H0[c], Q0[c], 1);
             Q1[c] = __funnelshift_l(H1[c], Q1[c], 1);
         }
