@@ -475,13 +475,13 @@ static int bits_round(nw_ctx *ctx, const uint8_t *pool, const PlaneSet &planes, 
         size_t k = k0;
         for (; k < items.size(); ++k) {
             BandBitsItem it = items[k];
-            const uint64_t r = band_bits_records(it.shape);
+            const uint64_t r = band_bits_kept(it.shape);
             if (want) {
                 if (!wave.empty() && (recs + r) * 16 > wave_budget) break;
                 it.ptr_off = recs;
                 recs += r;
             }
-            ctx->band_stats[6] += r * 64u;  // cells: 2 anti-diagonals x 32 rows per record
+            ctx->band_stats[6] += band_bits_cells(it.shape);
             wave.push_back(it);
             ww.push_back(iw[k]);
         }
@@ -513,7 +513,7 @@ static int bits_round(nw_ctx *ctx, const uint8_t *pool, const PlaneSet &planes, 
             }
             cert.push_back((uint32_t)q);
         }
-        if (want && (rc = band_bits_walk(ctx, pv, wave, cert, pool, cigar_pool, cigar_off, cigar_len,
+        if (want && (rc = band_bits_walk(ctx, planes, pv, wave, cert, pool, cigar_pool, cigar_off, cigar_len,
                                          (flags & NW_CIGAR_M) ? 1u : 0u)))
             return rc;
         k0 = k;

@@ -196,10 +196,10 @@ struct BandBitsShape {
     uint32_t words = 1;  // the band needs this many 32-row words (g * Q >= words)
 };
 // One banded pair of a round: pool offsets, sizes, score slot, window, and
-// its first pointer record (16 bytes per word and pair of anti-diagonals).
+// its first kept planes (16 bytes per word, every 192 anti-diagonals).
 struct BandBitsItem {
-    uint64_t a_off, b_off, ptr_off;  // pool byte offsets (the walk), first pointer record
-    int64_t a_slot, b_slot;          // the sequences' planar slots (the fill)
+    uint64_t a_off, b_off, ptr_off;  // pool byte offsets (the CIGARs), first kept planes
+    int64_t a_slot, b_slot;          // the sequences' planar slots (the fill and the walk)
     uint32_t m, n, out0;
     BandBitsShape shape;
 };
@@ -213,17 +213,18 @@ bool band_bits_shape(uint32_t m, uint32_t n, int32_t lo, int32_t hi, BandBitsSha
 // The same window spread over as many lanes as it has words (up to 32):
 // fewer instructions per lane and step, so a shorter time for the pair.
 void band_bits_fast(BandBitsShape *s);
-uint64_t band_bits_records(const BandBitsShape &s);  // pointer records of the pair
+uint64_t band_bits_cells(const BandBitsShape &s);  // cells of the pair's window, over all its chunks
+uint64_t band_bits_kept(const BandBitsShape &s);   // its kept planes (16-byte units)
 // The widest half-width whose band fits the window of an m x n pair.
 uint32_t band_bits_max_width(uint32_t m, uint32_t n);
 double band_bits_seconds(const BandBitsShape &s);    // estimated time of the pair on one warp
 // Fills the items (the paper's scoring: s' = 3 on a match, 1 on a
 // mismatch), writes scores[out0], returns the banded scores in item order,
-// and with `want` the pointer records at ptr + ptr_off.
+// and with `want` the kept planes at ptr + ptr_off (`kept` units in all).
 int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBitsItem> &items, bool want, int32_t gap, int32_t *scores, uint32_t score_cap,
-                   void *ptr, uint64_t ptr_records, std::vector<int32_t> &banded);
+                   void *ptr, uint64_t kept, std::vector<int32_t> &banded);
 // Walks the items `which` of a filled wave and writes their CIGARs.
-int band_bits_walk(nw_ctx *ctx, const void *ptr, const std::vector<BandBitsItem> &items,
+int band_bits_walk(nw_ctx *ctx, const PlaneSet &planes, const void *ptr, const std::vector<BandBitsItem> &items,
                    const std::vector<uint32_t> &which, const uint8_t *pool, char *cigar_pool,
                    const uint64_t *cigar_off, uint64_t *cigar_len, uint32_t mflag);
 

@@ -29,11 +29,20 @@
 //
 // The score is tracked at the window's top cell (its dH on a step without a
 // shift, its dV on a shift) and carried down the last anti-diagonal to
-// (m, n).  Pointer bits, per cell: L = T != s' (the diagonal loses), and
-// Hb = dV != 0 (the vertical move loses); the walk reads !L -> diagonal,
-// else !Hb -> vertical, else horizontal, the diagonal > vertical > horizontal
-// order of the scalar kernels.  One 16-byte record per word and pair of
-// anti-diagonals: (L, Hb) of the first, (L, Hb) of the second.
+// (m, n).
+//
+// Alignments.  The fill writes no pointers: every kBlockChunks chunks (192
+// anti-diagonals) it keeps the window's four planes (16 bytes per word).  The
+// walk then goes back block by block: it recomputes the pointer bits of the
+// block it stands in from the planes kept at its start -- only the 256 rows
+// around the path, because a cell of an anti-diagonal depends on the row
+// itself and its two neighbours one anti-diagonal pair earlier, so nothing
+// further than 96 rows away reaches the path within 192 anti-diagonals -- into
+// shared memory and follows the path through them.  Pointer bits, per cell:
+// L = T != s' (the diagonal loses), and Hb = dV != 0 (the vertical move
+// loses); the walk reads !L -> diagonal, else !Hb -> vertical, else
+// horizontal, the diagonal > vertical > horizontal order of the scalar
+// kernels.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -51,14 +60,20 @@ namespace nw {
 // 1.5x slower on the band workload: 27.3 against 18.0 ms per fill.
 constexpr int kBandBitsMaxQ = 4;
 constexpr int kBandBitsMaxWords = 32 * kBandBitsMaxQ;
-constexpr int kWalkWarps = 4;
+// Anti-diagonals between kept planes: kBlockChunks chunks of 64; the walk's
+// sub-window of kSubWords words covers the rows a block's path can depend on.
+constexpr int kBlockChunks = 2;
+constexpr int kSubWords = 8;
+constexpr int kSubPairs = 32 / kSubWords;                // pairs per warp of the walk
+constexpr int kBlockSteps = 32 * kBlockChunks;           // pairs of anti-diagonals per block
+static_assert(kSubWords * 32 >= 2 * (kBlockSteps + 1) + 16 + 32, "the sub-window must hold a block's dependencies");
 // Warps per CTA of the fill: at ~150 registers an SM holds 13 warps, so
 // CTAs of 4 warps fit 12 of them (CTAs of 8 only 8).
 constexpr int kBandWarps = 4;
 
 struct BandBitsTask {
     int64_t a_slot, b_slot; // planar slots of A (rows) and B (columns)
-    uint64_t ptr_off;       // first pointer record of the pair (16-byte units)
+    uint64_t ptr_off;       // first kept planes of the pair (16-byte units)
     uint32_t m, n;
     int32_t hi;             // window anchor: the band's upper diagonal, raised to the parity of m+n
     int32_t a_first;        // first anti-diagonal (a step without a shift), <= 0
@@ -79,8 +94,8 @@ struct BandBitsArgs {
     const BandBitsJob *jobs;
     uint32_t njobs;
     uint32_t *counter;
-    uint4 *ptr;
-    uint64_t ptr_cap;   // records at ptr (checked build)
+    uint4 *ptr;         // kept planes (H0, H1, V0, V1), per pair [block][word]
+    uint64_t ptr_cap;   // 16-byte units at ptr (checked build)
     int32_t *scores;
     int32_t *gathered;  // per task, in task order
     uint32_t score_cap;
@@ -99,15 +114,15 @@ __device__ __forceinline__ uint32_t range_mask(int32_t lo, int32_t hi) {
 
 // The cells of one word: inputs a (dH above), b (dV to the left), bases A,
 // B, mask mk of cells inside the grid (all ones unless RAMP; the others keep
-// the boundary's zero differences); outputs the new planes and the pointer
-// bits.  The paper's scoring: s' = 3 (match) or 1, where T != s' exactly
-// where the bases differ and a or b is 2 or 3.
-template <bool RAMP>
+// the boundary's zero differences); outputs the new planes and, with PTR, the
+// pointer bits.  The paper's scoring: s' = 3 (match) or 1, where T != s'
+// exactly where the bases differ and a or b is 2 or 3.
+template <bool RAMP, bool PTR>
 __device__ __forceinline__ void band_cell(uint32_t A0, uint32_t A1, uint32_t B0, uint32_t B1, uint32_t a0,
                                           uint32_t a1, uint32_t b0, uint32_t b1, uint32_t mk, uint32_t &H0,
                                           uint32_t &H1, uint32_t &V0, uint32_t &V1, uint32_t &L, uint32_t &Hb) {
     const uint32_t eq = lop3<kLutEq>(A0, B0, A1 ^ B1);
-    L = lop3<kLutOrAndNot>(a1, b1, eq);
+    if constexpr (PTR) L = lop3<kLutOrAndNot>(a1, b1, eq);
     bits_cell(eq, a0, a1, b0, b1, H0, H1, V0, V1);
     if constexpr (RAMP) {
         H0 &= mk;
@@ -115,105 +130,163 @@ __device__ __forceinline__ void band_cell(uint32_t A0, uint32_t A1, uint32_t B0,
         V0 &= mk;
         V1 &= mk;
     }
-    Hb = V0 | V1;
+    if constexpr (PTR) Hb = V0 | V1;
 }
 
-template <int Q, bool PTR>
+// A lane's Q words of the window: bases and difference planes.
+template <int Q>
+struct BandWords {
+    uint32_t A0[Q], A1[Q], B0[Q], B1[Q], H0[Q], H1[Q], V0[Q], V1[Q];
+};
+
+// The planar bases as the window reads them (clamped: bases outside belong to no cell that matters).
+struct BandBases {
+    const uint32_t *pl0, *pl1;
+    int64_t max_base, Ag, Bg;
+    __device__ uint32_t at(const uint32_t *pl, int64_t g) const {
+        return plane_window(pl, min(max(g, -kPlanePad), max_base));
+    }
+};
+
+// The bases of a lane's words before anti-diagonal ac, where the word W of
+// the lane's first word starts at row r (bit 0).
+template <int Q>
+__device__ __forceinline__ void band_bases(BandWords<Q> &w, const BandBases &bs, int32_t r, int32_t ac) {
+#pragma unroll
+    for (int v = 0; v < Q; ++v) {
+        const int64_t ra = bs.Ag + r + 32 * v - 1;                  // A index of the row of bit 0
+        w.A0[v] = bs.at(bs.pl0, ra);
+        w.A1[v] = bs.at(bs.pl1, ra);
+        const int64_t cb = bs.Bg + (ac - 1 - r - 32 * v - 31) - 1;  // B index of the column of bit 31
+        w.B0[v] = __brev(bs.at(bs.pl0, cb));
+        w.B1[v] = __brev(bs.at(bs.pl1, cb));
+    }
+}
+
+// The bases that enter a window during a chunk of 64 anti-diagonals: columns
+// at its top lane, rows at its bottom lane (0 on the other lanes, which take
+// their neighbour's bits).
+struct BandFeeds {
+    uint32_t B0, B1, A0, A1;
+    __device__ BandFeeds(const BandBases &bs, int32_t rc, int32_t ac, int32_t Hw, uint32_t nzt, uint32_t nzb) {
+        const int64_t fb = bs.Bg + (ac - rc) - 1, fa = bs.Ag + rc + Hw - 1;
+        B0 = nzt ? 0u : __brev(bs.at(bs.pl0, fb));
+        B1 = nzt ? 0u : __brev(bs.at(bs.pl1, fb));
+        A0 = nzb ? 0u : bs.at(bs.pl0, fa);
+        A1 = nzb ? 0u : bs.at(bs.pl1, fa);
+    }
+};
+
+// A pair of anti-diagonals of a window spread over groups of g lanes.  The
+// first has the lane's first word at row r (bit 0) and columns 1 .. at bits
+// below cmax; nzt, nzb: 0 on the group's top / bottom lane, else 1.  top()
+// runs after the first with the lane's first H word, after the second with
+// its first V word (the score's path); rec(v, L, Hb, L', Hb') takes the pointer bits.
+//
+// What bounds it: the logic pipe, 14 operations per word and anti-diagonal
+// (16 with pointers), the feeds and the choice at the group's ends being
+// multiply-adds, which issue beside it.
+template <int Q, bool RAMP, bool PTR, class Top, class Rec>
+__device__ __forceinline__ void band_two(BandWords<Q> &w, BandFeeds &f, uint32_t g, uint32_t nzt, uint32_t nzb,
+                                         int32_t r, int32_t cmax, Top top, Rec rec) {
+    uint32_t Ln[Q], Hn[Q];
+    {
+        // no shift; top lane: the fed columns, and above the window a horizontal gap, dH = 0
+        const uint32_t sB0 = muladd(__shfl_up_sync(kFull, w.B0[Q - 1], 1, g), nzt, f.B0);
+        const uint32_t sB1 = muladd(__shfl_up_sync(kFull, w.B1[Q - 1], 1, g), nzt, f.B1);
+        const uint32_t sH0 = mul(__shfl_up_sync(kFull, w.H0[Q - 1], 1, g), nzt);
+        const uint32_t sH1 = mul(__shfl_up_sync(kFull, w.H1[Q - 1], 1, g), nzt);
+        f.B0 = mul(f.B0, 2u);
+        f.B1 = mul(f.B1, 2u);
+#pragma unroll
+        for (int v = Q - 1; v >= 0; --v) {
+            w.B0[v] = __funnelshift_l(v ? w.B0[v - 1] : sB0, w.B0[v], 1);
+            w.B1[v] = __funnelshift_l(v ? w.B1[v - 1] : sB1, w.B1[v], 1);
+            const uint32_t a0 = __funnelshift_l(v ? w.H0[v - 1] : sH0, w.H0[v], 1);
+            const uint32_t a1 = __funnelshift_l(v ? w.H1[v - 1] : sH1, w.H1[v], 1);
+            const uint32_t mk = RAMP ? range_mask(1 - r - 32 * v, cmax - 32 * v - 1) : ~0u;
+            band_cell<RAMP, PTR>(w.A0[v], w.A1[v], w.B0[v], w.B1[v], a0, a1, w.V0[v], w.V1[v], mk, w.H0[v], w.H1[v],
+                                 w.V0[v], w.V1[v], Ln[v], Hn[v]);
+        }
+        top(0, w.H0[0], w.H1[0]);
+    }
+    {
+        // shift; bottom lane: the fed rows, and below the window a vertical gap, dV = 0
+        const uint32_t sA0 = muladd(__shfl_down_sync(kFull, w.A0[0], 1, g), nzb, f.A0);
+        const uint32_t sA1 = muladd(__shfl_down_sync(kFull, w.A1[0], 1, g), nzb, f.A1);
+        const uint32_t sV0 = mul(__shfl_down_sync(kFull, w.V0[0], 1, g), nzb);
+        const uint32_t sV1 = mul(__shfl_down_sync(kFull, w.V1[0], 1, g), nzb);
+        f.A0 >>= 1;
+        f.A1 >>= 1;
+#pragma unroll
+        for (int v = 0; v < Q; ++v) {
+            w.A0[v] = __funnelshift_r(w.A0[v], v + 1 < Q ? w.A0[v + 1] : sA0, 1);
+            w.A1[v] = __funnelshift_r(w.A1[v], v + 1 < Q ? w.A1[v + 1] : sA1, 1);
+            const uint32_t b0 = __funnelshift_r(w.V0[v], v + 1 < Q ? w.V0[v + 1] : sV0, 1);
+            const uint32_t b1 = __funnelshift_r(w.V1[v], v + 1 < Q ? w.V1[v + 1] : sV1, 1);
+            const uint32_t mk = RAMP ? range_mask(-r - 32 * v, cmax - 32 * v - 1) : ~0u;
+            uint32_t Ls = 0, Hs = 0;
+            band_cell<RAMP, PTR>(w.A0[v], w.A1[v], w.B0[v], w.B1[v], w.H0[v], w.H1[v], b0, b1, mk, w.H0[v], w.H1[v],
+                                 w.V0[v], w.V1[v], Ls, Hs);
+            if constexpr (PTR) rec(v, Ln[v], Hn[v], Ls, Hs);
+        }
+        top(1, w.V0[0], w.V1[0]);
+    }
+}
+
+template <int Q, bool KEEP>
 __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJob &job, uint32_t lane) {
     const uint32_t g = job.g;
     const uint32_t gl = lane & (g - 1), grp = lane / g;
     const bool active = grp < job.cnt;
     const uint32_t tid = job.t0 + (active ? grp : 0u);
     const BandBitsTask t = p.tasks[tid];
-    const int32_t gq = (int32_t)g * Q, Hw = 32 * gq;
+    const int32_t gq = (int32_t)g * Q, Hw = 32 * gq, wo = 32 * (int32_t)gl * Q;  // wo: the lane's first row in the window
     const int32_t a0 = t.a_first;
     const int32_t R = (a0 - t.hi - 1) >> 1;  // r0(a_first); a_first - hi is odd
-    const int64_t Ag = t.a_slot, Bg = t.b_slot;
-    auto ld = [&](const uint32_t *pl, int64_t gidx) {
-        return plane_window(pl, min(max(gidx, -kPlanePad), p.max_base));  // outside: bases of no cell that matters
-    };
-    uint32_t A0[Q], A1[Q], B0[Q], B1[Q], H0[Q], H1[Q], V0[Q], V1[Q], Ln[Q], Hn[Q];
+    const BandBases bs{p.pl0, p.pl1, p.max_base, t.a_slot, t.b_slot};
+    BandWords<Q> w;
+    band_bases<Q>(w, bs, R + wo, a0);
 #pragma unroll
-    for (int v = 0; v < Q; ++v) {
-        const int32_t W = (int32_t)gl * Q + v;
-        const int64_t ra = Ag + R + 32 * W - 1;                  // A index of the row of bit 0
-        A0[v] = ld(p.pl0, ra);
-        A1[v] = ld(p.pl1, ra);
-        const int64_t cb = Bg + (a0 - 1 - R - 32 * W - 31) - 1;  // B index of the column of bit 31
-        B0[v] = __brev(ld(p.pl0, cb));
-        B1[v] = __brev(ld(p.pl1, cb));
-        H0[v] = H1[v] = V0[v] = V1[v] = 0;
-    }
+    for (int v = 0; v < Q; ++v) w.H0[v] = w.H1[v] = w.V0[v] = w.V1[v] = 0;
     const uint32_t nzt = gl == 0 ? 0u : 1u, nzb = gl == g - 1 ? 0u : 1u;  // 0 on the group's top / bottom lane
-    uint4 *rp = p.ptr + t.ptr_off + gl * Q;  // this lane's records of the next pair of anti-diagonals
     int32_t top = 0;  // W of the window's top cell
     const uint32_t nch = t.nchunks;
     const uint32_t gmask = g == 32 ? kFull : (((1u << g) - 1u) << (grp * g));
+    uint4 *kp = KEEP ? p.ptr + t.ptr_off + gl * Q : nullptr;  // this lane's kept planes of the next block
+    uint32_t keep_in = 0;                                     // chunks until the next block starts
     for (uint32_t c = 0; c < job.nchunks; ++c) {
         const bool live = active && c < nch;
         const int32_t rc = R + 32 * (int32_t)c, ac = a0 + 64 * (int32_t)c;  // r0 and a of the chunk's first step
-        // new columns (top, one per step without a shift) and rows (bottom, one per shift) of the chunk
-        const int64_t fb = Bg + (ac - rc) - 1, fa = Ag + rc + Hw - 1;
-        // (0 on the lanes that take their neighbour's word instead)
-        uint32_t fB0 = nzt ? 0u : __brev(ld(p.pl0, fb)), fB1 = nzt ? 0u : __brev(ld(p.pl1, fb));
-        uint32_t fA0 = nzb ? 0u : ld(p.pl0, fa), fA1 = nzb ? 0u : ld(p.pl1, fa);
+        if constexpr (KEEP) {
+            if (keep_in == 0) {
+                keep_in = kBlockChunks;
+#pragma unroll
+                for (int v = 0; v < Q; ++v)
+                    if (live && in_range((uint64_t)(kp - p.ptr) + v, p.ptr_cap, p.err, kSiteBandBitsPtr))
+                        __stcg(kp + v, make_uint4(w.H0[v], w.H1[v], w.V0[v], w.V1[v]));
+                kp += gq;
+            }
+            --keep_in;
+        }
+        BandFeeds f(bs, rc, ac, Hw, nzt, nzb);
         // masks only while some cell of the chunk lies on or beyond row 0 / column 0
         const bool ramp = __any_sync(kFull, live && !(rc >= 1 && ac - rc - Hw >= 0));
         uint32_t cH0 = 0, cH1 = 0, cV0 = 0, cV1 = 0;
         auto steps = [&](auto ramp_tag) {
-            constexpr bool RAMP = decltype(ramp_tag)::value;
-            for (int32_t d = 0; d < 32; ++d) {
-                // ---- no shift: anti-diagonal ac + 2d, top row rc + d
-                {
-                    // top lane: the fed columns, and above the window a horizontal gap, dH = 0
-                    const uint32_t sB0 = muladd(__shfl_up_sync(kFull, B0[Q - 1], 1, g), nzt, fB0);
-                    const uint32_t sB1 = muladd(__shfl_up_sync(kFull, B1[Q - 1], 1, g), nzt, fB1);
-                    const uint32_t sH0 = muladd(__shfl_up_sync(kFull, H0[Q - 1], 1, g), nzt, 0u);
-                    const uint32_t sH1 = muladd(__shfl_up_sync(kFull, H1[Q - 1], 1, g), nzt, 0u);
-                    fB0 = muladd(fB0, 2u, 0u);
-                    fB1 = muladd(fB1, 2u, 0u);
-#pragma unroll
-                    for (int v = Q - 1; v >= 0; --v) {
-                        const int32_t W = (int32_t)gl * Q + v;
-                        B0[v] = __funnelshift_l(v ? B0[v - 1] : sB0, B0[v], 1);
-                        B1[v] = __funnelshift_l(v ? B1[v - 1] : sB1, B1[v], 1);
-                        const uint32_t a0v = __funnelshift_l(v ? H0[v - 1] : sH0, H0[v], 1);
-                        const uint32_t a1v = __funnelshift_l(v ? H1[v - 1] : sH1, H1[v], 1);
-                        const uint32_t mk = RAMP ? range_mask(1 - rc - d - 32 * W, ac - rc + d - 32 * W - 1) : ~0u;
-                        band_cell<RAMP>(A0[v], A1[v], B0[v], B1[v], a0v, a1v, V0[v], V1[v], mk, H0[v], H1[v], V0[v],
-                                        V1[v], Ln[v], Hn[v]);
-                    }
-                    cH0 = __funnelshift_r(cH0, H0[0], 1);
-                    cH1 = __funnelshift_r(cH1, H1[0], 1);
-                }
-                // ---- shift: anti-diagonal ac + 2d + 1, top row rc + d + 1
-                {
-                    // bottom lane: the fed rows, and below the window a vertical gap, dV = 0
-                    const uint32_t sA0 = muladd(__shfl_down_sync(kFull, A0[0], 1, g), nzb, fA0);
-                    const uint32_t sA1 = muladd(__shfl_down_sync(kFull, A1[0], 1, g), nzb, fA1);
-                    const uint32_t sV0 = muladd(__shfl_down_sync(kFull, V0[0], 1, g), nzb, 0u);
-                    const uint32_t sV1 = muladd(__shfl_down_sync(kFull, V1[0], 1, g), nzb, 0u);
-                    fA0 >>= 1;
-                    fA1 >>= 1;
-#pragma unroll
-                    for (int v = 0; v < Q; ++v) {
-                        const int32_t W = (int32_t)gl * Q + v;
-                        A0[v] = __funnelshift_r(A0[v], v + 1 < Q ? A0[v + 1] : sA0, 1);
-                        A1[v] = __funnelshift_r(A1[v], v + 1 < Q ? A1[v + 1] : sA1, 1);
-                        const uint32_t b0v = __funnelshift_r(V0[v], v + 1 < Q ? V0[v + 1] : sV0, 1);
-                        const uint32_t b1v = __funnelshift_r(V1[v], v + 1 < Q ? V1[v + 1] : sV1, 1);
-                        const uint32_t mk = RAMP ? range_mask(-rc - d - 32 * W, ac - rc + d - 32 * W - 1) : ~0u;
-                        uint32_t Ls, Hs;
-                        band_cell<RAMP>(A0[v], A1[v], B0[v], B1[v], H0[v], H1[v], b0v, b1v, mk, H0[v], H1[v], V0[v],
-                                        V1[v], Ls, Hs);
-                        if (PTR && live && in_range((uint64_t)(rp - p.ptr) + v, p.ptr_cap, p.err, kSiteBandBitsPtr))
-                            __stcg(rp + v, make_uint4(Ln[v], Hn[v], Ls, Hs));
-                    }
-                    cV0 = __funnelshift_r(cV0, V0[0], 1);
-                    cV1 = __funnelshift_r(cV1, V1[0], 1);
-                    rp += gq;
-                }
-            }
+            for (int32_t d = 0; d < 32; ++d)
+                band_two<Q, decltype(ramp_tag)::value, false>(
+                    w, f, g, nzt, nzb, rc + d + wo, ac - rc + d - wo,
+                    [&](int second, uint32_t x0, uint32_t x1) {
+                        if (!second) {
+                            cH0 = __funnelshift_r(cH0, x0, 1);
+                            cH1 = __funnelshift_r(cH1, x1, 1);
+                        } else {
+                            cV0 = __funnelshift_r(cV0, x0, 1);
+                            cV1 = __funnelshift_r(cV1, x1, 1);
+                        }
+                    },
+                    [](int, uint32_t, uint32_t, uint32_t, uint32_t) {});
         };
         if (ramp) steps(std::true_type{});
         else steps(std::false_type{});
@@ -225,9 +298,9 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
             int32_t sum = 0;
 #pragma unroll
             for (int v = 0; v < Q; ++v) {
-                const int32_t W = (int32_t)gl * Q + v;
-                const uint32_t vm = range_mask(1 - 32 * W, Pm - 32 * W), hm = range_mask(-32 * W, Pm - 1 - 32 * W);
-                sum += __popc(V0[v] & vm) + 2 * __popc(V1[v] & vm) - __popc(H0[v] & hm) - 2 * __popc(H1[v] & hm);
+                const int32_t o = wo + 32 * v;
+                const uint32_t vm = range_mask(1 - o, Pm - o), hm = range_mask(-o, Pm - 1 - o);
+                sum += __popc(w.V0[v] & vm) + 2 * __popc(w.V1[v] & vm) - __popc(w.H0[v] & hm) - 2 * __popc(w.H1[v] & hm);
             }
             for (uint32_t o = 1; o < g; o <<= 1) sum += __shfl_xor_sync(gmask, sum, o);
             if (gl == 0) {
@@ -239,7 +312,7 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
     }
 }
 
-template <bool PTR>
+template <bool KEEP>
 __global__ void __launch_bounds__(kBandWarps * 32) k_bits_band(BandBitsArgs p) {
     const uint32_t lane = threadIdx.x & 31u;
     for (;;) {
@@ -249,163 +322,163 @@ __global__ void __launch_bounds__(kBandWarps * 32) k_bits_band(BandBitsArgs p) {
         if (jid >= p.njobs) break;
         const BandBitsJob job = p.jobs[jid];
         switch (job.Q) {
-            case 1: band_job<1, PTR>(p, job, lane); break;
-            case 2: band_job<2, PTR>(p, job, lane); break;
-            case 3: band_job<3, PTR>(p, job, lane); break;
-            default: band_job<4, PTR>(p, job, lane); break;
+            case 1: band_job<1, KEEP>(p, job, lane); break;
+            case 2: band_job<2, KEEP>(p, job, lane); break;
+            case 3: band_job<3, KEEP>(p, job, lane); break;
+            default: band_job<4, KEEP>(p, job, lane); break;
         }
     }
 }
 
 // ---------------------------------------------------------------- the walk
 struct BitsWalkTask {
-    uint64_t ptr_off;    // the pair's first record
-    uint64_t moves_off;  // its move bytes
+    uint64_t ptr_off;         // the pair's first kept planes
+    uint64_t moves_off;       // its move bytes
+    int64_t a_slot, b_slot;   // planar slots of A (rows) and B (columns)
     uint32_t m, n, gq;
     int32_t hi, a_first;
-    uint32_t slot;       // its move count slot
+    uint32_t slot;            // its move count slot
 };
 
-// One warp per pair: it stages 32 records (64 anti-diagonals) of the three
-// words around the walk's position into shared memory, then walks from
-// (m, n) while the cells stay inside them; moves are written in walk order
-// (0 diagonal, 1 vertical, 2 horizontal), as the CIGAR assembly reads.
-// While the warp walks one block, the loads of the 32 records before it (the
-// same words) are in flight; they fill the second buffer, which the walk
-// continues in unless it left those words (then a new block is staged).
+struct BitsWalkArgs {
+    const uint32_t *pl0, *pl1;
+    int64_t max_base;
+    const uint4 *ptr;
+    const BitsWalkTask *tasks;
+    uint32_t ntasks;
+    uint8_t *moves;
+    uint64_t *nmoves;
+    uint32_t *err;
+};
+
+// Four pairs per warp, one per group of 8 lanes.  A group takes the block of
+// its cell, places its sub-window of 8 words (256 rows) around the cell's
+// row (at least 97 rows on either side unless the window itself ends),
+// starts from the planes kept at the block's start and recomputes the
+// block's anti-diagonals up to its own, their pointer records into shared
+// memory; then it walks.  A diagonal move keeps the cell's row in the window
+// (same word and bit) and goes one record back, so lane t reads the cells t
+// and t + 8 diagonal moves on; ballots of their L bits give the run's
+// length, its zero bytes are stored at once, and the Hb bit of the cell that
+// ends it gives the vertical or horizontal move.  Moves are written in walk
+// order (0 diagonal, 1 vertical, 2 horizontal), as the CIGAR assembly reads.
 //
-// RUNS: the whole warp walks, a run of diagonal moves at a time.  A
-// diagonal move keeps the cell's row in the window (same word and bit) and
-// goes one record row down, so lane t reads the cell t diagonal moves on;
-// a ballot of their L bits gives the run's length (its first lane whose
-// diagonal loses), the run's zero bytes are one store, and the cell that
-// ends it gives the vertical or horizontal move by its Hb bit.  Otherwise
-// lane 0 walks one move at a time.
-template <bool RUNS>
-__global__ void __launch_bounds__(kWalkWarps * 32) k_bits_walk(const uint4 *ptr, const BitsWalkTask *tasks,
-                                                               uint32_t ntasks, uint8_t *moves, uint64_t *nmoves,
-                                                               uint32_t *err) {
-    __shared__ uint4 tile[kWalkWarps][2][32][3];
-    const uint32_t lane = threadIdx.x & 31u, wb = threadIdx.x >> 5;
-    const uint32_t nw = gridDim.x * kWalkWarps;
-    for (uint32_t ti = blockIdx.x * kWalkWarps + wb; ti < ntasks; ti += nw) {
-        const BitsWalkTask tk = tasks[ti];
-        const uint4 *pp = ptr + tk.ptr_off;
-        uint8_t *mv = moves + tk.moves_off;
-        int32_t i = (int32_t)tk.m, j = (int32_t)tk.n;
-        uint64_t k = 0;
-        const int32_t gq = (int32_t)tk.gq;
-        bool ok = true, have = false;
-        int32_t ds_lo = 0, w_lo = 0, cur = 0;
-        while (ok && i > 0 && j > 0) {
-            const int32_t a = i + j, ds = (a - tk.a_first) >> 1;
-            const int32_t W = (i - ((a - tk.hi) >> 1)) >> 5;
-            bool staged = false;
-            if (!have || ds < ds_lo || ds > ds_lo + 31 || W < w_lo || W > w_lo + 2) {
-                // the 32 records ending at the walk's position, staged now
-                ds_lo = max(ds - 31, 0);
-                w_lo = max(min(W - 1, gq - 3), 0);
-                __syncwarp();
-                if (ds_lo + (int32_t)lane <= ds) {
-#pragma unroll
-                    for (int x = 0; x < 3; ++x)
-                        if (w_lo + x < gq)
-                            tile[wb][cur][lane][x] = __ldcg(pp + (uint64_t)(ds_lo + (int32_t)lane) * gq + w_lo + x);
-                }
-                __syncwarp();
-                have = staged = true;
+// Why recompute: the pointer records of a whole window are 0.25 bytes per
+// cell, which bounded the fill by HBM (10,000 pairs of 2-20 kb: 149 GB, 22 ms
+// at the measured copy rate, 36 ms measured with them), while the sub-window
+// is about a tenth of the window and its records never leave the SM.
+__global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
+    extern __shared__ uint4 tiles[];  // [group][record of the block][word]
+    const uint32_t lane = threadIdx.x, grp = lane / kSubWords, gl = lane % kSubWords;
+    uint4 *tile = tiles + grp * (kBlockSteps * kSubWords);
+    for (uint32_t w0 = blockIdx.x * kSubPairs; w0 < p.ntasks; w0 += gridDim.x * kSubPairs) {
+        const uint32_t ti = w0 + grp;
+        const bool mine = ti < p.ntasks;
+        const BitsWalkTask tk = p.tasks[mine ? ti : w0];
+        const int32_t gq = (int32_t)tk.gq, nw = min(gq, kSubWords);
+        const int32_t R = (tk.a_first - tk.hi - 1) >> 1;
+        const BandBases bs{p.pl0, p.pl1, p.max_base, tk.a_slot, tk.b_slot};
+        const uint32_t nzt = gl == 0 ? 0u : 1u, nzb = (int32_t)gl >= nw - 1 ? 0u : 1u;
+        uint8_t *mv = p.moves + tk.moves_off;
+        int32_t i = mine ? (int32_t)tk.m : 0, j = mine ? (int32_t)tk.n : 0;
+        uint32_t k = 0;
+        // every round makes a move in each walking group or ends its walk
+        while (__any_sync(kFull, i > 0 && j > 0)) {
+            bool on = i > 0 && j > 0;
+            const int32_t a = i + j, P = i - ((a - tk.hi) >> 1), wd = P >> 5;
+            if (on && (P < 0 || wd >= gq)) {
+                // the walk left the window, which a certified band excludes
+                if (gl == 0) raise_error(p.err, NW_ERR_ARG, 0x50000u + ti);
+                i = j = 0;
+                on = false;
             }
-            // the 32 records before the block: loads issued now, stored after the walk
-            const int32_t nds = ds_lo - 32, rec = nds + (int32_t)lane;
-            uint4 r[3];
-#pragma unroll
-            for (int x = 0; x < 3; ++x)
-                r[x] = (rec >= 0 && w_lo + x < gq) ? __ldcg(pp + (uint64_t)rec * gq + w_lo + x) : make_uint4(0, 0, 0, 0);
-            if (RUNS) {
-                // every pass makes a move or leaves the loop: at most m + n passes
-                const uint64_t k0 = k;
-                while (i > 0 && j > 0) {
-                    const int32_t a2 = i + j, rel = a2 - tk.a_first, x = (rel >> 1) - ds_lo, par = rel & 1;
-                    const int32_t P = i - ((a2 - tk.hi) >> 1), W2 = P >> 5, y = W2 - w_lo;
-                    if (x < 0 || x > 31 || y < 0 || y > 2 || W2 >= gq || P < 0) break;
-                    const uint32_t bit = (uint32_t)P & 31u;
-                    // lane t: the cell t diagonal moves on (record row x - t, same word and bit);
-                    // rows outside the block count as ending the run
-                    const int32_t xr = x - (int32_t)lane;
-                    uint32_t Lw = ~0u, Hw = 0u;
-                    if (xr >= 0 && ds_lo + xr >= 0) {
-                        const uint4 rc = tile[wb][cur][xr][y];
-                        Lw = par ? rc.z : rc.x;
-                        Hw = par ? rc.w : rc.y;
+            const int32_t cc = on ? (a - tk.a_first) >> 6 : 0, c0 = cc - cc % kBlockChunks;
+            const int32_t ws = on ? min(max(wd - ((P & 31) < 16 ? 4 : 3), 0), max(gq - kSubWords, 0)) : 0;
+            const int32_t as = tk.a_first + 64 * c0, r0 = R + 32 * c0 + 32 * ws;  // the block's first step, its top row
+            BandWords<1> w;
+            band_bases<1>(w, bs, r0 + 32 * (int32_t)gl, as);
+            uint4 h = make_uint4(0u, 0u, 0u, 0u);
+            if (on && c0 > 0 && (int32_t)gl < nw)
+                h = __ldcg(p.ptr + tk.ptr_off + (uint64_t)(c0 / kBlockChunks) * gq + ws + gl);
+            w.H0[0] = h.x;
+            w.H1[0] = h.y;
+            w.V0[0] = h.z;
+            w.V1[0] = h.w;
+            __syncwarp();
+            for (int32_t c = 0; c < kBlockChunks; ++c) {
+                const bool live = on && c0 + c <= cc;
+                if (!__any_sync(kFull, live)) break;
+                const int32_t rc = r0 + 32 * c, ac = as + 64 * c;
+                BandFeeds f(bs, rc, ac, 32 * nw, nzt, nzb);
+                const bool ramp = __any_sync(kFull, live && !(rc >= 1 && ac - rc - 32 * nw >= 0));
+                uint4 *out = tile + 32 * c * kSubWords + gl;
+                auto steps = [&](auto ramp_tag) {
+#pragma unroll 2
+                    for (int32_t d = 0; d < 32; ++d)
+                        band_two<1, decltype(ramp_tag)::value, true>(
+                            w, f, kSubWords, nzt, nzb, rc + d + 32 * (int32_t)gl, ac - rc + d - 32 * (int32_t)gl,
+                            [](int, uint32_t, uint32_t) {},
+                            [&](int, uint32_t Ln, uint32_t Hn, uint32_t Ls, uint32_t Hs) {
+                                out[d * kSubWords] = make_uint4(Ln, Hn, Ls, Hs);
+                            });
+                };
+                if (ramp) steps(std::true_type{});
+                else steps(std::false_type{});
+            }
+            __syncwarp();
+            // the walk through the block's records
+            while (__any_sync(kFull, on)) {
+                const int32_t a2 = i + j, rel = a2 - as, x = rel >> 1, par = rel & 1;
+                const int32_t P2 = i - ((a2 - tk.hi) >> 1), y = (P2 >> 5) - ws;
+                // (a block's path stays within its sub-window; the window's own ends are checked above)
+                on = on && rel >= 0 && i > 0 && j > 0 && P2 >= 0 && y >= 0 && y < nw;
+                const uint32_t bit = (uint32_t)P2 & 31u;
+                uint32_t L0 = 1u, L1 = 1u, h0 = 0u, h1 = 0u;  // cells outside the block end the run
+                if (on) {
+                    const int32_t x0 = x - (int32_t)gl, x1 = x0 - kSubWords;
+                    if (x0 >= 0) {
+                        const uint4 rc = tile[x0 * kSubWords + y];
+                        L0 = ((par ? rc.z : rc.x) >> bit) & 1u;
+                        h0 = ((par ? rc.w : rc.y) >> bit) & 1u;
                     }
-                    const uint32_t stop = __ballot_sync(kFull, (Lw >> bit) & 1u);
-                    const int32_t f = stop ? __ffs(stop) - 1 : 32;
-                    const int32_t run = min(f, min(i, j));
-                    if ((int32_t)lane < run) mv[k + lane] = 0;
-                    k += (uint64_t)run;
+                    if (x1 >= 0) {
+                        const uint4 rc = tile[x1 * kSubWords + y];
+                        L1 = ((par ? rc.z : rc.x) >> bit) & 1u;
+                        h1 = ((par ? rc.w : rc.y) >> bit) & 1u;
+                    }
+                }
+                const uint32_t sh = grp * kSubWords, gm = (1u << kSubWords) - 1u;
+                const uint32_t stop = ((__ballot_sync(kFull, L0) >> sh) & gm) |
+                                      (((__ballot_sync(kFull, L1) >> sh) & gm) << kSubWords);
+                const uint32_t hb = ((__ballot_sync(kFull, h0) >> sh) & gm) |
+                                    (((__ballot_sync(kFull, h1) >> sh) & gm) << kSubWords);
+                if (on) {
+                    const int32_t fr = stop ? __ffs(stop) - 1 : 2 * kSubWords;
+                    const int32_t run = min(fr, min(i, j));
+                    if ((int32_t)gl < run) mv[k + gl] = 0;
+                    if ((int32_t)gl + kSubWords < run) mv[k + gl + kSubWords] = 0;
+                    k += (uint32_t)run;
                     i -= run;
                     j -= run;
-                    const uint32_t hb = __shfl_sync(kFull, (Hw >> bit) & 1u, f & 31);
-                    if (run == f && f < 32 && x - f >= 0 && ds_lo + x - f >= 0 && i > 0 && j > 0) {
-                        const uint32_t mvc = hb ? 2u : 1u;
-                        if (lane == 0) mv[k] = (uint8_t)mvc;
+                    if (run == fr && fr < 2 * kSubWords && x - fr >= 0 && i > 0 && j > 0) {
+                        const uint32_t mvc = ((hb >> fr) & 1u) ? 2u : 1u;
+                        if (gl == 0) mv[k] = (uint8_t)mvc;
                         ++k;
                         i -= mvc == 1u;
                         j -= mvc == 2u;
-                    } else if (run == 0) {
-                        break;
                     }
                 }
-                // a block staged at the walk's own cell: no progress means the
-                // walk left the window, which a certified band excludes
-                if (staged && k == k0) {
-                    if (lane == 0) raise_error(err, NW_ERR_ARG, 0x50000u + ti);
-                    ok = false;
-                }
-            } else if (lane == 0) {
-                uint32_t steps = 0;
-                while (i > 0 && j > 0) {
-                    const int32_t a2 = i + j, rel = a2 - tk.a_first, d2 = rel >> 1;
-                    const int32_t P = i - ((a2 - tk.hi) >> 1), W2 = P >> 5;
-                    if (d2 < ds_lo || d2 > ds_lo + 31 || W2 < w_lo || W2 > w_lo + 2 || W2 >= gq || P < 0) break;
-                    const uint4 rc = tile[wb][cur][d2 - ds_lo][W2 - w_lo];
-                    const uint32_t bit = (uint32_t)P & 31u;
-                    const uint32_t L = (rel & 1) ? rc.z : rc.x, Hb = (rel & 1) ? rc.w : rc.y;
-                    const uint32_t mvc = !((L >> bit) & 1u) ? 0u : !((Hb >> bit) & 1u) ? 1u : 2u;
-                    mv[k++] = (uint8_t)mvc;
-                    i -= mvc != 2u;
-                    j -= mvc != 1u;
-                    ++steps;
-                }
-                // a block staged at the walk's own cell: no progress means the
-                // walk left the window, which a certified band excludes
-                if (staged && steps == 0) {
-                    raise_error(err, NW_ERR_ARG, 0x50000u + ti);
-                    ok = false;
-                }
             }
-            i = __shfl_sync(kFull, i, 0);
-            j = __shfl_sync(kFull, j, 0);
-            k = __shfl_sync(kFull, k, 0);
-            ok = __shfl_sync(kFull, ok, 0);
-            if (nds + 31 >= 0) {
-                // the prefetched block becomes the current one
-                __syncwarp();
-                if (rec >= 0) {
-#pragma unroll
-                    for (int x = 0; x < 3; ++x) tile[wb][cur ^ 1][lane][x] = r[x];
-                }
-                __syncwarp();
-                cur ^= 1;
-                ds_lo = nds;
-            } else {
-                have = false;
-            }
+            __syncwarp();
         }
-        const uint32_t rest = (uint32_t)(max(i, 0) + max(j, 0));
-        const uint8_t mvr = i > 0 ? 1 : 2;
-        for (uint32_t q = lane; q < rest; q += 32) mv[k + q] = mvr;
-        if (lane == 0) nmoves[tk.slot] = k + rest;
+        // row 0 / column 0: only horizontal / vertical moves remain
+        if (mine) {
+            const uint32_t rest = (uint32_t)(max(i, 0) + max(j, 0));
+            const uint8_t mvr = i > 0 ? 1 : 2;
+            for (uint32_t q = gl; q < rest; q += kSubWords) mv[k + q] = mvr;
+            if (gl == 0) p.nmoves[tk.slot] = (uint64_t)k + rest;
+        }
+        __syncwarp();
     }
 }
 
@@ -451,7 +524,11 @@ uint32_t band_bits_max_width(uint32_t m, uint32_t n) {
     return w > 0 ? (uint32_t)w : 0u;
 }
 
-uint64_t band_bits_records(const BandBitsShape &s) { return (uint64_t)s.nchunks * 32u * s.g * s.Q; }
+uint64_t band_bits_cells(const BandBitsShape &s) { return (uint64_t)s.nchunks * 64u * 32u * s.g * s.Q; }
+
+uint64_t band_bits_kept(const BandBitsShape &s) {
+    return (uint64_t)((s.nchunks + kBlockChunks - 1) / kBlockChunks) * s.g * s.Q;
+}
 
 double band_bits_seconds(const BandBitsShape &s) {
     // 64 anti-diagonals per chunk, ~20 instructions per word and ~14 per
@@ -460,7 +537,7 @@ double band_bits_seconds(const BandBitsShape &s) {
 }
 
 int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBitsItem> &items, bool want, int32_t gap, int32_t *scores, uint32_t score_cap,
-                   void *ptr, uint64_t ptr_records, std::vector<int32_t> &banded) {
+                   void *ptr, uint64_t kept, std::vector<int32_t> &banded) {
     int rc;
     banded.assign(items.size(), 0);
     if (items.empty()) return NW_OK;
@@ -532,7 +609,7 @@ int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBi
     a.njobs = (uint32_t)jobs.size();
     a.counter = cnt;
     a.ptr = (uint4 *)ptr;
-    a.ptr_cap = ptr_records;
+    a.ptr_cap = kept;
     a.scores = scores;
     a.gathered = dg;
     a.score_cap = score_cap;
@@ -571,7 +648,7 @@ int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBi
     return NW_OK;
 }
 
-int band_bits_walk(nw_ctx *ctx, const void *ptr, const std::vector<BandBitsItem> &items,
+int band_bits_walk(nw_ctx *ctx, const PlaneSet &planes, const void *ptr, const std::vector<BandBitsItem> &items,
                    const std::vector<uint32_t> &which, const uint8_t *pool, char *cigar_pool,
                    const uint64_t *cigar_off, uint64_t *cigar_len, uint32_t mflag) {
     if (which.empty()) return NW_OK;
@@ -595,8 +672,8 @@ int band_bits_walk(nw_ctx *ctx, const void *ptr, const std::vector<BandBitsItem>
     uint64_t mpos = 0;
     for (size_t q = 0; q < order.size(); ++q) {
         const BandBitsItem &it = items[order[q]];
-        wt[q] = BitsWalkTask{it.ptr_off, mpos, it.m, it.n, it.shape.g * it.shape.Q, it.shape.hi, it.shape.a_first,
-                             (uint32_t)q};
+        wt[q] = BitsWalkTask{it.ptr_off, mpos, it.a_slot, it.b_slot, it.m, it.n, it.shape.g * it.shape.Q, it.shape.hi,
+                             it.shape.a_first, (uint32_t)q};
         TraceTask x{};
         x.m = it.m;
         x.n = it.n;
@@ -625,17 +702,13 @@ int band_bits_walk(nw_ctx *ctx, const void *ptr, const std::vector<BandBitsItem>
     if (e != cudaSuccess) return cuda_fail(ctx, e, "walk tasks H2D");
     {
         LaunchTimer t(ctx, "bband_walk");
-        // every walk at once: each is a serial chain, so the launch's
-        // throughput is the number in flight (capping the CTAs per SM at
-        // 16 / 8 / 4 / 2 / 1 measured 8.6 / 9.3 / 10.1 / 14.9 / 24.2 ms per step
-        // on config 4, against 8.3 ms uncapped)
-        const uint32_t blocks = (uint32_t)std::min<size_t>((which.size() + kWalkWarps - 1) / kWalkWarps, 65535);
-        // runs of diagonal moves at a time; NW_BWALK_SERIAL=1 walks one move
-        // at a time on lane 0 (for comparisons)
-        const char *se = getenv("NW_BWALK_SERIAL");
-        auto walk = (se && *se == '1') ? k_bits_walk<false> : k_bits_walk<true>;
-        walk<<<blocks, kWalkWarps * 32, 0, ctx->stream>>>((const uint4 *)ptr, dw, (uint32_t)which.size(),
-                                                          (uint8_t *)mv, (uint64_t *)nm, ctx->d_err);
+        // one warp per CTA; its 48 KB of records let four CTAs share an SM (one warp per scheduler)
+        constexpr int smem = kSubPairs * kBlockSteps * kSubWords * (int)sizeof(uint4);
+        static_assert(smem <= 48 * 1024, "above the default limit of dynamic shared memory");
+        const uint32_t blocks = (uint32_t)std::min<size_t>((which.size() + kSubPairs - 1) / kSubPairs, 65535);
+        const BitsWalkArgs wa{planes.pl0, planes.pl1, planes.max_base, (const uint4 *)ptr, dw, (uint32_t)which.size(),
+                              (uint8_t *)mv, (uint64_t *)nm, ctx->d_err};
+        k_bits_walk<<<blocks, 32, smem, ctx->stream>>>(wa);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "walk launch");
