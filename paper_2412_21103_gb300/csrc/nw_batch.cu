@@ -216,9 +216,9 @@ static int check_band_scoring(nw_ctx *ctx, const nw_scoring &sc) {
 // run one after another.  Rates are GB300 measurements (cells/s): one warp
 // of the batched kernels, the whole batched kernel, and the scalar
 // single-pair kernel on a long pair; the bit-sliced one runs a chain of
-// m + n + m/31 steps of about 40 ns, then its walk.
+// m + n + m/31 steps of about 30 ns, then its walk.
 constexpr double kWarpRate = 2e9, kBatchRate = 3.5e12, kPairRate = 2e11, kPairFixed = 1e-3;
-constexpr double kBitsStepSeconds = 40e-9, kBitsPairFixed = 0.3e-3;
+constexpr double kBitsStepSeconds = 30e-9, kBitsPairFixed = 0.3e-3;
 
 struct PairCost {
     double secs;   // time of the pair on the single-pair path

@@ -31,13 +31,13 @@
 // shift, its dV on a shift) and carried down the last anti-diagonal to
 // (m, n).
 //
-// Alignments.  The fill writes no pointers: every kBlockChunks chunks (192
+// Alignments.  The fill writes no pointers: every kBlockChunks chunks (128
 // anti-diagonals) it keeps the window's four planes (16 bytes per word).  The
 // walk then goes back block by block: it recomputes the pointer bits of the
 // block it stands in from the planes kept at its start -- only the 256 rows
 // around the path, because a cell of an anti-diagonal depends on the row
 // itself and its two neighbours one anti-diagonal pair earlier, so nothing
-// further than 96 rows away reaches the path within 192 anti-diagonals -- into
+// further than 64 rows away reaches the path within 128 anti-diagonals -- into
 // shared memory and follows the path through them.  Pointer bits, per cell:
 // L = T != s' (the diagonal loses), and Hb = dV != 0 (the vertical move
 // loses); the walk reads !L -> diagonal, else !Hb -> vertical, else
@@ -133,10 +133,35 @@ __device__ __forceinline__ void band_cell(uint32_t A0, uint32_t A1, uint32_t B0,
     if constexpr (PTR) Hb = V0 | V1;
 }
 
-// A lane's Q words of the window: bases and difference planes.
+// A lane's Q words of the window: difference planes, the bases of the
+// chunk's start, and the words that follow them (in: the word above the
+// lane's first for B, below its last for A).  During a chunk the B bases of a
+// word slide up by 32 and its A bases down by 32, so both always lie in two
+// of these words and a step takes them by one funnel shift; after it each
+// word holds what its neighbour held.
 template <int Q>
 struct BandWords {
     uint32_t A0[Q], A1[Q], B0[Q], B1[Q], H0[Q], H1[Q], V0[Q], V1[Q];
+    uint32_t inA0, inA1, inB0, inB1;
+    __device__ __forceinline__ void next_chunk() {
+        uint32_t a0 = inA0, a1 = inA1, b0 = inB0, b1 = inB1;
+#pragma unroll
+        for (int v = 0; v < Q; ++v) {
+            const uint32_t x0 = B0[v], x1 = B1[v];
+            B0[v] = b0;
+            B1[v] = b1;
+            b0 = x0;
+            b1 = x1;
+        }
+#pragma unroll
+        for (int v = Q - 1; v >= 0; --v) {
+            const uint32_t x0 = A0[v], x1 = A1[v];
+            A0[v] = a0;
+            A1[v] = a1;
+            a0 = x0;
+            a1 = x1;
+        }
+    }
 };
 
 // The planar bases as the window reads them (clamped: bases outside belong to no cell that matters).
@@ -146,87 +171,62 @@ struct BandBases {
     __device__ uint32_t at(const uint32_t *pl, int64_t g) const {
         return plane_window(pl, min(max(g, -kPlanePad), max_base));
     }
-};
-
-// The bases of a lane's words before anti-diagonal ac, where the word W of
-// the lane's first word starts at row r (bit 0).
-template <int Q>
-__device__ __forceinline__ void band_bases(BandWords<Q> &w, const BandBases &bs, int32_t r, int32_t ac) {
-#pragma unroll
-    for (int v = 0; v < Q; ++v) {
-        const int64_t ra = bs.Ag + r + 32 * v - 1;                  // A index of the row of bit 0
-        w.A0[v] = bs.at(bs.pl0, ra);
-        w.A1[v] = bs.at(bs.pl1, ra);
-        const int64_t cb = bs.Bg + (ac - 1 - r - 32 * v - 31) - 1;  // B index of the column of bit 31
-        w.B0[v] = __brev(bs.at(bs.pl0, cb));
-        w.B1[v] = __brev(bs.at(bs.pl1, cb));
+    // words of 32 rows from row r on, and of 32 columns from column c down (bit 0 = the first)
+    __device__ uint2 rows(int32_t r) const {
+        const int64_t g = Ag + r - 1;
+        return make_uint2(at(pl0, g), at(pl1, g));
     }
-}
-
-// The bases that enter a window during a chunk of 64 anti-diagonals: columns
-// at its top lane, rows at its bottom lane (0 on the other lanes, which take
-// their neighbour's bits).
-struct BandFeeds {
-    uint32_t B0, B1, A0, A1;
-    __device__ BandFeeds(const BandBases &bs, int32_t rc, int32_t ac, int32_t Hw, uint32_t nzt, uint32_t nzb) {
-        const int64_t fb = bs.Bg + (ac - rc) - 1, fa = bs.Ag + rc + Hw - 1;
-        B0 = nzt ? 0u : __brev(bs.at(bs.pl0, fb));
-        B1 = nzt ? 0u : __brev(bs.at(bs.pl1, fb));
-        A0 = nzb ? 0u : bs.at(bs.pl0, fa);
-        A1 = nzb ? 0u : bs.at(bs.pl1, fa);
+    __device__ uint2 cols(int32_t c) const {
+        const int64_t g = Bg + c - 32;
+        return make_uint2(__brev(at(pl0, g)), __brev(at(pl1, g)));
     }
 };
 
-// A pair of anti-diagonals of a window spread over groups of g lanes.  The
-// first has the lane's first word at row r (bit 0) and columns 1 .. at bits
-// below cmax; nzt, nzb: 0 on the group's top / bottom lane, else 1.  top()
-// runs after the first with the lane's first H word, after the second with
-// its first V word (the score's path); rec(v, L, Hb, L', Hb') takes the pointer bits.
+// A pair of anti-diagonals, the d-th of its chunk, of a window spread over
+// groups of g lanes.  The first has the lane's first word at row r (bit 0)
+// and columns 1 .. at bits below cmax; nzt, nzb: 0 on the group's top /
+// bottom lane, else 1.  cA: the A words of the step before, then of this one.
+// top() runs after the first with the lane's first H word, after the second
+// with its first V word (the score's path); rec(v, L, Hb, L', Hb') takes the
+// pointer bits.
 //
 // What bounds it: the logic pipe, 14 operations per word and anti-diagonal
-// (16 with pointers), the feeds and the choice at the group's ends being
-// multiply-adds, which issue beside it.
+// (16 with pointers); the choice at the group's ends is a multiply-add,
+// which issues beside it.
 template <int Q, bool RAMP, bool PTR, class Top, class Rec>
-__device__ __forceinline__ void band_two(BandWords<Q> &w, BandFeeds &f, uint32_t g, uint32_t nzt, uint32_t nzb,
-                                         int32_t r, int32_t cmax, Top top, Rec rec) {
-    uint32_t Ln[Q], Hn[Q];
+__device__ __forceinline__ void band_two(BandWords<Q> &w, uint32_t (&cA0)[Q], uint32_t (&cA1)[Q], uint32_t d,
+                                         uint32_t g, uint32_t nzt, uint32_t nzb, int32_t r, int32_t cmax, Top top,
+                                         Rec rec) {
+    uint32_t Ln[Q], Hn[Q], cB0[Q], cB1[Q];
     {
-        // no shift; top lane: the fed columns, and above the window a horizontal gap, dH = 0
-        const uint32_t sB0 = muladd(__shfl_up_sync(kFull, w.B0[Q - 1], 1, g), nzt, f.B0);
-        const uint32_t sB1 = muladd(__shfl_up_sync(kFull, w.B1[Q - 1], 1, g), nzt, f.B1);
+        // no shift; above the window a horizontal gap, dH = 0
         const uint32_t sH0 = mul(__shfl_up_sync(kFull, w.H0[Q - 1], 1, g), nzt);
         const uint32_t sH1 = mul(__shfl_up_sync(kFull, w.H1[Q - 1], 1, g), nzt);
-        f.B0 = mul(f.B0, 2u);
-        f.B1 = mul(f.B1, 2u);
 #pragma unroll
         for (int v = Q - 1; v >= 0; --v) {
-            w.B0[v] = __funnelshift_l(v ? w.B0[v - 1] : sB0, w.B0[v], 1);
-            w.B1[v] = __funnelshift_l(v ? w.B1[v - 1] : sB1, w.B1[v], 1);
+            cB0[v] = __funnelshift_lc(v ? w.B0[v - 1] : w.inB0, w.B0[v], d + 1);
+            cB1[v] = __funnelshift_lc(v ? w.B1[v - 1] : w.inB1, w.B1[v], d + 1);
             const uint32_t a0 = __funnelshift_l(v ? w.H0[v - 1] : sH0, w.H0[v], 1);
             const uint32_t a1 = __funnelshift_l(v ? w.H1[v - 1] : sH1, w.H1[v], 1);
             const uint32_t mk = RAMP ? range_mask(1 - r - 32 * v, cmax - 32 * v - 1) : ~0u;
-            band_cell<RAMP, PTR>(w.A0[v], w.A1[v], w.B0[v], w.B1[v], a0, a1, w.V0[v], w.V1[v], mk, w.H0[v], w.H1[v],
+            band_cell<RAMP, PTR>(cA0[v], cA1[v], cB0[v], cB1[v], a0, a1, w.V0[v], w.V1[v], mk, w.H0[v], w.H1[v],
                                  w.V0[v], w.V1[v], Ln[v], Hn[v]);
         }
         top(0, w.H0[0], w.H1[0]);
     }
     {
-        // shift; bottom lane: the fed rows, and below the window a vertical gap, dV = 0
-        const uint32_t sA0 = muladd(__shfl_down_sync(kFull, w.A0[0], 1, g), nzb, f.A0);
-        const uint32_t sA1 = muladd(__shfl_down_sync(kFull, w.A1[0], 1, g), nzb, f.A1);
+        // shift; below the window a vertical gap, dV = 0
         const uint32_t sV0 = mul(__shfl_down_sync(kFull, w.V0[0], 1, g), nzb);
         const uint32_t sV1 = mul(__shfl_down_sync(kFull, w.V1[0], 1, g), nzb);
-        f.A0 >>= 1;
-        f.A1 >>= 1;
 #pragma unroll
         for (int v = 0; v < Q; ++v) {
-            w.A0[v] = __funnelshift_r(w.A0[v], v + 1 < Q ? w.A0[v + 1] : sA0, 1);
-            w.A1[v] = __funnelshift_r(w.A1[v], v + 1 < Q ? w.A1[v + 1] : sA1, 1);
+            cA0[v] = __funnelshift_rc(w.A0[v], v + 1 < Q ? w.A0[v + 1] : w.inA0, d + 1);
+            cA1[v] = __funnelshift_rc(w.A1[v], v + 1 < Q ? w.A1[v + 1] : w.inA1, d + 1);
             const uint32_t b0 = __funnelshift_r(w.V0[v], v + 1 < Q ? w.V0[v + 1] : sV0, 1);
             const uint32_t b1 = __funnelshift_r(w.V1[v], v + 1 < Q ? w.V1[v + 1] : sV1, 1);
             const uint32_t mk = RAMP ? range_mask(-r - 32 * v, cmax - 32 * v - 1) : ~0u;
             uint32_t Ls = 0, Hs = 0;
-            band_cell<RAMP, PTR>(w.A0[v], w.A1[v], w.B0[v], w.B1[v], w.H0[v], w.H1[v], b0, b1, mk, w.H0[v], w.H1[v],
+            band_cell<RAMP, PTR>(cA0[v], cA1[v], cB0[v], cB1[v], w.H0[v], w.H1[v], b0, b1, mk, w.H0[v], w.H1[v],
                                  w.V0[v], w.V1[v], Ls, Hs);
             if constexpr (PTR) rec(v, Ln[v], Hn[v], Ls, Hs);
         }
@@ -246,9 +246,18 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
     const int32_t R = (a0 - t.hi - 1) >> 1;  // r0(a_first); a_first - hi is odd
     const BandBases bs{p.pl0, p.pl1, p.max_base, t.a_slot, t.b_slot};
     BandWords<Q> w;
-    band_bases<Q>(w, bs, R + wo, a0);
 #pragma unroll
-    for (int v = 0; v < Q; ++v) w.H0[v] = w.H1[v] = w.V0[v] = w.V1[v] = 0;
+    for (int v = 0; v < Q; ++v) {
+        const uint2 x = bs.rows(R + wo + 32 * v), y = bs.cols(a0 - 1 - R - wo - 32 * v);
+        w.A0[v] = x.x;
+        w.A1[v] = x.y;
+        w.B0[v] = y.x;
+        w.B1[v] = y.y;
+        w.H0[v] = w.H1[v] = w.V0[v] = w.V1[v] = 0;
+    }
+    // the bases that enter the window during a chunk, loaded one chunk ahead
+    // (the top lane's columns, the bottom lane's rows)
+    uint2 fa = bs.rows(R + Hw), fb = bs.cols(a0 - R + 31);
     const uint32_t nzt = gl == 0 ? 0u : 1u, nzb = gl == g - 1 ? 0u : 1u;  // 0 on the group's top / bottom lane
     int32_t top = 0;  // W of the window's top cell
     const uint32_t nch = t.nchunks;
@@ -269,14 +278,29 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
             }
             --keep_in;
         }
-        BandFeeds f(bs, rc, ac, Hw, nzt, nzb);
+        {
+            const uint32_t b0 = __shfl_up_sync(kFull, w.B0[Q - 1], 1, g), b1 = __shfl_up_sync(kFull, w.B1[Q - 1], 1, g);
+            const uint32_t x0 = __shfl_down_sync(kFull, w.A0[0], 1, g), x1 = __shfl_down_sync(kFull, w.A1[0], 1, g);
+            w.inB0 = nzt ? b0 : fb.x;
+            w.inB1 = nzt ? b1 : fb.y;
+            w.inA0 = nzb ? x0 : fa.x;
+            w.inA1 = nzb ? x1 : fa.y;
+            fa = bs.rows(rc + 32 + Hw);
+            fb = bs.cols(ac + 64 - rc - 32 + 31);
+        }
         // masks only while some cell of the chunk lies on or beyond row 0 / column 0
         const bool ramp = __any_sync(kFull, live && !(rc >= 1 && ac - rc - Hw >= 0));
         uint32_t cH0 = 0, cH1 = 0, cV0 = 0, cV1 = 0;
+        uint32_t cA0[Q], cA1[Q];
+#pragma unroll
+        for (int v = 0; v < Q; ++v) {
+            cA0[v] = w.A0[v];
+            cA1[v] = w.A1[v];
+        }
         auto steps = [&](auto ramp_tag) {
             for (int32_t d = 0; d < 32; ++d)
                 band_two<Q, decltype(ramp_tag)::value, false>(
-                    w, f, g, nzt, nzb, rc + d + wo, ac - rc + d - wo,
+                    w, cA0, cA1, (uint32_t)d, g, nzt, nzb, rc + d + wo, ac - rc + d - wo,
                     [&](int second, uint32_t x0, uint32_t x1) {
                         if (!second) {
                             cH0 = __funnelshift_r(cH0, x0, 1);
@@ -290,6 +314,7 @@ __device__ __forceinline__ void band_job(const BandBitsArgs &p, const BandBitsJo
         };
         if (ramp) steps(std::true_type{});
         else steps(std::false_type{});
+        w.next_chunk();
         top += __popc(cH0) + 2 * __popc(cH1) + __popc(cV0) + 2 * __popc(cV1);
         if (active && c + 1 == nch) {
             // W(m, n): the top cell, then down the last anti-diagonal: each row
@@ -353,7 +378,7 @@ struct BitsWalkArgs {
 
 // Four pairs per warp, one per group of 8 lanes.  A group takes the block of
 // its cell, places its sub-window of 8 words (256 rows) around the cell's
-// row (at least 97 rows on either side unless the window itself ends),
+// row (at least 65 rows on either side unless the window itself ends),
 // starts from the planes kept at the block's start and recomputes the
 // block's anti-diagonals up to its own, their pointer records into shared
 // memory; then it walks.  A diagonal move keeps the cell's row in the window
@@ -382,6 +407,26 @@ __global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
         uint8_t *mv = p.moves + tk.moves_off;
         int32_t i = mine ? (int32_t)tk.m : 0, j = mine ? (int32_t)tk.n : 0;
         uint32_t k = 0;
+        // A block's inputs: the kept planes and, for each of its chunks and
+        // one more, the lane's A and B words.  The next block's are loaded
+        // while this one is computed, for the same sub-window.
+        struct Block {
+            uint4 h;
+            uint2 A[kBlockChunks + 1], B[kBlockChunks + 1];
+        };
+        auto load = [&](Block &blk, int32_t c0, int32_t ws) {
+            const int32_t as = tk.a_first + 64 * c0, r = R + 32 * c0 + 32 * (ws + (int32_t)gl);
+            blk.h = make_uint4(0u, 0u, 0u, 0u);
+            if (c0 > 0 && (int32_t)gl < nw)
+                blk.h = __ldcg(p.ptr + tk.ptr_off + (uint64_t)(c0 / kBlockChunks) * gq + ws + gl);
+#pragma unroll
+            for (int c = 0; c <= kBlockChunks; ++c) {
+                blk.A[c] = bs.rows(r + 32 * c);
+                blk.B[c] = bs.cols(as - 1 - r + 32 * c);
+            }
+        };
+        Block cur, ahead;
+        int32_t ahead_c0 = -1, ahead_ws = 0;
         // every round makes a move in each walking group or ends its walk
         while (__any_sync(kFull, i > 0 && j > 0)) {
             bool on = i > 0 && j > 0;
@@ -393,31 +438,47 @@ __global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
                 on = false;
             }
             const int32_t cc = on ? (a - tk.a_first) >> 6 : 0, c0 = cc - cc % kBlockChunks;
-            const int32_t ws = on ? min(max(wd - ((P & 31) < 16 ? 4 : 3), 0), max(gq - kSubWords, 0)) : 0;
+            int32_t ws = on ? min(max(wd - ((P & 31) < 16 ? 4 : 3), 0), max(gq - kSubWords, 0)) : 0;
+            // the words loaded ahead, when the path's rows lie far enough inside them
+            const bool hit = on && c0 == ahead_c0 && (ahead_ws == 0 || P - 32 * ahead_ws > kBlockSteps) &&
+                             (ahead_ws + kSubWords >= gq || P - 32 * ahead_ws < 32 * kSubWords - 1 - kBlockSteps);
+            if (hit) {
+                ws = ahead_ws;
+                cur = ahead;
+            }
+            if (on && !hit) load(cur, c0, ws);
+            ahead_c0 = on ? c0 - kBlockChunks : -1;
+            ahead_ws = ws;
+            if (ahead_c0 >= 0) load(ahead, ahead_c0, ahead_ws);
             const int32_t as = tk.a_first + 64 * c0, r0 = R + 32 * c0 + 32 * ws;  // the block's first step, its top row
             BandWords<1> w;
-            band_bases<1>(w, bs, r0 + 32 * (int32_t)gl, as);
-            uint4 h = make_uint4(0u, 0u, 0u, 0u);
-            if (on && c0 > 0 && (int32_t)gl < nw)
-                h = __ldcg(p.ptr + tk.ptr_off + (uint64_t)(c0 / kBlockChunks) * gq + ws + gl);
-            w.H0[0] = h.x;
-            w.H1[0] = h.y;
-            w.V0[0] = h.z;
-            w.V1[0] = h.w;
+            w.H0[0] = cur.h.x;
+            w.H1[0] = cur.h.y;
+            w.V0[0] = cur.h.z;
+            w.V1[0] = cur.h.w;
             __syncwarp();
+#pragma unroll
             for (int32_t c = 0; c < kBlockChunks; ++c) {
                 const bool live = on && c0 + c <= cc;
                 if (!__any_sync(kFull, live)) break;
                 const int32_t rc = r0 + 32 * c, ac = as + 64 * c;
-                BandFeeds f(bs, rc, ac, 32 * nw, nzt, nzb);
+                w.A0[0] = cur.A[c].x;
+                w.A1[0] = cur.A[c].y;
+                w.inA0 = cur.A[c + 1].x;
+                w.inA1 = cur.A[c + 1].y;
+                w.B0[0] = cur.B[c].x;
+                w.B1[0] = cur.B[c].y;
+                w.inB0 = cur.B[c + 1].x;
+                w.inB1 = cur.B[c + 1].y;
                 const bool ramp = __any_sync(kFull, live && !(rc >= 1 && ac - rc - 32 * nw >= 0));
                 uint4 *out = tile + 32 * c * kSubWords + gl;
+                uint32_t cA0[1] = {w.A0[0]}, cA1[1] = {w.A1[0]};
                 auto steps = [&](auto ramp_tag) {
-#pragma unroll 2
+#pragma unroll 4
                     for (int32_t d = 0; d < 32; ++d)
                         band_two<1, decltype(ramp_tag)::value, true>(
-                            w, f, kSubWords, nzt, nzb, rc + d + 32 * (int32_t)gl, ac - rc + d - 32 * (int32_t)gl,
-                            [](int, uint32_t, uint32_t) {},
+                            w, cA0, cA1, (uint32_t)d, kSubWords, nzt, nzb, rc + d + 32 * (int32_t)gl,
+                            ac - rc + d - 32 * (int32_t)gl, [](int, uint32_t, uint32_t) {},
                             [&](int, uint32_t Ln, uint32_t Hn, uint32_t Ls, uint32_t Hs) {
                                 out[d * kSubWords] = make_uint4(Ln, Hn, Ls, Hs);
                             });
@@ -531,9 +592,9 @@ uint64_t band_bits_kept(const BandBitsShape &s) {
 }
 
 double band_bits_seconds(const BandBitsShape &s) {
-    // 64 anti-diagonals per chunk, ~20 instructions per word and ~14 per
+    // 64 anti-diagonals per chunk, ~15 instructions per word and ~10 per
     // lane per step, two cycles each on a scheduler of its own, 2.07 GHz
-    return (double)s.nchunks * 64.0 * (20.0 * s.Q + 14.0) * 2.0 / 2.07e9;
+    return (double)s.nchunks * 64.0 * (15.0 * s.Q + 10.0) * 2.0 / 2.07e9;
 }
 
 int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBitsItem> &items, bool want, int32_t gap, int32_t *scores, uint32_t score_cap,
@@ -577,9 +638,14 @@ int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBi
         jobs.push_back(j);
     }
     // longest jobs first (ties in job order)
+    double work = 0, longest = 0;
     {
         std::vector<uint64_t> jk(jobs.size());
-        for (size_t q = 0; q < jobs.size(); ++q) jk[q] = (uint64_t)jobs[q].nchunks * (20 * jobs[q].Q + 14);
+        for (size_t q = 0; q < jobs.size(); ++q) {
+            jk[q] = (uint64_t)jobs[q].nchunks * (15 * jobs[q].Q + 10);
+            work += (double)jk[q];
+            longest = std::max(longest, (double)jk[q]);
+        }
         const std::vector<uint32_t> jo = radix_order_desc(std::move(jk));
         std::vector<BandBitsJob> sorted(jobs.size());
         for (size_t q = 0; q < jobs.size(); ++q) sorted[q] = jobs[jo[q]];
@@ -617,15 +683,16 @@ int band_bits_fill(nw_ctx *ctx, const PlaneSet &planes, const std::vector<BandBi
     a.err = ctx->d_err;
     auto kern = want ? k_bits_band<true> : k_bits_band<false>;
     htp.stop();
-    // Two CTAs per SM (two warps per scheduler), not the five the registers
-    // allow: the jobs are taken longest first, and a long job that shares
-    // its scheduler with four others runs at a fifth of its speed and ends
-    // the launch alone.  Measured on GB300 (config 4, 20,000 pairs, CTAs per
-    // SM 5 / 4 / 3 / 2 / 1): the fills took 54.4 / 48.1 / 41.2 / 37.7 /
-    // 45.0 ms.  NW_BBAND_OCC overrides (sweeps).
+    // Two CTAs per SM (two warps per scheduler), not the most the registers
+    // allow: the jobs are taken longest first, and a long job that shares its
+    // scheduler with others ends the launch alone.  One CTA where even beside
+    // one other the longest job would outlast the launch's ideal time (every
+    // scheduler busy).  Fills of both rounds on GB300, pairs of 2-20 kb, one /
+    // two CTAs: 2,000 pairs 5.9 / 6.8 ms, 10,000 pairs 11.4 / 12.2 ms, 20,000
+    // pairs 22.7 / 20.3 ms.  NW_BBAND_OCC overrides (sweeps).
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kBandWarps * 32, 0);
-    int cap = 2;
+    int cap = 2.0 * longest > work / (4.0 * ctx->sm_count) ? 1 : 2;
     if (const char *e = getenv("NW_BBAND_OCC")) cap = std::max(1, atoi(e));
     occ = std::min(occ, cap);
     uint32_t blocks = (uint32_t)std::max(occ, 1) * (uint32_t)ctx->sm_count;
