@@ -13,12 +13,19 @@
 //     F'(i,j) = max(F'(i-1,j), W(i-1,j) + go)
 //     W(i,j)  = max(W(i-1,j-1) + s - 2*ge, E'(i,j), F'(i,j))
 // with W(0,0) = 0, W(0,j) = W(i,0) = go, F'(0,j) = E'(i,0) = -inf and
-// H(m,n) = W(m,n) + ge*(m+n).  A cell is one byte permute (s - 2ge), three
-// DPX add-max (E', F', W) and one max.  The walk needs four bits per cell:
-// L (the diagonal candidate is below max(E', F')) and H (E' above F') in
-// the global kernels' pointer words, and in a second word array at the same
-// index the extension bits of the cell's gap states -- F: F'(i-1,j) >
-// W(i-1,j) + go, E: E'(i,j-1) > W(i,j-1) + go (a tie closes the gap).
+// H(m,n) = W(m,n) + ge*(m+n).  A cell is one byte permute (s - 2ge), two DPX
+// add-max (E', F'), an add and a three-input max (W).
+//
+// Alignments.  The fill writes no pointers: it keeps every stripe's bottom
+// row (which the next stripe reads anyway) and, every kTileSteps steps, the
+// state of a stripe's 32 lanes.  The trace then walks back from (m, n) tile by
+// tile -- a tile is one stripe and the steps between two kept states --
+// recomputing only the tiles the path crosses, up to the path's own step,
+// with four bits per cell in shared memory: L (the diagonal candidate is below
+// max(E', F')), H (E' above F'), and the extension bits of the cell's gap
+// states, F: F'(i-1,j) > W(i-1,j) + go, E: E'(i,j-1) > W(i,j-1) + go (a tie
+// closes the gap).  Writing the four bits of every cell cost the fill eight
+// more operations per cell (13 against 5) and 0.5 bytes.
 //
 // Batched by stripe jobs: every 32R-row stripe of every pair is one job,
 // jobs queued pair by pair (longest pairs first) and stripes in order, so a
@@ -41,17 +48,17 @@ namespace nw {
 namespace {
 
 constexpr int kAffWarps = 8;
-constexpr uint32_t kAffMinPeriod = 96;
 constexpr int32_t kAffNeg = -(1 << 27);   // -inf: far below any W, no add wraps
+constexpr uint32_t kTileSteps = 128;      // steps between a stripe's kept states
 
 struct AffTask {
     uint64_t a_off, b_off;
     uint32_t m, n;
     uint32_t out;
-    uint32_t ncg;        // pointer words per lane row
-    uint64_t ptr_off;    // word offset (the extension words follow at + ext_off)
-    uint64_t row_off;    // word offset of the pair's stripe rows: stripe s (< S-1) at row_off + 2*s*nr
     uint32_t nr;         // words per row half (n rounded up to 32)
+    uint64_t row_off;    // word offset of the pair's stripe rows: stripe s (< S-1) at row_off + 2*s*nr
+    uint64_t keep_off;   // 16-byte units: the pair's kept states, [stripe][state 1..][part][lane]
+    uint32_t keep_n;     // kept states per stripe
     uint32_t pad;
 };
 
@@ -72,11 +79,10 @@ struct AffArgs {
     uint64_t rows_cap;
     uint32_t *progress;  // per job: columns of its bottom row published
     int32_t *scores;
-    uint32_t *ptr;
-    uint64_t ext_off;    // words from a pointer word to its extension word
+    uint4 *keep;         // kept states
+    uint64_t keep_cap;
     uint32_t *err;
-    uint32_t out_cap;    // pairs at scores (checked build; the pointer words
-                         // of a launch are 2 * ext_off)
+    uint32_t out_cap;    // pairs at scores (checked build)
 };
 
 template <int R>
@@ -93,11 +99,6 @@ __device__ __forceinline__ uint32_t aff_rows(const uint8_t *s, uint32_t i0, uint
     return w;
 }
 
-__device__ __forceinline__ void aff_st_if(bool p, uint32_t *dst, uint32_t v) {
-    asm volatile("{.reg .pred q; setp.ne.b32 q, %0, 0; @q st.global.u32 [%1], %2;}" ::"r"((uint32_t)p), "l"(dst), "r"(v)
-                 : "memory");
-}
-
 // Warp-uniform bounded wait until *flag >= target (lane 0 spins; then every
 // lane acquires, so its following loads see what the producer published).
 __device__ __forceinline__ bool aff_wait(const uint32_t *flag, uint32_t target, uint32_t *err, uint32_t where) {
@@ -108,13 +109,129 @@ __device__ __forceinline__ bool aff_wait(const uint32_t *flag, uint32_t target, 
     return ok != 0;
 }
 
-template <int R, bool PTR>
+// A lane's R rows of a stripe: the systolic state between two steps.
+template <int R>
+struct AffLane {
+    static constexpr uint32_t kParts = (2 * R + 4) / 4;  // 16-byte parts of a kept state
+    uint32_t prof[R];
+    int32_t Wl[R], El[R];
+    int32_t dtop;        // W of the row above the lane's first, one column back
+    uint32_t xout;       // the last row's W (<< 2) and the column's base code, for the lane below
+    int32_t fout;        // its F'
+    uint32_t accL, accH, accF, accE;
+
+    __device__ __forceinline__ void rows(const AffArgs &p, const uint8_t *A, uint32_t i0, uint32_t m) {
+        const uint32_t codes = aff_rows<R>(A, i0, m);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const uint32_t c = (codes >> (2 * r)) & 3u;
+            prof[r] = c == 0 ? p.prof[0] : c == 1 ? p.prof[1] : c == 2 ? p.prof[2] : p.prof[3];
+        }
+    }
+    // column 0: W(i, 0) = go, E'(i, 0) = -inf
+    __device__ __forceinline__ void start(int32_t go, uint32_t i0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            Wl[r] = go;
+            El[r] = kAffNeg;
+        }
+        dtop = i0 == 0 ? 0 : go;  // W(i0, 0)
+        xout = 0;
+        fout = kAffNeg;
+    }
+    __device__ __forceinline__ void save(uint4 *k, uint64_t cap_left, uint32_t *err) const {
+        uint32_t v[4 * kParts];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            v[r] = (uint32_t)Wl[r];
+            v[R + r] = (uint32_t)El[r];
+        }
+        v[2 * R] = (uint32_t)dtop;
+        v[2 * R + 1] = xout;
+        v[2 * R + 2] = (uint32_t)fout;
+        v[2 * R + 3] = 0u;
+#pragma unroll
+        for (uint32_t q = 0; q < kParts; ++q)
+            if (in_range(q * 32u, cap_left, err, kSiteAffPtr))
+                __stcg(k + q * 32u, make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+    }
+    __device__ __forceinline__ void load(const uint4 *k) {
+        uint32_t v[4 * kParts];
+#pragma unroll
+        for (uint32_t q = 0; q < kParts; ++q) {
+            const uint4 x = __ldcg(k + q * 32u);
+            v[4 * q] = x.x;
+            v[4 * q + 1] = x.y;
+            v[4 * q + 2] = x.z;
+            v[4 * q + 3] = x.w;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            Wl[r] = (int32_t)v[r];
+            El[r] = (int32_t)v[R + r];
+        }
+        dtop = (int32_t)v[2 * R];
+        xout = v[2 * R + 1];
+        fout = (int32_t)v[2 * R + 2];
+    }
+    // The R cells of one column from the row above's word x (W << 2 | code)
+    // and F' fx; PTR appends the four bits of each cell to the accumulators
+    // (the last R bits of each are this column's, row 0 highest).
+    template <bool PTR>
+    __device__ __forceinline__ void column(int32_t go, uint32_t x, int32_t fx) {
+        const uint32_t sel = sext_selector(x & 3u);
+        int32_t u = (int32_t)x >> 2, d = dtop, fu = fx;
+        dtop = u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int32_t sv = (int32_t)prmt(prof[r], 0u, sel);
+            const int32_t e = __viaddmax_s32(Wl[r], go, El[r]);
+            const int32_t f = __viaddmax_s32(u, go, fu);
+            const int32_t w = __vimax3_s32(d + sv, e, f);
+            if constexpr (PTR) {
+                accL = ptr_append(accL, d + sv - max(e, f));
+                accH = ptr_append(accH, f - e);
+                accF = ptr_append(accF, u + go - fu);
+                accE = ptr_append(accE, Wl[r] + go - El[r]);
+            }
+            d = Wl[r];
+            Wl[r] = w;
+            El[r] = e;
+            u = w;
+            fu = f;
+        }
+        xout = ((uint32_t)u << 2) | (x & 3u);
+        fout = fu;
+    }
+};
+
+// Lane 0's inputs for the columns of a stripe: row 0 (W = go, F' = -inf) for
+// stripe 0, else the bottom row of the stripe above.
+struct AffAbove {
+    const uint8_t *B;
+    const uint32_t *inW, *inF;  // null for stripe 0
+    uint32_t n;
+    int32_t go;
+    __device__ __forceinline__ uint32_t w(uint32_t col) const {
+        if (col >= n) return 0u;
+        if (!inW) return ((uint32_t)go << 2) | base_at(B, col);
+        return __ldcg(inW + col);
+    }
+    __device__ __forceinline__ int32_t f(uint32_t col) const {
+        if (!inW || col >= n) return kAffNeg;
+        return (int32_t)__ldcg(inF + col);
+    }
+};
+
+// The fill; KEEP: also the stripes' states every kTileSteps steps (for the
+// trace).  What bounds it: the logic pipe, 4 operations per cell (prmt, two
+// add-max, max3; the add runs on either pipe) and about 12 per column of R
+// cells.
+template <int R, bool KEEP>
 __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
     constexpr uint32_t SH = 32u * R;
-    constexpr uint32_t CPW = PTR ? 16u / R : 1u;
     const int lane = threadIdx.x & 31;
     const int32_t go = p.go;
-    const uint32_t P0 = p.prof[0], P1 = p.prof[1], P2 = p.prof[2], P3 = p.prof[3];
 
     for (;;) {
         uint32_t jidx = 0;
@@ -124,8 +241,6 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
         const AffJob jb = p.jobs[jidx];
         const AffTask tk = p.tasks[jb.task];
         const uint32_t s = jb.stripe;
-        const uint8_t *A = p.pool + tk.a_off;
-        const uint8_t *B = p.pool + tk.b_off;
         const uint32_t m = tk.m, n = tk.n;
         if (m == 0 || n == 0) {   // a single job
             if (lane == 0 && in_range(tk.out, p.out_cap, p.err, kSiteAffScore))
@@ -135,122 +250,64 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
         const uint32_t S = (m + SH - 1) / SH;
         const uint32_t T = n + 31;
         const uint32_t lM = ((m - 1) % SH) / R, rM = (m - 1) % R;
-        uint32_t *pbase = PTR ? p.ptr + tk.ptr_off : nullptr;
         // the previous stripe's row (s > 0) and this stripe's (s < S - 1)
         const uint32_t *inW = s ? p.rows + tk.row_off + (size_t)(s - 1) * 2 * tk.nr : nullptr;
-        const uint32_t *inF = s ? inW + tk.nr : nullptr;
         uint32_t *outW = s + 1 < S ? p.rows + tk.row_off + (size_t)s * 2 * tk.nr : nullptr;
         uint32_t *outF = s + 1 < S ? outW + tk.nr : nullptr;
         const uint32_t *prev = s ? p.progress + (jidx - 1) : nullptr;   // stripe s-1 is the job before
         uint32_t *mine = p.progress + jidx;
-
-        uint32_t prof[R];
-        int32_t Wl[R], El[R];
-        uint32_t xout = 0, accL = 0, accH = 0, accF = 0, accE = 0;
-        int32_t fout = kAffNeg;
+        const AffAbove above{p.pool + tk.b_off, inW, s ? inW + tk.nr : nullptr, n, go};
+        AffLane<R> ln;
         const uint32_t i0 = s * SH + (uint32_t)lane * R;   // rows i0+1 .. i0+R (1-based)
-        {
-            const uint32_t codes = aff_rows<R>(A, i0, m);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const uint32_t c = (codes >> (2 * r)) & 3u;
-                prof[r] = c == 0 ? P0 : c == 1 ? P1 : c == 2 ? P2 : P3;
-                Wl[r] = go;        // W(i, 0)
-                El[r] = kAffNeg;   // E'(i, 0)
-            }
-        }
-        int32_t dtop = i0 == 0 ? 0 : go;   // W(i0, 0)
+        ln.rows(p, p.pool + tk.a_off, i0, m);
+        ln.start(go, i0);
+        uint4 *keep = KEEP ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * AffLane<R>::kParts * 32u + lane : nullptr;
         int32_t c = -lane;
-        // lane 0's inputs for column col: row 0 (W = go, F' = -inf) in stripe
-        // 0, the previous stripe's bottom row (published, see the waits) after
-        auto chunk_w = [&](uint32_t col) -> uint32_t {
-            if (col >= n) return 0u;
-            if (!s) return ((uint32_t)go << 2) | base_at(B, col);
-            return __ldcg(inW + col);
-        };
-        auto chunk_f = [&](uint32_t col) -> int32_t {
-            if (!s || col >= n) return kAffNeg;
-            return (int32_t)__ldcg(inF + col);
-        };
         bool alive = !s || aff_wait(prev, min(32u, n), p.err, jidx);
-        uint32_t stage = 0, stage_next = alive ? chunk_w((uint32_t)lane) : 0u;
-        int32_t fstage = kAffNeg, fstage_next = alive ? chunk_f((uint32_t)lane) : kAffNeg;
+        uint32_t stage = 0, stage_next = alive ? above.w((uint32_t)lane) : 0u;
+        int32_t fstage = kAffNeg, fstage_next = alive ? above.f((uint32_t)lane) : kAffNeg;
 
-        // the R cells of one column; u / fu: W and F' of the row above
-        auto column = [&](int32_t d, int32_t u, int32_t fu, uint32_t sel) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int32_t sv = (int32_t)prmt(prof[r], 0u, sel);
-                const int32_t e = __viaddmax_s32(Wl[r], go, El[r]);
-                const int32_t f = __viaddmax_s32(u, go, fu);
-                const int32_t mx = max(e, f);
-                const int32_t w = __viaddmax_s32(d, sv, mx);
-                if constexpr (PTR) {
-                    accL = ptr_append(accL, d + sv - mx);
-                    accH = ptr_append(accH, f - e);
-                    accF = ptr_append(accF, u + go - fu);
-                    accE = ptr_append(accE, Wl[r] + go - El[r]);
-                }
-                d = Wl[r];
-                Wl[r] = w;
-                El[r] = e;
-                u = w;
-                fu = f;
-            }
-            return make_int2(u, fu);
-        };
         // lane 31: this stripe's bottom row out, published every 32 columns
         auto row_out = [&](uint32_t col) {
             if (lane == 31 && outW && in_range((size_t)(outW - p.rows) + tk.nr + col, p.rows_cap, p.err, kSiteAffRing)) {
-                outW[col] = xout;
-                outF[col] = (uint32_t)fout;
+                outW[col] = ln.xout;
+                outF[col] = (uint32_t)ln.fout;
                 if (((col + 1) & 31u) == 0 || col + 1 == n) st_release(mine, col + 1);
             }
         };
 
         for (uint32_t t = 0; t < T && alive; ++t) {
             if ((t & 31u) == 0) {
+                if (KEEP && t && t % kTileSteps == 0) {
+                    ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
+                    keep += AffLane<R>::kParts * 32u;
+                }
                 stage = stage_next;
                 fstage = fstage_next;
                 if (s && t + 32 < n && !(alive = aff_wait(prev, min(t + 64u, n), p.err, jidx))) break;
-                stage_next = chunk_w(t + 32u + (uint32_t)lane);
-                fstage_next = chunk_f(t + 32u + (uint32_t)lane);
+                stage_next = above.w(t + 32u + (uint32_t)lane);
+                fstage_next = above.f(t + 32u + (uint32_t)lane);
                 if (__all_sync(kFull, c >= 0 && c + 32 <= (int32_t)n - 1)) {
-                    uint32_t cc = (uint32_t)c % CPW;
-                    uint32_t *prow = PTR ? pbase + (size_t)(s * 32u + lane) * tk.ncg : nullptr;
 #pragma unroll 4
                     for (uint32_t uu = 0; uu < 32u; ++uu) {
-                        uint32_t x = __shfl_up_sync(kFull, xout, 1);
-                        int32_t fx = __shfl_up_sync(kFull, fout, 1);
+                        uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                        int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
                         const uint32_t x0 = __shfl_sync(kFull, stage, uu);
                         const int32_t f0 = __shfl_sync(kFull, fstage, uu);
                         if (lane == 0) {
                             x = x0;
                             fx = f0;
                         }
-                        const int32_t up = (int32_t)x >> 2;
-                        const int2 o = column(dtop, up, fx, sext_selector(x & 3u));
-                        dtop = up;
-                        xout = ((uint32_t)o.x << 2) | (x & 3u);
-                        fout = o.y;
-                        const uint32_t col = (uint32_t)c + uu;
-                        if constexpr (PTR) {
-                            if (cc == CPW - 1 &&
-                                in_range((uint64_t)(prow - p.ptr) + col / CPW, p.ext_off, p.err, kSiteAffPtr)) {
-                                prow[col / CPW] = ptr_word(accL, accH);
-                                prow[p.ext_off + col / CPW] = ptr_word(accF, accE);
-                            }
-                            cc = (cc + 1) & (CPW - 1);
-                        }
-                        row_out(col);
+                        ln.template column<false>(go, x, fx);
+                        row_out((uint32_t)c + uu);
                     }
                     c += 32;
                     t += 31;
                     continue;
                 }
             }
-            uint32_t x = __shfl_up_sync(kFull, xout, 1);
-            int32_t fx = __shfl_up_sync(kFull, fout, 1);
+            uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+            int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
             const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
             const int32_t f0 = __shfl_sync(kFull, fstage, t & 31u);
             if (lane == 0) {
@@ -258,28 +315,13 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
                 fx = f0;
             }
             if (c >= 0 && c < (int32_t)n) {
-                const int32_t up = (int32_t)x >> 2;
-                const int2 o = column(dtop, up, fx, sext_selector(x & 3u));
-                dtop = up;
-                xout = ((uint32_t)o.x << 2) | (x & 3u);
-                fout = o.y;
-                if constexpr (PTR) {
-                    const uint32_t cc = (uint32_t)c % CPW;
-                    if (cc == CPW - 1 || c == (int32_t)n - 1) {
-                        const uint32_t miss = (CPW - 1 - cc) * R;
-                        const size_t wi = (size_t)(s * 32u + lane) * tk.ncg + (uint32_t)c / CPW;
-                        if (in_range(tk.ptr_off + wi, p.ext_off, p.err, kSiteAffPtr)) {
-                            pbase[wi] = ptr_word(accL << miss, accH << miss);
-                            pbase[p.ext_off + wi] = ptr_word(accF << miss, accE << miss);
-                        }
-                    }
-                }
+                ln.template column<false>(go, x, fx);
                 row_out((uint32_t)c);
                 if (s + 1 == S && (uint32_t)lane == lM && c == (int32_t)n - 1) {
                     int32_t wmn = 0;
 #pragma unroll
                     for (int r = 0; r < R; ++r)
-                        if ((uint32_t)r == rM) wmn = Wl[r];
+                        if ((uint32_t)r == rM) wmn = ln.Wl[r];
                     if (in_range(tk.out, p.out_cap, p.err, kSiteAffScore))
                         p.scores[tk.out] = wmn + p.ge * (int32_t)(m + n);
                 }
@@ -291,59 +333,143 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
     }
 }
 
-// The state-machine walk from (m, n), one thread per pair: in state H the
-// diagonal when L is clear, else the vertical gap (F) when H is clear, else
-// the horizontal one (E); in a gap state the move is emitted and the walk
-// stays in the gap while the cell's extension bit is set.  Row 0 / column
-// 0: only horizontal / vertical moves remain.  Moves in reverse order (0
-// diagonal, 1 vertical, 2 horizontal).
+// The four bits of a column's R cells as one word: fields L, H, F, E of 8
+// bits (R <= 8) or 16 (R = 16), row r at bit R - 1 - r of each field.
 template <int R>
-__global__ void k_affine_walk(const AffTask *tasks, uint32_t ntasks, const uint32_t *ptr, uint64_t ext_off,
-                              uint8_t *moves, const uint64_t *move_off, uint64_t *nmoves, uint32_t *err) {
-    constexpr uint32_t SH = 32u * R, CPW = 16u / R;
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < ntasks; q += gridDim.x * blockDim.x) {
-        const AffTask tk = tasks[q];
-        const uint32_t *pw = ptr + tk.ptr_off;
+struct AffBits {
+    using Word = uint32_t;
+    __device__ static __forceinline__ Word pack(uint32_t L, uint32_t H, uint32_t F, uint32_t E) {
+        return __byte_perm(__byte_perm(L, H, 0x0040), __byte_perm(F, E, 0x0040), 0x5410);
+    }
+    __device__ static __forceinline__ uint32_t bit(Word w, uint32_t field, uint32_t r) {
+        return (w >> (8u * field + (uint32_t)R - 1u - r)) & 1u;
+    }
+};
+template <>
+struct AffBits<16> {
+    using Word = uint2;
+    __device__ static __forceinline__ Word pack(uint32_t L, uint32_t H, uint32_t F, uint32_t E) {
+        return make_uint2(__byte_perm(L, H, 0x5410), __byte_perm(F, E, 0x5410));
+    }
+    __device__ static __forceinline__ uint32_t bit(Word w, uint32_t field, uint32_t r) {
+        return ((field < 2 ? w.x : w.y) >> (16u * (field & 1u) + 15u - r)) & 1u;
+    }
+};
+
+// The walk from (m, n), one warp per pair, longest pairs first.  The state
+// machine: in state H the diagonal when L is clear, else the vertical gap (F)
+// when H is clear, else the horizontal one (E); in a gap state the move is
+// emitted and the walk stays in the gap while the cell's extension bit is
+// set.  Row 0 / column 0: only horizontal / vertical moves remain.  Moves in
+// reverse order (0 diagonal, 1 vertical, 2 horizontal).  In state H the warp
+// takes a run of diagonal moves at a time: lane q reads the cell q diagonal
+// moves on, a ballot of the L bits gives the run.
+//
+// A cell of lane l and column c belongs to step c + l of its stripe; a tile
+// holds kTileSteps steps, from a kept state on, and the path's steps only
+// fall, so each tile is recomputed once, up to the step of the path's entry.
+template <int R>
+__global__ void __launch_bounds__(32) k_affine_trace(AffArgs p, uint32_t ntasks, uint8_t *moves,
+                                                     const uint64_t *move_off, uint64_t *nmoves) {
+    using Bits = AffBits<R>;
+    constexpr uint32_t SH = 32u * R;
+    __shared__ typename Bits::Word tile[kTileSteps * 32];  // [step][lane]
+    const uint32_t lane = threadIdx.x;
+    const int32_t go = p.go;
+    for (uint32_t q = blockIdx.x; q < ntasks; q += gridDim.x) {
+        const AffTask tk = p.tasks[q];
+        const uint32_t m = tk.m, n = tk.n;
         uint8_t *mv = moves + move_off[q];
-        uint32_t i = tk.m, j = tk.n;
+        uint32_t i = m, j = n, state = 0;   // state: 0 H, 1 F (vertical gap), 2 E (horizontal gap)
         uint64_t k = 0;
-        int state = 0;   // 0 H, 1 F (vertical gap), 2 E (horizontal gap)
         while (i > 0 && j > 0) {
-            if (!in_range(k, (uint64_t)tk.m + tk.n, err, kSiteAffMoves)) break;
-            const uint32_t i1 = i - 1, j1 = j - 1;
-            const size_t wi = (size_t)((i1 / SH) * 32u + (i1 % SH) / R) * tk.ncg + j1 / CPW;
-            const uint32_t o = (j1 % CPW) * R + (i1 % R);
-            if (state == 0) {
-                const uint32_t word = __ldg(pw + wi);
-                if (!((word >> (31u - o)) & 1u)) {
-                    mv[k++] = 0;
-                    --i;
-                    --j;
-                    continue;
+            // the tile of cell (i, j)
+            const uint32_t s = (i - 1) / SH, tc = (j - 1) + ((i - 1) % SH) / R, t0 = tc - tc % kTileSteps;
+            const uint32_t *inW = s ? p.rows + tk.row_off + (size_t)(s - 1) * 2 * tk.nr : nullptr;
+            const AffAbove above{p.pool + tk.b_off, inW, s ? inW + tk.nr : nullptr, n, go};
+            AffLane<R> ln;
+            const uint32_t i0 = s * SH + lane * R;
+            uint32_t stage = 0, stage_next = above.w(t0 + lane);
+            int32_t fstage = kAffNeg, fstage_next = above.f(t0 + lane);
+            ln.rows(p, p.pool + tk.a_off, i0, m);
+            if (t0)
+                ln.load(p.keep + tk.keep_off +
+                        ((uint64_t)s * tk.keep_n + (t0 / kTileSteps - 1)) * AffLane<R>::kParts * 32u + lane);
+            else
+                ln.start(go, i0);
+            ln.accL = ln.accH = ln.accF = ln.accE = 0;
+            __syncwarp();
+            for (uint32_t t = t0; t <= tc; ++t) {
+                if ((t & 31u) == 0) {
+                    stage = stage_next;
+                    fstage = fstage_next;
+                    stage_next = above.w(t + 32u + lane);
+                    fstage_next = above.f(t + 32u + lane);
                 }
-                state = ((word >> (15u - o)) & 1u) ? 2 : 1;
+                uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
+                const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
+                const int32_t f0 = __shfl_sync(kFull, fstage, t & 31u);
+                if (lane == 0) {
+                    x = x0;
+                    fx = f0;
+                }
+                if (t >= lane && t - lane < n) {
+                    ln.template column<true>(go, x, fx);
+                    tile[(t - t0) * 32u + lane] = Bits::pack(ln.accL, ln.accH, ln.accF, ln.accE);
+                }
             }
-            const uint32_t ext = __ldg(pw + ext_off + wi);
-            if (state == 1) {
-                mv[k++] = 1;
-                state = ((ext >> (31u - o)) & 1u) ? 1 : 0;
-                --i;
-            } else {
-                mv[k++] = 2;
-                state = ((ext >> (15u - o)) & 1u) ? 2 : 0;
-                --j;
+            __syncwarp();
+            // (uniform over the warp from here: every lane follows the same walk)
+            auto step_of = [&](uint32_t i_, uint32_t j_) { return (j_ - 1) + ((i_ - 1) % SH) / R; };
+            for (;;) {
+                if (i == 0 || j == 0 || (i - 1) / SH != s || step_of(i, j) < t0) break;
+                if (state == 0) {
+                    uint32_t stop = 1u, h = 0u;
+                    if (lane < i && lane < j) {
+                        const uint32_t iq = i - lane, jq = j - lane;
+                        if ((iq - 1) / SH == s && step_of(iq, jq) >= t0) {
+                            const uint32_t l = ((iq - 1) % SH) / R, r = (iq - 1) % R;
+                            const typename Bits::Word w = tile[(jq - 1 + l - t0) * 32u + l];
+                            stop = Bits::bit(w, 0, r);
+                            h = stop ? 2u + Bits::bit(w, 1, r) : 0u;  // the gap that ends the run, + 1
+                        }
+                    }
+                    const uint32_t b = __ballot_sync(kFull, stop);
+                    const uint32_t run = b ? (uint32_t)__ffs(b) - 1u : 32u;
+                    if (lane < run) mv[k + lane] = 0;
+                    k += run;
+                    i -= run;
+                    j -= run;
+                    h = __shfl_sync(kFull, h, run & 31u);
+                    if (run < 32u && h) state = h - 1u;
+                } else {
+                    const uint32_t l = ((i - 1) % SH) / R, r = (i - 1) % R;
+                    const typename Bits::Word w = tile[(j - 1 + l - t0) * 32u + l];
+                    if (lane == 0 && in_range(k, (uint64_t)m + n, p.err, kSiteAffMoves)) mv[k] = (uint8_t)state;
+                    ++k;
+                    if (state == 1) {
+                        state = Bits::bit(w, 2, r) ? 1u : 0u;
+                        --i;
+                    } else {
+                        state = Bits::bit(w, 3, r) ? 2u : 0u;
+                        --j;
+                    }
+                }
             }
         }
-        for (; j > 0; --j) mv[k++] = 2;
-        for (; i > 0; --i) mv[k++] = 1;
-        nmoves[q] = k;
+        const uint32_t rest = i + j;
+        const uint8_t mvr = i ? 1 : 2;
+        for (uint32_t x = lane; x < rest; x += 32) mv[k + x] = mvr;
+        if (lane == 0) nmoves[q] = k + rest;
+        __syncwarp();
     }
 }
 
-template <int R, bool PTR>
+template <int R, bool KEEP>
 int launch_affine_R(nw_ctx *ctx, AffArgs &aa) {
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_affine<R, PTR>, kAffWarps * 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_affine<R, KEEP>, kAffWarps * 32, 0);
     if (occ < 1) occ = 1;
     // every CTA resident: a job's warp may wait on an earlier job's warp
     uint32_t blocks = (uint32_t)occ * (uint32_t)ctx->sm_count;
@@ -354,13 +480,13 @@ int launch_affine_R(nw_ctx *ctx, AffArgs &aa) {
     if (rc) return rc;
     aa.counter = (uint32_t *)v;
     cudaMemsetAsync(aa.counter, 0, 4, ctx->stream);
-    LaunchTimer t(ctx, PTR ? "affine_fill_ptr" : "affine_score");
-    k_affine<R, PTR><<<blocks, kAffWarps * 32, 0, ctx->stream>>>(aa);
+    LaunchTimer t(ctx, KEEP ? "affine_fill_ptr" : "affine_score");
+    k_affine<R, KEEP><<<blocks, kAffWarps * 32, 0, ctx->stream>>>(aa);
     return NW_OK;
 }
 
-int launch_affine(nw_ctx *ctx, int R, bool ptr, AffArgs &aa) {
-    if (ptr) {
+int launch_affine(nw_ctx *ctx, int R, bool keep, AffArgs &aa) {
+    if (keep) {
         if (R == 4) return launch_affine_R<4, true>(ctx, aa);
         if (R == 16) return launch_affine_R<16, true>(ctx, aa);
         return launch_affine_R<8, true>(ctx, aa);
@@ -438,7 +564,8 @@ int affine_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const
     for (uint32_t k = 0; k < npairs; ++k) {
         AffTask &t = all[k];
         t = AffTask{a_off[k], b_off[k], a_len[k], b_len[k], k, 0, 0, 0, 0, 0};
-        if (want) t.ncg = ptr_words_per_lane_row(std::max(t.n, 1u), R);
+        // states before steps kTileSteps, 2 kTileSteps, .. of a stripe's n + 31
+        if (want && t.m && t.n) t.keep_n = (t.n + 30) / kTileSteps;
     }
     // longest pairs first: their stripe jobs start first
     std::stable_sort(all.begin(), all.end(), [](const AffTask &x, const AffTask &y) {
@@ -449,47 +576,45 @@ int affine_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const
         if ((rc = affine_jobs(ctx, all, R, aa))) return rc;
         return launch_affine(ctx, R, false, aa);
     }
-    // waves whose pointer words (two arrays) fit half the free budget
+    // waves whose kept states and stripe rows fit half the free budget
     const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
+    const uint32_t state_units = (2u * (uint32_t)R + 4u) / 4u * 32u;  // 16-byte units of a kept state
     size_t k0 = 0;
     while (k0 < all.size()) {
         std::vector<AffTask> wave;
         std::vector<uint64_t> moff;
-        uint64_t words = 0, mbytes = 0;
+        uint64_t units = 0, mbytes = 0, rbytes = 0;
         size_t k = k0;
         for (; k < all.size(); ++k) {
             AffTask t = all[k];
-            const uint64_t wds = (uint64_t)((t.m + SH - 1) / SH) * 32u * t.ncg;
-            if (!wave.empty() && (words + wds) * 8 > wave_budget) break;
-            t.ptr_off = words;
-            words += wds;
+            const uint64_t S = (t.m + SH - 1) / SH;
+            const uint64_t u = S * t.keep_n * state_units;
+            const uint64_t rb = S > 1 ? (S - 1) * 8 * (((uint64_t)t.n + 31) / 32 * 32) : 0;
+            if (!wave.empty() && (units + u) * 16 + rbytes + rb > wave_budget) break;
+            t.keep_off = units;
+            units += u;
+            rbytes += rb;
             moff.push_back(mbytes);
             mbytes += (uint64_t)t.m + t.n + 16;
             wave.push_back(t);
         }
         void *pv = nullptr, *mv = nullptr, *nm = nullptr;
-        if ((rc = scratch(ctx, "affine_ptr", words * 8 + 16, &pv))) return rc;
+        if ((rc = scratch(ctx, "affine_keep", units * 16 + 16, &pv))) return rc;
         if ((rc = scratch(ctx, "affine_moves", mbytes + 16, &mv))) return rc;
         if ((rc = scratch(ctx, "affine_nmoves", wave.size() * 8 + 16, &nm))) return rc;
         if ((rc = affine_jobs(ctx, wave, R, aa))) return rc;
         uint64_t *dmoff = nullptr;
         if ((rc = aff_upload(ctx, "affine_move_off", moff, &dmoff))) return rc;
-        aa.ptr = (uint32_t *)pv;
-        aa.ext_off = words;
+        aa.keep = (uint4 *)pv;
+        aa.keep_cap = units;
         if ((rc = launch_affine(ctx, R, true, aa))) return rc;
         {
             LaunchTimer t(ctx, "affine_walk");
-            const AffTask *dt = aa.tasks;
-            const uint32_t blocks = std::max<uint32_t>(1, ((uint32_t)wave.size() + 127) / 128);
-            if (R == 4)
-                k_affine_walk<4><<<blocks, 128, 0, ctx->stream>>>(dt, (uint32_t)wave.size(), (const uint32_t *)pv,
-                                                                  words, (uint8_t *)mv, dmoff, (uint64_t *)nm, ctx->d_err);
+            const uint32_t blocks = (uint32_t)std::min<size_t>(wave.size(), 65535), nt = (uint32_t)wave.size();
+            if (R == 4) k_affine_trace<4><<<blocks, 32, 0, ctx->stream>>>(aa, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
             else if (R == 16)
-                k_affine_walk<16><<<blocks, 128, 0, ctx->stream>>>(dt, (uint32_t)wave.size(), (const uint32_t *)pv,
-                                                                   words, (uint8_t *)mv, dmoff, (uint64_t *)nm, ctx->d_err);
-            else
-                k_affine_walk<8><<<blocks, 128, 0, ctx->stream>>>(dt, (uint32_t)wave.size(), (const uint32_t *)pv,
-                                                                  words, (uint8_t *)mv, dmoff, (uint64_t *)nm, ctx->d_err);
+                k_affine_trace<16><<<blocks, 32, 0, ctx->stream>>>(aa, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
+            else k_affine_trace<8><<<blocks, 32, 0, ctx->stream>>>(aa, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
         }
         std::vector<TraceTask> tt(wave.size());
         for (size_t q = 0; q < wave.size(); ++q) {

@@ -6,22 +6,33 @@
 // row-major order holding it and is walked back with the priority diagonal >
 // vertical > horizontal until a cell whose H is 0 (its start).
 //
-// Batched like the global kernel: one warp per pair, taken from an atomic
-// queue in descending cell order; lane k owns R rows of a 32R-row stripe
-// and walks the stripes back to back (lane 31 hands the stripe's bottom row
-// to lane 0 through a per-warp row buffer).  The floor rules out the W
-// domain of the global kernels (it would turn into a floor that grows along
-// every anti-diagonal), so the cell works on H itself: with m = max(H_up,
-// H_left), one cell is a byte permute (s), one max, one add (m + gap) and
-// one DPX add-max with ReLU, max(H_diag + s, m + gap, 0) -- the four
-// integer operations of the textbook cell.  Tracking the largest H costs
-// one more max per cell; when the end cell is wanted, each lane keeps per
-// row the largest H and the first column holding it (a DPX max that also
-// reports the comparison, and a select), folded into the lane's best when
-// the lane leaves the stripe.  Pointer bits are the global kernels' (L: the
-// diagonal candidate is below max(up, left) + gap; H: left above up), so
-// the walk reads them as usual and tracks H along the path to find the
-// start.
+// The floor rules out the W domain of the global kernels (it would turn into
+// a floor that grows along every anti-diagonal), so the cell works on H itself:
+// with m = max(H_up, H_left), one cell is a byte permute (s), one max, one add
+// (m + gap) and one DPX add-max with ReLU, max(H_diag + s, m + gap, 0), and
+// half a three-input max for the largest H.
+//
+// Batched by stripe jobs: every 32R-row stripe of every pair is one job, jobs
+// queued pair by pair (longest pairs first) and stripes in order, so a pair's
+// stripes run on several warps at once as a wavefront (one warp per pair left
+// the launch waiting on its longest pairs).  A warp takes the next job from an
+// atomic counter; lane k owns R rows of the stripe.  Lane 31 writes the
+// stripe's bottom row to the pair's row buffer and publishes every 32 columns
+// with a release store; the warp of the next stripe waits (a bounded spin) on
+// that word before it reads each chunk of 32 columns.  The job it waits on was
+// taken earlier by a warp of the same fully resident grid, so every wait ends.
+//
+// End cells and alignments.  The fill keeps no pointers and no positions: a
+// lane notes the chunk of 32 steps in which its rows first reached their
+// largest H (and whether another chunk reached it too), and every kTileSteps
+// steps the state of a stripe's lanes is kept.  The trace finds the pair's
+// best lane, recomputes the chunk (the whole stripe when several chunks tie) for
+// the first cell in row-major order, and walks back from it tile by tile -- a
+// tile is one stripe and the steps between two kept states -- recomputing only
+// the tiles the path crosses with the two pointer bits in shared memory (L:
+// the diagonal candidate is below max(up, left) + gap; H: left above up), and
+// tracking H along the path to find the start.  Pointers and positions for
+// every cell cost the fill 11 operations per cell, against 4.5.
 #include <algorithm>
 #include <vector>
 
@@ -31,32 +42,55 @@ namespace nw {
 namespace {
 
 constexpr int kLocalWarps = 8;
-constexpr uint32_t kLocalMinPeriod = 96;   // ring reuse distance (see the stripe hand-off)
+constexpr uint32_t kLocalMinPeriod = 96;   // columns a stripe counts at least (the limit on a pair's size)
+constexpr uint32_t kTileSteps = 128;       // steps between a stripe's kept states
 constexpr uint32_t kPadProfile = 0x80808080u;  // rows past the end: s = -128, never above a real row
 
 struct LocalTask {
     uint64_t a_off, b_off;
     uint32_t m, n;
     uint32_t out;        // pair index
-    uint32_t ncg;        // pointer words per lane row
-    uint64_t ptr_off;    // word offset of the pair's pointer words
+    uint32_t job0;       // its first stripe job
+    uint32_t nr;         // words per stripe row (n rounded up to 32)
+    uint32_t keep_n;     // kept states per stripe
+    uint64_t row_off;    // word offset of the pair's stripe rows
+    uint64_t keep_off;   // 16-byte units: its kept states, [stripe][state 1..][part][lane]
 };
+
+struct LocalJob {
+    uint32_t task, stripe;
+};
+
+// The largest H of a stripe: the first lane that reached it, the first chunk of
+// 32 steps in which it did, and whether the lane reached it in another too.
+struct LocalBest {
+    int32_t v;
+    uint32_t lane, t0, tie;
+};
+
+// What a launch produces: the scores alone, also the stripes' best lanes
+// (end cells), or also the kept states and all rows (alignments).
+enum LocalMode { kScore = 0, kEnds = 1, kKeep = 2 };
 
 struct LocalArgs {
     const uint8_t *pool;
     const LocalTask *tasks;
-    uint32_t ntasks;
+    const LocalJob *jobs;
+    uint32_t njobs;
     uint32_t *counter;
     uint32_t prof[4];    // byte d of prof[c] = s(c, d) as int8
-    int32_t gap;
-    uint32_t *ring;
-    uint32_t ring_stride;
+    int32_t match, mismatch, gap;
+    uint32_t *rows;      // stripe rows (H << 2 | base code): all of a pair's, or two in turn (turn)
+    uint32_t turn;
+    uint64_t rows_cap;
+    uint32_t *progress;  // per job: columns of its bottom row published
+    LocalBest *best;     // per job
     int32_t *scores;     // [out]
-    uint32_t *ends;      // [4*out]: i_start, j_start, i_end, j_end (POS)
-    uint32_t *ptr;
+    uint32_t *ends;      // [4*out]: i_start, j_start, i_end, j_end
+    uint4 *keep;
+    uint64_t keep_cap;
     uint32_t *err;
-    uint64_t ptr_cap;    // words at ptr, pairs at scores / ends (checked build)
-    uint32_t out_cap;
+    uint32_t out_cap;    // pairs at scores / ends (checked build)
 };
 
 template <int R>
@@ -73,103 +107,77 @@ __device__ __forceinline__ uint32_t rows_codes(const uint8_t *s, uint32_t i0, ui
     return w;
 }
 
-__device__ __forceinline__ void st_if(bool p, uint32_t *dst, uint32_t v) {
-    asm volatile("{.reg .pred q; setp.ne.b32 q, %0, 0; @q st.global.u32 [%1], %2;}" ::"r"((uint32_t)p), "l"(dst), "r"(v)
-                 : "memory");
+// Warp-uniform bounded wait until *flag >= target (lane 0 spins; then every
+// lane acquires, so its following loads see what the producer published).
+__device__ __forceinline__ bool local_wait(const uint32_t *flag, uint32_t target, uint32_t *err, uint32_t where) {
+    int ok = 1;
+    if ((threadIdx.x & 31) == 0) ok = wait_geq(flag, target, err, where) ? 1 : 0;
+    ok = __shfl_sync(kFull, ok, 0);
+    if (ok) (void)ld_acquire(flag);
+    return ok != 0;
 }
 
-// (v, i, j) beats (v2, i2, j2): larger value, then smaller row, then column.
-__device__ __forceinline__ bool first_max(int32_t v, uint32_t i, uint32_t j, int32_t v2, uint32_t i2, uint32_t j2) {
-    return v > v2 || (v == v2 && (i < i2 || (i == i2 && j < j2)));
-}
+// A lane's R rows of a stripe: the systolic state between two steps.
+template <int R>
+struct LocalLane {
+    static constexpr uint32_t kParts = (R + 5) / 4;  // 16-byte parts of a kept state
+    uint32_t prof[R];
+    int32_t Hl[R];
+    int32_t dtop;        // H of the row above the lane's first, one column back
+    uint32_t xout;       // the last row's H (<< 2) and the column's base code, for the lane below
+    uint32_t accL, accH;
 
-template <int R, bool PTR, bool POS>
-__global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
-    constexpr uint32_t SH = 32u * R;
-    constexpr uint32_t CPW = PTR ? 16u / R : 1u;
-    constexpr int RT = POS ? R : 1;
-    const int lane = threadIdx.x & 31;
-    const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint32_t *ring = p.ring + (size_t)gw * p.ring_stride;
-    const int32_t g = p.gap;
-    const uint32_t P0 = p.prof[0], P1 = p.prof[1], P2 = p.prof[2], P3 = p.prof[3];
-
-    for (;;) {
-        uint32_t idx = 0;
-        if (lane == 0) idx = atomicAdd(p.counter, 1u);
-        idx = __shfl_sync(kFull, idx, 0);
-        if (idx >= p.ntasks) break;
-        const LocalTask tk = p.tasks[idx];
-        const uint8_t *A = p.pool + tk.a_off;
-        const uint8_t *B = p.pool + tk.b_off;
-        const uint32_t m = tk.m, n = tk.n;
-        if (m == 0 || n == 0) {
-            if (lane == 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
-                p.scores[tk.out] = 0;
-                if (POS)
-                    for (int q = 0; q < 4; ++q) p.ends[4 * (size_t)tk.out + q] = (PTR || q >= 2) ? 0u : ~0u;
-            }
-            continue;
+    __device__ __forceinline__ void rows(const LocalArgs &p, const uint8_t *A, uint32_t i0, uint32_t m) {
+        const uint32_t codes = rows_codes<R>(A, i0, m);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const uint32_t c = (codes >> (2 * r)) & 3u;
+            prof[r] = i0 + r >= m ? kPadProfile
+                                  : c == 0 ? p.prof[0] : c == 1 ? p.prof[1] : c == 2 ? p.prof[2] : p.prof[3];
         }
-        const uint32_t S = (m + SH - 1) / SH;
-        const uint32_t P = max(n, kLocalMinPeriod);
-        const uint32_t T = S * P + 31;
-        uint32_t *pbase = PTR ? p.ptr + tk.ptr_off : nullptr;
-
-        uint32_t prof[R];
-        int32_t Hl[R];
-        int32_t rbest[RT];
-        uint32_t rcol[RT];
-        int32_t best = 0;            // the lane's largest H so far
-        uint32_t bi = 0, bj = 0;     // POS: its cell (row-major first)
-        int32_t dtop = 0;
-        uint32_t xout = 0, accL = 0, accH = 0;
-        auto init_rows = [&](uint32_t codes, uint32_t st) {
-            const uint32_t i0 = st * SH + (uint32_t)lane * R;
+    }
+    __device__ __forceinline__ void start() {  // column 0
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const uint32_t c = (codes >> (2 * r)) & 3u;
-                prof[r] = i0 + r >= m ? kPadProfile : c == 0 ? P0 : c == 1 ? P1 : c == 2 ? P2 : P3;
-                Hl[r] = 0;                          // column 0
-            }
+        for (int r = 0; r < R; ++r) Hl[r] = 0;
+        dtop = 0;
+        xout = 0;
+    }
+    __device__ __forceinline__ void save(uint4 *k, uint64_t cap_left, uint32_t *err) const {
+        uint32_t v[4 * kParts] = {};
 #pragma unroll
-            for (int r = 0; r < RT; ++r) {
-                rbest[r] = 0;
-                rcol[r] = 0;
-            }
-            dtop = 0;
-        };
-        // POS: the rows of stripe st (rows past m excluded) into the lane's
-        // best; rows in order, so an earlier row keeps a tie
-        auto fold = [&](uint32_t st) {
-            if constexpr (POS) {
-                const uint32_t i0 = st * SH + (uint32_t)lane * R;
+        for (int r = 0; r < R; ++r) v[r] = (uint32_t)Hl[r];
+        v[R] = (uint32_t)dtop;
+        v[R + 1] = xout;
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-                    if (i0 + r < m && rbest[r] > best) {
-                        best = rbest[r];
-                        bi = i0 + r + 1;
-                        bj = rcol[r] + 1;
-                    }
-            }
-        };
-        init_rows(rows_codes<R>(A, (uint32_t)lane * R, m), 0);
-        uint32_t next_rows = S > 1 ? rows_codes<R>(A, SH + (uint32_t)lane * R, m) : 0u;
-        int32_t c = -lane;
-        uint32_t s = 0;
-        // lane 0's input for global index gi: row 0 (H = 0) in stripe 0, the
-        // previous stripe's bottom row (written by lane 31 at least P - 94
-        // steps earlier, past the fences below) in later stripes
-        auto chunk_word = [&](uint32_t gi) -> uint32_t {
-            const uint32_t sg = gi / P, tg = gi - sg * P;
-            if (sg >= S || tg >= n) return 0u;
-            if (sg == 0) return base_at(B, tg);
-            return __ldcg(ring + tg);
-        };
-        uint32_t stage = 0, stage_next = chunk_word((uint32_t)lane);
-
-        // one cell: returns H, appends pointer bits, tracks the maxima
-        auto cell = [&](int r, int32_t d, int32_t u, uint32_t sel, int32_t col) -> int32_t {
+        for (uint32_t q = 0; q < kParts; ++q)
+            if (in_range(q * 32u, cap_left, err, kSiteLocalPtr))
+                __stcg(k + q * 32u, make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+    }
+    __device__ __forceinline__ void load(const uint4 *k) {
+        uint32_t v[4 * kParts];
+#pragma unroll
+        for (uint32_t q = 0; q < kParts; ++q) {
+            const uint4 x = __ldcg(k + q * 32u);
+            v[4 * q] = x.x;
+            v[4 * q + 1] = x.y;
+            v[4 * q + 2] = x.z;
+            v[4 * q + 3] = x.w;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) Hl[r] = (int32_t)v[r];
+        dtop = (int32_t)v[R];
+        xout = v[R + 1];
+    }
+    // The R cells of one column from the row above's word x (H << 2 | code);
+    // cm takes the largest H.  PTR appends the two bits of each cell to the
+    // accumulators (the last R bits of each are this column's, row 0 highest).
+    template <bool PTR>
+    __device__ __forceinline__ void column(int32_t g, uint32_t x, int32_t &cm) {
+        const uint32_t sel = sext_selector(x & 3u);
+        int32_t u = (int32_t)x >> 2, d = dtop;
+        dtop = u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
             const int32_t sv = (int32_t)prmt(prof[r], 0u, sel);
             const int32_t l = Hl[r];
             const int32_t mg = max(u, l) + g;
@@ -177,201 +185,371 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
             if constexpr (PTR) {
                 accL = ptr_append(accL, d + sv - mg);
                 accH = ptr_append(accH, u - l);
+            } else if (r & 1) {
+                cm = __vimax3_s32(cm, u, w);
             }
-            if constexpr (POS) {
-                bool keep;
-                rbest[r] = __vibmax_s32(rbest[r], w, &keep);
-                rcol[r] = keep ? rcol[r] : (uint32_t)col;
-            } else {
-                best = max(best, w);
-            }
-            return w;
-        };
+            d = l;
+            Hl[r] = w;
+            u = w;
+        }
+        xout = ((uint32_t)u << 2) | (x & 3u);
+    }
+};
 
-        for (uint32_t t = 0; t < T; ++t) {
+// Lane 0's inputs for the columns of a stripe: row 0 (H = 0) for stripe 0,
+// else the bottom row of the stripe above.
+struct LocalAbove {
+    const uint8_t *B;
+    const uint32_t *in;  // null for stripe 0
+    uint32_t n;
+    __device__ __forceinline__ uint32_t word(uint32_t col) const {
+        if (col >= n) return 0u;
+        return in ? __ldcg(in + col) : base_at(B, col);
+    }
+};
+
+// The fill.  What bounds it: the logic pipe, 3.5 operations per cell (prmt,
+// max, add-max, half a max3; the add runs on either pipe) and about ten per
+// column of R cells.
+template <int R, int MODE>
+__global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
+    constexpr uint32_t SH = 32u * R;
+    const int lane = threadIdx.x & 31;
+    const int32_t g = p.gap;
+
+    for (;;) {
+        uint32_t jidx = 0;
+        if (lane == 0) jidx = atomicAdd(p.counter, 1u);
+        jidx = __shfl_sync(kFull, jidx, 0);
+        if (jidx >= p.njobs) break;
+        const LocalJob jb = p.jobs[jidx];
+        const LocalTask tk = p.tasks[jb.task];
+        const uint32_t s = jb.stripe, m = tk.m, n = tk.n;
+        if (m == 0 || n == 0) {  // a single job: the score stays 0
+            if (MODE != kScore && lane == 0) p.best[jidx] = LocalBest{0, 0u, 0u, 0u};
+            continue;
+        }
+        const uint32_t S = (m + SH - 1) / SH;
+        const uint32_t T = n + 31;
+        // rows: all kept, or two in turn (the stripe below has read a column
+        // of the row before this one when this stripe's successor overwrites it)
+        auto row = [&](uint32_t q) { return p.rows + tk.row_off + (size_t)(p.turn ? q & 1u : q) * tk.nr; };
+        const uint32_t *in = s ? row(s - 1) : nullptr;
+        uint32_t *out = s + 1 < S ? row(s) : nullptr;
+        const uint32_t *prev = s ? p.progress + (jidx - 1) : nullptr;  // stripe s-1 is the job before
+        uint32_t *mine = p.progress + jidx;
+        const LocalAbove above{p.pool + tk.b_off, in, n};
+        LocalLane<R> ln;
+        const uint32_t i0 = s * SH + (uint32_t)lane * R;
+        ln.rows(p, p.pool + tk.a_off, i0, m);
+        ln.start();
+        uint4 *keep = MODE == kKeep ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * LocalLane<R>::kParts * 32u + lane
+                                    : nullptr;
+        int32_t best = 0, cm = 0;    // the lane's largest H before and in this chunk of 32 steps
+        uint32_t bt = 0, tie = 0;    // the chunk that first reached it, and whether another did
+        auto chunk_end = [&](uint32_t t) {
+            if (MODE != kScore) {
+                if (cm > best) {
+                    bt = t - 32u;
+                    tie = 0;
+                } else if (cm == best) {
+                    tie = 1u;
+                }
+                best = max(best, cm);
+                cm = 0;
+            }
+        };
+        int32_t c = -lane;
+        bool alive = !s || local_wait(prev, min(32u, n), p.err, jidx);
+        uint32_t stage = 0, stage_next = alive ? above.word((uint32_t)lane) : 0u;
+        auto row_out = [&](uint32_t col) {
+            if (lane == 31 && out && in_range((size_t)(out - p.rows) + col, p.rows_cap, p.err, kSiteLocalRing)) {
+                out[col] = ln.xout;
+                if (((col + 1) & 31u) == 0 || col + 1 == n) st_release(mine, col + 1);
+            }
+        };
+        uint32_t t = 0;
+        for (; t < T && alive; ++t) {
             if ((t & 31u) == 0) {
+                if (t) chunk_end(t);
+                if (MODE == kKeep && t && t % kTileSteps == 0) {
+                    ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
+                    keep += LocalLane<R>::kParts * 32u;
+                }
                 stage = stage_next;
-                __threadfence_block();
-                __syncwarp();
-                stage_next = chunk_word(t + 32u + (uint32_t)lane);
-                // 32 steps with every lane inside its stripe, short of its
-                // last column: no activity test, stripe change or flush
-                if (__all_sync(kFull, c >= 0 && s < S && c + 32 <= (int32_t)n - 1)) {
-                    const bool ring_out = lane == 31 && s + 1 < S;
-                    uint32_t cc = (uint32_t)c % CPW;
-                    uint32_t *prow = PTR ? pbase + (size_t)(s * 32u + lane) * tk.ncg : nullptr;
+                if (s && t + 32 < n && !(alive = local_wait(prev, min(t + 64u, n), p.err, jidx))) break;
+                stage_next = above.word(t + 32u + (uint32_t)lane);
+                if (__all_sync(kFull, c >= 0 && c + 32 <= (int32_t)n - 1)) {
 #pragma unroll 4
-                    for (uint32_t u = 0; u < 32u; ++u) {
-                        uint32_t x = __shfl_up_sync(kFull, xout, 1);
-                        const uint32_t x0 = __shfl_sync(kFull, stage, u);
+                    for (uint32_t uu = 0; uu < 32u; ++uu) {
+                        uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                        const uint32_t x0 = __shfl_sync(kFull, stage, uu);
                         if (lane == 0) x = x0;
-                        const int32_t up = (int32_t)x >> 2;
-                        const uint32_t sel = sext_selector(x & 3u);
-                        const int32_t col = c + (int32_t)u;
-                        int32_t d = dtop, uv = up;
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            const int32_t w = cell(r, d, uv, sel, col);
-                            d = Hl[r];
-                            Hl[r] = w;
-                            uv = w;
-                        }
-                        dtop = up;
-                        xout = ((uint32_t)uv << 2) | (x & 3u);
-                        if constexpr (PTR) {
-                            if (cc == CPW - 1 && in_range((uint64_t)(prow - p.ptr) + (uint32_t)col / CPW, p.ptr_cap,
-                                                          p.err, kSiteLocalPtr))
-                                prow[(uint32_t)col / CPW] = ptr_word(accL, accH);
-                            cc = (cc + 1) & (CPW - 1);
-                        }
-                        st_if(ring_out && in_range((uint64_t)col, p.ring_stride, p.err, kSiteLocalRing), ring + col,
-                              xout);
+                        ln.template column<false>(g, x, cm);
+                        row_out((uint32_t)c + uu);
                     }
                     c += 32;
                     t += 31;
                     continue;
                 }
             }
-            uint32_t x = __shfl_up_sync(kFull, xout, 1);
+            uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
             const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
             if (lane == 0) x = x0;
-            const bool act = c >= 0 && c < (int32_t)n && s < S;
-            if (act) {
-                const int32_t up = (int32_t)x >> 2;
-                const uint32_t sel = sext_selector(x & 3u);
-                int32_t d = dtop, uv = up;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int32_t w = cell(r, d, uv, sel, c);
-                    d = Hl[r];
-                    Hl[r] = w;
-                    uv = w;
-                }
-                dtop = up;
-                xout = ((uint32_t)uv << 2) | (x & 3u);
-                if constexpr (PTR) {
-                    const uint32_t cc = (uint32_t)c % CPW;
-                    if (cc == CPW - 1 || c == (int32_t)n - 1) {
-                        const uint32_t miss = (CPW - 1 - cc) * R;  // cells a row's last word lacks
-                        const size_t wi = (size_t)(s * 32u + lane) * tk.ncg + (uint32_t)c / CPW;
-                        if (in_range(tk.ptr_off + wi, p.ptr_cap, p.err, kSiteLocalPtr))
-                            pbase[wi] = ptr_word(accL << miss, accH << miss);
-                    }
-                }
-                if (lane == 31 && s + 1 < S && in_range((uint64_t)c, p.ring_stride, p.err, kSiteLocalRing))
-                    ring[c] = xout;
+            if (c >= 0 && c < (int32_t)n) {
+                ln.template column<false>(g, x, cm);
+                row_out((uint32_t)c);
             }
-            if (++c == (int32_t)P) {
-                fold(s);
-                c = 0;
-                ++s;
-                if (s < S) {
-                    init_rows(next_rows, s);
-                    next_rows = s + 1 < S ? rows_codes<R>(A, (s + 1) * SH + (uint32_t)lane * R, m) : 0u;
-                }
+            ++c;
+        }
+        if (!alive) return;   // a wait gave up (NW_ERR_TIMEOUT is raised): leave
+        chunk_end((t + 31u) / 32u * 32u);
+        if (MODE == kScore) best = cm;
+        // the stripe's largest H and its first lane
+        const int32_t top = __reduce_max_sync(kFull, best);
+        if (lane == 0 && top > 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) atomicMax(p.scores + tk.out, top);
+        if (MODE != kScore) {
+            const uint32_t first = (uint32_t)__ffs(__ballot_sync(kFull, best == top)) - 1u;
+            if ((uint32_t)lane == first) p.best[jidx] = LocalBest{top, first, bt, tie};
+        }
+        __syncwarp();
+    }
+}
+
+// The two bits of a column's R cells: fields L, H of 8 bits (R <= 8) or 16.
+template <int R>
+struct LocalBits {
+    using Word = uint16_t;
+    __device__ static __forceinline__ Word pack(uint32_t L, uint32_t H) { return (Word)__byte_perm(L, H, 0x0040); }
+    __device__ static __forceinline__ uint32_t bit(Word w, uint32_t field, uint32_t r) {
+        return ((uint32_t)w >> (8u * field + (uint32_t)R - 1u - r)) & 1u;
+    }
+};
+template <>
+struct LocalBits<16> {
+    using Word = uint32_t;
+    __device__ static __forceinline__ Word pack(uint32_t L, uint32_t H) { return __byte_perm(L, H, 0x5410); }
+    __device__ static __forceinline__ uint32_t bit(Word w, uint32_t field, uint32_t r) {
+        return (w >> (16u * field + 15u - r)) & 1u;
+    }
+};
+
+// A stripe's lanes again, from step t0 (a kept state, or its start) on.
+template <int R>
+struct LocalReplay {
+    LocalLane<R> ln;
+    LocalAbove above;
+    uint32_t t, stage, stage_next;
+    __device__ void begin(const LocalArgs &p, const LocalTask &tk, uint32_t s, uint32_t t0, uint32_t lane) {
+        constexpr uint32_t SH = 32u * R;
+        const uint32_t in = p.turn ? (s - 1) & 1u : s - 1;
+        above = LocalAbove{p.pool + tk.b_off, s ? p.rows + tk.row_off + (size_t)in * tk.nr : nullptr, tk.n};
+        t = t0;
+        stage = 0;
+        stage_next = above.word(t0 + lane);
+        ln.rows(p, p.pool + tk.a_off, s * SH + lane * R, tk.m);
+        ln.accL = ln.accH = 0;
+        if (t0)
+            ln.load(p.keep + tk.keep_off +
+                    ((uint64_t)s * tk.keep_n + (t0 / kTileSteps - 1)) * LocalLane<R>::kParts * 32u + lane);
+        else
+            ln.start();
+    }
+    // one step; whether the lane had a column
+    template <bool PTR>
+    __device__ __forceinline__ bool step(int32_t g, uint32_t lane) {
+        if ((t & 31u) == 0) {
+            stage = stage_next;
+            stage_next = above.word(t + 32u + lane);
+        }
+        uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+        const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
+        if (lane == 0) x = x0;
+        const bool act = t >= lane && t - lane < above.n;
+        int32_t cm = 0;
+        if (act) ln.template column<PTR>(g, x, cm);
+        ++t;
+        return act;
+    }
+};
+
+// End cells and, with WALK, the walk back from them: one warp per pair,
+// longest pairs first.  WALK follows the path to the first cell whose H is 0;
+// moves in reverse order (0 diagonal, 1 vertical, 2 horizontal).  A run of
+// diagonal moves is taken at a time: lane q reads the cell q diagonal moves
+// on, and H there follows from the matches before it (a ballot).  Without
+// WALK no states are kept: a stripe is replayed from its start.
+template <int R, bool WALK>
+__global__ void __launch_bounds__(32) k_local_trace(LocalArgs p, uint32_t ntasks, uint8_t *moves,
+                                                    const uint64_t *move_off, uint64_t *nmoves) {
+    using Bits = LocalBits<R>;
+    constexpr uint32_t SH = 32u * R;
+    __shared__ typename Bits::Word tile[WALK ? kTileSteps * 32 : 1];  // [step][lane]
+    const uint32_t lane = threadIdx.x;
+    for (uint32_t q = blockIdx.x; q < ntasks; q += gridDim.x) {
+        const LocalTask tk = p.tasks[q];
+        const uint32_t m = tk.m, n = tk.n, S = (m && n) ? (m + SH - 1) / SH : 1u;
+        // the first stripe with the largest H
+        int32_t bv = 0;
+        uint32_t bs = 0;
+        for (uint32_t s0 = 0; s0 < S; s0 += 32) {
+            const int32_t v = s0 + lane < S ? p.best[tk.job0 + s0 + lane].v : 0;
+            const int32_t top = __reduce_max_sync(kFull, v);
+            if (top > bv) {
+                bv = top;
+                bs = s0 + (uint32_t)__ffs(__ballot_sync(kFull, v == top)) - 1u;
             }
         }
-        // the pair's largest H (and its first cell) over the warp
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            const int32_t v2 = __shfl_xor_sync(kFull, best, o);
-            const uint32_t i2 = __shfl_xor_sync(kFull, bi, o), j2 = __shfl_xor_sync(kFull, bj, o);
-            if (POS ? first_max(v2, i2, j2, best, bi, bj) : v2 > best) {
-                best = v2;
-                bi = i2;
-                bj = j2;
+        uint32_t i = 0, j = 0;
+        LocalReplay<R> rp;
+        if (bv > 0) {
+            // the first cell in row-major order among the best lane's rows
+            const LocalBest b = p.best[tk.job0 + bs];
+            const uint32_t lo = b.tie ? 0u : b.t0, hi = b.tie ? n + 31u : min(b.t0 + 32u, n + 31u);
+            if (!WALK && p.turn) {
+                // the rows above were overwritten: sweep the stripes above again
+                for (uint32_t s = 0; s < bs; ++s) {
+                    rp.begin(p, tk, s, 0u, lane);
+                    uint32_t *out = p.rows + tk.row_off + (size_t)(s & 1u) * tk.nr;
+                    while (rp.t < n + 31u) {
+                        const uint32_t t = rp.t;
+                        if (rp.template step<false>(p.gap, lane) && lane == 31) __stcg(out + (t - 31u), rp.ln.xout);
+                    }
+                    __threadfence();
+                    __syncwarp();
+                }
             }
+            rp.begin(p, tk, bs, WALK ? lo - lo % kTileSteps : 0u, lane);
+            uint32_t first[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) first[r] = ~0u;
+            while (rp.t < hi) {
+                const uint32_t t = rp.t;
+                const bool act = rp.template step<false>(p.gap, lane);
+                if (act && t >= lo && lane == b.lane) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        if (rp.ln.Hl[r] == bv && first[r] == ~0u) first[r] = t - lane;
+                }
+            }
+#pragma unroll
+            for (int r = R - 1; r >= 0; --r)
+                if (first[r] != ~0u) {
+                    i = bs * SH + lane * R + (uint32_t)r + 1u;
+                    j = first[r] + 1u;
+                }
+            i = __shfl_sync(kFull, i, b.lane);
+            j = __shfl_sync(kFull, j, b.lane);
         }
         if (lane == 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
-            p.scores[tk.out] = best;
-            if (POS) {
-                p.ends[4 * (size_t)tk.out + 2] = bi;
-                p.ends[4 * (size_t)tk.out + 3] = bj;
-                // the start: the walk moves it from the end cell; without
-                // pointers it is not computed
-                p.ends[4 * (size_t)tk.out + 0] = PTR ? bi : ~0u;
-                p.ends[4 * (size_t)tk.out + 1] = PTR ? bj : ~0u;
+            p.ends[4 * (size_t)tk.out + 2] = i;
+            p.ends[4 * (size_t)tk.out + 3] = j;
+            if (!WALK) p.ends[4 * (size_t)tk.out + 0] = p.ends[4 * (size_t)tk.out + 1] = ~0u;  // not computed
+        }
+        if constexpr (WALK) {
+            const uint8_t *A = p.pool + tk.a_off, *B = p.pool + tk.b_off;
+            uint8_t *mv = moves + move_off[q];
+            int32_t h = bv;
+            uint64_t k = 0;
+            while (h > 0 && i > 0 && j > 0) {
+                // the tile of cell (i, j)
+                const uint32_t s = (i - 1) / SH, tc = (j - 1) + ((i - 1) % SH) / R, t0 = tc - tc % kTileSteps;
+                rp.begin(p, tk, s, t0, lane);
+                __syncwarp();
+                while (rp.t <= tc) {
+                    const uint32_t t = rp.t;
+                    if (rp.template step<true>(p.gap, lane))
+                        tile[(t - t0) * 32u + lane] = Bits::pack(rp.ln.accL, rp.ln.accH);
+                }
+                __syncwarp();
+                // (uniform over the warp from here: every lane follows the same walk)
+                auto step_of = [&](uint32_t i_, uint32_t j_) { return (j_ - 1) + ((i_ - 1) % SH) / R; };
+                while (h > 0 && i > 0 && j > 0 && (i - 1) / SH == s && step_of(i, j) >= t0) {
+                    uint32_t stop = 1u, gapm = 0u, same = 0u;
+                    if (lane < i && lane < j) {
+                        const uint32_t iq = i - lane, jq = j - lane;
+                        if ((iq - 1) / SH == s && step_of(iq, jq) >= t0) {
+                            const uint32_t l = ((iq - 1) % SH) / R, r = (iq - 1) % R;
+                            const typename Bits::Word w = tile[(jq - 1 + l - t0) * 32u + l];
+                            stop = Bits::bit(w, 0, r);
+                            gapm = stop ? 1u + Bits::bit(w, 1, r) : 0u;  // the gap move that ends the run
+                            same = base_at(A, iq - 1) == base_at(B, jq - 1);
+                        }
+                    }
+                    const uint32_t eq = __ballot_sync(kFull, same), before = (1u << lane) - 1u;
+                    const int32_t ne = __popc(eq & before);
+                    const int32_t hq = h - p.match * ne - p.mismatch * ((int32_t)lane - ne);  // H of the lane's cell
+                    const uint32_t b = __ballot_sync(kFull, stop || hq == 0);
+                    const uint32_t run = b ? (uint32_t)__ffs(b) - 1u : 32u;
+                    if (lane < run && in_range(k + lane, (uint64_t)m + n, p.err, kSiteLocalMoves)) mv[k + lane] = 0;
+                    k += run;
+                    i -= run;
+                    j -= run;
+                    const uint32_t lm = run < 32u ? (1u << run) - 1u : kFull;
+                    const int32_t nr = __popc(eq & lm);
+                    h -= p.match * nr + p.mismatch * ((int32_t)run - nr);
+                    gapm = __shfl_sync(kFull, gapm, run & 31u);
+                    if (run < 32u && h > 0 && gapm) {
+                        if (lane == 0 && in_range(k, (uint64_t)m + n, p.err, kSiteLocalMoves)) mv[k] = (uint8_t)gapm;
+                        ++k;
+                        h -= p.gap;
+                        i -= gapm == 1u;
+                        j -= gapm == 2u;
+                    }
+                }
+            }
+            if (lane == 0) {
+                if (in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
+                    p.ends[4 * (size_t)tk.out + 0] = i;
+                    p.ends[4 * (size_t)tk.out + 1] = j;
+                }
+                nmoves[q] = k;
             }
         }
         __syncwarp();
     }
 }
 
-// The walk back from each pair's end cell, one thread per pair: follows the
-// pointer words (layout [stripe][lane][column group]) and tracks H along
-// the path, stopping where it reaches 0.  Writes the moves in reverse order
-// (0 diagonal, 1 vertical, 2 horizontal), their count, and the start cell.
-template <int R>
-__global__ void k_local_walk(const LocalTask *tasks, uint32_t ntasks, const uint8_t *pool, const uint32_t *ptr,
-                             const int32_t *scores, uint32_t *ends, uint8_t *moves, const uint64_t *move_off,
-                             uint64_t *nmoves, uint32_t prof0, uint32_t prof1, uint32_t prof2, uint32_t prof3,
-                             int32_t gap, uint32_t *err) {
-    constexpr uint32_t SH = 32u * R, CPW = 16u / R;
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < ntasks; q += gridDim.x * blockDim.x) {
-        const LocalTask tk = tasks[q];
-        const uint8_t *A = pool + tk.a_off, *B = pool + tk.b_off;
-        const uint32_t *pw = ptr + tk.ptr_off;
-        uint32_t *e = ends + 4 * (size_t)tk.out;
-        uint32_t i = e[2], j = e[3];
-        int32_t h = scores[tk.out];
-        uint8_t *mv = moves + move_off[q];
-        uint64_t k = 0;
-        while (h > 0 && i > 0 && j > 0) {
-            const uint32_t i1 = i - 1, j1 = j - 1;
-            const uint32_t word = __ldg(pw + (size_t)((i1 / SH) * 32u + (i1 % SH) / R) * tk.ncg + j1 / CPW);
-            const uint32_t d = ptr_move(word, (j1 % CPW) * R + (i1 % R));
-            if (!in_range(k, (uint64_t)tk.m + tk.n, err, kSiteLocalMoves)) break;
-            mv[k++] = (uint8_t)d;
-            if (d == 0) {
-                const uint32_t ca = base_at(A, i1), cb = base_at(B, j1);
-                const uint32_t pr = ca == 0 ? prof0 : ca == 1 ? prof1 : ca == 2 ? prof2 : prof3;
-                h -= (int32_t)(int8_t)(pr >> (8 * cb));
-                --i;
-                --j;
-            } else {
-                h -= gap;
-                if (d == 1) --i;
-                else --j;
-            }
-        }
-        e[0] = i;
-        e[1] = j;
-        nmoves[q] = k;
-    }
-}
-
-template <int R, bool PTR, bool POS>
-int launch_local_R(nw_ctx *ctx, LocalArgs &la, uint32_t max_n) {
+template <int R, int MODE>
+int launch_local_R(nw_ctx *ctx, LocalArgs &la) {
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local<R, PTR, POS>, kLocalWarps * 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local<R, MODE>, kLocalWarps * 32, 0);
     if (occ < 1) occ = 1;
+    // every CTA resident: a job's warp may wait on an earlier job's warp
     uint32_t blocks = (uint32_t)occ * (uint32_t)ctx->sm_count;
-    const uint32_t need = (la.ntasks + kLocalWarps - 1) / kLocalWarps;
+    const uint32_t need = (la.njobs + kLocalWarps - 1) / kLocalWarps;
     if (blocks > need) blocks = need ? need : 1;
-    la.ring_stride = ((max_n + 31) / 32) * 32 + 32;
     void *v = nullptr;
-    int rc = scratch(ctx, "local_ring", (size_t)blocks * kLocalWarps * la.ring_stride * 4, &v);
+    int rc = scratch(ctx, "local_counter", 16, &v);
     if (rc) return rc;
-    la.ring = (uint32_t *)v;
-    if ((rc = scratch(ctx, "local_counter", 16, &v))) return rc;
     la.counter = (uint32_t *)v;
     cudaMemsetAsync(la.counter, 0, 4, ctx->stream);
-    LaunchTimer t(ctx, PTR ? "local_fill_ptr" : (POS ? "local_score_pos" : "local_score"));
-    k_local<R, PTR, POS><<<blocks, kLocalWarps * 32, 0, ctx->stream>>>(la);
+    LaunchTimer t(ctx, MODE == kKeep ? "local_fill_ptr" : (MODE == kEnds ? "local_score_pos" : "local_score"));
+    k_local<R, MODE><<<blocks, kLocalWarps * 32, 0, ctx->stream>>>(la);
     return NW_OK;
 }
 
-int launch_local(nw_ctx *ctx, int R, bool ptr, bool pos, LocalArgs &la, uint32_t max_n) {
-#define NW_LOCAL_CASES(PTRV, POSV)                                        \
-    switch (R) {                                                          \
-        case 4: return launch_local_R<4, PTRV, POSV>(ctx, la, max_n);     \
-        case 16: return launch_local_R<16, PTRV, POSV>(ctx, la, max_n);   \
-        default: return launch_local_R<8, PTRV, POSV>(ctx, la, max_n);    \
+int launch_local(nw_ctx *ctx, int R, LocalMode mode, LocalArgs &la) {
+#define NW_LOCAL_CASES(MODEV)                                    \
+    switch (R) {                                                 \
+        case 4: return launch_local_R<4, MODEV>(ctx, la);        \
+        case 16: return launch_local_R<16, MODEV>(ctx, la);      \
+        default: return launch_local_R<8, MODEV>(ctx, la);       \
     }
-    if (ptr) NW_LOCAL_CASES(true, true)
-    if (pos) NW_LOCAL_CASES(false, true)
-    NW_LOCAL_CASES(false, false)
+    if (mode == kKeep) NW_LOCAL_CASES(kKeep)
+    if (mode == kEnds) NW_LOCAL_CASES(kEnds)
+    NW_LOCAL_CASES(kScore)
 #undef NW_LOCAL_CASES
+}
+
+template <bool WALK>
+void launch_local_trace(nw_ctx *ctx, int R, const LocalArgs &la, uint32_t ntasks, uint8_t *moves,
+                        const uint64_t *move_off, uint64_t *nmoves) {
+    LaunchTimer t(ctx, WALK ? "local_walk" : "local_ends");
+    const uint32_t blocks = std::min<uint32_t>(ntasks, 65535);
+    if (R == 4) k_local_trace<4, WALK><<<blocks, 32, 0, ctx->stream>>>(la, ntasks, moves, move_off, nmoves);
+    else if (R == 16) k_local_trace<16, WALK><<<blocks, 32, 0, ctx->stream>>>(la, ntasks, moves, move_off, nmoves);
+    else k_local_trace<8, WALK><<<blocks, 32, 0, ctx->stream>>>(la, ntasks, moves, move_off, nmoves);
 }
 
 template <typename T>
@@ -402,9 +580,12 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     int R = 8;
     if (const char *e = getenv("NW_LOCAL_R")) R = atoi(e) == 4 ? 4 : atoi(e) == 16 ? 16 : 8;
     const uint32_t SH = 32u * R;
+    const LocalMode mode = want ? kKeep : ends ? kEnds : kScore;
     LocalArgs la{};
     la.pool = pool;
     local_profile(sc, la.prof);
+    la.match = sc.match;
+    la.mismatch = sc.mismatch;
     la.gap = sc.gap;
     la.scores = scores;
     la.ends = ends;
@@ -413,71 +594,87 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     std::vector<LocalTask> all(npairs);
     for (uint32_t k = 0; k < npairs; ++k) {
         LocalTask &t = all[k];
-        t = LocalTask{a_off[k], b_off[k], a_len[k], b_len[k], k, 0, 0};
-        // one warp steps through stripes x max(n, 96) columns: a 32-bit count
+        t = LocalTask{a_off[k], b_off[k], a_len[k], b_len[k], k, 0, 0, 0, 0, 0};
+        // a pair's stripe steps are limited to a 32-bit count
         if ((uint64_t)((t.m + SH - 1) / SH) * std::max(t.n, kLocalMinPeriod) >= (1ull << 31))
             return fail(ctx, NW_ERR_UNSUPPORTED, "pair %u too large for one warp (m*n/%u >= 2^31)", k, SH);
-        if (want) t.ncg = ptr_words_per_lane_row(std::max(t.n, kLocalMinPeriod), R);
+        t.nr = (t.n + 31) / 32 * 32;
+        // states before steps kTileSteps, 2 kTileSteps, .. of a stripe's n + 31
+        if (want && t.m && t.n) t.keep_n = (t.n + 30) / kTileSteps;
     }
     // longest first (the atomic queue then balances the tail)
     std::stable_sort(all.begin(), all.end(), [](const LocalTask &x, const LocalTask &y) {
         return (uint64_t)x.m * x.n > (uint64_t)y.m * y.n;
     });
     int rc;
-    if (!want) {
-        uint32_t max_n = 1;
-        for (const LocalTask &t : all) max_n = std::max(max_n, t.n);
-        LocalTask *dt = nullptr;
-        if ((rc = upload_vec(ctx, "local_tasks", all, &dt))) return rc;
-        la.tasks = dt;
-        la.ntasks = npairs;
-        return launch_local(ctx, R, false, ends != nullptr, la, max_n);
-    }
-    // CIGAR: waves whose pointer words fit half the free budget
+    cudaError_t e0 = cudaMemsetAsync(scores, 0, (size_t)npairs * 4, ctx->stream);  // the stripes' maxima are merged
+    if (e0 != cudaSuccess) return cuda_fail(ctx, e0, "local scores reset");
+    // waves whose stripe rows and kept states fit half the free budget
     const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
+    const uint32_t state_units = ((uint32_t)R + 5u) / 4u * 32u;  // 16-byte units of a kept state
     size_t k0 = 0;
     while (k0 < all.size()) {
         std::vector<LocalTask> wave;
+        std::vector<LocalJob> jobs;
         std::vector<uint64_t> moff;
-        uint64_t words = 0, mbytes = 0;
-        uint32_t max_n = 1;
+        uint64_t units = 0, rows = 0, mbytes = 0;
+        bool turn = mode == kScore;  // rows: two in turn
         size_t k = k0;
         for (; k < all.size(); ++k) {
             LocalTask t = all[k];
-            const uint64_t wds = (uint64_t)((t.m + SH - 1) / SH) * 32u * t.ncg;
-            if (!wave.empty() && (words + wds) * 4 > wave_budget) break;
-            t.ptr_off = words;
-            words += wds;
+            const uint32_t S = (t.m && t.n) ? (t.m + SH - 1) / SH : 1;
+            const uint64_t u = (uint64_t)S * t.keep_n * state_units;
+            uint64_t rw = (uint64_t)(mode == kScore ? std::min(S - 1, 2u) : S - 1) * t.nr;
+            if (!wave.empty() && ((turn && mode == kEnds) || (units + u) * 16 + (rows + rw) * 4 > wave_budget)) break;
+            // a lone pair whose rows alone exceed the budget keeps two and
+            // finds its end cell by sweeping the stripes above it again
+            if (mode == kEnds && wave.empty() && rw * 4 + (64u << 10) > scratch_headroom(ctx, "local_rows")) {
+                turn = true;
+                rw = (uint64_t)std::min(S - 1, 2u) * t.nr;
+            }
+            t.keep_off = units;
+            t.row_off = rows;
+            t.job0 = (uint32_t)jobs.size();
+            for (uint32_t s = 0; s < S; ++s) jobs.push_back(LocalJob{(uint32_t)wave.size(), s});
+            units += u;
+            rows += rw;
             moff.push_back(mbytes);
             mbytes += (uint64_t)t.m + t.n + 16;
-            max_n = std::max(max_n, t.n);
             wave.push_back(t);
         }
-        void *pv = nullptr, *mv = nullptr, *nm = nullptr;
-        if ((rc = scratch(ctx, "local_ptr", words * 4 + 16, &pv))) return rc;
-        if ((rc = scratch(ctx, "local_moves", mbytes + 16, &mv))) return rc;
-        if ((rc = scratch(ctx, "local_nmoves", wave.size() * 8 + 16, &nm))) return rc;
+        void *kv = nullptr, *rv = nullptr, *pv = nullptr, *bv = nullptr, *mv = nullptr, *nm = nullptr;
+        if ((rc = scratch(ctx, "local_rows", rows * 4 + 16, &rv))) return rc;
+        if ((rc = scratch(ctx, "local_progress", jobs.size() * 4 + 16, &pv))) return rc;
+        if (mode != kScore && (rc = scratch(ctx, "local_best", jobs.size() * sizeof(LocalBest) + 16, &bv))) return rc;
+        if (want) {
+            if ((rc = scratch(ctx, "local_keep", units * 16 + 16, &kv))) return rc;
+            if ((rc = scratch(ctx, "local_moves", mbytes + 16, &mv))) return rc;
+            if ((rc = scratch(ctx, "local_nmoves", wave.size() * 8 + 16, &nm))) return rc;
+        }
+        if ((e0 = cudaMemsetAsync(pv, 0, jobs.size() * 4, ctx->stream)) != cudaSuccess)
+            return cuda_fail(ctx, e0, "local progress reset");
         LocalTask *dt = nullptr;
+        LocalJob *dj = nullptr;
         uint64_t *dmoff = nullptr;
         if ((rc = upload_vec(ctx, "local_tasks", wave, &dt))) return rc;
-        if ((rc = upload_vec(ctx, "local_move_off", moff, &dmoff))) return rc;
+        if ((rc = upload_vec(ctx, "local_jobs", jobs, &dj))) return rc;
+        if (want && (rc = upload_vec(ctx, "local_move_off", moff, &dmoff))) return rc;
         la.tasks = dt;
-        la.ntasks = (uint32_t)wave.size();
-        la.ptr = (uint32_t *)pv;
-        la.ptr_cap = words;
-        if ((rc = launch_local(ctx, R, true, true, la, max_n))) return rc;
-        {
-            LaunchTimer t(ctx, "local_walk");
-            const uint32_t blocks = std::max<uint32_t>(1, ((uint32_t)wave.size() + 127) / 128);
-#define NW_WALK(RV)                                                                                               \
-    k_local_walk<RV><<<blocks, 128, 0, ctx->stream>>>(dt, (uint32_t)wave.size(), pool, (const uint32_t *)pv, scores, \
-                                                      ends, (uint8_t *)mv, dmoff, (uint64_t *)nm, la.prof[0],       \
-                                                      la.prof[1], la.prof[2], la.prof[3], sc.gap, ctx->d_err)
-            if (R == 4) NW_WALK(4);
-            else if (R == 16) NW_WALK(16);
-            else NW_WALK(8);
-#undef NW_WALK
-        }
+        la.jobs = dj;
+        la.njobs = (uint32_t)jobs.size();
+        la.rows = (uint32_t *)rv;
+        la.rows_cap = rows;
+        la.turn = turn;
+        la.progress = (uint32_t *)pv;
+        la.best = (LocalBest *)bv;
+        la.keep = (uint4 *)kv;
+        la.keep_cap = units;
+        const uint32_t nt = (uint32_t)wave.size();
+        k0 = k;
+        if ((rc = launch_local(ctx, R, mode, la))) return rc;
+        if (mode == kEnds) launch_local_trace<false>(ctx, R, la, nt, nullptr, nullptr, nullptr);
+        if (!want) continue;
+        launch_local_trace<true>(ctx, R, la, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
         std::vector<TraceTask> tt(wave.size());
         for (size_t q = 0; q < wave.size(); ++q) {
             const LocalTask &t = wave[q];
@@ -497,7 +694,6 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         TraceTask *dtt = nullptr;
         if ((rc = upload_vec(ctx, "local_trace_tasks", tt, &dtt))) return rc;
         if ((rc = launch_finish(ctx, tt[0], dtt, (uint32_t)tt.size(), (flags & NW_CIGAR_M) ? 1u : 0u))) return rc;
-        k0 = k;
     }
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? NW_OK : cuda_fail(ctx, e, "local launch");
