@@ -33,10 +33,11 @@
 // one after another on one warp (which left a batch waiting on its longest
 // pair).  A warp takes the next job from an atomic counter; lane k owns R
 // rows of the stripe and a step hands the lane below two values (W with the
-// base code, and F').  Lane 31 writes the stripe's bottom row (W and F')
-// to the job's row buffer and publishes every 32 columns with a release
-// store to the job's progress word; the warp of the next stripe waits (a
-// bounded spin) on that word before it reads each chunk of 32 columns.
+// base code, and F').  Every 32 steps the warp writes what lane 31 produced of
+// the stripe's bottom row (W and F', through shared memory) to the job's row
+// buffer and publishes it with a release store to the job's progress word; the
+// warp of the next stripe waits (a bounded spin) on that word before it reads
+// a chunk of 32 columns that it has not seen published yet.
 // The job it waits on was taken earlier by a warp of the same persistent,
 // fully resident grid, so every wait ends.
 #include <algorithm>
@@ -50,6 +51,7 @@ namespace {
 constexpr int kAffWarps = 8;
 constexpr int32_t kAffNeg = -(1 << 27);   // -inf: far below any W, no add wraps
 constexpr uint32_t kTileSteps = 128;      // steps between a stripe's kept states
+constexpr int kTraceWarps = 3;            // tiles the trace replays at once
 
 struct AffTask {
     uint64_t a_off, b_off;
@@ -97,16 +99,6 @@ __device__ __forceinline__ uint32_t aff_rows(const uint8_t *s, uint32_t i0, uint
         }
     }
     return w;
-}
-
-// Warp-uniform bounded wait until *flag >= target (lane 0 spins; then every
-// lane acquires, so its following loads see what the producer published).
-__device__ __forceinline__ bool aff_wait(const uint32_t *flag, uint32_t target, uint32_t *err, uint32_t where) {
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = wait_geq(flag, target, err, where) ? 1 : 0;
-    ok = __shfl_sync(kFull, ok, 0);
-    if (ok) (void)ld_acquire(flag);
-    return ok != 0;
 }
 
 // A lane's R rows of a stripe: the systolic state between two steps.
@@ -189,7 +181,7 @@ struct AffLane {
             const int32_t f = __viaddmax_s32(u, go, fu);
             const int32_t w = __vimax3_s32(d + sv, e, f);
             if constexpr (PTR) {
-                accL = ptr_append(accL, d + sv - max(e, f));
+                accL = ptr_append(accL, d + sv - w);
                 accH = ptr_append(accH, f - e);
                 accF = ptr_append(accF, u + go - fu);
                 accE = ptr_append(accE, Wl[r] + go - El[r]);
@@ -232,6 +224,9 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
     constexpr uint32_t SH = 32u * R;
     const int lane = threadIdx.x & 31;
     const int32_t go = p.go;
+    // a chunk's inputs of lane 0 and outputs of lane 31, per warp
+    __shared__ uint2 ins_[kAffWarps][32], outs_[kAffWarps][32];
+    uint2 *ins = ins_[threadIdx.x >> 5], *outs = outs_[threadIdx.x >> 5];
 
     for (;;) {
         uint32_t jidx = 0;
@@ -263,70 +258,75 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
         ln.start(go, i0);
         uint4 *keep = KEEP ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * AffLane<R>::kParts * 32u + lane : nullptr;
         int32_t c = -lane;
-        bool alive = !s || aff_wait(prev, min(32u, n), p.err, jidx);
-        uint32_t stage = 0, stage_next = alive ? above.w((uint32_t)lane) : 0u;
-        int32_t fstage = kAffNeg, fstage_next = alive ? above.f((uint32_t)lane) : kAffNeg;
-
-        // lane 31: this stripe's bottom row out, published every 32 columns
-        auto row_out = [&](uint32_t col) {
-            if (lane == 31 && outW && in_range((size_t)(outW - p.rows) + tk.nr + col, p.rows_cap, p.err, kSiteAffRing)) {
-                outW[col] = ln.xout;
-                outF[col] = (uint32_t)ln.fout;
-                if (((col + 1) & 31u) == 0 || col + 1 == n) st_release(mine, col + 1);
+        uint32_t seen = 0;
+        bool alive = !s || warp_wait_geq(prev, min(32u, n), seen, p.err, jidx);
+        uint32_t w_next = alive ? above.w((uint32_t)lane) : 0u;
+        int32_t f_next = alive ? above.f((uint32_t)lane) : kAffNeg;
+        // the last chunk's bottom row (columns t - 63 .. t - 32 of lane 31) out, and published
+        auto row_out = [&](uint32_t t) {
+            if (!outW) return;
+            __syncwarp();
+            const int32_t col = (int32_t)t - 63 + lane;
+            if (col >= 0 && col < (int32_t)n &&
+                in_range((size_t)(outW - p.rows) + tk.nr + (uint32_t)col, p.rows_cap, p.err, kSiteAffRing)) {
+                const uint2 v = outs[lane];
+                __stcg(outW + col, v.x);
+                __stcg(outF + col, v.y);
             }
+            __syncwarp();
+            if (lane == 0) st_release(mine, min(t - 31u, n));
         };
 
-        for (uint32_t t = 0; t < T && alive; ++t) {
-            if ((t & 31u) == 0) {
-                if (KEEP && t && t % kTileSteps == 0) {
-                    ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
-                    keep += AffLane<R>::kParts * 32u;
-                }
-                stage = stage_next;
-                fstage = fstage_next;
-                if (s && t + 32 < n && !(alive = aff_wait(prev, min(t + 64u, n), p.err, jidx))) break;
-                stage_next = above.w(t + 32u + (uint32_t)lane);
-                fstage_next = above.f(t + 32u + (uint32_t)lane);
-                if (__all_sync(kFull, c >= 0 && c + 32 <= (int32_t)n - 1)) {
+        for (uint32_t t = 0; t < T && alive; t += 32) {
+            if (KEEP && t && t % kTileSteps == 0) {
+                ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
+                keep += AffLane<R>::kParts * 32u;
+            }
+            __syncwarp();
+            ins[lane] = make_uint2(w_next, (uint32_t)f_next);
+            __syncwarp();
+            if (s && t + 32 < n && !(alive = warp_wait_geq(prev, min(t + 64u, n), seen, p.err, jidx))) break;
+            w_next = above.w(t + 32u + (uint32_t)lane);
+            f_next = above.f(t + 32u + (uint32_t)lane);
+            if (__all_sync(kFull, c >= 0 && c + 32 <= (int32_t)n - 1)) {
 #pragma unroll 4
-                    for (uint32_t uu = 0; uu < 32u; ++uu) {
-                        uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
-                        int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
-                        const uint32_t x0 = __shfl_sync(kFull, stage, uu);
-                        const int32_t f0 = __shfl_sync(kFull, fstage, uu);
-                        if (lane == 0) {
-                            x = x0;
-                            fx = f0;
-                        }
-                        ln.template column<false>(go, x, fx);
-                        row_out((uint32_t)c + uu);
+                for (uint32_t uu = 0; uu < 32u; ++uu) {
+                    uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                    int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
+                    const uint2 in = ins[uu];
+                    if (lane == 0) {
+                        x = in.x;
+                        fx = (int32_t)in.y;
                     }
-                    c += 32;
-                    t += 31;
-                    continue;
+                    ln.template column<false>(go, x, fx);
+                    if (lane == 31) outs[uu] = make_uint2(ln.xout, (uint32_t)ln.fout);
                 }
-            }
-            uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
-            int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
-            const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
-            const int32_t f0 = __shfl_sync(kFull, fstage, t & 31u);
-            if (lane == 0) {
-                x = x0;
-                fx = f0;
-            }
-            if (c >= 0 && c < (int32_t)n) {
-                ln.template column<false>(go, x, fx);
-                row_out((uint32_t)c);
-                if (s + 1 == S && (uint32_t)lane == lM && c == (int32_t)n - 1) {
-                    int32_t wmn = 0;
+                c += 32;
+            } else {
+                for (uint32_t uu = 0; uu < 32u && t + uu < T; ++uu) {
+                    uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                    int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
+                    const uint2 in = ins[uu];
+                    if (lane == 0) {
+                        x = in.x;
+                        fx = (int32_t)in.y;
+                    }
+                    if (c >= 0 && c < (int32_t)n) {
+                        ln.template column<false>(go, x, fx);
+                        if (lane == 31) outs[uu] = make_uint2(ln.xout, (uint32_t)ln.fout);
+                        if (s + 1 == S && (uint32_t)lane == lM && c == (int32_t)n - 1) {
+                            int32_t wmn = 0;
 #pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        if ((uint32_t)r == rM) wmn = ln.Wl[r];
-                    if (in_range(tk.out, p.out_cap, p.err, kSiteAffScore))
-                        p.scores[tk.out] = wmn + p.ge * (int32_t)(m + n);
+                            for (int r = 0; r < R; ++r)
+                                if ((uint32_t)r == rM) wmn = ln.Wl[r];
+                            if (in_range(tk.out, p.out_cap, p.err, kSiteAffScore))
+                                p.scores[tk.out] = wmn + p.ge * (int32_t)(m + n);
+                        }
+                    }
+                    ++c;
                 }
             }
-            ++c;
+            row_out(t + 32u);
         }
         __syncwarp();
         if (!alive) return;   // a wait gave up (NW_ERR_TIMEOUT is raised): leave
@@ -356,7 +356,7 @@ struct AffBits<16> {
     }
 };
 
-// The walk from (m, n), one warp per pair, longest pairs first.  The state
+// The walk from (m, n), one CTA per pair, longest pairs first.  The state
 // machine: in state H the diagonal when L is clear, else the vertical gap (F)
 // when H is clear, else the horizontal one (E); in a gap state the move is
 // emitted and the walk stays in the gap while the cell's extension bit is
@@ -368,13 +368,20 @@ struct AffBits<16> {
 // A cell of lane l and column c belongs to step c + l of its stripe; a tile
 // holds kTileSteps steps, from a kept state on, and the path's steps only
 // fall, so each tile is recomputed once, up to the step of the path's entry.
+// The CTA's warps replay kTraceWarps tiles of the path's stripe at once, the one
+// of its cell and the ones before it (a path crosses about 2.3 tiles of a
+// stripe), then the first warp walks: one warp doing both was bound by its
+// longest pair's chain of steps (700 pairs of 1-5 kb 1.7 ms; 2,000 are bound by the
+// replayed steps themselves, 2.1 ms either way).
 template <int R>
-__global__ void __launch_bounds__(32) k_affine_trace(AffArgs p, uint32_t ntasks, uint8_t *moves,
-                                                     const uint64_t *move_off, uint64_t *nmoves) {
+__global__ void __launch_bounds__(32 * kTraceWarps) k_affine_trace(AffArgs p, uint32_t ntasks, uint8_t *moves,
+                                                                   const uint64_t *move_off, uint64_t *nmoves) {
     using Bits = AffBits<R>;
     constexpr uint32_t SH = 32u * R;
-    __shared__ typename Bits::Word tile[kTileSteps * 32];  // [step][lane]
-    const uint32_t lane = threadIdx.x;
+    extern __shared__ uint4 tiles_[];  // [tile][step][lane]
+    __shared__ uint32_t at[3];         // i, j, state between the warps
+    typename Bits::Word *tiles = reinterpret_cast<typename Bits::Word *>(tiles_);
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const int32_t go = p.go;
     for (uint32_t q = blockIdx.x; q < ntasks; q += gridDim.x) {
         const AffTask tk = p.tasks[q];
@@ -382,47 +389,61 @@ __global__ void __launch_bounds__(32) k_affine_trace(AffArgs p, uint32_t ntasks,
         uint8_t *mv = moves + move_off[q];
         uint32_t i = m, j = n, state = 0;   // state: 0 H, 1 F (vertical gap), 2 E (horizontal gap)
         uint64_t k = 0;
-        while (i > 0 && j > 0) {
-            // the tile of cell (i, j)
-            const uint32_t s = (i - 1) / SH, tc = (j - 1) + ((i - 1) % SH) / R, t0 = tc - tc % kTileSteps;
-            const uint32_t *inW = s ? p.rows + tk.row_off + (size_t)(s - 1) * 2 * tk.nr : nullptr;
-            const AffAbove above{p.pool + tk.b_off, inW, s ? inW + tk.nr : nullptr, n, go};
-            AffLane<R> ln;
-            const uint32_t i0 = s * SH + lane * R;
-            uint32_t stage = 0, stage_next = above.w(t0 + lane);
-            int32_t fstage = kAffNeg, fstage_next = above.f(t0 + lane);
-            ln.rows(p, p.pool + tk.a_off, i0, m);
-            if (t0)
-                ln.load(p.keep + tk.keep_off +
-                        ((uint64_t)s * tk.keep_n + (t0 / kTileSteps - 1)) * AffLane<R>::kParts * 32u + lane);
-            else
-                ln.start(go, i0);
-            ln.accL = ln.accH = ln.accF = ln.accE = 0;
-            __syncwarp();
-            for (uint32_t t = t0; t <= tc; ++t) {
-                if ((t & 31u) == 0) {
-                    stage = stage_next;
-                    fstage = fstage_next;
-                    stage_next = above.w(t + 32u + lane);
-                    fstage_next = above.f(t + 32u + lane);
-                }
-                uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
-                int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
-                const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
-                const int32_t f0 = __shfl_sync(kFull, fstage, t & 31u);
-                if (lane == 0) {
-                    x = x0;
-                    fx = f0;
-                }
-                if (t >= lane && t - lane < n) {
-                    ln.template column<true>(go, x, fx);
-                    tile[(t - t0) * 32u + lane] = Bits::pack(ln.accL, ln.accH, ln.accF, ln.accE);
+        for (;;) {
+            if (threadIdx.x == 0) {
+                at[0] = i;
+                at[1] = j;
+                at[2] = state;
+            }
+            __syncthreads();
+            i = at[0];
+            j = at[1];
+            state = at[2];
+            if (i == 0 || j == 0) break;
+            // the tile of cell (i, j) and the ones before it in its stripe
+            const uint32_t s = (i - 1) / SH, tc = (j - 1) + ((i - 1) % SH) / R, tl = tc / kTileSteps;
+            const uint32_t ntile = min(tl + 1u, (uint32_t)kTraceWarps), t0 = (tl + 1u - ntile) * kTileSteps;
+            if (warp < ntile) {
+                typename Bits::Word *tile = tiles + warp * kTileSteps * 32u;
+                const uint32_t tw = t0 + warp * kTileSteps, te = min(tc, tw + kTileSteps - 1u);
+                const uint32_t *inW = s ? p.rows + tk.row_off + (size_t)(s - 1) * 2 * tk.nr : nullptr;
+                const AffAbove above{p.pool + tk.b_off, inW, s ? inW + tk.nr : nullptr, n, go};
+                AffLane<R> ln;
+                const uint32_t i0 = s * SH + lane * R;
+                uint32_t stage = 0, stage_next = above.w(tw + lane);
+                int32_t fstage = kAffNeg, fstage_next = above.f(tw + lane);
+                ln.rows(p, p.pool + tk.a_off, i0, m);
+                if (tw)
+                    ln.load(p.keep + tk.keep_off +
+                            ((uint64_t)s * tk.keep_n + (tw / kTileSteps - 1)) * AffLane<R>::kParts * 32u + lane);
+                else
+                    ln.start(go, i0);
+                ln.accL = ln.accH = ln.accF = ln.accE = 0;
+                for (uint32_t t = tw; t <= te; ++t) {
+                    if ((t & 31u) == 0) {
+                        stage = stage_next;
+                        fstage = fstage_next;
+                        stage_next = above.w(t + 32u + lane);
+                        fstage_next = above.f(t + 32u + lane);
+                    }
+                    uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                    int32_t fx = __shfl_up_sync(kFull, ln.fout, 1);
+                    const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
+                    const int32_t f0 = __shfl_sync(kFull, fstage, t & 31u);
+                    if (lane == 0) {
+                        x = x0;
+                        fx = f0;
+                    }
+                    if (t >= lane && t - lane < n) {
+                        ln.template column<true>(go, x, fx);
+                        tile[(t - tw) * 32u + lane] = Bits::pack(ln.accL, ln.accH, ln.accF, ln.accE);
+                    }
                 }
             }
-            __syncwarp();
-            // (uniform over the warp from here: every lane follows the same walk)
+            __syncthreads();
+            // (uniform over the first warp from here: every lane follows the same walk)
             auto step_of = [&](uint32_t i_, uint32_t j_) { return (j_ - 1) + ((i_ - 1) % SH) / R; };
-            for (;;) {
+            while (warp == 0) {
                 if (i == 0 || j == 0 || (i - 1) / SH != s || step_of(i, j) < t0) break;
                 if (state == 0) {
                     uint32_t stop = 1u, h = 0u;
@@ -430,7 +451,7 @@ __global__ void __launch_bounds__(32) k_affine_trace(AffArgs p, uint32_t ntasks,
                         const uint32_t iq = i - lane, jq = j - lane;
                         if ((iq - 1) / SH == s && step_of(iq, jq) >= t0) {
                             const uint32_t l = ((iq - 1) % SH) / R, r = (iq - 1) % R;
-                            const typename Bits::Word w = tile[(jq - 1 + l - t0) * 32u + l];
+                            const typename Bits::Word w = tiles[(jq - 1 + l - t0) * 32u + l];
                             stop = Bits::bit(w, 0, r);
                             h = stop ? 2u + Bits::bit(w, 1, r) : 0u;  // the gap that ends the run, + 1
                         }
@@ -445,7 +466,7 @@ __global__ void __launch_bounds__(32) k_affine_trace(AffArgs p, uint32_t ntasks,
                     if (run < 32u && h) state = h - 1u;
                 } else {
                     const uint32_t l = ((i - 1) % SH) / R, r = (i - 1) % R;
-                    const typename Bits::Word w = tile[(j - 1 + l - t0) * 32u + l];
+                    const typename Bits::Word w = tiles[(j - 1 + l - t0) * 32u + l];
                     if (lane == 0 && in_range(k, (uint64_t)m + n, p.err, kSiteAffMoves)) mv[k] = (uint8_t)state;
                     ++k;
                     if (state == 1) {
@@ -458,11 +479,13 @@ __global__ void __launch_bounds__(32) k_affine_trace(AffArgs p, uint32_t ntasks,
                 }
             }
         }
-        const uint32_t rest = i + j;
-        const uint8_t mvr = i ? 1 : 2;
-        for (uint32_t x = lane; x < rest; x += 32) mv[k + x] = mvr;
-        if (lane == 0) nmoves[q] = k + rest;
-        __syncwarp();
+        if (warp == 0) {
+            const uint32_t rest = i + j;
+            const uint8_t mvr = i ? 1 : 2;
+            for (uint32_t x = lane; x < rest; x += 32) mv[k + x] = mvr;
+            if (lane == 0) nmoves[q] = k + rest;
+        }
+        __syncthreads();
     }
 }
 
@@ -494,6 +517,27 @@ int launch_affine(nw_ctx *ctx, int R, bool keep, AffArgs &aa) {
     if (R == 4) return launch_affine_R<4, false>(ctx, aa);
     if (R == 16) return launch_affine_R<16, false>(ctx, aa);
     return launch_affine_R<8, false>(ctx, aa);
+}
+
+template <int R>
+int launch_affine_trace_R(nw_ctx *ctx, const AffArgs &aa, uint32_t ntasks, uint8_t *moves, const uint64_t *move_off,
+                          uint64_t *nmoves) {
+    constexpr int smem = kTraceWarps * (int)kTileSteps * 32 * (int)sizeof(typename AffBits<R>::Word);
+    if (smem + 64 > 48 * 1024) {  // (with the static words)
+        // one value for every caller: the attribute belongs to the process
+        const cudaError_t e = cudaFuncSetAttribute(k_affine_trace<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "affine trace shared memory");
+    }
+    k_affine_trace<R><<<std::min<uint32_t>(ntasks, 65535), 32 * kTraceWarps, smem, ctx->stream>>>(aa, ntasks, moves,
+                                                                                               move_off, nmoves);
+    return NW_OK;
+}
+
+int launch_affine_trace(nw_ctx *ctx, int R, const AffArgs &aa, uint32_t ntasks, uint8_t *moves,
+                        const uint64_t *move_off, uint64_t *nmoves) {
+    if (R == 4) return launch_affine_trace_R<4>(ctx, aa, ntasks, moves, move_off, nmoves);
+    if (R == 16) return launch_affine_trace_R<16>(ctx, aa, ntasks, moves, move_off, nmoves);
+    return launch_affine_trace_R<8>(ctx, aa, ntasks, moves, move_off, nmoves);
 }
 
 template <typename T>
@@ -610,11 +654,8 @@ int affine_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const
         if ((rc = launch_affine(ctx, R, true, aa))) return rc;
         {
             LaunchTimer t(ctx, "affine_walk");
-            const uint32_t blocks = (uint32_t)std::min<size_t>(wave.size(), 65535), nt = (uint32_t)wave.size();
-            if (R == 4) k_affine_trace<4><<<blocks, 32, 0, ctx->stream>>>(aa, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
-            else if (R == 16)
-                k_affine_trace<16><<<blocks, 32, 0, ctx->stream>>>(aa, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
-            else k_affine_trace<8><<<blocks, 32, 0, ctx->stream>>>(aa, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
+            if ((rc = launch_affine_trace(ctx, R, aa, (uint32_t)wave.size(), (uint8_t *)mv, dmoff, (uint64_t *)nm)))
+                return rc;
         }
         std::vector<TraceTask> tt(wave.size());
         for (size_t q = 0; q < wave.size(); ++q) {

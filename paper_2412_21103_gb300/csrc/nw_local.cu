@@ -16,22 +16,23 @@
 // queued pair by pair (longest pairs first) and stripes in order, so a pair's
 // stripes run on several warps at once as a wavefront (one warp per pair left
 // the launch waiting on its longest pairs).  A warp takes the next job from an
-// atomic counter; lane k owns R rows of the stripe.  Lane 31 writes the
-// stripe's bottom row to the pair's row buffer and publishes every 32 columns
-// with a release store; the warp of the next stripe waits (a bounded spin) on
-// that word before it reads each chunk of 32 columns.  The job it waits on was
-// taken earlier by a warp of the same fully resident grid, so every wait ends.
+// atomic counter; lane k owns R rows of the stripe.  Every 32 steps the warp
+// writes what lane 31 produced of the stripe's bottom row (through shared
+// memory) to the pair's row buffer and publishes it with a release store; the
+// warp of the next stripe waits (a bounded spin) on that word before it reads a
+// chunk of 32 columns that it has not seen published yet.  The job it waits on
+// was taken earlier by a warp of the same fully resident grid, so every wait
+// ends.
 //
 // End cells and alignments.  The fill keeps no pointers and no positions: a
-// lane notes the chunk of 32 steps in which its rows first reached their
-// largest H (and whether another chunk reached it too), and every kTileSteps
-// steps the state of a stripe's lanes is kept.  The trace finds the pair's
-// best lane, recomputes the chunk (the whole stripe when several chunks tie) for
-// the first cell in row-major order, and walks back from it tile by tile -- a
-// tile is one stripe and the steps between two kept states -- recomputing only
-// the tiles the path crosses with the two pointer bits in shared memory (L:
-// the diagonal candidate is below max(up, left) + gap; H: left above up), and
-// tracking H along the path to find the start.  Pointers and positions for
+// lane notes the first and the last chunk of 32 steps in which its rows reached
+// their largest H, and every kTileSteps steps the state of a stripe's lanes is
+// kept.  The trace finds the pair's best lane, recomputes those chunks for the
+// first cell in row-major order, and walks back from it tile by tile -- a tile
+// is one stripe and the steps between two kept states -- recomputing only the
+// tiles the path crosses (a warp each) with the two pointer bits in shared
+// memory (L: the diagonal candidate is below max(up, left) + gap; H: left above
+// up), and tracking H along the path to find the start.  Pointers and positions for
 // every cell cost the fill 11 operations per cell, against 4.5.
 #include <algorithm>
 #include <vector>
@@ -44,6 +45,7 @@ namespace {
 constexpr int kLocalWarps = 8;
 constexpr uint32_t kLocalMinPeriod = 96;   // columns a stripe counts at least (the limit on a pair's size)
 constexpr uint32_t kTileSteps = 128;       // steps between a stripe's kept states
+constexpr int kTraceWarps = 3;             // tiles the trace replays at once
 constexpr uint32_t kPadProfile = 0x80808080u;  // rows past the end: s = -128, never above a real row
 
 struct LocalTask {
@@ -61,11 +63,11 @@ struct LocalJob {
     uint32_t task, stripe;
 };
 
-// The largest H of a stripe: the first lane that reached it, the first chunk of
-// 32 steps in which it did, and whether the lane reached it in another too.
+// The largest H of a stripe: the first lane that reached it, and the first
+// and the last chunk of 32 steps in which it did.
 struct LocalBest {
     int32_t v;
-    uint32_t lane, t0, tie;
+    uint32_t lane, t0, t1;
 };
 
 // What a launch produces: the scores alone, also the stripes' best lanes
@@ -105,16 +107,6 @@ __device__ __forceinline__ uint32_t rows_codes(const uint8_t *s, uint32_t i0, ui
         }
     }
     return w;
-}
-
-// Warp-uniform bounded wait until *flag >= target (lane 0 spins; then every
-// lane acquires, so its following loads see what the producer published).
-__device__ __forceinline__ bool local_wait(const uint32_t *flag, uint32_t target, uint32_t *err, uint32_t where) {
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = wait_geq(flag, target, err, where) ? 1 : 0;
-    ok = __shfl_sync(kFull, ok, 0);
-    if (ok) (void)ld_acquire(flag);
-    return ok != 0;
 }
 
 // A lane's R rows of a stripe: the systolic state between two steps.
@@ -216,6 +208,9 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
     constexpr uint32_t SH = 32u * R;
     const int lane = threadIdx.x & 31;
     const int32_t g = p.gap;
+    // a chunk's inputs of lane 0 and outputs of lane 31, per warp
+    __shared__ uint32_t ins_[kLocalWarps][32], outs_[kLocalWarps][32];
+    uint32_t *ins = ins_[threadIdx.x >> 5], *outs = outs_[threadIdx.x >> 5];
 
     for (;;) {
         uint32_t jidx = 0;
@@ -246,71 +241,70 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         uint4 *keep = MODE == kKeep ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * LocalLane<R>::kParts * 32u + lane
                                     : nullptr;
         int32_t best = 0, cm = 0;    // the lane's largest H before and in this chunk of 32 steps
-        uint32_t bt = 0, tie = 0;    // the chunk that first reached it, and whether another did
-        auto chunk_end = [&](uint32_t t) {
-            if (MODE != kScore) {
-                if (cm > best) {
-                    bt = t - 32u;
-                    tie = 0;
-                } else if (cm == best) {
-                    tie = 1u;
+        uint32_t bt = 0, bl = 0;     // the first and the last chunk that reached it
+        int32_t c = -lane;
+        uint32_t seen = 0;
+        bool alive = !s || warp_wait_geq(prev, min(32u, n), seen, p.err, jidx);
+        uint32_t next = alive ? above.word((uint32_t)lane) : 0u;
+        // the last chunk's bottom row (columns t - 63 .. t - 32 of lane 31) out, and published
+        auto row_out = [&](uint32_t t) {
+            if (!out) return;
+            __syncwarp();
+            const int32_t col = (int32_t)t - 63 + lane;
+            if (col >= 0 && col < (int32_t)n &&
+                in_range((size_t)(out - p.rows) + (uint32_t)col, p.rows_cap, p.err, kSiteLocalRing))
+                __stcg(out + col, outs[lane]);
+            __syncwarp();
+            if (lane == 0) st_release(mine, min(t - 31u, n));
+        };
+        for (uint32_t t = 0; t < T && alive; t += 32) {
+            if (MODE == kKeep && t && t % kTileSteps == 0) {
+                ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
+                keep += LocalLane<R>::kParts * 32u;
+            }
+            __syncwarp();
+            ins[lane] = next;
+            __syncwarp();
+            if (s && t + 32 < n && !(alive = warp_wait_geq(prev, min(t + 64u, n), seen, p.err, jidx))) break;
+            next = above.word(t + 32u + (uint32_t)lane);
+            if (__all_sync(kFull, c >= 0 && c + 32 <= (int32_t)n - 1)) {
+#pragma unroll 4
+                for (uint32_t uu = 0; uu < 32u; ++uu) {
+                    uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                    const uint32_t in = ins[uu];
+                    if (lane == 0) x = in;
+                    ln.template column<false>(g, x, cm);
+                    if (lane == 31) outs[uu] = ln.xout;
                 }
+                c += 32;
+            } else {
+                for (uint32_t uu = 0; uu < 32u && t + uu < T; ++uu) {
+                    uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
+                    const uint32_t in = ins[uu];
+                    if (lane == 0) x = in;
+                    if (c >= 0 && c < (int32_t)n) {
+                        ln.template column<false>(g, x, cm);
+                        if (lane == 31) outs[uu] = ln.xout;
+                    }
+                    ++c;
+                }
+            }
+            row_out(t + 32u);
+            if (MODE != kScore) {
+                if (cm > best) bt = t;
+                if (cm >= best) bl = t;
                 best = max(best, cm);
                 cm = 0;
             }
-        };
-        int32_t c = -lane;
-        bool alive = !s || local_wait(prev, min(32u, n), p.err, jidx);
-        uint32_t stage = 0, stage_next = alive ? above.word((uint32_t)lane) : 0u;
-        auto row_out = [&](uint32_t col) {
-            if (lane == 31 && out && in_range((size_t)(out - p.rows) + col, p.rows_cap, p.err, kSiteLocalRing)) {
-                out[col] = ln.xout;
-                if (((col + 1) & 31u) == 0 || col + 1 == n) st_release(mine, col + 1);
-            }
-        };
-        uint32_t t = 0;
-        for (; t < T && alive; ++t) {
-            if ((t & 31u) == 0) {
-                if (t) chunk_end(t);
-                if (MODE == kKeep && t && t % kTileSteps == 0) {
-                    ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
-                    keep += LocalLane<R>::kParts * 32u;
-                }
-                stage = stage_next;
-                if (s && t + 32 < n && !(alive = local_wait(prev, min(t + 64u, n), p.err, jidx))) break;
-                stage_next = above.word(t + 32u + (uint32_t)lane);
-                if (__all_sync(kFull, c >= 0 && c + 32 <= (int32_t)n - 1)) {
-#pragma unroll 4
-                    for (uint32_t uu = 0; uu < 32u; ++uu) {
-                        uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
-                        const uint32_t x0 = __shfl_sync(kFull, stage, uu);
-                        if (lane == 0) x = x0;
-                        ln.template column<false>(g, x, cm);
-                        row_out((uint32_t)c + uu);
-                    }
-                    c += 32;
-                    t += 31;
-                    continue;
-                }
-            }
-            uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
-            const uint32_t x0 = __shfl_sync(kFull, stage, t & 31u);
-            if (lane == 0) x = x0;
-            if (c >= 0 && c < (int32_t)n) {
-                ln.template column<false>(g, x, cm);
-                row_out((uint32_t)c);
-            }
-            ++c;
         }
         if (!alive) return;   // a wait gave up (NW_ERR_TIMEOUT is raised): leave
-        chunk_end((t + 31u) / 32u * 32u);
         if (MODE == kScore) best = cm;
         // the stripe's largest H and its first lane
         const int32_t top = __reduce_max_sync(kFull, best);
         if (lane == 0 && top > 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) atomicMax(p.scores + tk.out, top);
         if (MODE != kScore) {
             const uint32_t first = (uint32_t)__ffs(__ballot_sync(kFull, best == top)) - 1u;
-            if ((uint32_t)lane == first) p.best[jidx] = LocalBest{top, first, bt, tie};
+            if ((uint32_t)lane == first) p.best[jidx] = LocalBest{top, first, bt, bl};
         }
         __syncwarp();
     }
@@ -373,19 +367,24 @@ struct LocalReplay {
     }
 };
 
-// End cells and, with WALK, the walk back from them: one warp per pair,
-// longest pairs first.  WALK follows the path to the first cell whose H is 0;
+// End cells and, with WALK, the walk back from them: one CTA per pair,
+// longest pairs first.  WALK: its warps replay kTraceWarps tiles of the path's
+// stripe at once, the one of its cell and the ones before it (a path crosses
+// about 2.3 tiles of a stripe), then the first warp follows the path to the first cell whose H is 0;
 // moves in reverse order (0 diagonal, 1 vertical, 2 horizontal).  A run of
 // diagonal moves is taken at a time: lane q reads the cell q diagonal moves
 // on, and H there follows from the matches before it (a ballot).  Without
 // WALK no states are kept: a stripe is replayed from its start.
 template <int R, bool WALK>
-__global__ void __launch_bounds__(32) k_local_trace(LocalArgs p, uint32_t ntasks, uint8_t *moves,
-                                                    const uint64_t *move_off, uint64_t *nmoves) {
+__global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(LocalArgs p, uint32_t ntasks,
+                                                                              uint8_t *moves, const uint64_t *move_off,
+                                                                              uint64_t *nmoves) {
     using Bits = LocalBits<R>;
     constexpr uint32_t SH = 32u * R;
-    __shared__ typename Bits::Word tile[WALK ? kTileSteps * 32 : 1];  // [step][lane]
-    const uint32_t lane = threadIdx.x;
+    extern __shared__ uint4 tiles_[];  // [tile][step][lane]
+    __shared__ int32_t at[3];          // i, j, h between the warps
+    typename Bits::Word *tiles = reinterpret_cast<typename Bits::Word *>(tiles_);
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     for (uint32_t q = blockIdx.x; q < ntasks; q += gridDim.x) {
         const LocalTask tk = p.tasks[q];
         const uint32_t m = tk.m, n = tk.n, S = (m && n) ? (m + SH - 1) / SH : 1u;
@@ -402,10 +401,10 @@ __global__ void __launch_bounds__(32) k_local_trace(LocalArgs p, uint32_t ntasks
         }
         uint32_t i = 0, j = 0;
         LocalReplay<R> rp;
-        if (bv > 0) {
+        if (bv > 0 && warp == 0) {
             // the first cell in row-major order among the best lane's rows
             const LocalBest b = p.best[tk.job0 + bs];
-            const uint32_t lo = b.tie ? 0u : b.t0, hi = b.tie ? n + 31u : min(b.t0 + 32u, n + 31u);
+            const uint32_t lo = b.t0, hi = min(b.t1 + 32u, n + 31u);
             if (!WALK && p.turn) {
                 // the rows above were overwritten: sweep the stripes above again
                 for (uint32_t s = 0; s < bs; ++s) {
@@ -441,7 +440,7 @@ __global__ void __launch_bounds__(32) k_local_trace(LocalArgs p, uint32_t ntasks
             i = __shfl_sync(kFull, i, b.lane);
             j = __shfl_sync(kFull, j, b.lane);
         }
-        if (lane == 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
+        if (threadIdx.x == 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
             p.ends[4 * (size_t)tk.out + 2] = i;
             p.ends[4 * (size_t)tk.out + 3] = j;
             if (!WALK) p.ends[4 * (size_t)tk.out + 0] = p.ends[4 * (size_t)tk.out + 1] = ~0u;  // not computed
@@ -451,26 +450,40 @@ __global__ void __launch_bounds__(32) k_local_trace(LocalArgs p, uint32_t ntasks
             uint8_t *mv = moves + move_off[q];
             int32_t h = bv;
             uint64_t k = 0;
-            while (h > 0 && i > 0 && j > 0) {
-                // the tile of cell (i, j)
-                const uint32_t s = (i - 1) / SH, tc = (j - 1) + ((i - 1) % SH) / R, t0 = tc - tc % kTileSteps;
-                rp.begin(p, tk, s, t0, lane);
-                __syncwarp();
-                while (rp.t <= tc) {
-                    const uint32_t t = rp.t;
-                    if (rp.template step<true>(p.gap, lane))
-                        tile[(t - t0) * 32u + lane] = Bits::pack(rp.ln.accL, rp.ln.accH);
+            for (;;) {
+                if (threadIdx.x == 0) {
+                    at[0] = (int32_t)i;
+                    at[1] = (int32_t)j;
+                    at[2] = h;
                 }
-                __syncwarp();
-                // (uniform over the warp from here: every lane follows the same walk)
+                __syncthreads();
+                i = (uint32_t)at[0];
+                j = (uint32_t)at[1];
+                h = at[2];
+                if (!(h > 0 && i > 0 && j > 0)) break;
+                // the tile of cell (i, j) and the ones before it in its stripe
+                const uint32_t s = (i - 1) / SH, tc = (j - 1) + ((i - 1) % SH) / R, tl = tc / kTileSteps;
+                const uint32_t ntile = min(tl + 1u, (uint32_t)kTraceWarps), t0 = (tl + 1u - ntile) * kTileSteps;
+                if (warp < ntile) {
+                    typename Bits::Word *tile = tiles + warp * kTileSteps * 32u;
+                    const uint32_t tw = t0 + warp * kTileSteps, te = min(tc, tw + kTileSteps - 1u);
+                    rp.begin(p, tk, s, tw, lane);
+                    while (rp.t <= te) {
+                        const uint32_t t = rp.t;
+                        if (rp.template step<true>(p.gap, lane))
+                            tile[(t - tw) * 32u + lane] = Bits::pack(rp.ln.accL, rp.ln.accH);
+                    }
+                }
+                __syncthreads();
+                // (uniform over the first warp from here: every lane follows the same walk)
                 auto step_of = [&](uint32_t i_, uint32_t j_) { return (j_ - 1) + ((i_ - 1) % SH) / R; };
-                while (h > 0 && i > 0 && j > 0 && (i - 1) / SH == s && step_of(i, j) >= t0) {
+                while (warp == 0 && h > 0 && i > 0 && j > 0 && (i - 1) / SH == s && step_of(i, j) >= t0) {
                     uint32_t stop = 1u, gapm = 0u, same = 0u;
                     if (lane < i && lane < j) {
                         const uint32_t iq = i - lane, jq = j - lane;
                         if ((iq - 1) / SH == s && step_of(iq, jq) >= t0) {
                             const uint32_t l = ((iq - 1) % SH) / R, r = (iq - 1) % R;
-                            const typename Bits::Word w = tile[(jq - 1 + l - t0) * 32u + l];
+                            const typename Bits::Word w = tiles[(jq - 1 + l - t0) * 32u + l];
                             stop = Bits::bit(w, 0, r);
                             gapm = stop ? 1u + Bits::bit(w, 1, r) : 0u;  // the gap move that ends the run
                             same = base_at(A, iq - 1) == base_at(B, jq - 1);
@@ -498,13 +511,14 @@ __global__ void __launch_bounds__(32) k_local_trace(LocalArgs p, uint32_t ntasks
                     }
                 }
             }
-            if (lane == 0) {
+            if (threadIdx.x == 0) {
                 if (in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
                     p.ends[4 * (size_t)tk.out + 0] = i;
                     p.ends[4 * (size_t)tk.out + 1] = j;
                 }
                 nmoves[q] = k;
             }
+            __syncthreads();
         }
         __syncwarp();
     }
@@ -542,14 +556,28 @@ int launch_local(nw_ctx *ctx, int R, LocalMode mode, LocalArgs &la) {
 #undef NW_LOCAL_CASES
 }
 
-template <bool WALK>
-void launch_local_trace(nw_ctx *ctx, int R, const LocalArgs &la, uint32_t ntasks, uint8_t *moves,
-                        const uint64_t *move_off, uint64_t *nmoves) {
+template <int R, bool WALK>
+int launch_local_trace_R(nw_ctx *ctx, const LocalArgs &la, uint32_t ntasks, uint8_t *moves, const uint64_t *move_off,
+                         uint64_t *nmoves) {
+    constexpr int smem = WALK ? kTraceWarps * (int)kTileSteps * 32 * (int)sizeof(typename LocalBits<R>::Word) : 0;
+    if (smem + 64 > 48 * 1024) {  // (with the static words)
+        // one value for every caller: the attribute belongs to the process
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_local_trace<R, WALK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "local trace shared memory");
+    }
     LaunchTimer t(ctx, WALK ? "local_walk" : "local_ends");
-    const uint32_t blocks = std::min<uint32_t>(ntasks, 65535);
-    if (R == 4) k_local_trace<4, WALK><<<blocks, 32, 0, ctx->stream>>>(la, ntasks, moves, move_off, nmoves);
-    else if (R == 16) k_local_trace<16, WALK><<<blocks, 32, 0, ctx->stream>>>(la, ntasks, moves, move_off, nmoves);
-    else k_local_trace<8, WALK><<<blocks, 32, 0, ctx->stream>>>(la, ntasks, moves, move_off, nmoves);
+    k_local_trace<R, WALK><<<std::min<uint32_t>(ntasks, 65535), WALK ? 32 * kTraceWarps : 32, smem, ctx->stream>>>(
+        la, ntasks, moves, move_off, nmoves);
+    return NW_OK;
+}
+
+template <bool WALK>
+int launch_local_trace(nw_ctx *ctx, int R, const LocalArgs &la, uint32_t ntasks, uint8_t *moves,
+                       const uint64_t *move_off, uint64_t *nmoves) {
+    if (R == 4) return launch_local_trace_R<4, WALK>(ctx, la, ntasks, moves, move_off, nmoves);
+    if (R == 16) return launch_local_trace_R<16, WALK>(ctx, la, ntasks, moves, move_off, nmoves);
+    return launch_local_trace_R<8, WALK>(ctx, la, ntasks, moves, move_off, nmoves);
 }
 
 template <typename T>
@@ -672,9 +700,9 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         const uint32_t nt = (uint32_t)wave.size();
         k0 = k;
         if ((rc = launch_local(ctx, R, mode, la))) return rc;
-        if (mode == kEnds) launch_local_trace<false>(ctx, R, la, nt, nullptr, nullptr, nullptr);
+        if (mode == kEnds && (rc = launch_local_trace<false>(ctx, R, la, nt, nullptr, nullptr, nullptr))) return rc;
         if (!want) continue;
-        launch_local_trace<true>(ctx, R, la, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm);
+        if ((rc = launch_local_trace<true>(ctx, R, la, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm))) return rc;
         std::vector<TraceTask> tt(wave.size());
         for (size_t q = 0; q < wave.size(); ++q) {
             const LocalTask &t = wave[q];
