@@ -218,6 +218,7 @@ static int check_band_scoring(nw_ctx *ctx, const nw_scoring &sc) {
 // single-pair kernel on a long pair; the bit-sliced one runs a chain of
 // m + n + m/31 steps of about 30 ns, then its walk.
 constexpr double kWarpRate = 2e9, kBatchRate = 3.5e12, kPairRate = 2e11, kPairFixed = 1e-3;
+constexpr double kBitsBatchRate = 2.5e13;  // the bit-sliced score kernel, all lanes busy
 constexpr double kBitsStepSeconds = 30e-9, kBitsPairFixed = 0.3e-3;
 
 struct PairCost {
@@ -955,11 +956,17 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     {
         std::vector<double> wc(tasks.size()), fc(tasks.size());
         std::vector<PairCost> ps(tasks.size());
+        double total = 0, longest = 0;
         for (size_t q = 0; q < tasks.size(); ++q) {
             wc[q] = fc[q] = (double)tasks[q].m * tasks[q].n;
+            total += wc[q];
+            longest = std::max(longest, wc[q]);
             ps[q] = single_pair_cost(tasks[q].m, tasks[q].n, sc);
         }
-        std::vector<size_t> strag = pick_stragglers(wc, fc, ps, ctx->sm_count);
+        // (no pair outlasts the batch: nothing to route)
+        const double rate = !want && bits_scoring_ok(sc) ? kBitsBatchRate : kBatchRate;
+        std::vector<size_t> strag;
+        if (longest / kWarpRate > total / rate) strag = pick_stragglers(wc, fc, ps, ctx->sm_count, rate);
         if (want) {
             const uint64_t room = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
             std::vector<char> in(tasks.size(), 0);
@@ -996,21 +1003,22 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     // choice (tuned on score-only launches of the whole list)
     int R = pick_rows(tasks);
     if (!want || ctx->autotune) {
-        std::vector<BatchTask> lpt = tasks;
-        sort_lpt(lpt);
-        BatchTask *dt = nullptr;
-        if ((rc = upload(ctx, (pre + "_tasks").c_str(), lpt, &dt))) return rc;
-        BatchArgs bs = ba;
-        bs.tasks = dt;
-        bs.ntasks = npairs;
-        bs.score_cap = score_slots(lpt.data(), npairs);
         // score-only: the bit-sliced kernel (rows per lane 32) where the
         // scoring fits two bit planes
         const bool bits = !want && bits_scoring_ok(sc);
+        const uint32_t cap = score_slots(tasks.data(), npairs);
         BitsPlan bp;
-        if (bits) {
-            std::vector<BatchTask> bt = lpt;
-            if ((rc = bits_prepare(ctx, pool, bt, sc, scores, bs.score_cap, pre, &bp))) return rc;
+        if (bits && (rc = bits_prepare(ctx, pool, tasks, sc, scores, cap, pre, &bp))) return rc;
+        std::vector<BatchTask> lpt;
+        BatchArgs bs = ba;
+        if (!bits || ctx->autotune) {  // the scalar kernel runs, or is timed
+            lpt = tasks;
+            sort_lpt(lpt);
+            BatchTask *dt = nullptr;
+            if ((rc = upload(ctx, (pre + "_tasks").c_str(), lpt, &dt))) return rc;
+            bs.tasks = dt;
+            bs.ntasks = npairs;
+            bs.score_cap = cap;
         }
         auto run = [&](int r) { return r == 32 ? bits_launch(ctx, bp) : launch_batch(ctx, r, false, bs, max_n, 0, pre); };
         if ((rc = tune_rows(ctx, lpt, bits ? 32 : R, run, &R, bits))) return rc;
@@ -1355,28 +1363,14 @@ extern "C" int nw_score_all_pairs(nw_ctx *ctx, const uint8_t *pool2b, const uint
         if (replayed) return copy_back();
         pre = "g" + std::to_string(++ctx->graph_seq);
     }
-    // n(n-1)/2 pairs (Eq. 2), each written to both triangle entries
+    // n(n-1)/2 pairs (Eq. 2), each written to both triangle entries: on the
+    // bit-sliced kernel where the scoring fits two bit planes (rows per lane
+    // 32), else -- or as the autotuner finds -- on the scalar batch kernel
+    const bool bits = bits_scoring_ok(sc);
+    BitsPlan bp;
+    if (bits && (rc = bits_prepare_all(ctx, pool, off, len, nseq, sc, dout, pre, &bp))) return rc;
     std::vector<BatchTask> tasks;
-    tasks.reserve((size_t)nseq * (nseq - 1) / 2);
     uint32_t max_n = 1;
-    for (uint32_t i = 0; i < nseq; ++i)
-        for (uint32_t j = i + 1; j < nseq; ++j) {
-            BatchTask t{};
-            // rows: the sequence whose 256-row stripes waste fewer padded rows
-            const uint32_t SH = 256;
-            const uint32_t wi = (len[i] + SH - 1) / SH * SH - len[i], wj = (len[j] + SH - 1) / SH * SH - len[j];
-            const bool rows_i = (uint64_t)wi * len[j] <= (uint64_t)wj * len[i] || len[j] < kMinPeriod;
-            const uint32_t r = rows_i ? i : j, c = rows_i ? j : i;
-            t.a_off = off[r];
-            t.m = len[r];
-            t.b_off = off[c];
-            t.n = len[c];
-            t.out0 = i * nseq + j;
-            t.out1 = j * nseq + i;
-            max_n = std::max(max_n, t.n);
-            tasks.push_back(t);
-        }
-    sort_lpt(tasks);
     const Profile pf = make_profile(sc);
     BatchArgs ba{};
     ba.pool = pool;
@@ -1384,22 +1378,35 @@ extern "C" int nw_score_all_pairs(nw_ctx *ctx, const uint8_t *pool2b, const uint
     ba.gap = pf.gap;
     ba.scores = dout;
     ba.err = ctx->d_err;
-    ba.ntasks = (uint32_t)tasks.size();
     ba.score_cap = nseq * nseq;
+    if (!bits || ctx->autotune) {
+        tasks.reserve((size_t)nseq * (nseq - 1) / 2);
+        for (uint32_t i = 0; i < nseq; ++i)
+            for (uint32_t j = i + 1; j < nseq; ++j) {
+                BatchTask t{};
+                // rows: the sequence whose 256-row stripes waste fewer padded rows
+                const uint32_t SH = 256;
+                const uint32_t wi = (len[i] + SH - 1) / SH * SH - len[i], wj = (len[j] + SH - 1) / SH * SH - len[j];
+                const bool rows_i = (uint64_t)wi * len[j] <= (uint64_t)wj * len[i] || len[j] < kMinPeriod;
+                const uint32_t r = rows_i ? i : j, c = rows_i ? j : i;
+                t.a_off = off[r];
+                t.m = len[r];
+                t.b_off = off[c];
+                t.n = len[c];
+                t.out0 = i * nseq + j;
+                t.out1 = j * nseq + i;
+                max_n = std::max(max_n, t.n);
+                tasks.push_back(t);
+            }
+        sort_lpt(tasks);
+        BatchTask *dt = nullptr;
+        if ((rc = upload(ctx, (pre + "_tasks").c_str(), tasks, &dt))) return rc;
+        ba.tasks = dt;
+        ba.ntasks = (uint32_t)tasks.size();
+    }
     std::vector<uint32_t> lens(len, len + nseq);
     uint32_t *dlen = nullptr;
     if ((rc = upload(ctx, (pre + "_len").c_str(), lens, &dlen))) return rc;
-    // the bit-sliced kernel where the scoring fits two bit planes (rows per
-    // lane 32), else -- or as the autotuner finds -- the scalar batch kernel
-    const bool bits = bits_scoring_ok(sc);
-    BitsPlan bp;
-    if (bits) {
-        std::vector<BatchTask> bt = tasks;
-        if ((rc = bits_prepare(ctx, pool, bt, sc, dout, nseq * nseq, pre, &bp))) return rc;
-    }
-    BatchTask *dt = nullptr;
-    if ((rc = upload(ctx, (pre + "_tasks").c_str(), tasks, &dt))) return rc;
-    ba.tasks = dt;
     auto run = [&](int r) { return r == 32 ? bits_launch(ctx, bp) : launch_batch(ctx, r, false, ba, max_n, 0, pre); };
     int R = 16;
     if ((rc = tune_rows(ctx, tasks, bits ? 32 : pick_rows(tasks), run, &R, bits))) return rc;

@@ -35,9 +35,11 @@
 // last stripe's outgoing words with population counts.
 #include <algorithm>
 #include <cstdlib>
+#include <cstring>
 #include <vector>
 
 #include "nw_bits.cuh"
+#include "nw_order.h"
 
 namespace nw {
 
@@ -156,6 +158,25 @@ __device__ __forceinline__ void bits_stripe(const BitsArgs &p, uint32_t C, uint3
     }
 }
 
+// Row and column of the q-th pair of a class: the columns before the class's
+// rows pair with all of them, a column among them with the rows after it.
+__device__ __forceinline__ void class_pair(const BitsClass &k, uint32_t q, uint32_t &r, uint32_t &c) {
+    const uint32_t rows = k.r1 - k.r0, whole = k.r0 * rows;
+    if (q < whole) {
+        c = q / rows;
+        r = k.r0 + q % rows;
+        return;
+    }
+    // the x-th column among the rows starts at x (2 rows - x - 1) / 2
+    const uint64_t t = q - whole, b = 2ull * rows - 1ull;
+    uint64_t x = (uint64_t)(((double)b - sqrt(fmax((double)(b * b) - 8.0 * (double)t, 0.0))) * 0.5);
+    if (x > rows - 2ull) x = rows - 2ull;
+    while (x > 0 && x * (b - x) / 2ull > t) --x;
+    while ((x + 1ull) * (b - x - 1ull) / 2ull <= t) ++x;
+    c = k.r0 + (uint32_t)x;
+    r = c + 1u + (uint32_t)(t - x * (b - x) / 2ull);
+}
+
 template <bool GEN>
 __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -168,11 +189,29 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
         if (jid >= p.njobs) break;
         const BitsJob job = p.jobs[jid];
         const bool active = lane < job.cnt;
-        const BatchTask tk = p.tasks[job.t0 + (active ? lane : 0u)];
-        const uint32_t m = tk.m, n = tk.n;
+        uint32_t m, n, aw, bw, out0, out1;
+        if (p.tasks) {
+            const BitsTask tk = p.tasks[job.t0 + (active ? lane : 0u)];
+            m = tk.m;
+            n = tk.n;
+            aw = tk.aw;
+            bw = tk.bw;
+            out0 = tk.out0;
+            out1 = tk.out1;
+        } else {
+            uint32_t r, c;
+            class_pair(p.classes[job.cls], job.t0 + (active ? lane : 0u), r, c);
+            const BitsSeq a = p.seqs[r], b = p.seqs[c];
+            m = a.len;
+            n = b.len;
+            aw = a.w;
+            bw = b.w;
+            out0 = a.id * p.nseq + b.id;
+            out1 = b.id * p.nseq + a.id;
+        }
         const uint32_t S = job.S, C = job.C;
         int32_t W = 0;
-        const int64_t Ag = (int64_t)tk.a_off, Bg = (int64_t)tk.b_off;  // planar slots
+        const int64_t Ag = (int64_t)aw * 32 - kPlanePad, Bg = (int64_t)bw * 32 - kPlanePad;  // planar slots
         const int32_t top0 = (int32_t)m - 32 * (int32_t)S;             // row above bit 0 of stripe 0
         for (uint32_t s = 0; s < S; ++s) {
             const int64_t abase = max(Ag + top0 + 32 * (int64_t)s, Ag - 32);
@@ -182,8 +221,8 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
         }
         if (active) {
             const int32_t sc = W + p.gap * (int32_t)(m + n);
-            if (in_range(tk.out0, p.score_cap, p.err, kSiteBatchScore)) p.scores[tk.out0] = sc;
-            if (tk.out1 != ~0u && in_range(tk.out1, p.score_cap, p.err, kSiteBatchScore)) p.scores[tk.out1] = sc;
+            if (in_range(out0, p.score_cap, p.err, kSiteBatchScore)) p.scores[out0] = sc;
+            if (out1 != ~0u && in_range(out1, p.score_cap, p.err, kSiteBatchScore)) p.scores[out1] = sc;
         }
     }
 }
@@ -199,27 +238,45 @@ __device__ __forceinline__ uint32_t even_bits(uint64_t x) {
     return (uint32_t)x;
 }
 
-// Planar copy of the launch's sequences: one warp per sequence; word w of
-// its slot holds bit k of the codes of its bases 32w .. 32w+31 (bases past
-// its end read as 0).
+// Planar copy of a sequence by a warp: word w of its slot holds bit k of the
+// codes of its bases 32w .. 32w+31 (bases past its end read as 0).
+__device__ __forceinline__ void plane_copy(const uint8_t *src, uint32_t nbytes, uint32_t dst, uint32_t lane,
+                                           uint32_t *pl0, uint32_t *pl1) {
+    const uint32_t words = (nbytes + 7) / 8;
+    for (uint32_t w = lane; w < words; w += 32) {
+        uint64_t v = 0;
+        const uint32_t b0 = 8 * w;
+        if (b0 + 8 <= nbytes) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v |= (uint64_t)src[b0 + k] << (8 * k);
+        } else {
+            for (uint32_t k = 0; b0 + k < nbytes; ++k) v |= (uint64_t)src[b0 + k] << (8 * k);
+        }
+        pl0[dst + w] = even_bits(v);
+        pl1[dst + w] = even_bits(v >> 1);
+    }
+}
+
+// The launch's distinct sequences, one warp per sequence.
 __global__ void k_planes(const uint8_t *pool, const PlaneSeg *segs, uint32_t nsegs, uint32_t *pl0, uint32_t *pl1) {
     const uint32_t lane = threadIdx.x & 31u;
     for (uint32_t sg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; sg < nsegs; sg += (gridDim.x * blockDim.x) >> 5) {
         const PlaneSeg seg = segs[sg];
         const uint8_t *src = pool ? pool + seg.src : reinterpret_cast<const uint8_t *>(seg.src);  // offset or address
-        const uint32_t words = (seg.nbytes + 7) / 8;
-        for (uint32_t w = lane; w < words; w += 32) {
-            uint64_t v = 0;
-            const uint32_t b0 = 8 * w;
-            if (b0 + 8 <= seg.nbytes) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) v |= (uint64_t)src[b0 + k] << (8 * k);
-            } else {
-                for (uint32_t k = 0; b0 + k < seg.nbytes; ++k) v |= (uint64_t)src[b0 + k] << (8 * k);
-            }
-            pl0[seg.dst + w] = even_bits(v);
-            pl1[seg.dst + w] = even_bits(v >> 1);
-        }
+        plane_copy(src, seg.nbytes, seg.dst, lane, pl0, pl1);
+    }
+}
+
+// Both sequences of every task, into the task's own slots.
+__global__ void k_planes_tasks(const uint8_t *pool, const BitsTask *tasks, uint32_t ntasks, uint32_t *pl0,
+                               uint32_t *pl1) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < 2 * ntasks;
+         k += (gridDim.x * blockDim.x) >> 5) {
+        const BitsTask t = tasks[k >> 1];
+        if (!t.m || !t.n) continue;  // no slots
+        if (k & 1u) plane_copy(pool + t.b_off, (t.n + 3) / 4, t.bw, lane, pl0, pl1);
+        else plane_copy(pool + t.a_off, (t.m + 3) / 4, t.aw, lane, pl0, pl1);
     }
 }
 
@@ -308,74 +365,35 @@ bool bits_scoring_ok(const nw_scoring &sc) {
     return sx >= 0 && sx <= sm && sm <= 3;
 }
 
-template <typename T>
-static int bits_upload(nw_ctx *ctx, const std::string &slot, const std::vector<T> &v, T **dev) {
-    void *d = nullptr;
-    int rc = scratch(ctx, slot.c_str(), v.size() * sizeof(T) + 16, &d);
-    if (rc) return rc;
-    if (!v.empty()) {
-        cudaError_t e = cudaMemcpyAsync(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // the host vector is temporary
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "bit-sliced task upload");
-    }
-    *dev = (T *)d;
-    return NW_OK;
-}
+// Stripes and chunks per stripe of an m x n pair.
+static uint32_t stripes_of(uint32_t m) { return (m + 31) / 32; }
+static uint32_t chunks_of(uint32_t n) { return (n + 62) / 32; }
 
-int bits_prepare(nw_ctx *ctx, const uint8_t *pool, std::vector<BatchTask> &tasks, const nw_scoring &sc,
-                 int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan) {
+// The launch's tables in one upload, its constants, grid and row buffers.
+// `head`: the task table, or the sequence and class tables (16-byte padded).
+static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_t> &head, std::vector<BitsJob> &jobs,
+                            uint32_t maxC, const nw_scoring &sc, int32_t *scores, uint32_t score_cap,
+                            const std::string &prefix, BitsPlan *plan, void **dhead) {
     int rc;
-    *plan = BitsPlan{};
-    if (tasks.empty()) return NW_OK;
-    // rows: the orientation with fewer stripe-chunks (the score is symmetric)
-    auto S_of = [](uint32_t m) { return (m + 31) / 32; };
-    auto C_of = [](uint32_t n) { return (n + 62) / 32; };
-    for (auto &t : tasks) {
-        if (t.m == 0 || t.n == 0) continue;
-        if ((uint64_t)S_of(t.n) * C_of(t.m) < (uint64_t)S_of(t.m) * C_of(t.n)) {
-            std::swap(t.a_off, t.b_off);
-            std::swap(t.m, t.n);
-        }
-    }
-    // jobs: equal stripe counts, widest first, at most 32 pairs each
-    auto S_task = [&](const BatchTask &t) { return (t.m && t.n) ? S_of(t.m) : 0u; };
-    std::stable_sort(tasks.begin(), tasks.end(), [&](const BatchTask &x, const BatchTask &y) {
-        const uint32_t sx = S_task(x), sy = S_task(y);
-        if (sx != sy) return sx > sy;
-        return x.n > y.n;
-    });
-    std::vector<BitsJob> jobs;
-    uint32_t maxC = 1;
-    for (uint32_t k = 0; k < tasks.size();) {
-        const uint32_t S = S_task(tasks[k]);
-        BitsJob j{k, 0, S, S ? C_of(tasks[k].n) : 0};
-        while (k < tasks.size() && j.cnt < 32 && S_task(tasks[k]) == S) {
-            ++j.cnt;
-            ++k;
-        }
-        maxC = std::max(maxC, j.C);
-        jobs.push_back(j);
-    }
-    std::stable_sort(jobs.begin(), jobs.end(),
-                     [](const BitsJob &x, const BitsJob &y) { return (uint64_t)x.S * x.C > (uint64_t)y.S * y.C; });
-
-    void *v = nullptr;
-    // the tasks address their sequences by planar slot
-    for (auto &t : tasks) {
-        if (!t.m || !t.n) continue;
-        t.a_off = (uint64_t)plan->planes.add(t.a_off, t.m);
-        t.b_off = (uint64_t)plan->planes.add(t.b_off, t.n);
-    }
+    // longest jobs first, ties in job order
+    std::vector<uint64_t> keys(jobs.size());
+    for (size_t q = 0; q < jobs.size(); ++q) keys[q] = (uint64_t)jobs[q].S * jobs[q].C;
+    const std::vector<uint32_t> jo = radix_order_desc(std::move(keys));
+    const size_t jobs_at = (head.size() + 15) / 16 * 16;
+    head.resize(jobs_at + jobs.size() * sizeof(BitsJob));
+    BitsJob *hj = reinterpret_cast<BitsJob *>(head.data() + jobs_at);
+    for (size_t q = 0; q < jobs.size(); ++q) hj[q] = jobs[jo[q]];
     if ((rc = plan->planes.prepare(ctx, prefix))) return rc;
     BitsArgs &ba = plan->ba;
     ba.pl0 = plan->planes.pl0;
     ba.pl1 = plan->planes.pl1;
-    BatchTask *dt = nullptr;
-    BitsJob *dj = nullptr;
-    if ((rc = bits_upload(ctx, prefix + "_bits_tasks", tasks, &dt))) return rc;
-    if ((rc = bits_upload(ctx, prefix + "_bits_jobs", jobs, &dj))) return rc;
-    ba.tasks = dt;
-    ba.jobs = dj;
+    void *v = nullptr;
+    if ((rc = scratch(ctx, (prefix + "_bits_plan").c_str(), head.size() + 16, &v))) return rc;
+    cudaError_t e = cudaMemcpyAsync(v, head.data(), head.size(), cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // the host table is temporary
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "bit-sliced plan upload");
+    *dhead = v;
+    ba.jobs = reinterpret_cast<const BitsJob *>((const uint8_t *)v + jobs_at);
     ba.njobs = (uint32_t)jobs.size();
     ba.scores = scores;
     ba.score_cap = score_cap;
@@ -413,10 +431,133 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, std::vector<BatchTask> &tasks
     return NW_OK;
 }
 
+int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> &tasks, const nw_scoring &sc,
+                 int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan) {
+    *plan = BitsPlan{};
+    if (tasks.empty()) return NW_OK;
+    HostTimer ht(ctx, "bits_plan");
+    // rows: the orientation with fewer stripe-chunks (the score is symmetric);
+    // order: equal stripe counts, widest first
+    const size_t n = tasks.size();
+    std::vector<uint64_t> keys(n);
+    std::vector<uint8_t> turned(n);
+    uint64_t bytes = 0, extent = 0;
+    for (size_t k = 0; k < n; ++k) {
+        const BatchTask &t = tasks[k];
+        if (!t.m || !t.n) {
+            keys[k] = std::max(t.m, t.n);  // no stripes
+            continue;
+        }
+        turned[k] = (uint64_t)stripes_of(t.n) * chunks_of(t.m) < (uint64_t)stripes_of(t.m) * chunks_of(t.n);
+        const uint32_t rows = turned[k] ? t.n : t.m, cols = turned[k] ? t.m : t.n;
+        keys[k] = (uint64_t)stripes_of(rows) << 32 | cols;
+        bytes += (t.m + 3) / 4 + (t.n + 3) / 4;
+        extent = std::max(extent, std::max(t.a_off + (t.m + 3) / 4, t.b_off + (t.n + 3) / 4));
+    }
+    const std::vector<uint32_t> order = radix_order_desc(std::move(keys));
+    // Planar copies: a slot for each of a task's sequences, unless the tasks
+    // read their sequences several times over (then the distinct sequences,
+    // found by hashing, which costs the host more than the device saves
+    // otherwise: 20,000 pairs of distinct reads, 1 ms).
+    const bool own = bytes <= 2 * extent;
+    uint64_t words = 2;
+    if (!own) plan->planes.reserve(std::min<size_t>(2 * n, 1u << 16));
+    std::vector<uint8_t> head(n * sizeof(BitsTask));
+    BitsTask *ht_ = reinterpret_cast<BitsTask *>(head.data());
+    std::vector<BitsJob> jobs;
+    uint32_t maxC = 1;
+    for (size_t q = 0; q < n; ++q) {
+        const BatchTask &t = tasks[order[q]];
+        BitsTask b{t.a_off, t.b_off, 2, 2, t.m, t.n, t.out0, t.out1};
+        if (turned[order[q]]) {
+            std::swap(b.a_off, b.b_off);
+            std::swap(b.m, b.n);
+        }
+        const uint32_t S = (b.m && b.n) ? stripes_of(b.m) : 0u;
+        if (S && own) {
+            b.aw = (uint32_t)words;
+            b.bw = b.aw + (b.m + 31) / 32 + 2;
+            words = (uint64_t)b.bw + (b.n + 31) / 32 + 2;
+            if (words >= (1ull << 32)) return fail(ctx, NW_ERR_ARG, "planar copy of more than 2^37 bases");
+        } else if (S) {
+            b.aw = PlaneSet::word_of(plan->planes.add(b.a_off, b.m));
+            b.bw = PlaneSet::word_of(plan->planes.add(b.b_off, b.n));
+        }
+        ht_[q] = b;
+        if (jobs.empty() || jobs.back().S != S || jobs.back().cnt == 32)
+            jobs.push_back(BitsJob{(uint32_t)q, 0, S, S ? chunks_of(b.n) : 0, 0});
+        ++jobs.back().cnt;
+        maxC = std::max(maxC, jobs.back().C);
+    }
+    if (own) {
+        plan->planes.reserve_words(words - 2);
+        plan->ntasks = (uint32_t)n;
+    }
+    void *dh = nullptr;
+    const int rc = bits_finish_plan(ctx, pool, head, jobs, maxC, sc, scores, score_cap, prefix, plan, &dh);
+    plan->ba.tasks = (const BitsTask *)dh;
+    return rc;
+}
+
+int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, const uint32_t *len, uint32_t nseq,
+                     const nw_scoring &sc, int32_t *scores, const std::string &prefix, BitsPlan *plan) {
+    *plan = BitsPlan{};
+    HostTimer ht(ctx, "bits_plan");
+    std::vector<uint64_t> keys(nseq);
+    for (uint32_t i = 0; i < nseq; ++i) keys[i] = len[i];
+    const std::vector<uint32_t> order = radix_order_desc(std::move(keys));
+    plan->planes.reserve(nseq);
+    const size_t classes_at = (nseq * sizeof(BitsSeq) + 15) / 16 * 16;
+    std::vector<BitsSeq> seqs(nseq);
+    for (uint32_t q = 0; q < nseq; ++q) {
+        const uint32_t i = order[q];
+        seqs[q] = BitsSeq{len[i] ? PlaneSet::word_of(plan->planes.add(off[i], len[i])) : 2u, len[i], i};
+    }
+    std::vector<BitsClass> classes;
+    std::vector<BitsJob> jobs;
+    uint32_t maxC = 1;
+    for (uint32_t r0 = 0; r0 < nseq;) {
+        const uint32_t S = stripes_of(seqs[r0].len);
+        uint32_t r1 = r0;
+        while (r1 < nseq && stripes_of(seqs[r1].len) == S) ++r1;
+        const uint32_t rows = r1 - r0, pairs = r0 * rows + rows * (rows - 1) / 2;
+        // the pairs run through the columns in order: a job's first column is its widest
+        uint32_t c = 0;
+        auto end_of = [&](uint32_t col) {  // pairs of the columns up to col
+            const uint32_t x = col < r0 ? 0u : col - r0 + 1u;
+            return col < r0 ? (col + 1u) * rows : r0 * rows + (uint32_t)((uint64_t)x * (2ull * rows - x - 1u) / 2u);
+        };
+        for (uint32_t q = 0; q < pairs; q += 32) {
+            while (end_of(c) <= q) ++c;
+            jobs.push_back(BitsJob{q, std::min(32u, pairs - q), S, S ? chunks_of(seqs[c].len) : 0,
+                                   (uint32_t)classes.size()});
+            maxC = std::max(maxC, jobs.back().C);
+        }
+        classes.push_back(BitsClass{r0, r1});
+        r0 = r1;
+    }
+    std::vector<uint8_t> head(classes_at + classes.size() * sizeof(BitsClass));
+    memcpy(head.data(), seqs.data(), nseq * sizeof(BitsSeq));
+    memcpy(head.data() + classes_at, classes.data(), classes.size() * sizeof(BitsClass));
+    void *dh = nullptr;
+    const int rc = bits_finish_plan(ctx, pool, head, jobs, maxC, sc, scores, nseq * nseq, prefix, plan, &dh);
+    plan->ba.seqs = (const BitsSeq *)dh;
+    plan->ba.classes = (const BitsClass *)((const uint8_t *)dh + classes_at);
+    plan->ba.nseq = nseq;
+    return rc;
+}
+
 int bits_launch(nw_ctx *ctx, const BitsPlan &plan) {
     if (plan.ba.njobs == 0) return NW_OK;
     cudaMemsetAsync(plan.ba.counter, 0, 4, ctx->stream);
-    if (int rc = plan.planes.enqueue(ctx, plan.pool)) return rc;
+    if (plan.ntasks) {
+        LaunchTimer t(ctx, "planes");
+        const uint32_t blocks = std::min<uint32_t>((plan.ntasks + 3) / 4, 4096);
+        k_planes_tasks<<<blocks, 256, 0, ctx->stream>>>(plan.pool, plan.ba.tasks, plan.ntasks, plan.planes.planes(),
+                                                        plan.planes.planes() + plan.planes.plane_words());
+    } else if (int rc = plan.planes.enqueue(ctx, plan.pool)) {
+        return rc;
+    }
     {
         LaunchTimer t(ctx, "bits_score");
         if (plan.gen) k_bits_score<true><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(plan.ba);

@@ -80,14 +80,38 @@ struct BitsScoring {
     uint32_t M1, M0, X1, X0;
 };
 
+// One pair of a score-only launch: byte offsets in the pool, the first words
+// of its sequences' planar slots, and its score's destinations.
+struct BitsTask {
+    uint64_t a_off, b_off;
+    uint32_t aw, bw;
+    uint32_t m, n;
+    uint32_t out0, out1;  // out1 == ~0u: none
+};
+
+// All-vs-all launches name their pairs instead of listing them.  The
+// sequences are sorted longest first; a class holds the rows [r0, r1) of
+// equal stripe count, and its pairs are all (column c < row r), by c and then
+// r, so that 32 consecutive pairs have one stripe count and nearly one width.
+struct BitsSeq {
+    uint32_t w, len, id;  // first word of the planar slot, bases, index in the caller's list
+};
+struct BitsClass {
+    uint32_t r0, r1;
+};
+
 struct BitsJob {
-    uint32_t t0, cnt;  // tasks [t0, t0 + cnt), cnt <= 32, one per lane
+    uint32_t t0, cnt;  // tasks (or pairs of the class) [t0, t0 + cnt), cnt <= 32, one per lane
     uint32_t S, C;     // stripes, chunks per stripe (the job's largest)
+    uint32_t cls;      // all-vs-all: the class
 };
 
 struct BitsArgs {
     const uint32_t *pl0, *pl1;  // planar sequences: bit k of global base g at word (g+64)>>5, bit (g+64)&31
-    const BatchTask *tasks;     // a_off / b_off: the sequences' slots (global base indices)
+    const BitsTask *tasks;      // or, all-vs-all:
+    const BitsSeq *seqs;
+    const BitsClass *classes;
+    uint32_t nseq;
     const BitsJob *jobs;
     uint32_t njobs;
     uint32_t *counter;
@@ -117,6 +141,10 @@ class PlaneSet {
     // Slot (global base index of base 0) of the sequence at pool byte `off`
     // with `len` bases, added on first use.
     int64_t add(uint64_t off, uint32_t len);
+    // First word of a slot that add() returned.
+    static uint32_t word_of(int64_t slot) { return (uint32_t)((slot + kPlanePad) / 32); }
+    // Room for `words` words of slots laid out by the caller from word 2 on.
+    void reserve_words(uint64_t words) { words_ += words; }
     // Enqueues the copy (one H2D table, one kernel); pl0 / pl1 receive the
     // two planes, max_base the largest base index a 32-bit window may start at.
     // With a null pool the offsets given to add() are device addresses.
@@ -127,6 +155,8 @@ class PlaneSet {
     int enqueue(nw_ctx *ctx, const uint8_t *pool) const;
     const uint32_t *pl0 = nullptr, *pl1 = nullptr;
     int64_t max_base = 0;
+    uint32_t *planes() const { return planes_; }
+    uint64_t plane_words() const { return words_ + 4; }  // words from one plane to the next
 
   private:
     // open addressing (linear probing, at most half full): one table of
@@ -151,16 +181,21 @@ struct BitsPlan {
     BitsArgs ba{};
     uint32_t blocks = 0;
     const uint8_t *pool = nullptr;
-    PlaneSet planes;
+    uint32_t ntasks = 0;      // tasks whose sequences have slots of their own
+    PlaneSet planes;          // or the distinct sequences
     bool gen = false;
 };
 
 // 0 <= s'(mismatch) <= s'(match) <= 3, s' = s - 2*gap: every difference fits two bits.
 bool bits_scoring_ok(const nw_scoring &sc);
-// Orients, groups and uploads the tasks (reordered in place), sizes the
-// scratch; scores[out0] (and scores[out1]) receive each task's score.
-int bits_prepare(nw_ctx *ctx, const uint8_t *pool, std::vector<BatchTask> &tasks,
-                 const nw_scoring &sc, int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan);
+// Orients, groups and uploads the tasks, sizes the scratch; scores[out0] (and
+// scores[out1]) receive each task's score.
+int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> &tasks, const nw_scoring &sc,
+                 int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan);
+// The same for every pair of nseq sequences (the off-diagonal entries of the
+// nseq x nseq matrix `scores`).
+int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, const uint32_t *len, uint32_t nseq,
+                     const nw_scoring &sc, int32_t *scores, const std::string &prefix, BitsPlan *plan);
 // Enqueues the planar copy of the pool and the fill (no host copies: it can
 // be captured into a graph).
 int bits_launch(nw_ctx *ctx, const BitsPlan &plan);
