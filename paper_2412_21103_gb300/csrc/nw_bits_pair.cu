@@ -500,7 +500,7 @@ int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &job
             const uint8_t *b = pool ? pool + j.b_off : (const uint8_t *)(uintptr_t)j.b_off;
             tts.push_back(TraceTask{(const uint32_t *)(L.rec + descs[q].rec_off), descs[q].rec_rows, j.m, j.n,
                                     (uint8_t *)mv + moff, (uint64_t *)nm + q, a, b, j.cigar, j.cigar_len, kNoBand, 0,
-                                    nullptr, nullptr});
+                                    nullptr, nullptr, 32});
             moff += (uint64_t)j.m + j.n + 16;
         }
         if (tts.size() > 1) {

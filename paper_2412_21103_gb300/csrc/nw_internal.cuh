@@ -355,6 +355,7 @@ struct TraceTask {
                            // paused in device memory: {i, j, k lo, k hi, done}
     const uint32_t *origin;  // null: the moves start at (0, 0); else at (origin[0], origin[1])
                              // (a local alignment's start cell, read by the CIGAR assembly)
+    uint32_t lanes;          // bit-sliced records: bit stripes side by side (launch_trace_bits)
 };
 constexpr int32_t kNoBand = INT32_MIN;
 // Traceback + CIGAR for `ntasks` tasks: `host` describes them on the host
@@ -362,9 +363,10 @@ constexpr int32_t kNoBand = INT32_MIN;
 // passed by value).  Pairs of kParMinStripes stripes or more walk their
 // stripes in parallel (see nw_trace.cu).
 int launch_trace(nw_ctx *ctx, int R, const TraceTask *host, const TraceTask *dev, uint32_t ntasks, uint32_t mflag);
-// The same on the bit-sliced single-pair records (ptr: (L, Hb) word pairs,
-// [warp][step pair][lane] with ncg step pairs per warp; stripes of 31 rows
-// from the top, see nw_bits_pair.cu).
+// The same on bit-sliced records (ptr: (L, Hb) word pairs of bit stripes of 31
+// rows from the top, `lanes` of them side by side: bit stripe s at step pair
+// q lies in row (s / lanes) * ncg + 16 * (s % lanes) + q, lane s % lanes; see
+// nw_bits_pair.cu).  Tasks in descending order of m + n.
 int launch_trace_bits(nw_ctx *ctx, const TraceTask *host, const TraceTask *dev, uint32_t ntasks, uint32_t mflag);
 // The two halves of launch_trace: the walk (resumable through `state`) and
 // the CIGAR assembly from the finished move list.

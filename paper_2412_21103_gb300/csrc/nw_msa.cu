@@ -12,9 +12,9 @@
 // columns, the most 'I' ops any alignment puts there; center base p lands in
 // column p + G[0] + ... + G[p]; a row's I-bases fill their slot from its
 // left; a 'D' op leaves '-' in the center's column.  The merge reads the
-// RLE CIGARs on the device: one thread per sequence finds its insertion
+// RLE CIGARs on the device: one warp per sequence finds its insertion
 // runs (atomic max into G), one block scans G into column offsets, one
-// thread per sequence writes its row.
+// warp per sequence writes its row.
 #include <algorithm>
 #include <vector>
 
@@ -74,20 +74,44 @@ __global__ void k_argmax(const int64_t *sums, uint32_t nseq, uint32_t *center) {
     }
 }
 
-// Calls f(op, count) for every run of a run-length encoded CIGAR; returns
-// false on a character that is neither a digit nor an op.
+// Calls f(op, count) for every run of a run-length encoded CIGAR, in order and
+// with the whole warp; returns false on a character that is neither a digit
+// nor an op, or when f does.  The warp reads 32 characters at a time; a ballot
+// finds the ops, and each op's lane has its number from the digits before it
+// (a shuffle per place, the digits left over from the characters before
+// carried along), so the only serial work is one pass per run.
 template <typename F>
-__device__ bool for_runs(const char *c, uint64_t len, F f) {
-    uint64_t num = 0;
-    for (uint64_t q = 0; q < len; ++q) {
-        const char ch = c[q];
-        if (ch >= '0' && ch <= '9') {
-            num = num * 10u + (uint64_t)(ch - '0');
-            continue;
+__device__ bool for_runs(const char *c, uint64_t len, uint32_t lane, F f) {
+    uint64_t open = 0;  // the number that the characters before end with
+    for (uint64_t q0 = 0; q0 < len; q0 += 32) {
+        const bool in = q0 + lane < len;
+        const char ch = in ? c[q0 + lane] : '=';
+        const bool digit = ch >= '0' && ch <= '9';
+        const bool op = ch == '=' || ch == 'X' || ch == 'M' || ch == 'I' || ch == 'D';
+        uint32_t ops = __ballot_sync(kFull, in && !digit);
+        const uint32_t bad = __ballot_sync(kFull, in && !digit && !op);
+        // the number of the digits up to and with this lane: v digits-to-here, p its power of ten
+        uint64_t v = digit ? (uint64_t)(ch - '0') : 0u, p = digit ? 10u : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t v2 = __shfl_up_sync(kFull, v, o), p2 = __shfl_up_sync(kFull, p, o);
+            if ((int)lane >= o) {
+                v += p * v2;  // p is 0 once a lane that is no digit lies between
+                p *= p2;
+            }
         }
-        if (ch != '=' && ch != 'X' && ch != 'M' && ch != 'I' && ch != 'D') return false;
-        if (!f(ch, num)) return false;
-        num = 0;
+        v += p * open;  // digits from the first character on continue the open number
+        const uint32_t last = (uint32_t)min((unsigned long long)(len - q0), 32ull) - 1u;
+        const uint64_t next_open = __shfl_sync(kFull, v, last);
+        while (ops) {
+            const uint32_t at = (uint32_t)__ffs(ops) - 1u;
+            ops &= ops - 1u;
+            if ((bad >> at) & 1u) return false;
+            const uint64_t before = __shfl_sync(kFull, v, at ? at - 1u : 0u);
+            const uint64_t cnt = at ? before : open;
+            if (!f((char)__shfl_sync(kFull, (int)ch, at), cnt)) return false;
+        }
+        open = next_open;
     }
     return true;
 }
@@ -97,22 +121,26 @@ __device__ bool for_runs(const char *c, uint64_t len, F f) {
 // bases (NW_ERR_ARG into the error word, detail k, otherwise).
 __global__ void k_slot_gaps(const char *cigar_pool, const uint64_t *cigar_off, const uint64_t *cigar_len,
                             const uint32_t *len, uint32_t nseq, uint32_t C, uint32_t *G, uint32_t *err) {
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nseq; k += gridDim.x * blockDim.x) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nseq; k += (gridDim.x * blockDim.x) >> 5) {
         uint64_t p = 0, i = 0, ins = 0;
-        const bool ok = for_runs(cigar_pool + cigar_off[k], cigar_len[k], [&](char op, uint64_t cnt) {
+        auto slot = [&]() {
+            if (lane == 0 && ins && p <= C) atomicMax(G + p, ins < 0xffffffffull ? (uint32_t)ins : 0xffffffffu);
+        };
+        const bool ok = for_runs(cigar_pool + cigar_off[k], cigar_len[k], lane, [&](char op, uint64_t cnt) {
             if (op == 'I') {
                 ins += cnt;
                 i += cnt;
             } else {
-                if (ins && p <= C) atomicMax(G + p, ins < 0xffffffffull ? (uint32_t)ins : 0xffffffffu);
+                slot();
                 ins = 0;
                 p += cnt;
                 if (op != 'D') i += cnt;
             }
             return p <= C && i <= len[k];
         });
-        if (ins && p <= C) atomicMax(G + p, ins < 0xffffffffull ? (uint32_t)ins : 0xffffffffu);
-        if (!ok || p != C || i != len[k]) raise_error(err, NW_ERR_ARG, k);
+        slot();
+        if (lane == 0 && (!ok || p != C || i != len[k])) raise_error(err, NW_ERR_ARG, k);
     }
 }
 
@@ -161,30 +189,34 @@ __global__ void k_merge_rows(const uint8_t *pool, const uint64_t *off, const uin
                              uint32_t *err) {
     if (*(volatile const uint32_t *)err) return;  // a CIGAR failed its check
     const uint64_t cols = *ncols;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < nseq; k += gridDim.x * blockDim.x) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nseq; k += (gridDim.x * blockDim.x) >> 5) {
         char *row = msa + (uint64_t)k * ld;
         const uint8_t *s = pool + off[k];
         uint64_t p = 0, i = 0, used = 0;
-        for_runs(cigar_pool + cigar_off[k], cigar_len[k], [&](char op, uint64_t cnt) {
-            for (uint64_t r = 0; r < cnt; ++r) {
-                if (op == 'I') {
-                    const uint64_t col = start[p] + used++;
-                    if (in_range(col, cols, err, kSiteMsaRow)) row[col] = "ACGT"[base_at(s, i)];
-                    ++i;
-                } else if (op == 'D') {
-                    ++p;
-                    used = 0;
-                } else {
-                    const uint64_t col = start[p] + G[p];
-                    if (in_range(col, cols, err, kSiteMsaRow)) row[col] = "ACGT"[base_at(s, i)];
-                    ++i;
-                    ++p;
-                    used = 0;
+        for_runs(cigar_pool + cigar_off[k], cigar_len[k], lane, [&](char op, uint64_t cnt) {
+            // a run's bases by the lanes
+            if (op == 'I') {
+                for (uint64_t r = lane; r < cnt; r += 32) {
+                    const uint64_t col = start[p] + used + r;
+                    if (in_range(col, cols, err, kSiteMsaRow)) row[col] = "ACGT"[base_at(s, i + r)];
                 }
+                used += cnt;
+                i += cnt;
+            } else if (cnt) {
+                if (op != 'D') {
+                    for (uint64_t r = lane; r < cnt; r += 32) {
+                        const uint64_t col = start[p + r] + G[p + r];
+                        if (in_range(col, cols, err, kSiteMsaRow)) row[col] = "ACGT"[base_at(s, i + r)];
+                    }
+                    i += cnt;
+                }
+                p += cnt;
+                used = 0;
             }
             return true;
         });
-        if (ld > cols) row[cols] = '\0';
+        if (lane == 0 && ld > cols) row[cols] = '\0';
     }
 }
 
@@ -203,7 +235,7 @@ static int merge_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, c
     if ((rc = scratch(ctx, "msa_ncols", 16, &dn))) return rc;
     cudaError_t e = cudaMemsetAsync(dG, 0, ((size_t)C + 1) * 4, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "msa memset");
-    const uint32_t blocks = std::max<uint32_t>(1, (nseq + 127) / 128);
+    const uint32_t blocks = std::max<uint32_t>(1, (nseq + 3) / 4);  // a warp per sequence
     {
         LaunchTimer t(ctx, "msa_gaps");
         k_slot_gaps<<<blocks, 128, 0, ctx->stream>>>(cigar_pool, (const uint64_t *)dcoff, cigar_len,

@@ -125,6 +125,10 @@ __global__ void __launch_bounds__(32) k_traceback(TraceTask one, const TraceTask
 // moves are those of the plain walk, one for one.
 constexpr uint32_t kWalkDone = 0, kWalkJoined = 1, kWalkFull = 2, kWalkBand = 3, kWalkNone = 4;
 constexpr int kWalkWarps = 4;
+constexpr int kRunWarps = 4;               // warps per CTA of the walk by runs
+// Bit-sliced records: pairs up to this many moves walk from their end by runs,
+// about 0.4 us per 31 rows; longer ones in linked pieces, 120-250 us each.
+constexpr uint64_t kRunMaxMoves = 16384;
 constexpr uint32_t kParMinStripes = 3;     // shorter pairs walk sequentially,
 constexpr uint64_t kParMinMoves = 8192;    // and so do pairs of a batch with m + n below this (the
                                            // other pairs' walks keep the GPU busy, and the
@@ -198,10 +202,10 @@ struct ScalarLayout {
 };
 
 // Bit-sliced single-pair fill: bit stripes of 31 rows from the top (bit
-// stripe s: rows 31s + 1 .. 31s + 31).  Bit stripe s is lane l = s % 32 of
-// warp w = s / 32, and its step t is the warp's step tau = t + 32l; one
-// record (L, Hb) per bit stripe and step, laid out [warp][tau / 2][lane] in
-// 16-byte pairs of steps (ncg = pairs per warp).  Bit p of the step-t
+// stripe s: rows 31s + 1 .. 31s + 31).  Bit stripe s is lane l = s % lanes of
+// group w = s / lanes, and its step t is the group's step tau = t + 32l; one
+// record (L, Hb) per bit stripe and step, laid out [group][tau / 2][lane] in
+// 16-byte pairs of steps (ncg = pairs from one group to the next).  Bit p of the step-t
 // record is the cell of row 31s + p + 1 and column t + 1 - p; L = 0 where
 // the diagonal predecessor attains the maximum, Hb = 0 where the upper one
 // does.  The walk's stripes are G bit stripes each, so that a speculative
@@ -222,9 +226,10 @@ struct BitsLayout {
     }
     __device__ static void load(const TraceTask &p, uint32_t g, uint32_t key, uint32_t *tile, uint32_t lane) {
         const uint32_t s = g * G + (key >> 24);
-        const uint32_t w = s >> 5, l = s & 31u;
+        const uint32_t w = s / p.lanes, l = s % p.lanes;
         const size_t row = (size_t)w * p.ncg + (size_t)(key & 0xffffffu) * 32u + 16u * l;  // tau = 64 tile + 32 l
-        reinterpret_cast<uint4 *>(tile)[lane] = __ldcg(reinterpret_cast<const uint4 *>(p.ptr) + (row + lane) * 32u + l);
+        reinterpret_cast<uint4 *>(tile)[lane] =
+            __ldcg(reinterpret_cast<const uint4 *>(p.ptr) + (row + lane) * p.lanes + l);
     }
     __device__ static uint32_t move(const TraceTask &, const uint32_t *tile, uint32_t, uint32_t, uint32_t a1,
                                     uint32_t b1) {
@@ -234,6 +239,102 @@ struct BitsLayout {
     }
 };
 constexpr uint32_t kBitsWalkGroup = 8;  // bit stripes per walk stripe (248 rows)
+
+// The whole walk on the bit-sliced records, one warp per pair, a run of
+// diagonal moves at a time.  A diagonal move lowers the bit by one and the
+// step by two within a bit stripe, so when lane x holds the pair of steps x
+// before the walk's own (and the pair 32 further, in a second register), the
+// cells of a run of diagonal moves lie in successive lanes: ballots of their
+// L bits give the run's length and the Hb bits the move that ends it, with no
+// memory access within a stripe of 31 rows.  The next stripe's steps are
+// loaded when this one is entered, where the diagonal will leave it, with 16
+// steps to spare before and some 50 after; a path that misses them loads again.
+//
+// One move at a time from staged tiles, in pieces walked ahead from guessed
+// cells and linked, took 136 us in four launches on a 1,000 x 1,000 pair and
+// 1.7 ms on a batch of 3,000 pairs walked from their ends.
+__global__ void __launch_bounds__(kRunWarps * 32) k_tb_runs(TraceTask one, const TraceTask *many, uint32_t ntasks) {
+    constexpr uint32_t RS = 31u;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t ti = blockIdx.x * kRunWarps + (threadIdx.x >> 5);
+    if (ti >= ntasks) return;
+    const TraceTask &p = many ? many[ti] : one;
+    const uint4 *rec = reinterpret_cast<const uint4 *>(p.ptr);
+    const int32_t lanes = (int32_t)p.lanes, n = (int32_t)p.n;
+    const int32_t qmax = 16 * ((n + 61) / 32) - 1;  // a stripe's last step pair
+    uint8_t *mv = p.moves;
+    struct Steps {
+        int32_t q;      // lane 0's step pair
+        uint4 a, b;     // pairs q - lane and q - 32 - lane
+    };
+    auto load = [&](Steps &w, int32_t s, int32_t q) {
+        w.q = min(max(q, 0), qmax);
+        const int32_t l = s % lanes;
+        const uint4 *base = rec + ((int64_t)(s / lanes) * p.ncg + 16 * l) * lanes + l;
+        const int32_t qa = w.q - (int32_t)lane, qb = qa - 32;
+        w.a = qa >= 0 ? __ldcg(base + (int64_t)qa * lanes) : make_uint4(0u, 0u, 0u, 0u);
+        w.b = qb >= 0 ? __ldcg(base + (int64_t)qb * lanes) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    int32_t i = (int32_t)p.m, j = n;
+    uint32_t k = 0;
+    if (i > 0 && j > 0) {
+        int32_t s = (i - 1) / (int32_t)RS, bit = (i - 1) - (int32_t)RS * s, t = j - 1 + bit;
+        Steps cur, next;
+        load(cur, s, t >> 1);
+        if (s > 0) load(next, s - 1, (j - bit - 2 + 30 + 16) >> 1);
+        while (i > 0 && j > 0) {
+            const int32_t x0 = cur.q - (t >> 1);
+            const bool par = t & 1;
+            const int32_t y0 = (int32_t)lane - x0, y1 = y0 + 32;
+            const uint32_t L0 = par ? cur.a.z : cur.a.x, h0 = par ? cur.a.w : cur.a.y;
+            const uint32_t L1 = par ? cur.b.z : cur.b.x, h1 = par ? cur.b.w : cur.b.y;
+            // lane's cell y diagonal moves on: row bit - y; past the stripe's top the run ends
+            const uint32_t s0 = y0 < 0 ? 0u : y0 > bit ? 1u : (L0 >> (bit - y0)) & 1u;
+            const uint32_t s1 = y1 > bit ? 1u : (L1 >> ((bit - y1) & 31)) & 1u;
+            const uint32_t g0 = y0 < 0 || y0 > bit ? 0u : (h0 >> (bit - y0)) & 1u;
+            const uint32_t g1 = y1 > bit ? 0u : (h1 >> ((bit - y1) & 31)) & 1u;
+            const uint64_t stop = (((uint64_t)__ballot_sync(kFull, s1) << 32) | __ballot_sync(kFull, s0)) >> x0;
+            const uint64_t gap = (((uint64_t)__ballot_sync(kFull, g1) << 32) | __ballot_sync(kFull, g0)) >> x0;
+            const int32_t f = stop ? __ffsll((long long)stop) - 1 : 64 - x0;
+            const int32_t run = min(f, j);
+            if ((int32_t)lane < run) mv[k + lane] = 0;  // (at most 31: a run ends with its stripe)
+            k += (uint32_t)run;
+            i -= run;
+            j -= run;
+            t -= 2 * run;
+            const bool gapped = run == f && f <= bit && stop != 0u && j > 0;
+            bit -= run;
+            if (gapped) {
+                const uint32_t mvc = ((gap >> f) & 1u) ? 2u : 1u;
+                if (lane == 0) mv[k] = (uint8_t)mvc;
+                ++k;
+                --t;
+                if (mvc == 1u) {
+                    --i;
+                    --bit;
+                } else {
+                    --j;
+                }
+            }
+            if (bit < 0) {
+                if (i <= 0) break;
+                --s;
+                bit = (int32_t)RS - 1;
+                t = j - 1 + bit;
+                const int32_t q = t >> 1;
+                if (next.q >= q && next.q - q <= 28) cur = next;  // a whole stripe of diagonal moves lies ahead
+                else load(cur, s, q);
+                if (s > 0) load(next, s - 1, (j - bit - 2 + 30 + 16) >> 1);
+            } else if (cur.q - (t >> 1) > 62) {
+                load(cur, s, t >> 1);
+            }
+        }
+    }
+    const uint32_t rest = (uint32_t)(max(i, 0) + max(j, 0));
+    const uint8_t mvr = i > 0 ? 1 : 2;
+    for (uint32_t q = lane; q < rest; q += 32) mv[k + q] = mvr;
+    if (lane == 0) *p.nmoves = (uint64_t)k + rest;
+}
 
 // Walk from (i, j) inside stripe s until the walk leaves the stripe or
 // reaches row / column 0 (kWalkDone), steps on a cell of the spec path in
@@ -774,8 +875,22 @@ int launch_trace(nw_ctx *ctx, int R, const TraceTask *host, const TraceTask *dev
 
 int launch_trace_bits(nw_ctx *ctx, const TraceTask *host, const TraceTask *dev, uint32_t ntasks, uint32_t mflag) {
     if (ntasks == 0) return NW_OK;
-    const int rc = launch_walks<BitsLayout<kBitsWalkGroup>>(ctx, host, dev, ntasks);
-    return rc ? rc : launch_finish(ctx, host[0], dev, ntasks, mflag);
+    // the long pairs lead
+    uint32_t nlong = 0;
+    while (nlong < ntasks && (uint64_t)host[nlong].m + host[nlong].n > kRunMaxMoves) ++nlong;
+    if (nlong) {
+        const int rc = launch_walks<BitsLayout<kBitsWalkGroup>>(ctx, host, dev, nlong);
+        if (rc) return rc;
+    }
+    if (nlong < ntasks) {
+        LaunchTimer t(ctx, "tb_runs");
+        const uint32_t ns = ntasks - nlong;
+        k_tb_runs<<<(ns + kRunWarps - 1) / kRunWarps, kRunWarps * 32, 0, ctx->stream>>>(
+            host[nlong], dev ? dev + nlong : nullptr, ns);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "walk launch");
+    return launch_finish(ctx, host[0], dev, ntasks, mflag);
 }
 
 }  // namespace nw
