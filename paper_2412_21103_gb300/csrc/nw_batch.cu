@@ -950,6 +950,9 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
         max_n = std::max(max_n, t.n);
         tasks[q] = t;
     }
+    // alignments whose scoring fits two bit planes run on groups of lanes of
+    // the bit-sliced kernel, the others on the scalar batch kernel
+    const bool groups = want && bits_scoring_ok(sc) && !getenv("NW_PAIR_SCALAR");
     // pairs that would leave the GPU idle on one warp take the single-pair
     // kernel, and so do pairs whose pointer matrix alone exceeds half the
     // remaining budget (the single-pair path recomputes from checkpoints)
@@ -963,16 +966,30 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
             longest = std::max(longest, wc[q]);
             ps[q] = single_pair_cost(tasks[q].m, tasks[q].n, sc);
         }
+        // alignments on the bit-sliced groups: a pair's time on its warp,
+        // against the GPU's 4 x 152 schedulers
+        double rate = !want && bits_scoring_ok(sc) ? kBitsBatchRate : kBatchRate;
+        if (groups) {
+            rate = kWarpRate * 4.0 * ctx->sm_count;
+            total = longest = 0;
+            for (size_t q = 0; q < tasks.size(); ++q) {
+                wc[q] = bits_group_seconds(tasks[q].m, tasks[q].n) * kWarpRate;
+                total += wc[q];
+                longest = std::max(longest, wc[q]);
+            }
+        }
         // (no pair outlasts the batch: nothing to route)
-        const double rate = !want && bits_scoring_ok(sc) ? kBitsBatchRate : kBatchRate;
         std::vector<size_t> strag;
         if (longest / kWarpRate > total / rate) strag = pick_stragglers(wc, fc, ps, ctx->sm_count, rate);
         if (want) {
             const uint64_t room = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
             std::vector<char> in(tasks.size(), 0);
             for (size_t q : strag) in[q] = 1;
-            for (size_t q = 0; q < tasks.size(); ++q)
-                if (!in[q] && ((uint64_t)tasks[q].m + 512) * ((uint64_t)tasks[q].n + 128) / 4 > room) strag.push_back(q);
+            for (size_t q = 0; q < tasks.size(); ++q) {
+                const uint64_t need = groups ? bits_group_bytes(tasks[q].m, tasks[q].n)
+                                             : ((uint64_t)tasks[q].m + 512) * ((uint64_t)tasks[q].n + 128) / 4;
+                if (!in[q] && need > room) strag.push_back(q);
+            }
         }
         if (!strag.empty()) {
             std::vector<char> routed(tasks.size(), 0);
@@ -1030,6 +1047,20 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
             return NW_OK;
         }
     }
+    if (groups) {
+        std::vector<PairJob> jobs(npairs);
+        for (uint32_t q = 0; q < npairs; ++q) {
+            const BatchTask &t = tasks[q];
+            jobs[q] = PairJob{t.a_off, t.b_off, t.m, t.n, scores + t.out0, cigar_pool + cigar_off[t.out0],
+                              cigar_len + t.out0};
+        }
+        // the scalar kernel's pointer slot of an earlier call is idle here
+        uint64_t need = 0;
+        for (const PairJob &j : jobs) need += bits_group_bytes(j.m, j.n);
+        if (need > scratch_headroom(ctx, "bgroup_rec") / 2) free_prefix(ctx, "batch_ptr");
+        return bits_groups(ctx, pool, jobs, sc, (flags & NW_CIGAR_M) ? 1u : 0u);
+    }
+    free_prefix(ctx, "bgroup_rec");  // idle here: another scoring's slot
     // CIGAR: waves whose pointer words fit half of the remaining budget.
     // (a wave always takes at least one pair; scratch() reports NW_ERR_OOM if
     // even that does not fit)

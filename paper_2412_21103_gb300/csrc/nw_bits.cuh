@@ -221,6 +221,13 @@ struct PairJob {
 int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &jobs, const nw_scoring &sc, bool want,
                uint32_t mflag);
 
+// Many pairs with alignments, each on a group of lanes of one warp, in waves
+// whose records fit the budget (any lengths, also 0; want is implied).
+int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pairs, const nw_scoring &sc,
+                uint32_t mflag);
+double bits_group_seconds(uint32_t m, uint32_t n);  // estimated time of a pair on one warp there
+uint64_t bits_group_bytes(uint32_t m, uint32_t n);  // its records on a whole warp
+
 // ---- the certified band on the bit-sliced window (nw_bits_band.cu)
 // Window of one pair: g lanes (a power of two) x Q words of 32 rows, its
 // anchor diagonal hi (the band's upper diagonal raised to the parity of

@@ -33,12 +33,21 @@
 // diagonal predecessor attains the maximum (T = s'), bit p of Hb is 0 where
 // the upper one does (dV = 0).  They are laid out [warp][tau][lane], two
 // steps per 16-byte store, so a warp's stores are contiguous.
+//
+// Batches.  k_bits_group runs pairs of a batch on groups of G lanes of one warp
+// (32 / G pairs per warp): lane l takes the stripes l, l + G, l + 2G, .. of its
+// pair one after another, again one chunk of 32 steps behind lane l - 1, and
+// lane 0 reads what the group's last lane wrote of the stripe above (a row
+// buffer in global memory) a pass earlier.  Nothing waits, so the launch is an
+// ordinary one whose warps take jobs from a queue, longest first.
 #include <algorithm>
 #include <cstdlib>
+#include <cstring>
 #include <numeric>
 #include <vector>
 
 #include "nw_bits.cuh"
+#include "nw_order.h"
 
 namespace nw {
 
@@ -200,11 +209,12 @@ __device__ __forceinline__ void pair_step(int u, PairState &st, uint32_t A0, uin
     st.Qo1 = __funnelshift_l(st.G1, st.Qo1, 1);
 }
 
-// 32 steps; with PTR the records of steps 2v, 2v + 1 go to recp[v * 32].
+// 32 steps; with PTR the records of steps 2v, 2v + 1 go to recp[v * lanes]
+// (where `write`).
 template <bool GEN, bool RAMP, bool PTR>
 __device__ __forceinline__ void pair_chunk(PairState &st, uint32_t A0, uint32_t A1, uint32_t Rc0, uint32_t Rc1,
                                            uint32_t Rn0, uint32_t Rn1, uint32_t nz, uint32_t gmul, uint32_t rz,
-                                           const BitsScoring &g, uint4 *recp) {
+                                           const BitsScoring &g, uint4 *recp, uint32_t lanes = 32u, bool write = true) {
     uint32_t Lp = 0, Hp = 0;
 #pragma unroll
     for (int u = 0; u < 32; ++u) {
@@ -212,7 +222,7 @@ __device__ __forceinline__ void pair_chunk(PairState &st, uint32_t A0, uint32_t 
         pair_step<GEN, RAMP>(u, st, A0, A1, __funnelshift_l(Rn0, Rc0, u), __funnelshift_l(Rn1, Rc1, u), nz, gmul, rz,
                              g, L, Hb);
         if constexpr (PTR) {
-            if (u & 1) __stcg(recp + (size_t)(u >> 1) * 32u, make_uint4(Lp, Hp, L, Hb));
+            if ((u & 1) && write) __stcg(recp + (size_t)(u >> 1) * lanes, make_uint4(Lp, Hp, L, Hb));
             Lp = L;
             Hp = Hb;
         }
@@ -319,6 +329,148 @@ __global__ void __launch_bounds__(kPairWarps * 32, 1) k_bits_pair(PairLaunch L) 
         }
     }
     if (last) *p.score = W + p.gap * (int32_t)(p.m + p.n);
+}
+
+// ------------------------------------------------ a batch on groups of lanes
+struct GroupTask {
+    int64_t Ag, Bg;     // slots of a (rows) and b (columns)
+    uint32_t m, n, S, C;
+    uint32_t period;    // chunks from one pass of a lane to its next: max(C, G + 2)
+    uint32_t K;         // chunks until the last lane is done
+    uint32_t pm;        // bit of row m in the last stripe
+    uint32_t pad;
+    uint64_t rec_off;   // records (uint4 units), K * 16 rows of G
+    uint64_t row_off;   // its row buffer (C entries)
+    int32_t *score;
+};
+struct GroupJob {
+    uint32_t t0, cnt;   // tasks [t0, t0 + cnt), one per group
+    uint32_t G, K;      // lanes per group, the job's most chunks
+};
+struct GroupLaunch {
+    const uint32_t *pl0, *pl1;
+    const GroupTask *tasks;
+    const GroupJob *jobs;
+    uint32_t njobs;
+    uint32_t *counter;
+    uint4 *rec;
+    uint64_t rec_cap;
+    uint2 *rows;
+    int32_t gap;
+    BitsScoring g;
+    uint32_t *err;
+};
+
+// What bounds it: the logic pipe (see pair_step), two warps per scheduler.
+template <bool GEN>
+__global__ void __launch_bounds__(kPairWarps * 32) k_bits_group(GroupLaunch L) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (;;) {
+        uint32_t jid = 0;
+        if (lane == 0) jid = atomicAdd(L.counter, 1u);
+        jid = __shfl_sync(kFull, jid, 0);
+        if (jid >= L.njobs) break;
+        const GroupJob job = L.jobs[jid];
+        const uint32_t G = job.G, l = lane & (G - 1u), grp = lane / G;
+        const bool mine = grp < job.cnt;
+        const GroupTask t = L.tasks[job.t0 + (mine ? grp : 0u)];
+        const uint32_t S = t.S, nz = l == 0 ? 0u : 1u;
+        const int32_t C = (int32_t)t.C, period = (int32_t)t.period;
+        uint2 *row = L.rows + t.row_off;
+        uint4 *recp = L.rec + t.rec_off + l;
+        auto base = [&](uint32_t s, const uint32_t *pl) {
+            return plane_window(pl, s < S ? t.Ag + (int64_t)kPairRows * s : t.Ag - 32);
+        };
+        auto b_next = [&](int32_t c, const uint32_t *pl) {
+            return plane_window(pl, t.Bg + 32 * (int64_t)min(max(c, 0), C - 1) + 1);
+        };
+        auto word = [&](int32_t c) { return c < C ? __ldcg(row + c) : make_uint2(0u, 0u); };
+        PairState st{};
+        int32_t W = 0, c = -(int32_t)l;  // the lane's chunk within its pass
+        uint32_t s = l;                  // its stripe
+        uint32_t A0 = 0, A1 = 0, An0 = 0, An1 = 0, Ri0 = 0, Ri1 = 0, Fn0 = 0, Fn1 = 0;
+        if (S) {
+            A0 = base(s, L.pl0);
+            A1 = base(s, L.pl1);
+            An0 = base(s + G, L.pl0);
+            An1 = base(s + G, L.pl1);
+            Ri0 = __brev(plane_window(L.pl0, t.Bg - 31));
+            Ri1 = __brev(plane_window(L.pl1, t.Bg - 31));
+            Fn0 = b_next(c, L.pl0);
+            Fn1 = b_next(c, L.pl1);
+        }
+        uint32_t Rc0 = 0, Rc1 = 0;
+        bool last = s + 1 == S;
+        uint32_t gmul = 1u << (31u - (last ? t.pm : kPairRows - 1));
+        // the first lane's input words: chunk c's, the next chunk's, and what was loaded ahead
+        uint2 prev = make_uint2(0u, 0u), nx = prev, pre0 = prev, pre1 = prev;
+        for (uint32_t k = 0; k < job.K; ++k) {
+            __syncwarp();  // the row words of earlier chunks are written
+            if (c == period) {
+                c = 0;
+                s += G;
+                A0 = An0;
+                A1 = An1;
+                An0 = base(s + G, L.pl0);
+                An1 = base(s + G, L.pl1);
+                last = s + 1 == S;
+                gmul = 1u << (31u - (last ? t.pm : kPairRows - 1));
+            }
+            if (c == 0) {
+                // (G stays: the lane below still reads this lane's last stripe)
+                st.H0 = st.H1 = st.V0 = st.V1 = 0;
+                Rc0 = Ri0;
+                Rc1 = Ri1;
+            }
+            const bool act = mine && s < S && c >= 0 && c < C;
+            if (l == 0) {
+                if (c == 0) {
+                    prev = pre0;
+                    nx = pre1;
+                } else {
+                    prev = nx;
+                    nx = pre1;
+                }
+                st.Qi0 = st.Y0 = __funnelshift_r(nx.x, prev.x, 2);
+                st.Qi1 = st.Y1 = __funnelshift_r(nx.y, prev.y, 2);
+                if (c + 1 == period) {
+                    pre0 = s + G < S ? word(0) : make_uint2(0u, 0u);
+                    pre1 = s + G < S ? word(1) : make_uint2(0u, 0u);
+                } else {
+                    pre1 = s > 0 && s < S ? word(c + 2) : make_uint2(0u, 0u);
+                }
+            }
+            const uint32_t Rn0 = __brev(Fn0), Rn1 = __brev(Fn1);
+            if (S) {
+                const int32_t cn = c + 1 == period ? 0 : c + 1;
+                Fn0 = b_next(cn, L.pl0);
+                Fn1 = b_next(cn, L.pl1);
+            }
+            const bool write = mine && k < t.K && in_range((uint64_t)(recp - L.rec) + 15u * G, L.rec_cap, L.err, kSiteBandBitsPtr);
+            if (__any_sync(kFull, act && c == 0)) {
+                const uint32_t rz = c == 0 ? 0u : ~0u;
+                pair_chunk<GEN, true, true>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, nz, gmul, rz, L.g, recp, G, write);
+            } else {
+                pair_chunk<GEN, false, true>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, nz, gmul, ~0u, L.g, recp, G, write);
+            }
+            recp += 16u * G;
+            Rc0 = Rn0;
+            Rc1 = Rn1;
+            // outgoing bits: bit b is column 32c + 2 - b of the stripe's bottom row
+            if (act && l == G - 1u && s + 1 < S) __stcg(row + c, make_uint2(st.Qo0, st.Qo1));
+            if (act && last) {
+                const int32_t top = 32 * c + 32 - (int32_t)t.pm;
+                const int32_t lo = max(top - (int32_t)t.n, 0), hi = min(31, top - 1);
+                if (lo <= hi) {
+                    const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
+                    W += __popc(st.Qo0 & mk) + 2 * __popc(st.Qo1 & mk);
+                }
+            }
+            ++c;
+        }
+        if (mine && l == (S ? (S - 1u) & (G - 1u) : 0u)) *t.score = W + L.gap * (int32_t)(t.m + t.n);
+        __syncwarp();
+    }
 }
 
 // ------------------------------------------------------------------ host
@@ -512,6 +664,174 @@ int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &job
         }
         if ((rc = launch_trace_bits(ctx, tts.data(), tts.size() > 1 ? (const TraceTask *)dt : nullptr,
                                     (uint32_t)tts.size(), mflag)))
+            return rc;
+    }
+    return NW_OK;
+}
+
+namespace {
+// A pair on G lanes of a warp: its chunks, and its 16-byte record units.
+struct GroupGeom {
+    uint32_t S, C, period, K;
+    uint64_t rec;
+};
+GroupGeom group_geom(uint32_t m, uint32_t n, uint32_t G) {
+    GroupGeom g{};
+    if (!m || !n) return g;
+    g.S = (m + kPairRows - 1) / kPairRows;
+    g.C = (uint32_t)(((uint64_t)n + kPairRows - 1 + 31u) / 32u);
+    g.period = std::max(g.C, G + 2);
+    g.K = (g.S - 1) / G * g.period + g.C + (g.S - 1) % G;
+    g.rec = (uint64_t)g.K * 16u * G;
+    return g;
+}
+constexpr double kGroupStep = 45.0 / 2.07e9;  // a step of a warp, two per scheduler in flight
+}  // namespace
+
+double bits_group_seconds(uint32_t m, uint32_t n) {
+    uint32_t G = 1;
+    while (G < 32 && G * kPairRows < m) G *= 2;
+    return (double)group_geom(m, n, G).K * 32.0 * kGroupStep;
+}
+
+uint64_t bits_group_bytes(uint32_t m, uint32_t n) { return group_geom(m, n, 32).rec * 16u; }
+
+int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pairs, const nw_scoring &sc,
+                uint32_t mflag) {
+    if (pairs.empty()) return NW_OK;
+    int rc;
+    HostTimer ht(ctx, "bits_groups");
+    const bool gen = gen_of(sc);
+    const size_t np = pairs.size();
+    PlaneSet ps;
+    ps.reserve(std::min<size_t>(2 * np, 1u << 16));
+    std::vector<int64_t> ag(np, 0), bg(np, 0);
+    double work = 0;  // lane-chunks
+    for (size_t k = 0; k < np; ++k) {
+        if (!pairs[k].m || !pairs[k].n) continue;
+        ag[k] = ps.add(pairs[k].a_off, pairs[k].m);
+        bg[k] = ps.add(pairs[k].b_off, pairs[k].n);
+        const GroupGeom g = group_geom(pairs[k].m, pairs[k].n, 1);
+        work += (double)g.S * g.C;
+    }
+    if ((rc = ps.launch(ctx, pool, "bgroup"))) return rc;
+    // Lanes per pair: the fewest (fewer lanes leave fewer idle while a pair
+    // starts and ends) that bring the pair's own time under half of the time
+    // the batch takes with every scheduler busy, at least four (records of 64
+    // bytes per store) where the pair has that many stripes.
+    const double half = 0.5 * work / (4.0 * ctx->sm_count);  // in chunks of a warp at 32 lanes .. of one lane
+    std::vector<uint8_t> lanes(np);
+    std::vector<uint64_t> by_moves(np);
+    for (size_t k = 0; k < np; ++k) {
+        uint32_t G = 1;
+        const uint32_t S = (pairs[k].m + kPairRows - 1) / kPairRows;
+        while (G < 32 && G < S && (G < 4 || (double)group_geom(pairs[k].m, pairs[k].n, G).K > half / 32.0)) G *= 2;
+        lanes[k] = (uint8_t)G;
+        by_moves[k] = (uint64_t)pairs[k].m + pairs[k].n;
+    }
+    const std::vector<uint32_t> order = radix_order_desc(std::move(by_moves));  // longest first, as the walks want them
+    GroupLaunch L{};
+    L.pl0 = ps.pl0;
+    L.pl1 = ps.pl1;
+    L.gap = sc.gap;
+    L.err = ctx->d_err;
+    const int32_t sm = sc.match - 2 * sc.gap, sx = sc.mismatch - 2 * sc.gap;
+    L.g.M1 = (sm & 2) ? ~0u : 0u;
+    L.g.M0 = (sm & 1) ? ~0u : 0u;
+    L.g.X1 = (sx & 2) ? ~0u : 0u;
+    L.g.X0 = (sx & 1) ? ~0u : 0u;
+    const void *kern = gen ? (const void *)k_bits_group<true> : (const void *)k_bits_group<false>;
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kPairWarps * 32, 0);
+    occ = std::max(1, std::min(occ, 2));
+    // waves of pairs whose records fit half of what their slot may grow to
+    const uint64_t room = scratch_headroom(ctx, "bgroup_rec") / 2 / 16;
+    for (size_t next = 0; next < np;) {
+        std::vector<uint32_t> wave;
+        uint64_t rec = 0, rows = 0, moves = 0;
+        for (; next < np; ++next) {
+            const PairJob &j = pairs[order[next]];
+            const GroupGeom g = group_geom(j.m, j.n, lanes[order[next]]);
+            if (!wave.empty() && rec + g.rec > room) break;
+            wave.push_back(order[next]);
+            rec += g.rec;
+            rows += g.C;
+            moves += (uint64_t)j.m + j.n + 16;
+        }
+        const size_t nt = wave.size();
+        void *rv = nullptr, *wv = nullptr, *mv = nullptr, *nm = nullptr, *dv = nullptr;
+        // (a walk may read up to 32 rows past a stripe's last)
+        if ((rc = scratch(ctx, "bgroup_rec", (rec + 32u * 32u) * 16 + 16, &rv))) return rc;
+        if ((rc = scratch(ctx, "bgroup_rows", rows * sizeof(uint2) + 16, &wv))) return rc;
+        if ((rc = scratch(ctx, "bgroup_moves", moves + 16, &mv))) return rc;
+        if ((rc = scratch(ctx, "bgroup_nmoves", nt * 8 + 16, &nm))) return rc;
+        // tasks by lanes, then chunks; jobs of 32 / G of them, longest first
+        std::vector<uint64_t> keys(nt);
+        for (size_t q = 0; q < nt; ++q) {
+            const PairJob &j = pairs[wave[q]];
+            keys[q] = (uint64_t)lanes[wave[q]] << 32 | group_geom(j.m, j.n, lanes[wave[q]]).K;
+        }
+        const std::vector<uint32_t> to = radix_order_desc(std::move(keys));
+        std::vector<GroupTask> tasks(nt);
+        std::vector<TraceTask> tts(nt);
+        std::vector<GroupJob> jobs;
+        std::vector<uint64_t> jk;
+        uint64_t rec_off = 0, row_off = 0, moff = 0;
+        for (size_t q = 0; q < nt; ++q) {  // records in the walks' order
+            const PairJob &j = pairs[wave[q]];
+            const uint32_t G = lanes[wave[q]];
+            const GroupGeom g = group_geom(j.m, j.n, G);
+            const uint8_t *a = pool ? pool + j.a_off : (const uint8_t *)(uintptr_t)j.a_off;
+            const uint8_t *b = pool ? pool + j.b_off : (const uint8_t *)(uintptr_t)j.b_off;
+            tts[q] = TraceTask{(const uint32_t *)((uint4 *)rv + rec_off), 16u * g.period, j.m, j.n, (uint8_t *)mv + moff,
+                               (uint64_t *)nm + q, a, b, j.cigar, j.cigar_len, kNoBand, 0, nullptr, nullptr, G};
+            rec_off += g.rec;
+            moff += (uint64_t)j.m + j.n + 16;
+        }
+        for (size_t q = 0; q < nt; ++q) {
+            const uint32_t w = to[q], k = wave[w], G = lanes[k];
+            const PairJob &j = pairs[k];
+            const GroupGeom g = group_geom(j.m, j.n, G);
+            GroupTask &t = tasks[q];
+            t = GroupTask{ag[k], bg[k], j.m, j.n, g.S, g.C, g.period, g.K, g.S ? (j.m - 1) - kPairRows * (g.S - 1) : 0u,
+                          0u, (uint64_t)((const uint4 *)tts[w].ptr - (const uint4 *)rv), row_off, j.score};
+            row_off += g.C;
+            if (jobs.empty() || jobs.back().G != G || jobs.back().cnt == 32u / G) {
+                jobs.push_back(GroupJob{(uint32_t)q, 0, G, g.K});
+                jk.push_back(g.K);
+            }
+            ++jobs.back().cnt;
+        }
+        const std::vector<uint32_t> jo = radix_order_desc(std::move(jk));
+        // one upload: tasks, jobs, walks
+        const size_t at_j = nt * sizeof(GroupTask), at_t = (at_j + jobs.size() * sizeof(GroupJob) + 15) / 16 * 16;
+        std::vector<uint8_t> tab(at_t + nt * sizeof(TraceTask));
+        memcpy(tab.data(), tasks.data(), at_j);
+        for (size_t q = 0; q < jobs.size(); ++q) memcpy(tab.data() + at_j + q * sizeof(GroupJob), &jobs[jo[q]], sizeof(GroupJob));
+        memcpy(tab.data() + at_t, tts.data(), nt * sizeof(TraceTask));
+        if ((rc = scratch(ctx, "bgroup_tab", tab.size() + 16, &dv))) return rc;
+        void *cv = nullptr;
+        if ((rc = scratch(ctx, "bgroup_counter", 16, &cv))) return rc;
+        cudaError_t e = cudaMemcpyAsync(dv, tab.data(), tab.size(), cudaMemcpyHostToDevice, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(cv, 0, 4, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // the tables are host memory of this call
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "group table upload");
+        L.tasks = (const GroupTask *)dv;
+        L.jobs = (const GroupJob *)((const uint8_t *)dv + at_j);
+        L.njobs = (uint32_t)jobs.size();
+        L.counter = (uint32_t *)cv;
+        L.rec = (uint4 *)rv;
+        L.rec_cap = rec;
+        L.rows = (uint2 *)wv;
+        {
+            LaunchTimer t(ctx, "bgroup_fill_ptr");
+            const uint32_t blocks = std::min<uint32_t>((L.njobs + kPairWarps - 1) / kPairWarps,
+                                                       (uint32_t)occ * (uint32_t)ctx->sm_count);
+            if (gen) k_bits_group<true><<<blocks, kPairWarps * 32, 0, ctx->stream>>>(L);
+            else k_bits_group<false><<<blocks, kPairWarps * 32, 0, ctx->stream>>>(L);
+        }
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, "group launch");
+        if ((rc = launch_trace_bits(ctx, tts.data(), (const TraceTask *)((const uint8_t *)dv + at_t), (uint32_t)nt, mflag)))
             return rc;
     }
     return NW_OK;

@@ -264,16 +264,27 @@ __global__ void __launch_bounds__(kRunWarps * 32) k_tb_runs(TraceTask one, const
     const int32_t qmax = 16 * ((n + 61) / 32) - 1;  // a stripe's last step pair
     uint8_t *mv = p.moves;
     struct Steps {
-        int32_t q;      // lane 0's step pair
-        uint4 a, b;     // pairs q - lane and q - 32 - lane
+        int32_t q;   // lane 0's step pair
+        uint4 a, b;  // pairs q - lane and q - 32 - lane, their L bits inverted
+    };
+    auto pairs = [&](int32_t s, int32_t q) {
+        const int32_t l = s % lanes, qa = q - (int32_t)lane;
+        const uint4 *base = rec + ((int64_t)(s / lanes) * p.ncg + 16 * l) * lanes + l;
+        uint4 v = qa >= 0 ? __ldcg(base + (int64_t)qa * lanes) : make_uint4(0u, 0u, 0u, 0u);
+        v.x = ~v.x;
+        v.z = ~v.z;
+        return v;
     };
     auto load = [&](Steps &w, int32_t s, int32_t q) {
         w.q = min(max(q, 0), qmax);
-        const int32_t l = s % lanes;
-        const uint4 *base = rec + ((int64_t)(s / lanes) * p.ncg + 16 * l) * lanes + l;
-        const int32_t qa = w.q - (int32_t)lane, qb = qa - 32;
-        w.a = qa >= 0 ? __ldcg(base + (int64_t)qa * lanes) : make_uint4(0u, 0u, 0u, 0u);
-        w.b = qb >= 0 ? __ldcg(base + (int64_t)qb * lanes) : make_uint4(0u, 0u, 0u, 0u);
+        w.a = pairs(s, w.q);
+        w.b = pairs(s, w.q - 32);
+    };
+    // bit e - lane of a word (0 where that is none)
+    auto row = [&](uint32_t word, int32_t e) {
+        uint32_t d;
+        asm("shr.u32 %0, %1, %2;" : "=r"(d) : "r"(word), "r"((uint32_t)(e - (int32_t)lane)));
+        return d & 1u;
     };
     int32_t i = (int32_t)p.m, j = n;
     uint32_t k = 0;
@@ -282,51 +293,48 @@ __global__ void __launch_bounds__(kRunWarps * 32) k_tb_runs(TraceTask one, const
         Steps cur, next;
         load(cur, s, t >> 1);
         if (s > 0) load(next, s - 1, (j - bit - 2 + 30 + 16) >> 1);
-        while (i > 0 && j > 0) {
-            const int32_t x0 = cur.q - (t >> 1);
+        for (;;) {
+            // lane x0 + y has the cell y diagonal moves on, at bit - y: the
+            // sum e of lane and bit is the same for all of them (and none
+            // is left past the stripe's top, where the run ends)
+            const int32_t x0 = cur.q - (t >> 1), e = bit + x0;
             const bool par = t & 1;
-            const int32_t y0 = (int32_t)lane - x0, y1 = y0 + 32;
-            const uint32_t L0 = par ? cur.a.z : cur.a.x, h0 = par ? cur.a.w : cur.a.y;
-            const uint32_t L1 = par ? cur.b.z : cur.b.x, h1 = par ? cur.b.w : cur.b.y;
-            // lane's cell y diagonal moves on: row bit - y; past the stripe's top the run ends
-            const uint32_t s0 = y0 < 0 ? 0u : y0 > bit ? 1u : (L0 >> (bit - y0)) & 1u;
-            const uint32_t s1 = y1 > bit ? 1u : (L1 >> ((bit - y1) & 31)) & 1u;
-            const uint32_t g0 = y0 < 0 || y0 > bit ? 0u : (h0 >> (bit - y0)) & 1u;
-            const uint32_t g1 = y1 > bit ? 0u : (h1 >> ((bit - y1) & 31)) & 1u;
-            const uint64_t stop = (((uint64_t)__ballot_sync(kFull, s1) << 32) | __ballot_sync(kFull, s0)) >> x0;
-            const uint64_t gap = (((uint64_t)__ballot_sync(kFull, g1) << 32) | __ballot_sync(kFull, g0)) >> x0;
-            const int32_t f = stop ? __ffsll((long long)stop) - 1 : 64 - x0;
+            const uint32_t g0 = __ballot_sync(kFull, row(par ? cur.a.z : cur.a.x, e));
+            const uint32_t g1 = __ballot_sync(kFull, row(par ? cur.b.z : cur.b.x, e - 32));
+            const uint32_t h0 = __ballot_sync(kFull, row(par ? cur.a.w : cur.a.y, e));
+            const uint32_t h1 = __ballot_sync(kFull, row(par ? cur.b.w : cur.b.y, e - 32));
+            const uint32_t go = __funnelshift_r(g0, g1, (uint32_t)x0), hb = __funnelshift_r(h0, h1, (uint32_t)x0);
+            const int32_t f = __ffs((int)~go) - 1;  // at most 31: the stripe's rows
             const int32_t run = min(f, j);
-            if ((int32_t)lane < run) mv[k + lane] = 0;  // (at most 31: a run ends with its stripe)
+            if ((int32_t)lane < run) mv[k + lane] = 0;
             k += (uint32_t)run;
             i -= run;
             j -= run;
             t -= 2 * run;
-            const bool gapped = run == f && f <= bit && stop != 0u && j > 0;
             bit -= run;
-            if (gapped) {
-                const uint32_t mvc = ((gap >> f) & 1u) ? 2u : 1u;
+            if (bit >= 0 && j > 0) {  // the cell that ends the run
+                const uint32_t mvc = ((hb >> f) & 1u) + 1u;
                 if (lane == 0) mv[k] = (uint8_t)mvc;
                 ++k;
                 --t;
-                if (mvc == 1u) {
-                    --i;
-                    --bit;
-                } else {
-                    --j;
-                }
+                const int32_t v = mvc == 1u;
+                i -= v;
+                bit -= v;
+                j -= 1 - v;
             }
+            if (i <= 0 || j <= 0) break;
             if (bit < 0) {
-                if (i <= 0) break;
                 --s;
                 bit = (int32_t)RS - 1;
                 t = j - 1 + bit;
                 const int32_t q = t >> 1;
-                if (next.q >= q && next.q - q <= 28) cur = next;  // a whole stripe of diagonal moves lies ahead
+                if (next.q >= q && next.q - q < 32) cur = next;
                 else load(cur, s, q);
                 if (s > 0) load(next, s - 1, (j - bit - 2 + 30 + 16) >> 1);
-            } else if (cur.q - (t >> 1) > 62) {
-                load(cur, s, t >> 1);
+            } else if (cur.q - (t >> 1) >= 32) {
+                cur.q -= 32;
+                cur.a = cur.b;
+                cur.b = pairs(s, cur.q - 32);
             }
         }
     }
