@@ -258,27 +258,38 @@ __global__ void __launch_bounds__(kRunWarps * 32) k_tb_runs(TraceTask one, const
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t ti = blockIdx.x * kRunWarps + (threadIdx.x >> 5);
     if (ti >= ntasks) return;
-    const TraceTask &p = many ? many[ti] : one;
-    const uint4 *rec = reinterpret_cast<const uint4 *>(p.ptr);
-    const int32_t lanes = (int32_t)p.lanes, n = (int32_t)p.n;
-    const int32_t qmax = 16 * ((n + 61) / 32) - 1;  // a stripe's last step pair
-    uint8_t *mv = p.moves;
+    struct {
+        const uint32_t *ptr;
+        uint8_t *moves;
+        uint64_t *nmoves;
+        uint32_t m, n, ncg, lanes;
+    } p;
+    if (many) {
+        const TraceTask &x = many[ti];
+        p = {x.ptr, x.moves, x.nmoves, x.m, x.n, x.ncg, x.lanes};
+    } else {
+        p = {one.ptr, one.moves, one.nmoves, one.m, one.n, one.ncg, one.lanes};
+    }
+    const int32_t lanes = (int32_t)p.lanes, n = (int32_t)p.n;  // (lanes: a power of two)
+    const int32_t qmax = 16 * ((n + 61) / 32) - 1;             // a stripe's last step pair
+    uint8_t *mv = p.moves + lane;
     struct Steps {
         int32_t q;   // lane 0's step pair
-        uint4 a, b;  // pairs q - lane and q - 32 - lane, their L bits inverted
+        uint4 a, b;  // pairs q - lane and q - 32 - lane
     };
-    auto pairs = [&](int32_t s, int32_t q) {
-        const int32_t l = s % lanes, qa = q - (int32_t)lane;
-        const uint4 *base = rec + ((int64_t)(s / lanes) * p.ncg + 16 * l) * lanes + l;
-        uint4 v = qa >= 0 ? __ldcg(base + (int64_t)qa * lanes) : make_uint4(0u, 0u, 0u, 0u);
-        v.x = ~v.x;
-        v.z = ~v.z;
-        return v;
+    // this lane's pair 0 of bit stripe s
+    const int32_t sh = 31 - __clz(lanes);
+    auto stripe = [&](int32_t s) {
+        const int32_t l = s & (lanes - 1);
+        return reinterpret_cast<const uint4 *>(p.ptr) + (((int64_t)(s >> sh) * p.ncg + 16 * l - (int32_t)lane) << sh) + l;
     };
-    auto load = [&](Steps &w, int32_t s, int32_t q) {
+    auto pairs = [&](const uint4 *base, int32_t q) {
+        return q >= (int32_t)lane ? __ldcg(base + ((int64_t)q << sh)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    auto load = [&](Steps &w, const uint4 *base, int32_t q) {
         w.q = min(max(q, 0), qmax);
-        w.a = pairs(s, w.q);
-        w.b = pairs(s, w.q - 32);
+        w.a = pairs(base, w.q);
+        w.b = pairs(base, w.q - 32);
     };
     // bit e - lane of a word (0 where that is none)
     auto row = [&](uint32_t word, int32_t e) {
@@ -291,56 +302,75 @@ __global__ void __launch_bounds__(kRunWarps * 32) k_tb_runs(TraceTask one, const
     if (i > 0 && j > 0) {
         int32_t s = (i - 1) / (int32_t)RS, bit = (i - 1) - (int32_t)RS * s, t = j - 1 + bit;
         Steps cur, next;
-        load(cur, s, t >> 1);
-        if (s > 0) load(next, s - 1, (j - bit - 2 + 30 + 16) >> 1);
+        const uint4 *base = stripe(s);
+        load(cur, base, t >> 1);
+        if (s > 0) load(next, stripe(s - 1), (j - bit - 2 + 30 + 16) >> 1);
+        // the words of the walk, L bits inverted (done when a block is taken up, not when it is loaded)
+        auto take = [&]() {
+            cur.a.x = ~cur.a.x;
+            cur.a.z = ~cur.a.z;
+            cur.b.x = ~cur.b.x;
+            cur.b.z = ~cur.b.z;
+        };
+        take();
+        int32_t x0 = 0;       // the walk's step pair is lane x0's
+        uint32_t par = t & 1;  // its step within the pair
         for (;;) {
             // lane x0 + y has the cell y diagonal moves on, at bit - y: the
-            // sum e of lane and bit is the same for all of them (and none
+            // sum of lane and bit is the same for all of them (and none
             // is left past the stripe's top, where the run ends)
-            const int32_t x0 = cur.q - (t >> 1), e = bit + x0;
-            const bool par = t & 1;
+            const int32_t e = bit + x0;
             const uint32_t g0 = __ballot_sync(kFull, row(par ? cur.a.z : cur.a.x, e));
             const uint32_t g1 = __ballot_sync(kFull, row(par ? cur.b.z : cur.b.x, e - 32));
             const uint32_t h0 = __ballot_sync(kFull, row(par ? cur.a.w : cur.a.y, e));
             const uint32_t h1 = __ballot_sync(kFull, row(par ? cur.b.w : cur.b.y, e - 32));
             const uint32_t go = __funnelshift_r(g0, g1, (uint32_t)x0), hb = __funnelshift_r(h0, h1, (uint32_t)x0);
-            const int32_t f = __ffs((int)~go) - 1;  // at most 31: the stripe's rows
-            const int32_t run = min(f, j);
-            if ((int32_t)lane < run) mv[k + lane] = 0;
-            k += (uint32_t)run;
-            i -= run;
-            j -= run;
-            t -= 2 * run;
-            bit -= run;
-            if (bit >= 0 && j > 0) {  // the cell that ends the run
-                const uint32_t mvc = ((hb >> f) & 1u) + 1u;
-                if (lane == 0) mv[k] = (uint8_t)mvc;
-                ++k;
-                --t;
-                const int32_t v = mvc == 1u;
-                i -= v;
-                bit -= v;
-                j -= 1 - v;
+            const int32_t f = __clz((int)__brev(~go));  // at most 31: the stripe's rows
+            if (f <= bit && f < j) {
+                // f diagonal moves, then the gap move of the cell that ends them
+                const int32_t v = (int32_t)(((hb >> f) & 1u) ^ 1u);
+                if ((int32_t)lane <= f) mv[k] = (int32_t)lane < f ? 0 : (uint8_t)(2 - v);
+                k += (uint32_t)f + 1u;
+                i -= f + v;
+                j -= f + 1 - v;
+                bit -= f + v;
+                x0 += f + 1 - (int32_t)par;
+                par ^= 1u;
+            } else {
+                const int32_t run = min(f, j);
+                if ((int32_t)lane < run) mv[k] = 0;
+                k += (uint32_t)run;
+                i -= run;
+                j -= run;
+                bit -= run;
+                x0 += run;
             }
-            if (i <= 0 || j <= 0) break;
-            if (bit < 0) {
+            if (bit < 0 || j <= 0) {
+                if (i <= 0 || j <= 0) break;
                 --s;
                 bit = (int32_t)RS - 1;
                 t = j - 1 + bit;
+                par = t & 1;
                 const int32_t q = t >> 1;
+                base = stripe(s);
                 if (next.q >= q && next.q - q < 32) cur = next;
-                else load(cur, s, q);
-                if (s > 0) load(next, s - 1, (j - bit - 2 + 30 + 16) >> 1);
-            } else if (cur.q - (t >> 1) >= 32) {
+                else load(cur, base, q);
+                x0 = cur.q - q;
+                if (s > 0) load(next, stripe(s - 1), (j - bit - 2 + 30 + 16) >> 1);
+                take();
+            } else if (x0 >= 32) {
+                x0 -= 32;
                 cur.q -= 32;
                 cur.a = cur.b;
-                cur.b = pairs(s, cur.q - 32);
+                cur.b = pairs(base, cur.q - 32);
+                cur.b.x = ~cur.b.x;
+                cur.b.z = ~cur.b.z;
             }
         }
     }
     const uint32_t rest = (uint32_t)(max(i, 0) + max(j, 0));
     const uint8_t mvr = i > 0 ? 1 : 2;
-    for (uint32_t q = lane; q < rest; q += 32) mv[k + q] = mvr;
+    for (uint32_t q = lane; q < rest; q += 32) mv[k + q - lane] = mvr;
     if (lane == 0) *p.nmoves = (uint64_t)k + rest;
 }
 
