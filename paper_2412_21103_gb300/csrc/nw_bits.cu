@@ -227,17 +227,6 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
     }
 }
 
-// Compacts the even bits of x into the low 32 bits.
-__device__ __forceinline__ uint32_t even_bits(uint64_t x) {
-    x &= 0x5555555555555555ull;
-    x = (x | (x >> 1)) & 0x3333333333333333ull;
-    x = (x | (x >> 2)) & 0x0F0F0F0F0F0F0F0Full;
-    x = (x | (x >> 4)) & 0x00FF00FF00FF00FFull;
-    x = (x | (x >> 8)) & 0x0000FFFF0000FFFFull;
-    x = (x | (x >> 16)) & 0x00000000FFFFFFFFull;
-    return (uint32_t)x;
-}
-
 // Planar copy of a sequence by a warp: word w of its slot holds bit k of the
 // codes of its bases 32w .. 32w+31 (bases past its end read as 0).
 __device__ __forceinline__ void plane_copy(const uint8_t *src, uint32_t nbytes, uint32_t dst, uint32_t lane,

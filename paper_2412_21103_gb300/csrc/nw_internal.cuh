@@ -143,6 +143,17 @@ __device__ __forceinline__ uint32_t base_at(const uint8_t *s2b, uint64_t k) {
     return (s2b[k >> 2] >> ((k & 3) * 2)) & 3u;
 }
 
+// Compacts the even bits of x into the low 32 bits.
+__device__ __forceinline__ uint32_t even_bits(uint64_t x) {
+    x &= 0x5555555555555555ull;
+    x = (x | (x >> 1)) & 0x3333333333333333ull;
+    x = (x | (x >> 2)) & 0x0F0F0F0F0F0F0F0Full;
+    x = (x | (x >> 4)) & 0x00FF00FF00FF00FFull;
+    x = (x | (x >> 8)) & 0x0000FFFF0000FFFFull;
+    x = (x | (x >> 16)) & 0x00000000FFFFFFFFull;
+    return (uint32_t)x;
+}
+
 // Scoring handed to kernels: prof[c] is the row profile of a query base c,
 // byte d of prof[c] = s'(c, d) as int8.
 struct Profile {
