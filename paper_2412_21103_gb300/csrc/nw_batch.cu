@@ -952,7 +952,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     }
     // alignments whose scoring fits two bit planes run on groups of lanes of
     // the bit-sliced kernel, the others on the scalar batch kernel
-    const bool groups = want && bits_scoring_ok(sc) && !getenv("NW_PAIR_SCALAR");
+    const bool groups = want && bits_batch_ok(sc) && !getenv("NW_PAIR_SCALAR");
     // pairs that would leave the GPU idle on one warp take the single-pair
     // kernel, and so do pairs whose pointer matrix alone exceeds half the
     // remaining budget (the single-pair path recomputes from checkpoints)
@@ -968,7 +968,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
         }
         // alignments on the bit-sliced groups: a pair's time on its warp,
         // against the GPU's 4 x 152 schedulers
-        double rate = !want && bits_scoring_ok(sc) ? kBitsBatchRate : kBatchRate;
+        double rate = !want && bits_batch_ok(sc) ? kBitsBatchRate : kBatchRate;
         if (groups) {
             rate = kWarpRate * 4.0 * ctx->sm_count;
             total = longest = 0;
@@ -1022,7 +1022,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     if (!want || ctx->autotune) {
         // score-only: the bit-sliced kernel (rows per lane 32) where the
         // scoring fits two bit planes
-        const bool bits = !want && bits_scoring_ok(sc);
+        const bool bits = !want && bits_batch_ok(sc);
         const uint32_t cap = score_slots(tasks.data(), npairs);
         BitsPlan bp;
         if (bits && (rc = bits_prepare(ctx, pool, tasks, sc, scores, cap, pre, &bp))) return rc;

@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <numeric>
 #include <vector>
 
 #include "nw_bits.cuh"
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
             else bits_stripe<GEN, false>(p, C, n, Bg, A0, A1, ~0u, s + 1 == S, rows, W);
         }
         if (active) {
-            const int32_t sc = W + p.gap * (int32_t)(m + n);
+            const int32_t sc = W * p.unit + p.gap * (int32_t)(m + n);
             if (in_range(out0, p.score_cap, p.err, kSiteBatchScore)) p.scores[out0] = sc;
             if (out1 != ~0u && in_range(out1, p.score_cap, p.err, kSiteBatchScore)) p.scores[out1] = sc;
         }
@@ -349,9 +350,20 @@ int PlaneSet::launch(nw_ctx *ctx, const uint8_t *pool, const std::string &prefix
     return rc ? rc : enqueue(ctx, pool);
 }
 
+BitsUnits bits_units(const nw_scoring &sc) {
+    const int32_t sm = sc.match - 2 * sc.gap, sx = sc.mismatch - 2 * sc.gap;
+    const int32_t unit = sm > 0 && sx >= 0 ? std::gcd(sm, sx) : 1;
+    return BitsUnits{sm / unit, sx / unit, unit};
+}
+
 bool bits_scoring_ok(const nw_scoring &sc) {
     const int32_t sm = sc.match - 2 * sc.gap, sx = sc.mismatch - 2 * sc.gap;
     return sx >= 0 && sx <= sm && sm <= 3;
+}
+
+bool bits_batch_ok(const nw_scoring &sc) {
+    const BitsUnits u = bits_units(sc);
+    return u.sx >= 0 && u.sx <= u.sm && u.sm <= 3;
 }
 
 // Stripes and chunks per stripe of an m x n pair.
@@ -388,12 +400,10 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
     ba.score_cap = score_cap;
     ba.gap = sc.gap;
     ba.err = ctx->d_err;
-    const int32_t sm = sc.match - 2 * sc.gap, sx = sc.mismatch - 2 * sc.gap;
-    ba.g.M1 = (sm & 2) ? ~0u : 0u;
-    ba.g.M0 = (sm & 1) ? ~0u : 0u;
-    ba.g.X1 = (sx & 2) ? ~0u : 0u;
-    ba.g.X0 = (sx & 1) ? ~0u : 0u;
-    plan->gen = !(sm == 3 && sx == 1);
+    const BitsUnits u = bits_units(sc);
+    ba.unit = u.unit;
+    ba.g = u.planes();
+    plan->gen = u.gen();
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, plan->gen ? k_bits_score<true> : k_bits_score<false>,
                                                   kBitsWarps * 32, 0);

@@ -78,7 +78,7 @@ struct PairLaunch {
     uint4 *rec;                 // records, per pair [warp][rec_rows][32 lanes] (two steps each), or null
     uint64_t *ring;             // per pair [warp][C][2] tagged outgoing words of lane 31
     uint32_t epoch;             // tag of this launch (never 0)
-    int32_t gap;
+    int32_t unit, gap;
     BitsScoring g;
     uint32_t *err;
 };
@@ -92,7 +92,7 @@ struct PairBitsArgs {
     uint64_t *ring;
     uint32_t epoch;
     int32_t *score;
-    int32_t gap;
+    int32_t unit, gap;
     BitsScoring g;
     uint32_t *err;
 };
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, 1) k_bits_pair(PairLaunch L) 
     if (w >= pd.nwarps) return;
     const PairBitsArgs p{L.pl0, L.pl1, pd.Ag, pd.Bg, pd.m, pd.n, pd.S, pd.C, pd.nwarps, pd.pm,
                          PTR ? L.rec + pd.rec_off : nullptr, pd.rec_rows, L.ring + pd.ring_off, L.epoch, pd.score,
-                         L.gap, L.g, L.err};
+                         L.unit, L.gap, L.g, L.err};
     const uint32_t S = p.S, C = p.C;
     const uint32_t s = 32u * w + lane;
     const bool valid = s < S;
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kPairWarps * 32, 1) k_bits_pair(PairLaunch L) 
             }
         }
     }
-    if (last) *p.score = W + p.gap * (int32_t)(p.m + p.n);
+    if (last) *p.score = W * p.unit + p.gap * (int32_t)(p.m + p.n);
 }
 
 // ------------------------------------------------ a batch on groups of lanes
@@ -356,7 +356,7 @@ struct GroupLaunch {
     uint4 *rec;
     uint64_t rec_cap;
     uint2 *rows;
-    int32_t gap;
+    int32_t unit, gap;
     BitsScoring g;
     uint32_t *err;
 };
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_bits_group(GroupLaunch L) {
             }
             ++c;
         }
-        if (mine && l == (S ? (S - 1u) & (G - 1u) : 0u)) *t.score = W + L.gap * (int32_t)(t.m + t.n);
+        if (mine && l == (S ? (S - 1u) & (G - 1u) : 0u)) *t.score = W * L.unit + L.gap * (int32_t)(t.m + t.n);
         __syncwarp();
     }
 }
@@ -513,9 +513,7 @@ uint32_t resident_warps(nw_ctx *ctx, bool gen, bool want) {
     return (uint32_t)std::max(occ, 1) * (uint32_t)ctx->sm_count;
 }
 
-bool gen_of(const nw_scoring &sc) {
-    return !(sc.match - 2 * sc.gap == 3 && sc.mismatch - 2 * sc.gap == 1);
-}
+bool gen_of(const nw_scoring &sc) { return bits_units(sc).gen(); }
 }  // namespace
 
 bool bits_pair_takes(nw_ctx *ctx, uint32_t m, uint32_t n, const nw_scoring &sc, bool want) {
@@ -545,13 +543,11 @@ int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &job
     PairLaunch L{};
     L.pl0 = ps.pl0;
     L.pl1 = ps.pl1;
+    const BitsUnits units = bits_units(sc);
+    L.unit = units.unit;
     L.gap = sc.gap;
+    L.g = units.planes();
     L.err = ctx->d_err;
-    const int32_t sm = sc.match - 2 * sc.gap, sx = sc.mismatch - 2 * sc.gap;
-    L.g.M1 = (sm & 2) ? ~0u : 0u;
-    L.g.M0 = (sm & 1) ? ~0u : 0u;
-    L.g.X1 = (sx & 2) ? ~0u : 0u;
-    L.g.X0 = (sx & 1) ? ~0u : 0u;
     // longest chains first; a wave takes pairs while their warps are all
     // resident at once and their records fit the budget
     std::vector<size_t> order(jobs.size());
@@ -733,13 +729,11 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
     GroupLaunch L{};
     L.pl0 = ps.pl0;
     L.pl1 = ps.pl1;
+    const BitsUnits units = bits_units(sc);
+    L.unit = units.unit;
     L.gap = sc.gap;
+    L.g = units.planes();
     L.err = ctx->d_err;
-    const int32_t sm = sc.match - 2 * sc.gap, sx = sc.mismatch - 2 * sc.gap;
-    L.g.M1 = (sm & 2) ? ~0u : 0u;
-    L.g.M0 = (sm & 1) ? ~0u : 0u;
-    L.g.X1 = (sx & 2) ? ~0u : 0u;
-    L.g.X0 = (sx & 1) ? ~0u : 0u;
     const void *kern = gen ? (const void *)k_bits_group<true> : (const void *)k_bits_group<false>;
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kPairWarps * 32, 0);

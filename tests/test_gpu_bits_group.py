@@ -2,7 +2,8 @@
 the walk by runs, against the oracle: rows at and around multiples of a bit
 stripe (31), of a group's stripes and of a pass, columns at and around the
 chunks of 32 steps (where a pass follows the one before without a gap), long
-gaps, unrelated pairs, empty sides, two-plane scorings, 'M' CIGARs, and a
+gaps, unrelated pairs, empty sides, two-plane scorings (as they are, and in
+units of a common divisor), 'M' CIGARs, and a
 budget that splits the batch into waves."""
 import numpy as np
 import pytest
@@ -36,7 +37,7 @@ def _check(ctx, pairs, sc, flags=0):
         assert s[k] == v and c[k] == want, (k, pairs[k][0].size, pairs[k][1].size)
 
 
-@pytest.mark.parametrize("sc", [(1, -1, -1), (1, 0, -1), (1, -2, -1)])
+@pytest.mark.parametrize("sc", [(1, -1, -1), (1, 0, -1), (1, -2, -1), (2, -1, -2), (2, -2, -2), (4, -2, -1)])
 def test_shapes(sc):
     import torch
     import paper_2412_21103_gb300 as nw
@@ -47,6 +48,10 @@ def test_shapes(sc):
         _check(ctx, pairs, sc)
         assert ctx.kernel_stats()["bgroup_fill_ptr"][0] > 0
         _check(ctx, pairs[:40], sc, nw.NW_CIGAR_M)
+        pool, off, lens = nw.pool_of([s for p in pairs for s in p])
+        s, _ = nw.nw_align_batch(ctx, pool, off[0::2], lens[0::2], off[1::2], lens[1::2], sc, 0)
+        assert list(s) == oracle.score_many(pairs, *sc)
+        assert ctx.kernel_stats()["bits_score"][0] > 0
 
 
 def test_many_pairs_take_few_lanes_and_waves():
