@@ -17,22 +17,36 @@
 // anti-diagonal (bit p = row top + p); the cell above a bit is the bit below
 // it on the previous anti-diagonal and the cell to its left is the same bit,
 // so one anti-diagonal step is a fixed sequence of funnel shifts and
-// three-input logic operations (LOP3) on whole words: about 20 instructions
-// for 32 cells, where the scalar kernels spend 3 per cell.
+// three-input logic operations (LOP3) on whole words.
 //
-// Work split.  One pair per lane.  Stripes of 32 rows are aligned to the
-// bottom of the grid (the last stripe's bit 31 is row m); rows <= 0 of the
-// first stripe are padding, forced to the boundary's zero differences by a
-// row mask.  A stripe sweeps the anti-diagonals that cross it, in chunks of
-// 32 steps: bit 0 meets column t+1 at step t, bit 31 column t-30.  The
-// previous stripe's bottom row arrives as 32 input bits per chunk and the
-// stripe's own bottom row leaves through the same shift register (one funnel
-// shift per plane and step does both); the words go through a per-warp row
-// buffer in global memory, [chunk][lane], so a warp's accesses coalesce.
-// The lanes of a warp hold pairs of equal stripe count and similar width
-// (a "job"), so they run in lockstep; jobs are taken longest first from an
-// atomic counter.  The score is W(m,n) = sum over j of dH(m,j), read from the
-// last stripe's outgoing words with population counts.
+// Work split.  One pair per lane.  A lane holds K = 1, 2 or 4 words of each
+// plane, rows dealt out in turn: bit p of word w is row K*p + w of a stripe of
+// 32*K rows.  So the cell above word w is the same bit of word w - 1 one step
+// earlier -- no shift --, only word 0 takes a funnel shift of word K - 1; and
+// the B window of word w is the one word 0 had w steps before, so K windows
+// are kept, and each step one of them moves by one bit.  The shifts (the
+// upper dH, the stripe boundary and the B window, two planes each) cost a step
+// 6 operations for all K words, the cells 10 a word: 16, 13 or 11.5 a word.
+//
+// Stripes are aligned to the bottom of the grid (the last row of the last
+// stripe is row m) and follow one another without a gap: the row r of a
+// stripe starts r steps after its row 0, on a period of whole chunks of 32
+// columns, so while the last rows finish a stripe the first ones are in the
+// next.  A step starts one row: its bit of A is replaced and its dV cleared.
+// The rows <= 0 of the first stripe are padding: what they hold is kept from
+// row 1 by a mask on its upper dH.  The previous stripe's bottom row arrives
+// as 32 input bits per chunk and the stripe's own leaves through the same
+// shift register; the words go through a per-warp buffer in global memory,
+// [chunk][lane], so a warp's accesses coalesce.  The lanes of a warp hold
+// pairs of equal stripe count and similar width (a "job"), so they run in
+// lockstep; jobs are taken longest first from an atomic counter.  The score is
+// W(m,n) = sum over j of dH(m,j), read from the last stripe's outgoing words
+// with population counts.
+//
+// What bounds it: the logic pipe.  All-vs-all of 512 sequences of 500 to
+// 1,500 bases: 3.2 ms; with one word a lane and a gap of 31 steps after each
+// stripe 4.2 ms.  (K = 1, 2, 4 for all: 4.3, 3.4, 3.25 ms; 20,000 pairs of
+// reads of 50 to 600 bases .43, .36, .34 ms.)
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -44,119 +58,178 @@
 
 namespace nw {
 
-// One anti-diagonal step of the 32 cells of a lane.  (H, V): the dH, dV
-// planes of the previous anti-diagonal; Q: the shift register of the stripe
-// boundary (bit 31 = the input bit of this step, the output bit enters at
-// bit 0).  bw: the B window (bit p = base of column t+1-p), A: the row bases,
-// rmask: rows of the grid (the padding rows of a pair's first stripe, FIRST,
-// keep the boundary's zero differences).  RAMP: the first chunk of a stripe,
-// where bits p > u lie in column <= 0 and their dV is forced to the
-// boundary's 0.
-//
-// What bounds it: the logic pipe, 16 operations for 32 cells (two B window
-// shifts, two for equality, two to bring the upper dH into line, eight for
-// the update, two for the shift register).
-template <bool GEN, bool RAMP, bool FIRST>
-__device__ __forceinline__ void bits_step(int u, uint32_t &H0, uint32_t &H1, uint32_t &V0, uint32_t &V1, uint32_t &Q0,
-                                          uint32_t &Q1, uint32_t A0, uint32_t A1, uint32_t bw0, uint32_t bw1,
-                                          uint32_t rmask, const BitsScoring &g, uint32_t X1r, uint32_t X0r) {
-    const uint32_t a0 = __funnelshift_l(Q0, H0, 1), a1 = __funnelshift_l(Q1, H1, 1);  // dH of the cell above
-    const uint32_t b0 = V0, b1 = V1;                                                  // dV of the cell to the left
-    if constexpr (!GEN) {
-        const uint32_t eq = lop3<kLutEq>(A0, bw0, A1 ^ bw1);  // A_i == B_j
-        bits_cell(eq, a0, a1, b0, b1, H0, H1, V0, V1);
-        if constexpr (FIRST) {
-            H0 &= rmask;
-            H1 &= rmask;
-            V0 &= rmask;
-            V1 &= rmask;
-        }
-        if constexpr (RAMP) {
-            const uint32_t mk = (2u << u) - 1u;  // bits in column >= 1
-            V0 &= mk;
-            V1 &= mk;
-        }
-    } else {
-        const uint32_t x = lop3<kLutXorOrNotC>(A1, bw1, rmask);
-        const uint32_t eq = lop3<kLutEq>(A0, bw0, x);  // A_i == B_j (0 on padding rows)
-        const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);  // the low bit of max(a, b), from a
-        const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);  // ... from b
-        const uint32_t e1 = lop3<kLutSel>(eq, g.M1, X1r), e0 = lop3<kLutSel>(eq, g.M0, X0r);
-        const uint32_t m0 = p | q, m1 = a1 | b1;
-        const uint32_t T0 = lop3<kLutAndNotOr>(m0, e1, m1) | lop3<kLutAndNotOr>(e0, m1, e1);
-        const uint32_t T1 = m1 | e1;
-        const uint32_t ca = lop3<kLutAndNot>(a0, T0, 0u), cb = lop3<kLutAndNot>(b0, T0, 0u);  // borrows
-        if constexpr (RAMP) {
-            const uint32_t mk = (2u << u) - 1u;
-            V0 = lop3<kLutXorAnd>(T0, a0, mk);
-            V1 = lop3<kLutXor3>(T1, a1, ca) & mk;
-        } else {
-            V0 = T0 ^ a0;
-            V1 = lop3<kLutXor3>(T1, a1, ca);
-        }
-        H0 = T0 ^ b0;
-        H1 = lop3<kLutXor3>(T1, b1, cb);
-    }
-    Q0 = __funnelshift_l(H0, Q0, 1);
-    Q1 = __funnelshift_l(H1, Q1, 1);
+// The cell update for any scoring of two bit planes (see bits_cell).
+__device__ __forceinline__ void bits_cell_gen(const BitsScoring &g, uint32_t eq, uint32_t a0, uint32_t a1, uint32_t b0,
+                                              uint32_t b1, uint32_t &H0, uint32_t &H1, uint32_t &V0, uint32_t &V1) {
+    const uint32_t p = lop3<kLutAndOrNot>(a0, a1, b1);  // the low bit of max(a, b), from a
+    const uint32_t q = lop3<kLutAndOrNot>(b0, b1, a1);  // ... from b
+    const uint32_t e1 = lop3<kLutSel>(eq, g.M1, g.X1), e0 = lop3<kLutSel>(eq, g.M0, g.X0);
+    const uint32_t m0 = p | q, m1 = a1 | b1;
+    const uint32_t T0 = lop3<kLutAndNotOr>(m0, e1, m1) | lop3<kLutAndNotOr>(e0, m1, e1);
+    const uint32_t T1 = m1 | e1;
+    const uint32_t ca = lop3<kLutAndNot>(a0, T0, 0u), cb = lop3<kLutAndNot>(b0, T0, 0u);  // borrows
+    V0 = T0 ^ a0;
+    V1 = lop3<kLutXor3>(T1, a1, ca);
+    H0 = T0 ^ b0;
+    H1 = lop3<kLutXor3>(T1, b1, cb);
 }
 
-template <bool GEN, bool RAMP, bool FIRST>
-__device__ __forceinline__ void bits_chunk(uint32_t &H0, uint32_t &H1, uint32_t &V0, uint32_t &V1, uint32_t &Q0,
-                                           uint32_t &Q1, uint32_t A0, uint32_t A1, uint32_t Rc0, uint32_t Rc1,
-                                           uint32_t Rn0, uint32_t Rn1, uint32_t rmask, const BitsScoring &g,
-                                           uint32_t X1r, uint32_t X0r) {
+// A lane's state: difference planes, row bases and B windows of K words, the
+// next stripe's row bases, and the mask that clears row 1's upper dH.
+template <int K>
+struct BitsLane {
+    uint32_t H0[K], H1[K], V0[K], V1[K], A0[K], A1[K], N0[K], N1[K], B0[K], B1[K], top[K];
+};
+
+// 32 steps.  X: the chunk's columns, the first at bit 31; Q: the shift register
+// of the stripe boundary (bit 31 = the input bit of the step, the output bit
+// enters at bit 0).  TRANS: rows of a stripe start, one a step, from bit `q` on.
+// FIRST: rows of the first stripe are at work; `lift`: the rows that start are
+// beyond them.
+template <bool GEN, int K, bool FIRST, bool TRANS>
+__device__ __forceinline__ void bits_chunk(BitsLane<K> &s, uint32_t X0, uint32_t X1, uint32_t &Q0, uint32_t &Q1,
+                                           uint32_t q, uint32_t lift, const BitsScoring &g) {
+    uint32_t tb = 1u << q;
+#pragma unroll 1
+    for (int it = 0; it < 8; ++it) {
 #pragma unroll
-    for (int u = 0; u < 32; ++u)
-        bits_step<GEN, RAMP, FIRST>(u, H0, H1, V0, V1, Q0, Q1, A0, A1, __funnelshift_l(Rn0, Rc0, u),
-                                    __funnelshift_l(Rn1, Rc1, u), rmask, g, X1r, X0r);
+        for (int u = 0; u < 4; ++u) {
+            constexpr auto mod = [](int x) { return (x + 4) % K; };
+            const int w0 = mod(u);
+            s.B0[w0] = __funnelshift_l(u ? mul(X0, 1u << u) : X0, s.B0[w0], 1);
+            s.B1[w0] = __funnelshift_l(u ? mul(X1, 1u << u) : X1, s.B1[w0], 1);
+            if constexpr (TRANS) {
+                const uint32_t bit = u / K ? mul(tb, 1u << (u / K)) : tb;
+                s.A0[w0] = lop3<kLutSel>(bit, s.N0[w0], s.A0[w0]);
+                s.A1[w0] = lop3<kLutSel>(bit, s.N1[w0], s.A1[w0]);
+                s.V0[w0] &= ~bit;
+                s.V1[w0] &= ~bit;
+                if constexpr (FIRST) s.top[w0] |= bit & lift;
+            }
+            uint32_t a0 = __funnelshift_l(Q0, s.H0[K - 1], 1), a1 = __funnelshift_l(Q1, s.H1[K - 1], 1);
+            const uint32_t h0 = a0, h1 = a1;
+#pragma unroll
+            for (int w = K - 1; w >= 0; --w) {
+                a0 = w ? s.H0[w ? w - 1 : 0] : h0;
+                a1 = w ? s.H1[w ? w - 1 : 0] : h1;
+                if constexpr (FIRST) {
+                    a0 &= s.top[w];
+                    a1 &= s.top[w];
+                }
+                const uint32_t eq = lop3<kLutEq>(s.A0[w], s.B0[mod(u - w)], s.A1[w] ^ s.B1[mod(u - w)]);  // A_i == B_j
+                if constexpr (GEN) bits_cell_gen(g, eq, a0, a1, s.V0[w], s.V1[w], s.H0[w], s.H1[w], s.V0[w], s.V1[w]);
+                else bits_cell(eq, a0, a1, s.V0[w], s.V1[w], s.H0[w], s.H1[w], s.V0[w], s.V1[w]);
+            }
+            Q0 = __funnelshift_l(s.H0[K - 1], Q0, 1);
+            Q1 = __funnelshift_l(s.H1[K - 1], Q1, 1);
+        }
+        X0 = mul(X0, 16u);
+        X1 = mul(X1, 16u);
+        if constexpr (TRANS) tb <<= 4 / K;
+    }
 }
 
-// One stripe of a job, lane by lane: its chunks in order, the words of the
-// row above in and of its bottom row out through `rows`.  The B window that
-// follows a chunk and the row's words are loaded one chunk ahead.
-// FIRST: stripe 0 (nothing comes in; padding rows).
-template <bool GEN, bool FIRST>
-__device__ __forceinline__ void bits_stripe(const BitsArgs &p, uint32_t C, uint32_t n, int64_t Bg, uint32_t A0,
-                                            uint32_t A1, uint32_t rmask, bool last, uint2 *rows, int32_t &W) {
-    const uint32_t X1r = p.g.X1 & rmask, X0r = p.g.X0 & rmask;
-    uint32_t H0 = 0, H1 = 0, V0 = 0, V1 = 0;
-    uint32_t Rc0 = __brev(plane_window(p.pl0, Bg - 31)), Rc1 = __brev(plane_window(p.pl1, Bg - 31));
-    uint32_t Fn0 = plane_window(p.pl0, Bg + 1), Fn1 = plane_window(p.pl1, Bg + 1);
-    uint2 prev = make_uint2(0u, 0u), nx = make_uint2(0u, 0u);
-    if constexpr (!FIRST) {
-        prev = __ldcg(rows);
-        if (C > 1) nx = __ldcg(rows + 32u);
+__device__ __forceinline__ uint32_t even_bits32(uint32_t x) {  // into the low 16 bits
+    x &= 0x55555555u;
+    x = (x | (x >> 1)) & 0x33333333u;
+    x = (x | (x >> 2)) & 0x0F0F0F0Fu;
+    x = (x | (x >> 4)) & 0x00FF00FFu;
+    return (x | (x >> 8)) & 0x0000FFFFu;
+}
+
+// 32*K rows from row `row` on (before the first base: unspecified), dealt out in turn to K words.
+template <int K>
+__device__ __forceinline__ void deal_rows(const uint32_t *pl, int64_t Ag, int32_t row, uint32_t (&out)[K]) {
+    uint32_t c[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) c[j] = plane_window(pl, Ag + max(row + 32 * j, -32));
+    if constexpr (K == 1) {
+        out[0] = c[0];
+    } else if constexpr (K == 2) {
+        out[0] = even_bits32(c[0]) | even_bits32(c[1]) << 16;
+        out[1] = even_bits32(c[0] >> 1) | even_bits32(c[1] >> 1) << 16;
+    } else {
+        static_assert(K == 4);
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            const uint32_t lo = even_bits32(c[0] >> o) | even_bits32(c[1] >> o) << 16;
+            const uint32_t hi = even_bits32(c[2] >> o) | even_bits32(c[3] >> o) << 16;
+            out[o] = even_bits32(lo) | even_bits32(hi) << 16;
+            out[o + 2] = even_bits32(lo >> 1) | even_bits32(hi >> 1) << 16;
+        }
     }
-    for (uint32_t c = 0; c < C; ++c) {
-        const uint32_t Rn0 = __brev(Fn0), Rn1 = __brev(Fn1);
-        const int64_t gb = Bg + 32 * (int64_t)min(c + 1, C - 1) + 1;
-        Fn0 = plane_window(p.pl0, gb);
-        Fn1 = plane_window(p.pl1, gb);
+}
+
+// W(m, n) of a lane's pair, in the steps of its job: job.T chunks, a stripe
+// every job.C.
+template <bool GEN, int K>
+__device__ __forceinline__ int32_t bits_pairs_of(const BitsArgs &p, const BitsJob &job, uint32_t m, uint32_t n,
+                                                 int64_t Ag, int64_t Bg, uint2 *rows) {
+    constexpr int32_t SH = 32 * K;
+    const uint32_t S = job.S, C = job.C;
+    const int32_t pad = SH * (int32_t)S - (int32_t)m;  // rows above row 1 in stripe 0
+    const int32_t ncol = (int32_t)((n + 31) / 32);     // chunks that hold columns of this pair
+    BitsLane<K> s;
+#pragma unroll
+    for (int w = 0; w < K; ++w) {
+        s.H0[w] = s.H1[w] = s.V0[w] = s.V1[w] = s.A0[w] = s.A1[w] = s.N0[w] = s.N1[w] = s.B0[w] = s.B1[w] = 0;
+        s.top[w] = pad % K == w ? ~(1u << (pad / K)) : ~0u;
+    }
+    const auto cols = [&](const uint32_t *pl, uint32_t cl) {
+        return __brev(plane_window(pl, Bg + 32 * (int64_t)min((int32_t)cl, ncol)));
+    };
+    uint32_t X0 = cols(p.pl0, 0), X1 = cols(p.pl1, 0);
+    uint2 prev = make_uint2(0u, 0u), nx = make_uint2(0u, 0u);
+    int32_t W = 0;
+    uint32_t stripe = 0, cl = 0;   // of the stripe's row 0
+    uint32_t started = 0, lift = 0;  // chunks since a stripe began; all ones once it is not the first
+    for (uint32_t c = 0; c < job.T; ++c) {
+        if (cl == 0 && stripe < S) {
+            started = 0;
+            lift = stripe ? ~0u : 0u;
+            const int32_t row = SH * (int32_t)stripe - pad;
+            deal_rows<K>(p.pl0, Ag, row, s.N0);
+            deal_rows<K>(p.pl1, Ag, row, s.N1);
+        }
+        const uint32_t cn = cl + 1 == C ? 0u : cl + 1;
+        const uint32_t Y0 = cols(p.pl0, cn), Y1 = cols(p.pl1, cn);  // the next chunk's columns
+        // The bottom row of the stripe above: its column 32x is bit 0 of the
+        // word of chunk x + K - 1, the 31 columns that follow are the high bits
+        // of the word after it.  Loaded one chunk ahead; the buffer holds the
+        // last C chunks' words.
         uint32_t Q0 = 0, Q1 = 0;
-        if constexpr (!FIRST) {
-            // input bits: the previous stripe's bottom row, columns 32c+1 .. 32c+32,
-            // column 32c+1 at bit 31
+        if (stripe) {
             Q0 = __funnelshift_r(nx.x, prev.x, 1);
             Q1 = __funnelshift_r(nx.y, prev.y, 1);
-            prev = nx;
-            nx = c + 2 < C ? __ldcg(rows + (size_t)(c + 2) * 32u) : make_uint2(0u, 0u);
         }
-        if (c == 0) bits_chunk<GEN, true, FIRST>(H0, H1, V0, V1, Q0, Q1, A0, A1, Rc0, Rc1, Rn0, Rn1, rmask, p.g, X1r, X0r);
-        else bits_chunk<GEN, false, FIRST>(H0, H1, V0, V1, Q0, Q1, A0, A1, Rc0, Rc1, Rn0, Rn1, rmask, p.g, X1r, X0r);
-        // outgoing bits: bit b is column 32c+1-b of the stripe's bottom row
-        if (!last) {
-            __stcg(rows + (size_t)c * 32u, make_uint2(Q0, Q1));
+        prev = nx;
+        if (S > 1 && c + 2 >= C) {
+            uint32_t r = cl + 1 + K;
+            if (r >= C) r -= C;
+            nx = __ldcg(rows + (size_t)r * 32u);
+        }
+        if (c < C + K || S == 1) {
+            if (started < (uint32_t)K) bits_chunk<GEN, K, true, true>(s, X0, X1, Q0, Q1, started * (32 / K), lift, p.g);
+            else bits_chunk<GEN, K, true, false>(s, X0, X1, Q0, Q1, 0u, 0u, p.g);
         } else {
-            const int32_t lo = max(32 * (int32_t)c + 1 - (int32_t)n, 0), hi = min(31, 32 * (int32_t)c);
-            if (lo <= hi) {
-                const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
-                W += __popc(Q0 & mk) + 2 * __popc(Q1 & mk);
-            }
+            if (started < (uint32_t)K) bits_chunk<GEN, K, false, true>(s, X0, X1, Q0, Q1, started * (32 / K), 0u, p.g);
+            else bits_chunk<GEN, K, false, false>(s, X0, X1, Q0, Q1, 0u, 0u, p.g);
         }
-        Rc0 = Rn0;
-        Rc1 = Rn1;
+        ++started;
+        // outgoing bits: bit b is column 32 (c - K + 1) - b of the bottom row, from the stripe's first chunk on
+        if (S > 1 && c < (S - 1) * C + K) __stcg(rows + (size_t)cl * 32u, make_uint2(Q0, Q1));
+        const int32_t e = 32 * ((int32_t)c - (int32_t)((S - 1) * C) - K + 1);
+        const int32_t lo = max(e + 1 - (int32_t)n, 0), hi = min(31, e);
+        if (lo <= hi) {
+            const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
+            W += __popc(Q0 & mk) + 2 * __popc(Q1 & mk);
+        }
+        X0 = Y0;
+        X1 = Y1;
+        cl = cn;
+        if (cl == 0) ++stripe;
     }
+    return W;
 }
 
 // Row and column of the q-th pair of a class: the columns before the class's
@@ -210,15 +283,12 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
             out0 = a.id * p.nseq + b.id;
             out1 = b.id * p.nseq + a.id;
         }
-        const uint32_t S = job.S, C = job.C;
         int32_t W = 0;
         const int64_t Ag = (int64_t)aw * 32 - kPlanePad, Bg = (int64_t)bw * 32 - kPlanePad;  // planar slots
-        const int32_t top0 = (int32_t)m - 32 * (int32_t)S;             // row above bit 0 of stripe 0
-        for (uint32_t s = 0; s < S; ++s) {
-            const int64_t abase = max(Ag + top0 + 32 * (int64_t)s, Ag - 32);
-            const uint32_t A0 = plane_window(p.pl0, abase), A1 = plane_window(p.pl1, abase);
-            if (s == 0) bits_stripe<GEN, true>(p, C, n, Bg, A0, A1, ~0u << min(max(-top0, 0), 31), S == 1, rows, W);
-            else bits_stripe<GEN, false>(p, C, n, Bg, A0, A1, ~0u, s + 1 == S, rows, W);
+        if (job.S) {
+            if (job.K == 4) W = bits_pairs_of<GEN, 4>(p, job, m, n, Ag, Bg, rows);
+            else if (job.K == 2) W = bits_pairs_of<GEN, 2>(p, job, m, n, Ag, Bg, rows);
+            else W = bits_pairs_of<GEN, 1>(p, job, m, n, Ag, Bg, rows);
         }
         if (active) {
             const int32_t sc = W * p.unit + p.gap * (int32_t)(m + n);
@@ -366,9 +436,55 @@ bool bits_batch_ok(const nw_scoring &sc) {
     return u.sx >= 0 && u.sx <= u.sm && u.sm <= 3;
 }
 
-// Stripes and chunks per stripe of an m x n pair.
-static uint32_t stripes_of(uint32_t m) { return (m + 31) / 32; }
-static uint32_t chunks_of(uint32_t n) { return (n + 62) / 32; }
+// How a pair of m rows runs: K words a lane, S stripes, and the operations of
+// a step.
+struct BitsShape {
+    uint32_t K, S, ops;
+    uint32_t period(uint32_t n) const { return S > 1 ? std::max((n + 31) / 32, K + 3) : (n + 31) / 32; }
+    uint32_t chunks(uint32_t n) const { return (S - 1) * period(n) + (n + 32 * K + 30) / 32; }
+    uint64_t work(uint32_t n) const { return (uint64_t)ops * chunks(n); }
+};
+
+// The K with the least work at as many columns as rows, by the rows' words (a
+// pair's columns are mostly as many or more): more words take fewer shifts a
+// word, but pad the rows to 32*K and want a period of K + 3 chunks for the row
+// buffer (a word is read K + 1 chunks after its stripe's first, one chunk
+// ahead of its use).  From 64 words on the padding no longer matters.
+// NW_BITS_WORDS: one K for all (sweeps).
+class BitsShapes {
+  public:
+    BitsShapes() {
+        const char *e = getenv("NW_BITS_WORDS");
+        const uint32_t force = e ? (uint32_t)atoi(e) : 0u;
+        for (uint32_t w = 1; w <= kWords; ++w) {
+            uint64_t best = ~0ull;
+            for (uint32_t l = 0; l < 3; ++l) {
+                const BitsShape c = shape(w, l);
+                const uint64_t x = force ? (force != c.K) : c.work(32 * w);
+                if (x < best) {
+                    best = x;
+                    by_words_[w] = c;
+                }
+            }
+        }
+    }
+    BitsShape of(uint32_t m) const {  // m = 0: no stripes
+        const uint32_t w = (m + 31) / 32;
+        if (w <= kWords) return by_words_[w];
+        return shape(w, by_words_[kWords].K / 2);
+    }
+
+  private:
+    static constexpr uint32_t kWords = 64;
+    // K = 2^l
+    static BitsShape shape(uint32_t w, uint32_t l) { return BitsShape{1u << l, (w + (1u << l) - 1) >> l, (10u << l) + 6}; }
+    BitsShape by_words_[kWords + 1] = {};
+};
+
+// A job of pairs of at most n columns.
+static BitsJob job_of(const BitsShape &s, uint32_t n, uint32_t t0, uint32_t cnt, uint32_t cls) {
+    return BitsJob{t0, cnt, s.S, s.S ? s.period(n) : 0u, s.S ? s.chunks(n) : 0u, s.K, cls};
+}
 
 // The launch's tables in one upload, its constants, grid and row buffers.
 // `head`: the task table, or the sequence and class tables (16-byte padded).
@@ -378,7 +494,7 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
     int rc;
     // longest jobs first, ties in job order
     std::vector<uint64_t> keys(jobs.size());
-    for (size_t q = 0; q < jobs.size(); ++q) keys[q] = (uint64_t)jobs[q].S * jobs[q].C;
+    for (size_t q = 0; q < jobs.size(); ++q) keys[q] = (uint64_t)jobs[q].T * (10 * jobs[q].K + 6);
     const std::vector<uint32_t> jo = radix_order_desc(std::move(keys));
     const size_t jobs_at = (head.size() + 15) / 16 * 16;
     head.resize(jobs_at + jobs.size() * sizeof(BitsJob));
@@ -409,9 +525,8 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
                                                   kBitsWarps * 32, 0);
     // One CTA of 8 warps per SM (two warps per scheduler), not the most the
     // registers allow: with more, the longest jobs -- taken first -- share
-    // their scheduler with the rest and finish the launch alone.  Measured on
-    // GB300 (all-vs-all of 512 sequences, CTAs per SM 8 / 3 / 2 / 1): 17.6k /
-    // 17.7k / 22.4k / 23.7k GCUPS.  NW_BITS_OCC overrides (sweeps).
+    // their scheduler with the rest and finish the launch alone.  All-vs-all of
+    // 512 sequences: 3.25 ms, with two CTAs 3.6.  NW_BITS_OCC overrides (sweeps).
     int cap = 1;
     if (const char *e = getenv("NW_BITS_OCC")) cap = std::max(1, atoi(e));
     occ = std::min(occ, cap);
@@ -435,8 +550,9 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> 
     *plan = BitsPlan{};
     if (tasks.empty()) return NW_OK;
     HostTimer ht(ctx, "bits_plan");
-    // rows: the orientation with fewer stripe-chunks (the score is symmetric);
-    // order: equal stripe counts, widest first
+    // rows: the orientation with less work (the score is symmetric); order:
+    // equal shapes, widest first
+    const BitsShapes shapes;
     const size_t n = tasks.size();
     std::vector<uint64_t> keys(n);
     std::vector<uint8_t> turned(n);
@@ -447,9 +563,13 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> 
             keys[k] = std::max(t.m, t.n);  // no stripes
             continue;
         }
-        turned[k] = (uint64_t)stripes_of(t.n) * chunks_of(t.m) < (uint64_t)stripes_of(t.m) * chunks_of(t.n);
-        const uint32_t rows = turned[k] ? t.n : t.m, cols = turned[k] ? t.m : t.n;
-        keys[k] = (uint64_t)stripes_of(rows) << 32 | cols;
+        BitsShape sh = shapes.of(t.m);
+        if ((t.m + 31) / 32 != (t.n + 31) / 32) {
+            const BitsShape sn = shapes.of(t.n);
+            turned[k] = sn.work(t.m) < sh.work(t.n);
+            if (turned[k]) sh = sn;
+        }
+        keys[k] = (uint64_t)sh.S << 36 | (uint64_t)sh.K << 32 | (turned[k] ? t.m : t.n);
         bytes += (t.m + 3) / 4 + (t.n + 3) / 4;
         extent = std::max(extent, std::max(t.a_off + (t.m + 3) / 4, t.b_off + (t.n + 3) / 4));
     }
@@ -472,19 +592,19 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> 
             std::swap(b.a_off, b.b_off);
             std::swap(b.m, b.n);
         }
-        const uint32_t S = (b.m && b.n) ? stripes_of(b.m) : 0u;
-        if (S && own) {
+        const BitsShape sh = shapes.of(b.n ? b.m : 0);
+        if (sh.S && own) {
             b.aw = (uint32_t)words;
             b.bw = b.aw + (b.m + 31) / 32 + 2;
             words = (uint64_t)b.bw + (b.n + 31) / 32 + 2;
             if (words >= (1ull << 32)) return fail(ctx, NW_ERR_ARG, "planar copy of more than 2^37 bases");
-        } else if (S) {
+        } else if (sh.S) {
             b.aw = PlaneSet::word_of(plan->planes.add(b.a_off, b.m));
             b.bw = PlaneSet::word_of(plan->planes.add(b.b_off, b.n));
         }
         ht_[q] = b;
-        if (jobs.empty() || jobs.back().S != S || jobs.back().cnt == 32)
-            jobs.push_back(BitsJob{(uint32_t)q, 0, S, S ? chunks_of(b.n) : 0, 0});
+        if (jobs.empty() || jobs.back().S != sh.S || jobs.back().K != sh.K || jobs.back().cnt == 32)
+            jobs.push_back(job_of(sh, b.n, (uint32_t)q, 0, 0));
         ++jobs.back().cnt;
         maxC = std::max(maxC, jobs.back().C);
     }
@@ -512,13 +632,15 @@ int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, cons
         const uint32_t i = order[q];
         seqs[q] = BitsSeq{len[i] ? PlaneSet::word_of(plan->planes.add(off[i], len[i])) : 2u, len[i], i};
     }
+    const BitsShapes shapes;
     std::vector<BitsClass> classes;
     std::vector<BitsJob> jobs;
     uint32_t maxC = 1;
     for (uint32_t r0 = 0; r0 < nseq;) {
-        const uint32_t S = stripes_of(seqs[r0].len);
-        uint32_t r1 = r0;
-        while (r1 < nseq && stripes_of(seqs[r1].len) == S) ++r1;
+        const BitsShape sh = shapes.of(seqs[r0].len);
+        uint32_t r1 = r0 + 1;
+        for (; r1 < nseq; ++r1)
+            if (const BitsShape x = shapes.of(seqs[r1].len); x.S != sh.S || x.K != sh.K) break;
         const uint32_t rows = r1 - r0, pairs = r0 * rows + rows * (rows - 1) / 2;
         // the pairs run through the columns in order: a job's first column is its widest
         uint32_t c = 0;
@@ -528,8 +650,7 @@ int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, cons
         };
         for (uint32_t q = 0; q < pairs; q += 32) {
             while (end_of(c) <= q) ++c;
-            jobs.push_back(BitsJob{q, std::min(32u, pairs - q), S, S ? chunks_of(seqs[c].len) : 0,
-                                   (uint32_t)classes.size()});
+            jobs.push_back(job_of(sh, seqs[c].len, q, std::min(32u, pairs - q), (uint32_t)classes.size()));
             maxC = std::max(maxC, jobs.back().C);
         }
         classes.push_back(BitsClass{r0, r1});

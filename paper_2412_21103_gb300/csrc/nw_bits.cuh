@@ -22,7 +22,6 @@ __device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
 // Truth tables from the canonical inputs a = 0xF0, b = 0xCC, c = 0xAA.
 constexpr uint32_t kA = 0xF0, kB = 0xCC, kC = 0xAA;
 constexpr uint32_t lut(uint32_t v) { return v & 0xFFu; }
-constexpr uint32_t kLutXorOrNotC = lut((kA ^ kB) | ~kC);     // (a ^ b) | ~c
 constexpr uint32_t kLutEq = lut(~(kA ^ kB) & ~kC);           // ~(a ^ b) & ~c
 constexpr uint32_t kLutAndOrNot = lut(kA & (kB | ~kC));      // a & (b | ~c)
 constexpr uint32_t kLutXor3 = lut(kA ^ kB ^ kC);             // a ^ b ^ c
@@ -91,8 +90,8 @@ struct BitsTask {
 
 // All-vs-all launches name their pairs instead of listing them.  The
 // sequences are sorted longest first; a class holds the rows [r0, r1) of
-// equal stripe count, and its pairs are all (column c < row r), by c and then
-// r, so that 32 consecutive pairs have one stripe count and nearly one width.
+// equal shape (words a lane, stripes), and its pairs are all (column c < row r), by c and then
+// r, so that 32 consecutive pairs have one shape and nearly one width.
 struct BitsSeq {
     uint32_t w, len, id;  // first word of the planar slot, bases, index in the caller's list
 };
@@ -102,7 +101,8 @@ struct BitsClass {
 
 struct BitsJob {
     uint32_t t0, cnt;  // tasks (or pairs of the class) [t0, t0 + cnt), cnt <= 32, one per lane
-    uint32_t S, C;     // stripes, chunks per stripe (the job's largest)
+    uint32_t S, C, T;  // stripes, chunks from one to the next, chunks in all (of the job's widest pair)
+    uint32_t K;        // words a lane
     uint32_t cls;      // all-vs-all: the class
 };
 

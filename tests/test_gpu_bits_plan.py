@@ -48,3 +48,27 @@ def test_batch_slots(repeated):
         got, _ = nw.nw_align_batch(ctx, pool, off[a], ln[a], off[b], ln[b], (1, -1, -1), 0)
     for k, (i, j) in enumerate(pairs):
         assert got[k] == oracle.score(seqs[i], seqs[j], 1, -1, -1), (i, j)
+
+
+@pytest.mark.parametrize("words", [1, 2, 4])
+@pytest.mark.parametrize("sc", [(1, -1, -1), (1, 0, -1)])
+def test_words_per_lane(words, sc, monkeypatch):
+    """Every number of words a lane on rows around multiples of its stripes and
+    columns around its shortest period, lanes of one warp differing in both."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    monkeypatch.setenv("NW_BITS_WORDS", str(words))
+    h = 32 * words
+    rows = [1, 2, h - 1, h, h + 1, 2 * h - 3, 2 * h, 3 * h - 31, 5 * h + 1]
+    cols = [1, 3, 31, 32, 33, 65, 32 * (words + 2), 32 * (words + 3), 32 * (words + 3) + 1, 32 * (words + 5) - 1, 700]
+    rs = seqgen.Stream(43)
+    root = rs.bases(800)
+    pairs = []
+    for m in rows:
+        for n in cols:
+            a = root[:m]
+            pairs.append((a, seqgen.mutate_distinct(root, rs, 0.2)[0][:n]))
+    pool, off, ln = nw.pool_of([s for p in pairs for s in p])
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        got, _ = nw.nw_align_batch(ctx, pool, off[0::2], ln[0::2], off[1::2], ln[1::2], sc, 0)
+    assert list(got) == oracle.score_many(pairs, *sc)
