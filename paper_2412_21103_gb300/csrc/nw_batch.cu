@@ -422,17 +422,18 @@ static int bits_round(nw_ctx *ctx, const uint8_t *pool, const PlaneSet &planes, 
     int rc;
     HostTimer ht_prep(ctx, "bband_round_prep");
     {
-        // pairs that would take longer on their warp than the whole round
-        // ideally takes (the GPU's 4 x 152 schedulers busy) spread their
+        // pairs that would take longer on their warp than the round's
+        // ideal time (the GPU's 4 x 152 schedulers busy) spread their
         // window over more lanes (NW_BBAND_FAST=0 keeps every pair on the
         // throughput shape)
         const char *fe = getenv("NW_BBAND_FAST");
         const bool fast_on = !(fe && *fe == '0');
         double total = 0;
-        for (const auto &it : items) total += band_bits_seconds(it.shape);
-        const double ideal = total / (4.0 * ctx->sm_count);
+        for (const auto &it : items) total += band_bits_seconds(it.shape) * it.shape.g / 32.0;
+        const double limit = total / (4.0 * ctx->sm_count);
         for (auto &it : items)
-            if (fast_on && band_bits_seconds(it.shape) > ideal) band_bits_fast(&it.shape);
+            while (fast_on && band_bits_seconds(it.shape) > limit && band_bits_spread(&it.shape)) {
+            }
     }
     {
         // one warp of this kernel runs its pair at about the scalar batch

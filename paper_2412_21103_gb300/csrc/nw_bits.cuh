@@ -269,9 +269,9 @@ int band_bits_max_q();
 // most max_q words each; false when it needs more than 128 words (4,096
 // rows).
 bool band_bits_shape(uint32_t m, uint32_t n, int32_t lo, int32_t hi, BandBitsShape *s, int max_q);
-// The same window spread over as many lanes as it has words (up to 32):
-// fewer instructions per lane and step, so a shorter time for the pair.
-void band_bits_fast(BandBitsShape *s);
+// The same window spread over twice the lanes: fewer instructions per lane and
+// step, so a shorter time for the pair; false when it cannot be spread further.
+bool band_bits_spread(BandBitsShape *s);
 uint64_t band_bits_cells(const BandBitsShape &s);  // cells of the pair's window, over all its chunks
 uint64_t band_bits_kept(const BandBitsShape &s);   // its kept planes (16-byte units)
 // The widest half-width whose band fits the window of an m x n pair.

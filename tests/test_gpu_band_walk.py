@@ -2,7 +2,8 @@
 in a sub-window around the path.  Exact against the oracle where that can go
 wrong: pairs whose last anti-diagonal lies at, just before and just after a
 block's end, windows of fewer, as many and more words than the sub-window,
-and paths that drift across a block by long gaps."""
+paths that drift across a block by long gaps, and
+walks split into stretches that join or do not."""
 import os
 
 import numpy as np
@@ -14,8 +15,13 @@ import seqgen
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("w", [3, 200, 250, 600])
-def test_blocks_windows_and_drift(w):
+@pytest.mark.parametrize("w,stretch", [(3, None), (200, None), (250, None), (600, None), (3, 1), (100, 1), (200, 2),
+                                       (300, 7), (600, 3)])
+def test_blocks_windows_and_drift(w, stretch, monkeypatch):
+    if stretch:
+        # blocks of a stretch: with one or two the ways between them often miss
+        # the next stretch, and the pair is walked as a whole
+        monkeypatch.setenv("NW_BBAND_STRETCH", str(stretch))
     import torch
     import paper_2412_21103_gb300 as nw
     rs = seqgen.Stream(7100 + w)
