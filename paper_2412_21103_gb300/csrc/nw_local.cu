@@ -8,9 +8,10 @@
 //
 // The floor rules out the W domain of the global kernels (it would turn into
 // a floor that grows along every anti-diagonal), so the cell works on H itself:
-// with m = max(H_up, H_left), one cell is a byte permute (s), one max, one add
-// (m + gap) and one DPX add-max with ReLU, max(H_diag + s, m + gap, 0), and
-// half a three-input max for the largest H.
+// with G = H + gap kept beside H, one cell is a score (a byte permute, or a word
+// from shared memory), two adds (H_diag + s, and G) and one DPX three-input max
+// with ReLU, max(H_diag + s, G_up, G_left, 0), and half a three-input max for
+// the largest H.
 //
 // Batched by stripe jobs: every 32R-row stripe of every pair is one job, jobs
 // queued pair by pair (longest pairs first) and stripes in order, so a pair's
@@ -114,7 +115,7 @@ template <int R>
 struct LocalLane {
     static constexpr uint32_t kParts = (R + 5) / 4;  // 16-byte parts of a kept state
     uint32_t prof[R];
-    int32_t Hl[R];
+    int32_t Hl[R], Gl[R];  // H of the column before, and with the gap's score added (in the fill)
     int32_t dtop;        // H of the row above the lane's first, one column back
     uint32_t xout;       // the last row's H (<< 2) and the column's base code, for the lane below
     uint32_t accL, accH;
@@ -128,9 +129,23 @@ struct LocalLane {
                                   : c == 0 ? p.prof[0] : c == 1 ? p.prof[1] : c == 2 ? p.prof[2] : p.prof[3];
         }
     }
-    __device__ __forceinline__ void start() {  // column 0
+    // the lane's table: kTabRows scores for each base of B
+    __device__ __forceinline__ void table(int4 *tab) const {
 #pragma unroll
-        for (int r = 0; r < R; ++r) Hl[r] = 0;
+        for (uint32_t b = 0; b < 4; ++b)
+#pragma unroll
+            for (int q = 0; q < kTabRows / 4; ++q) {
+                const uint32_t *pr = prof + (R - kTabRows) + 4 * q, sel = sext_selector(b);
+                tab[(b * (kTabRows / 4) + q) * 32] = make_int4((int32_t)prmt(pr[0], 0u, sel), (int32_t)prmt(pr[1], 0u, sel),
+                                                               (int32_t)prmt(pr[2], 0u, sel), (int32_t)prmt(pr[3], 0u, sel));
+            }
+    }
+    __device__ __forceinline__ void start(int32_t g) {  // column 0
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            Hl[r] = 0;
+            Gl[r] = g;
+        }
         dtop = 0;
         xout = 0;
     }
@@ -145,7 +160,7 @@ struct LocalLane {
             if (in_range(q * 32u, cap_left, err, kSiteLocalPtr))
                 __stcg(k + q * 32u, make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
     }
-    __device__ __forceinline__ void load(const uint4 *k) {
+    __device__ __forceinline__ void load(const uint4 *k, int32_t g) {
         uint32_t v[4 * kParts];
 #pragma unroll
         for (uint32_t q = 0; q < kParts; ++q) {
@@ -156,33 +171,53 @@ struct LocalLane {
             v[4 * q + 3] = x.w;
         }
 #pragma unroll
-        for (int r = 0; r < R; ++r) Hl[r] = (int32_t)v[r];
+        for (int r = 0; r < R; ++r) {
+            Hl[r] = (int32_t)v[r];
+            Gl[r] = Hl[r] + g;
+        }
         dtop = (int32_t)v[R];
         xout = v[R + 1];
     }
     // The R cells of one column from the row above's word x (H << 2 | code);
     // cm takes the largest H.  PTR appends the two bits of each cell to the
     // accumulators (the last R bits of each are this column's, row 0 highest).
-    template <bool PTR>
-    __device__ __forceinline__ void column(int32_t g, uint32_t x, int32_t &cm) {
+    // TAB: the scores of the lane's last kTabRows rows come from shared memory,
+    // where the rows before them leave the time for it.
+    static constexpr int kTabRows = R >= 8 ? R / 2 : 0;
+    template <bool PTR, bool TAB>
+    __device__ __forceinline__ void column(int32_t g, uint32_t x, int32_t &cm, const int4 *tab) {
         const uint32_t sel = sext_selector(x & 3u);
-        int32_t u = (int32_t)x >> 2, d = dtop;
+        int32_t tv[kTabRows ? kTabRows : 1];
+        if constexpr (TAB) {
+#pragma unroll
+            for (int q = 0; q < kTabRows / 4; ++q) {
+                const int4 v = tab[((x & 3u) * (kTabRows / 4) + q) * 32];
+                tv[4 * q] = v.x;
+                tv[4 * q + 1] = v.y;
+                tv[4 * q + 2] = v.z;
+                tv[4 * q + 3] = v.w;
+            }
+        }
+        int32_t u = (int32_t)x >> 2, d = dtop, ug = u + g;
         dtop = u;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int32_t sv = (int32_t)prmt(prof[r], 0u, sel);
+            const int k = r - (R - kTabRows);
+            const int32_t sv = TAB && k >= 0 ? tv[k >= 0 ? k : 0] : (int32_t)prmt(prof[r], 0u, sel);
             const int32_t l = Hl[r];
-            const int32_t mg = max(u, l) + g;
-            const int32_t w = __viaddmax_s32_relu(d, sv, mg);
             if constexpr (PTR) {
+                const int32_t mg = max(u, l) + g;
                 accL = ptr_append(accL, d + sv - mg);
                 accH = ptr_append(accH, u - l);
-            } else if (r & 1) {
-                cm = __vimax3_s32(cm, u, w);
+                Hl[r] = __viaddmax_s32_relu(d, sv, mg);
+                Gl[r] = Hl[r] + g;
+            } else {
+                Hl[r] = __vimax3_s32_relu(d + sv, ug, Gl[r]);
+                ug = Gl[r] = Hl[r] + g;
+                if (r & 1) cm = __vimax3_s32(cm, u, Hl[r]);
             }
             d = l;
-            Hl[r] = w;
-            u = w;
+            u = Hl[r];
         }
         xout = ((uint32_t)u << 2) | (x & 3u);
     }
@@ -200,9 +235,11 @@ struct LocalAbove {
     }
 };
 
-// The fill.  What bounds it: the logic pipe, 3.5 operations per cell (prmt,
-// max, add-max, half a max3; the add runs on either pipe) and about ten per
-// column of R cells.
+// The fill.  What bounds it: the logic pipe, 2 operations per cell (half a
+// prmt, max3, half a max3; the adds run on either pipe) and about ten per
+// column of R cells, 79% busy; the rest are waits for the stripe above.  4,000
+// pairs of 2 to 10 kb: 10.3 ms; with max, add and add-max per cell (3.5
+// operations) 12.4, with prmt for every row 10.7.
 template <int R, int MODE>
 __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
     constexpr uint32_t SH = 32u * R;
@@ -211,6 +248,9 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
     // a chunk's inputs of lane 0 and outputs of lane 31, per warp
     __shared__ uint32_t ins_[kLocalWarps][32], outs_[kLocalWarps][32];
     uint32_t *ins = ins_[threadIdx.x >> 5], *outs = outs_[threadIdx.x >> 5];
+    constexpr int kTab = 4 * LocalLane<R>::kTabRows / 4 * 32;  // a warp's scores, [base][four rows][lane]
+    __shared__ int4 tabs_[kTab ? kLocalWarps * kTab : 1];
+    int4 *tab = tabs_ + (kTab ? (threadIdx.x >> 5) * kTab + lane : 0);
 
     for (;;) {
         uint32_t jidx = 0;
@@ -237,7 +277,8 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         LocalLane<R> ln;
         const uint32_t i0 = s * SH + (uint32_t)lane * R;
         ln.rows(p, p.pool + tk.a_off, i0, m);
-        ln.start();
+        ln.table(tab);
+        ln.start(p.gap);
         uint4 *keep = MODE == kKeep ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * LocalLane<R>::kParts * 32u + lane
                                     : nullptr;
         int32_t best = 0, cm = 0;    // the lane's largest H before and in this chunk of 32 steps
@@ -273,7 +314,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
                     uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
                     const uint32_t in = ins[uu];
                     if (lane == 0) x = in;
-                    ln.template column<false>(g, x, cm);
+                    ln.template column<false, true>(g, x, cm, tab);
                     if (lane == 31) outs[uu] = ln.xout;
                 }
                 c += 32;
@@ -283,7 +324,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
                     const uint32_t in = ins[uu];
                     if (lane == 0) x = in;
                     if (c >= 0 && c < (int32_t)n) {
-                        ln.template column<false>(g, x, cm);
+                        ln.template column<false, true>(g, x, cm, tab);
                         if (lane == 31) outs[uu] = ln.xout;
                     }
                     ++c;
@@ -345,9 +386,9 @@ struct LocalReplay {
         ln.accL = ln.accH = 0;
         if (t0)
             ln.load(p.keep + tk.keep_off +
-                    ((uint64_t)s * tk.keep_n + (t0 / kTileSteps - 1)) * LocalLane<R>::kParts * 32u + lane);
+                    ((uint64_t)s * tk.keep_n + (t0 / kTileSteps - 1)) * LocalLane<R>::kParts * 32u + lane, p.gap);
         else
-            ln.start();
+            ln.start(p.gap);
     }
     // one step; whether the lane had a column
     template <bool PTR>
@@ -361,7 +402,7 @@ struct LocalReplay {
         if (lane == 0) x = x0;
         const bool act = t >= lane && t - lane < above.n;
         int32_t cm = 0;
-        if (act) ln.template column<PTR>(g, x, cm);
+        if (act) ln.template column<PTR, false>(g, x, cm, nullptr);
         ++t;
         return act;
     }
