@@ -612,23 +612,6 @@ __global__ void k_bits_peaks(BitsWalkArgs p) {
     }
 }
 
-// n bytes by a warp, both sides at any alignment.
-__device__ __forceinline__ void copy_moves(uint8_t *dst, const uint8_t *src, uint32_t n, uint32_t lane) {
-    const uint32_t head = min(n, (uint32_t)(-(intptr_t)dst & 3));
-    if (lane < head) dst[lane] = src[lane];
-    dst += head;
-    src += head;
-    n -= head;
-    const uint32_t sh = (uint32_t)((uintptr_t)src & 3);
-    const uint32_t *s = reinterpret_cast<const uint32_t *>(src - sh);
-    uint32_t *d = reinterpret_cast<uint32_t *>(dst);
-    const uint32_t words = n / 4;
-#pragma unroll 4
-    for (uint32_t q = lane; q < words; q += 32) d[q] = sh ? __funnelshift_r(s[q], s[q + 1], 8 * sh) : s[q];
-    const uint32_t done = 4 * words;
-    if (lane < n - done) dst[done + lane] = src[done + lane];
-}
-
 // A pair's moves from its stretches: each from the cell where the way from the
 // one before joined it.  One warp per pair.
 __global__ void k_bits_link(BitsWalkArgs p) {
@@ -647,7 +630,7 @@ __global__ void k_bits_link(BitsWalkArgs p) {
             const BitsWalkEnd e = p.ends[w];
             l.w = kNoStretch;
             if (e.i < 0) break;
-            copy_moves(dst + l.moves, p.own + wk.moves_off + l.from, e.k - l.from, lane);
+            copy_bytes(dst + l.moves, p.own + wk.moves_off + l.from, e.k - l.from, lane, 32);
             l.moves += e.k - l.from;
             l.i = e.i;
             l.j = e.j;
@@ -657,7 +640,7 @@ __global__ void k_bits_link(BitsWalkArgs p) {
             }
             const BitsWalkEnd x = p.joints[w];
             if (x.i < 0) break;
-            copy_moves(dst + l.moves, p.own + wk.joint_off, x.k, lane);
+            copy_bytes(dst + l.moves, p.own + wk.joint_off, x.k, lane, 32);
             l.moves += x.k;
             l.i = x.i;
             l.j = x.j;

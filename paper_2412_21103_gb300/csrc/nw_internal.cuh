@@ -154,6 +154,24 @@ __device__ __forceinline__ uint32_t even_bits(uint64_t x) {
     return (uint32_t)x;
 }
 
+// n bytes by `threads` threads, both sides at any alignment; reads up to 7 bytes
+// past the source.
+__device__ __forceinline__ void copy_bytes(uint8_t *dst, const uint8_t *src, uint32_t n, uint32_t rank, uint32_t threads) {
+    const uint32_t head = min(n, (uint32_t)(-(intptr_t)dst & 3));
+    if (rank < head) dst[rank] = src[rank];
+    dst += head;
+    src += head;
+    n -= head;
+    const uint32_t sh = (uint32_t)((uintptr_t)src & 3);
+    const uint32_t *s = reinterpret_cast<const uint32_t *>(src - sh);
+    uint32_t *d = reinterpret_cast<uint32_t *>(dst);
+    const uint32_t words = n / 4;
+#pragma unroll 4
+    for (uint32_t q = rank; q < words; q += threads) d[q] = sh ? __funnelshift_r(s[q], s[q + 1], 8 * sh) : s[q];
+    const uint32_t done = 4 * words;
+    if (rank < n - done) dst[done + rank] = src[done + rank];
+}
+
 // Scoring handed to kernels: prof[c] is the row profile of a query base c,
 // byte d of prof[c] = s'(c, d) as int8.
 struct Profile {
