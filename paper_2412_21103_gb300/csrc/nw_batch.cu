@@ -233,6 +233,27 @@ static PairCost single_pair_cost(uint32_t m, uint32_t n, const nw_scoring &sc) {
     return PairCost{(double)m * n / kPairRate + kPairFixed, 0.0};
 }
 
+// Whether a score batch runs on the bit planes, one pair per lane.  A scoring
+// that fits them as it is always does (its long pairs leave for the single-pair
+// kernel, see pick_stragglers).  One that fits them in units of a common divisor
+// has no such kernel, so it does where the longest pair's time on its lane (a
+// step of 128 rows is about 86 operations, 2.2 cycles each) is within what the
+// scalar kernel takes: 40 pairs of 400 to 3,000 bases 8.4 ms against 2.1.
+static bool bits_scores_pay(nw_ctx *ctx, const std::vector<BatchTask> &tasks, const nw_scoring &sc) {
+    if (bits_scoring_ok(sc)) return true;
+    if (!bits_batch_ok(sc)) return false;
+    double longest = 0, total = 0, cells = 0, most = 0;
+    for (const BatchTask &t : tasks) {
+        const double r = std::min(t.m, t.n), c = std::max(t.m, t.n), secs = (r / 128.0 + 1.0) * (c + 128.0) * 86.0 * 2.2 / 2.0e9;
+        const double padded = std::ceil(r / 128.0) * 128.0 * (std::max(c, (double)kMinPeriod) + 31.0);
+        longest = std::max(longest, secs);
+        total += secs;
+        cells += padded;
+        most = std::max(most, padded);
+    }
+    return std::max(longest, total / 32.0 / (4.0 * ctx->sm_count)) <= std::max(cells / kBatchRate, most / kWarpRate);
+}
+
 // warp_cells[k]: cells pair k costs on one warp (scaled for slower
 // kernels), full_cells[k]: its full grid, costs[k] (or, when empty,
 // full_cells[k] / kPairRate + kPairFixed on the scalar kernel): its cost on
@@ -954,6 +975,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     // alignments whose scoring fits two bit planes run on groups of lanes of
     // the bit-sliced kernel, the others on the scalar batch kernel
     const bool groups = want && bits_batch_ok(sc) && !getenv("NW_PAIR_SCALAR");
+    const bool score_bits = !want && bits_scores_pay(ctx, tasks, sc);
     // pairs that would leave the GPU idle on one warp take the single-pair
     // kernel, and so do pairs whose pointer matrix alone exceeds half the
     // remaining budget (the single-pair path recomputes from checkpoints)
@@ -969,7 +991,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
         }
         // alignments on the bit-sliced groups: a pair's time on its warp,
         // against the GPU's 4 x 152 schedulers
-        double rate = !want && bits_batch_ok(sc) ? kBitsBatchRate : kBatchRate;
+        double rate = score_bits ? kBitsBatchRate : kBatchRate;
         if (groups) {
             rate = kWarpRate * 4.0 * ctx->sm_count;
             total = longest = 0;
@@ -1023,7 +1045,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     if (!want || ctx->autotune) {
         // score-only: the bit-sliced kernel (rows per lane 32) where the
         // scoring fits two bit planes
-        const bool bits = !want && bits_batch_ok(sc);
+        const bool bits = score_bits;
         const uint32_t cap = score_slots(tasks.data(), npairs);
         BitsPlan bp;
         if (bits && (rc = bits_prepare(ctx, pool, tasks, sc, scores, cap, pre, &bp))) return rc;

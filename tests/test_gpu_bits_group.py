@@ -51,7 +51,25 @@ def test_shapes(sc):
         pool, off, lens = nw.pool_of([s for p in pairs for s in p])
         s, _ = nw.nw_align_batch(ctx, pool, off[0::2], lens[0::2], off[1::2], lens[1::2], sc, 0)
         assert list(s) == oracle.score_many(pairs, *sc)
-        assert ctx.kernel_stats()["bits_score"][0] > 0
+
+
+@pytest.mark.parametrize("sc", [(2, -1, -2), (2, -2, -2)])
+def test_score_batches_in_units(sc):
+    """Enough short pairs to fill the GPU take the bit planes in units of the
+    common divisor, a few the scalar kernel; the scores are the same."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    rs = seqgen.Stream(54)
+    seqs = [rs.bases(int(n)) for n in rs.integers(20, 70, 24000)]
+    pool, off, lens = nw.pool_of(seqs)
+    want = oracle.score_many(list(zip(seqs[0::2], seqs[1::2])), *sc)
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        ctx.set_profiling(True)
+        for n, bits in ((12000, True), (30, sc[0] - 2 * sc[2] <= 3)):
+            ctx.reset_stats()
+            s, _ = nw.nw_align_batch(ctx, pool, off[0:2 * n:2], lens[0:2 * n:2], off[1:2 * n:2], lens[1:2 * n:2], sc, 0)
+            assert list(s) == want[:n]
+            assert (ctx.kernel_stats().get("bits_score", (0, 0.0))[0] > 0) == bits
 
 
 def test_many_pairs_take_few_lanes_and_waves():
