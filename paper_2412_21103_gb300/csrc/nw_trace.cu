@@ -127,8 +127,10 @@ constexpr uint32_t kWalkDone = 0, kWalkJoined = 1, kWalkFull = 2, kWalkBand = 3,
 constexpr int kWalkWarps = 4;
 constexpr int kRunWarps = 4;               // warps per CTA of the walk by runs
 // Bit-sliced records: pairs up to this many moves walk from their end by runs,
-// about 0.4 us per 31 rows; longer ones in linked pieces, 120-250 us each.
-constexpr uint64_t kRunMaxMoves = 16384;
+// about 0.4 us per 31 rows; longer ones in linked pieces, 120-250 us each.  A
+// lone pair of 8 kb takes .79 ms in all by runs and .67 in pieces, one of 4 kb
+// about .40 either way.
+constexpr uint64_t kRunMaxMoves = 16384, kRunMaxMovesOne = 8192;
 constexpr uint32_t kParMinStripes = 3;     // shorter pairs walk sequentially,
 constexpr uint64_t kParMinMoves = 8192;    // and so do pairs of a batch with m + n below this (the
                                            // other pairs' walks keep the GPU busy, and the
@@ -937,7 +939,8 @@ int launch_trace_bits(nw_ctx *ctx, const TraceTask *host, const TraceTask *dev, 
     if (ntasks == 0) return NW_OK;
     // the long pairs lead
     uint32_t nlong = 0;
-    while (nlong < ntasks && (uint64_t)host[nlong].m + host[nlong].n > kRunMaxMoves) ++nlong;
+    const uint64_t most = ntasks == 1 ? kRunMaxMovesOne : kRunMaxMoves;
+    while (nlong < ntasks && (uint64_t)host[nlong].m + host[nlong].n > most) ++nlong;
     if (nlong) {
         const int rc = launch_walks<BitsLayout<kBitsWalkGroup>>(ctx, host, dev, nlong);
         if (rc) return rc;
