@@ -51,12 +51,12 @@ W_OPS_PER_CELL = 3           # what the W-domain kernels issue for it: prmt + ad
 PEAK_KINDS = (0, 2, 4)       # nw_peak_int kinds: DPX add-max, max, prmt (lane-ops/s each)
 CELL_KINDS = (5, 6, 7)       # nw_peak_int kinds: score-only cells in three instruction mixes (cells/s)
 # The bit-sliced kernels (bits_score, bband_*) update 32 cells of an anti-diagonal
-# with whole-word operations.  Their algorithmic work per 32 cells: 14 logic
-# ops of the difference update (match word 2, T = max(s', a, b) 6, dV 3, dH 3)
-# and 2 funnel shifts that bring the upper neighbour's difference into line;
-# the pointer planes add 2 (L, Hb).
-BITS_OPS_PER_32 = 16
-BITS_PTR_OPS_PER_32 = 18
+# with whole-word operations.  Their algorithmic work per 32 cells: 10 logic
+# operations (match word 2, the two differences 8); the single-pair kernel, a
+# word per lane, adds 2 funnel shifts that bring the upper neighbour's difference
+# into line and 2 for its pointer planes (L, Hb).
+BITS_OPS_PER_32 = 10
+BITS_PAIR_OPS_PER_32 = 14
 BITS_PEAK_KINDS = (8, 10)    # nw_peak_int kinds: 3-input logic op, funnel shift (lane-ops/s)
 BITS_CELL_KIND = 11          # nw_peak_int kind: one bit-sliced step, 32 cells (cells/s)
 BITS_KERNELS = ("bits_score", "bband_fill_ptr", "bband_score", "bpair_fill_ptr")
@@ -65,8 +65,7 @@ BITS_KERNELS = ("bits_score", "bband_fill_ptr", "bband_score", "bpair_fill_ptr")
 # time is the wavefront's chain of m + n + m/31 steps, each 24 logic ops of
 # one warp (the 16-lane logic pipe of one scheduler: 2 cycles each).
 PAIR_ROWS = 31
-PAIR_ALU_OPS_PER_STEP = 24
-HBM_PEAK_FALLBACK = 6800.0   # GB/s, when MEASURED_PEAKS.json is absent
+PAIR_ALU_OPS_PER_STEP = 18
 STEPS_DEFAULT = {"pair32k": 100, "pair1k": 200, "allpairs": 20, "centerstar": 20, "local": 10, "affine": 10, "band": 3}
 
 
@@ -937,7 +936,8 @@ def run_ours(args):
                      "unit": "Gop/s", "frac": (achieved / peak_ops) if achieved else None,
                      "traffic": dram_traffic(work.dominant, args.workload),
                      "traffic_note": "DRAM bytes per launch (ncu, profiles/dram_traffic.json); "
-                                     "algorithmic: 0.25 B/cell of pointers for *_ptr kernels, ~0 for score-only",
+                                     "algorithmic: 0.25 B/cell of pointers for batch_fill_ptr, kept states of about "
+                                     "0.1 B/cell for local_fill_ptr and affine_fill_ptr, ~0 for score-only",
                      "ops_per_cell": OPS_PER_CELL, "kernel_ms": dom_avg_ms, "cells_per_launch": kcells,
                      "peak_source": "measured live: slowest of nw_peak_int kinds 0/2/4 (DPX add-max, max, prmt; "
                                     "independent chains on every SM)",
@@ -1001,29 +1001,18 @@ def pair_chain(m, n, kernel_ms, sm_mhz):
     return out
 
 
-def measured_hbm_gbs():
-    """The driver's measured copy bandwidth (GB/s) and where it came from."""
-    try:
-        v = float(json.load(open(os.path.join(HERE, "MEASURED_PEAKS.json")))["hbm_gbs"])
-        return v, "MEASURED_PEAKS.json hbm_gbs (STREAM-style copy, measured on this pool's GB300)"
-    except (OSError, KeyError, ValueError):
-        return HBM_PEAK_FALLBACK, "fallback 6.8 TB/s (no MEASURED_PEAKS.json)"
-
-
 def bits_roofline(kernel, workload, cells, kernel_ms, bits_peak, bits_cell_peak, scalar_peak):
-    """Roofline of a bit-sliced kernel.  Score-only (bits_score): bound by the
-    ALU issue of its word operations, 16 per 32 cells, against the slowest of
-    the measured LOP3 / funnel-shift rates.  With pointers (bband_fill_ptr): it
-    also writes 0.25 B per window cell, so the line reports the HBM side as
-    the bound (pointer bytes per launch over the kernel's time against the
-    measured copy bandwidth) with the ALU side beside it."""
+    """Roofline of a bit-sliced kernel: bound by the ALU issue of its word
+    operations, 10 per 32 cells (the single-pair kernel: 14), against the
+    slowest of the measured LOP3 / funnel-shift rates.  The banded fill keeps
+    its planes every 64 anti-diagonals, 1/128 B per window cell."""
     if not kernel_ms or not cells:
         return {"bound": "alu", "kernel": kernel, "achieved": None, "peak": bits_peak, "unit": "Gop/s",
                 "frac": None, "traffic": dram_traffic(kernel, workload)}
     sec = kernel_ms * 1e-3
-    ptr = kernel in ("bband_fill_ptr", "bpair_fill_ptr")
-    ops32 = BITS_PTR_OPS_PER_32 if ptr else BITS_OPS_PER_32
-    rows = PAIR_ROWS if kernel == "bpair_fill_ptr" else 32  # grid cells per word step
+    pair = kernel == "bpair_fill_ptr"
+    ops32 = BITS_PAIR_OPS_PER_32 if pair else BITS_OPS_PER_32
+    rows = PAIR_ROWS if pair else 32  # grid cells per word step
     alu_achieved = cells * ops32 / rows / sec / 1e9
     gcups = cells / sec / 1e9
     alu = {"bound": "alu", "achieved": alu_achieved, "peak": bits_peak, "unit": "Gop/s",
@@ -1039,18 +1028,9 @@ def bits_roofline(kernel, workload, cells, kernel_ms, bits_peak, bits_cell_peak,
                       "word op here updates a bit of 32 cells"}
     base = {"kernel": kernel, "kernel_ms": kernel_ms, "cells_per_launch": cells,
             "traffic": dram_traffic(kernel, workload),
-            "traffic_note": "DRAM bytes per launch (ncu, profiles/dram_traffic.json); algorithmic: 0.25 B per "
-                            "window cell of pointers for bband_fill_ptr, ~0 for score-only"}
-    if not ptr:
-        return {**alu, **base, "cell_peak": cell, "scalar_unit": scalar}
-    if kernel == "bpair_fill_ptr":
-        return {**alu, **base, "cell_peak": cell, "scalar_unit": scalar}
-    hbm, src = measured_hbm_gbs()
-    bytes_ = cells * 0.25
-    achieved = bytes_ / sec / 1e9
-    return {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-            "bytes_per_launch": bytes_, "peak_source": src, **base, "alu": alu, "cell_peak": cell,
-            "scalar_unit": scalar}
+            "traffic_note": "DRAM bytes per launch (ncu, profiles/dram_traffic.json); algorithmic: 1/128 B per "
+                            "window cell of kept planes for bband_fill_ptr, ~0 for score-only"}
+    return {**alu, **base, "cell_peak": cell, "scalar_unit": scalar}
 
 
 class _Null:

@@ -323,8 +323,8 @@ int nw_local_align_batch(nw_ctx *ctx, const uint8_t *pool2b, const uint64_t *a_o
  * strictly better than opening (a tie closes the gap); on row 0 / column 0
  * only horizontal / vertical moves remain.  With gap_open = 0 the result
  * equals nw_align_batch with gap = gap_extend, move for move.  Memory and
- * arguments as nw_align_batch (NW_HOST_IO, NW_CIGAR, NW_CIGAR_M; pointer
- * words take 0.5 byte per cell).  Scores in [-40, 40], both gap scores <=
+ * arguments as nw_align_batch (NW_HOST_IO, NW_CIGAR, NW_CIGAR_M; kept
+ * rows and states take about 0.11 byte per cell).  Scores in [-40, 40], both gap scores <=
  * 0, mismatch <= match, max(match - 2*gap_extend, 0) * min(m,n) below 2^29;
  * a pair whose one-warp sweep would exceed 2^31 stripe steps is
  * NW_ERR_UNSUPPORTED. */

@@ -255,7 +255,7 @@ struct BandBitsShape {
     uint32_t words = 1;  // the band needs this many 32-row words (g * Q >= words)
 };
 // One banded pair of a round: pool offsets, sizes, score slot, window, and
-// its first kept planes (16 bytes per word, every 128 anti-diagonals).
+// its first kept planes (16 bytes per word, every 64 anti-diagonals).
 struct BandBitsItem {
     uint64_t a_off, b_off, ptr_off;  // pool byte offsets (the CIGARs), first kept planes
     int64_t a_slot, b_slot;          // the sequences' planar slots (the fill and the walk)
