@@ -13,8 +13,9 @@
 //     F'(i,j) = max(F'(i-1,j), W(i-1,j) + go)
 //     W(i,j)  = max(W(i-1,j-1) + s - 2*ge, E'(i,j), F'(i,j))
 // with W(0,0) = 0, W(0,j) = W(i,0) = go, F'(0,j) = E'(i,0) = -inf and
-// H(m,n) = W(m,n) + ge*(m+n).  A cell is one byte permute (s - 2ge), two DPX
-// add-max (E', F'), an add and a three-input max (W).
+// H(m,n) = W(m,n) + ge*(m+n).  A cell is a score (s - 2ge: from shared
+// memory, or a byte permute), two DPX add-max (E', F'), an add and a three-input
+// max (W).
 //
 // Alignments.  The fill writes no pointers: it keeps every stripe's bottom
 // row (which the next stripe reads anyway) and, every kTileSteps steps, the
@@ -169,14 +170,40 @@ struct AffLane {
     // The R cells of one column from the row above's word x (W << 2 | code)
     // and F' fx; PTR appends the four bits of each cell to the accumulators
     // (the last R bits of each are this column's, row 0 highest).
-    template <bool PTR>
-    __device__ __forceinline__ void column(int32_t go, uint32_t x, int32_t fx) {
+    // TAB: the scores of the lane's last kTabRows rows come from shared memory by
+    // the column's base, four to a load, not by a byte permute each.
+    static constexpr int kTabRows = R >= 8 ? 8 : 0;
+    // the lane's table: kTabRows scores for each base of B
+    __device__ __forceinline__ void table(int4 *tab) const {
+#pragma unroll
+        for (uint32_t b = 0; b < 4; ++b)
+#pragma unroll
+            for (int q = 0; q < kTabRows / 4; ++q) {
+                const uint32_t *pr = prof + (R - kTabRows) + 4 * q, sel = sext_selector(b);
+                tab[(b * (kTabRows / 4) + q) * 32] = make_int4((int32_t)prmt(pr[0], 0u, sel), (int32_t)prmt(pr[1], 0u, sel),
+                                                               (int32_t)prmt(pr[2], 0u, sel), (int32_t)prmt(pr[3], 0u, sel));
+            }
+    }
+    template <bool PTR, bool TAB>
+    __device__ __forceinline__ void column(int32_t go, uint32_t x, int32_t fx, const int4 *tab) {
         const uint32_t sel = sext_selector(x & 3u);
+        int32_t tv[kTabRows ? kTabRows : 1];
+        if constexpr (TAB) {
+#pragma unroll
+            for (int q = 0; q < kTabRows / 4; ++q) {
+                const int4 v = tab[((x & 3u) * (kTabRows / 4) + q) * 32];
+                tv[4 * q] = v.x;
+                tv[4 * q + 1] = v.y;
+                tv[4 * q + 2] = v.z;
+                tv[4 * q + 3] = v.w;
+            }
+        }
         int32_t u = (int32_t)x >> 2, d = dtop, fu = fx;
         dtop = u;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int32_t sv = (int32_t)prmt(prof[r], 0u, sel);
+            const int k = r - (R - kTabRows);
+            const int32_t sv = TAB && k >= 0 ? tv[k >= 0 ? k : 0] : (int32_t)prmt(prof[r], 0u, sel);
             const int32_t e = __viaddmax_s32(Wl[r], go, El[r]);
             const int32_t f = __viaddmax_s32(u, go, fu);
             const int32_t w = __vimax3_s32(d + sv, e, f);
@@ -216,9 +243,10 @@ struct AffAbove {
 };
 
 // The fill; KEEP: also the stripes' states every kTileSteps steps (for the
-// trace).  What bounds it: the logic pipe, 4 operations per cell (prmt, two
-// add-max, max3; the add runs on either pipe) and about 12 per column of R
-// cells.
+// trace).  What bounds it: the logic pipe, 3 operations per cell (two add-max,
+// max3; the add runs on either pipe) and about 12 per column of R cells.
+// 2,000 pairs of 1 to 5 kb: 5.2 ms; with a prmt for every row 5.9, for half of
+// them 5.55.
 template <int R, bool KEEP>
 __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
     constexpr uint32_t SH = 32u * R;
@@ -227,6 +255,9 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
     // a chunk's inputs of lane 0 and outputs of lane 31, per warp
     __shared__ uint2 ins_[kAffWarps][32], outs_[kAffWarps][32];
     uint2 *ins = ins_[threadIdx.x >> 5], *outs = outs_[threadIdx.x >> 5];
+    constexpr int kTab = 4 * AffLane<R>::kTabRows / 4 * 32;  // a warp's scores, [base][four rows][lane]
+    __shared__ int4 tabs_[kTab ? kAffWarps * kTab : 1];
+    int4 *tab = tabs_ + (kTab ? (threadIdx.x >> 5) * kTab + lane : 0);
 
     for (;;) {
         uint32_t jidx = 0;
@@ -255,6 +286,7 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
         AffLane<R> ln;
         const uint32_t i0 = s * SH + (uint32_t)lane * R;   // rows i0+1 .. i0+R (1-based)
         ln.rows(p, p.pool + tk.a_off, i0, m);
+        ln.table(tab);
         ln.start(go, i0);
         uint4 *keep = KEEP ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * AffLane<R>::kParts * 32u + lane : nullptr;
         int32_t c = -lane;
@@ -298,7 +330,7 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
                         x = in.x;
                         fx = (int32_t)in.y;
                     }
-                    ln.template column<false>(go, x, fx);
+                    ln.template column<false, true>(go, x, fx, tab);
                     if (lane == 31) outs[uu] = make_uint2(ln.xout, (uint32_t)ln.fout);
                 }
                 c += 32;
@@ -312,7 +344,7 @@ __global__ void __launch_bounds__(kAffWarps * 32) k_affine(AffArgs p) {
                         fx = (int32_t)in.y;
                     }
                     if (c >= 0 && c < (int32_t)n) {
-                        ln.template column<false>(go, x, fx);
+                        ln.template column<false, true>(go, x, fx, tab);
                         if (lane == 31) outs[uu] = make_uint2(ln.xout, (uint32_t)ln.fout);
                         if (s + 1 == S && (uint32_t)lane == lM && c == (int32_t)n - 1) {
                             int32_t wmn = 0;
@@ -435,7 +467,7 @@ __global__ void __launch_bounds__(32 * kTraceWarps) k_affine_trace(AffArgs p, ui
                         fx = f0;
                     }
                     if (t >= lane && t - lane < n) {
-                        ln.template column<true>(go, x, fx);
+                        ln.template column<true, false>(go, x, fx, nullptr);
                         tile[(t - tw) * 32u + lane] = Bits::pack(ln.accL, ln.accH, ln.accF, ln.accE);
                     }
                 }

@@ -181,9 +181,9 @@ struct LocalLane {
     // The R cells of one column from the row above's word x (H << 2 | code);
     // cm takes the largest H.  PTR appends the two bits of each cell to the
     // accumulators (the last R bits of each are this column's, row 0 highest).
-    // TAB: the scores of the lane's last kTabRows rows come from shared memory,
-    // where the rows before them leave the time for it.
-    static constexpr int kTabRows = R >= 8 ? R / 2 : 0;
+    // TAB: the scores of the lane's last kTabRows rows come from shared memory by
+    // the column's base, four to a load, not by a byte permute each.
+    static constexpr int kTabRows = R >= 8 ? 8 : 0;
     template <bool PTR, bool TAB>
     __device__ __forceinline__ void column(int32_t g, uint32_t x, int32_t &cm, const int4 *tab) {
         const uint32_t sel = sext_selector(x & 3u);
@@ -235,11 +235,11 @@ struct LocalAbove {
     }
 };
 
-// The fill.  What bounds it: the logic pipe, 2 operations per cell (half a
-// prmt, max3, half a max3; the adds run on either pipe) and about ten per
-// column of R cells, 79% busy; the rest are waits for the stripe above.  4,000
-// pairs of 2 to 10 kb: 10.3 ms; with max, add and add-max per cell (3.5
-// operations) 12.4, with prmt for every row 10.7.
+// The fill.  What bounds it: the logic pipe, 1.5 operations per cell (max3,
+// half a max3; the adds run on either pipe) and about ten per column of R
+// cells, and waits for the stripe above.  4,000 pairs of 2 to 10 kb: 9.8 ms;
+// with max, add and add-max per cell (3.5 operations) 12.4, with a prmt for
+// every row 10.7, for half of them 10.3.
 template <int R, int MODE>
 __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
     constexpr uint32_t SH = 32u * R;
