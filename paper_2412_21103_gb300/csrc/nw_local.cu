@@ -722,6 +722,12 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         }
         if ((e0 = cudaMemsetAsync(pv, 0, jobs.size() * 4, ctx->stream)) != cudaSuccess)
             return cuda_fail(ctx, e0, "local progress reset");
+        // A fill that gives up (a wait's limit, or an error that the context
+        // holds from an earlier call) leaves jobs undone.  Their best reads 0,
+        // so the trace starts only from stripes that were finished -- and then
+        // every stripe above them was: a stripe reads all of the one above.
+        if (mode != kScore && (e0 = cudaMemsetAsync(bv, 0, jobs.size() * sizeof(LocalBest), ctx->stream)) != cudaSuccess)
+            return cuda_fail(ctx, e0, "local best reset");
         LocalTask *dt = nullptr;
         LocalJob *dj = nullptr;
         uint64_t *dmoff = nullptr;
