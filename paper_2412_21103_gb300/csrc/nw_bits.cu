@@ -54,6 +54,7 @@
 #include <vector>
 
 #include "nw_bits.cuh"
+#include "nw_bits_shape.h"
 #include "nw_order.h"
 
 namespace nw {
@@ -183,7 +184,8 @@ __device__ __forceinline__ int32_t bits_pairs_of(const BitsArgs &p, const BitsJo
     int32_t W = 0;
     uint32_t stripe = 0, cl = 0;   // of the stripe's row 0
     uint32_t started = 0, lift = 0;  // chunks since a stripe began; all ones once it is not the first
-    for (uint32_t c = 0; c < job.T; ++c) {
+    const uint64_t last = bits_last_row(S, C, K);
+    for (uint64_t c = 0; c < job.T; ++c) {
         if (cl == 0 && stripe < S) {
             started = 0;
             lift = stripe ? ~0u : 0u;
@@ -217,9 +219,9 @@ __device__ __forceinline__ int32_t bits_pairs_of(const BitsArgs &p, const BitsJo
         }
         ++started;
         // outgoing bits: bit b is column 32 (c - K + 1) - b of the bottom row, from the stripe's first chunk on
-        if (S > 1 && c < (S - 1) * C + K) __stcg(rows + (size_t)cl * 32u, make_uint2(Q0, Q1));
-        const int32_t e = 32 * ((int32_t)c - (int32_t)((S - 1) * C) - K + 1);
-        const int32_t lo = max(e + 1 - (int32_t)n, 0), hi = min(31, e);
+        if (S > 1 && c <= last) __stcg(rows + (size_t)cl * 32u, make_uint2(Q0, Q1));
+        int32_t lo, hi;
+        bits_last_row_span(c, last, n, lo, hi);
         if (lo <= hi) {
             const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
             W += __popc(Q0 & mk) + 2 * __popc(Q1 & mk);
@@ -436,15 +438,6 @@ bool bits_batch_ok(const nw_scoring &sc) {
     return u.sx >= 0 && u.sx <= u.sm && u.sm <= 3;
 }
 
-// How a pair of m rows runs: K words a lane, S stripes, and the operations of
-// a step.
-struct BitsShape {
-    uint32_t K, S, ops;
-    uint32_t period(uint32_t n) const { return S > 1 ? std::max((n + 31) / 32, K + 3) : (n + 31) / 32; }
-    uint32_t chunks(uint32_t n) const { return (S - 1) * period(n) + (n + 32 * K + 30) / 32; }
-    uint64_t work(uint32_t n) const { return (uint64_t)ops * chunks(n); }
-};
-
 // The K with the least work at as many columns as rows, by the rows' words (a
 // pair's columns are mostly as many or more): more words take fewer shifts a
 // word, but pad the rows to 32*K and want a period of K + 3 chunks for the row
@@ -483,7 +476,7 @@ class BitsShapes {
 
 // A job of pairs of at most n columns.
 static BitsJob job_of(const BitsShape &s, uint32_t n, uint32_t t0, uint32_t cnt, uint32_t cls) {
-    return BitsJob{t0, cnt, s.S, s.S ? s.period(n) : 0u, s.S ? s.chunks(n) : 0u, s.K, cls};
+    return BitsJob{s.S ? s.chunks(n) : 0u, t0, cnt, s.S, s.S ? s.period(n) : 0u, s.K, cls};
 }
 
 // The launch's tables in one upload, its constants, grid and row buffers.
@@ -494,7 +487,7 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
     int rc;
     // longest jobs first, ties in job order
     std::vector<uint64_t> keys(jobs.size());
-    for (size_t q = 0; q < jobs.size(); ++q) keys[q] = (uint64_t)jobs[q].T * (10 * jobs[q].K + 6);
+    for (size_t q = 0; q < jobs.size(); ++q) keys[q] = jobs[q].T * (10 * jobs[q].K + 6);
     const std::vector<uint32_t> jo = radix_order_desc(std::move(keys));
     const size_t jobs_at = (head.size() + 15) / 16 * 16;
     head.resize(jobs_at + jobs.size() * sizeof(BitsJob));

@@ -100,8 +100,9 @@ struct BitsClass {
 };
 
 struct BitsJob {
+    uint64_t T;        // chunks in all (of the job's widest pair)
     uint32_t t0, cnt;  // tasks (or pairs of the class) [t0, t0 + cnt), cnt <= 32, one per lane
-    uint32_t S, C, T;  // stripes, chunks from one to the next, chunks in all (of the job's widest pair)
+    uint32_t S, C;     // stripes, chunks from one to the next
     uint32_t K;        // words a lane
     uint32_t cls;      // all-vs-all: the class
 };

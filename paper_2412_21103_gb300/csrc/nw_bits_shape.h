@@ -1,0 +1,44 @@
+// Shapes and counts of the bit-sliced score kernel (nw_bits.cu): plain
+// arithmetic, for the host plan and the kernel alike.
+#pragma once
+
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define NW_HOST_DEVICE __host__ __device__ __forceinline__
+#else
+#define NW_HOST_DEVICE inline
+#endif
+
+namespace nw {
+
+// How a pair of m rows runs: K words a lane, S stripes, and the operations of
+// a step.  Chunks in all are counted in 64 bits: two sequences of 2^30 bases
+// have 2^23 stripes of 2^25 chunks.
+struct BitsShape {
+    uint32_t K, S, ops;
+    uint32_t period(uint32_t n) const {
+        const uint32_t words = (n + 31) / 32;
+        return S > 1 && words < K + 3 ? K + 3 : words;
+    }
+    uint64_t chunks(uint32_t n) const { return (uint64_t)(S - 1) * period(n) + (n + 32 * K + 30) / 32; }
+    uint64_t work(uint32_t n) const { return ops * chunks(n); }
+};
+
+// The chunk from which on the last stripe's bottom row leaves: its bit 0 is
+// column 0 there, and column 32 d - b is bit b of the d-th chunk after it.
+NW_HOST_DEVICE uint64_t bits_last_row(uint32_t S, uint32_t C, uint32_t K) { return (uint64_t)(S - 1) * C + K - 1; }
+
+// The bits [lo, hi] of chunk c that are columns 0 .. n-1 of that row (lo > hi:
+// none).  Chunks of earlier stripes hold none: the difference is formed only
+// from `last` on, where it is small.
+NW_HOST_DEVICE void bits_last_row_span(uint64_t c, uint64_t last, uint32_t n, int32_t &lo, int32_t &hi) {
+    lo = 1;
+    hi = 0;
+    if (c < last) return;
+    const int32_t e = (int32_t)(32 * (c - last));
+    lo = e + 1 > (int32_t)n ? e + 1 - (int32_t)n : 0;
+    hi = e < 31 ? e : 31;
+}
+
+}  // namespace nw
