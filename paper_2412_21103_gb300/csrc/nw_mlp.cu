@@ -527,7 +527,8 @@ constexpr size_t feature_bytes(uint32_t n) { return (size_t)(n + 31) / 32 * size
 
 static int launch_features(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const uint32_t *a_len,
                            const uint64_t *b_off, const uint32_t *b_len, uint32_t npairs, uint32_t maxn, float *feat) {
-    if (feature_bytes(maxn) > 48 * 1024) {
+    // (the default limit counts the kernel's static words too)
+    if (feature_bytes(maxn) + kBins * sizeof(uint32_t) > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_features, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)feature_bytes(kFeatMaxB));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "feature kernel shared memory");
