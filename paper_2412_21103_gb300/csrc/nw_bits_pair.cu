@@ -651,6 +651,11 @@ int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &job
                                     nullptr, nullptr, 32});
             moff += (uint64_t)j.m + j.n + 16;
         }
+        // by moves, as the walks want them: the wave's order (by chain) puts a
+        // tall pair before a wide one of more moves
+        std::stable_sort(tts.begin(), tts.end(), [](const TraceTask &x, const TraceTask &y) {
+            return (uint64_t)x.m + x.n > (uint64_t)y.m + y.n;
+        });
         if (tts.size() > 1) {
             if ((rc = scratch(ctx, "bpair_tt", tts.size() * sizeof(TraceTask), &dt))) return rc;
             cudaError_t e = cudaMemcpyAsync(dt, tts.data(), tts.size() * sizeof(TraceTask), cudaMemcpyHostToDevice,
