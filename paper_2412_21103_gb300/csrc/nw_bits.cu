@@ -538,10 +538,12 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
     return NW_OK;
 }
 
-int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> &tasks, const nw_scoring &sc,
-                 int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan) {
+// bits_prepare with the distinct sequences' slots (`shared`) or with one for each
+// of a task's sequences where that is the cheaper plan; *own: which it took.
+static int bits_prepare_slots(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> &tasks, const nw_scoring &sc,
+                              int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan, bool shared,
+                              bool *own_out) {
     *plan = BitsPlan{};
-    if (tasks.empty()) return NW_OK;
     HostTimer ht(ctx, "bits_plan");
     // rows: the orientation with less work (the score is symmetric); order:
     // equal shapes, widest first
@@ -570,8 +572,14 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> 
     // Planar copies: a slot for each of a task's sequences, unless the tasks
     // read their sequences several times over (then the distinct sequences,
     // found by hashing, which costs the host more than the device saves
-    // otherwise: 20,000 pairs of distinct reads, 1 ms).
-    const bool own = bytes <= 2 * extent;
+    // otherwise: 20,000 pairs of distinct reads, 1 ms) -- or may do so, when
+    // the slots (as many bytes as the packed bases, and at most 24 more a
+    // sequence) would take more than a quarter of the scratch that is left: few
+    // sequences far up in a large pool.
+    const uint64_t slots = bytes + 48 * (uint64_t)n;
+    const bool own = !shared && bytes <= 2 * extent && slots < (1ull << 35) &&
+                     slots <= scratch_headroom(ctx, (prefix + "_planes").c_str()) / 4;
+    *own_out = own;
     uint64_t words = 2;
     if (!own) plan->planes.reserve(std::min<size_t>(2 * n, 1u << 16));
     std::vector<uint8_t> head(n * sizeof(BitsTask));
@@ -590,7 +598,6 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> 
             b.aw = (uint32_t)words;
             b.bw = b.aw + (b.m + 31) / 32 + 2;
             words = (uint64_t)b.bw + (b.n + 31) / 32 + 2;
-            if (words >= (1ull << 32)) return fail(ctx, NW_ERR_ARG, "planar copy of more than 2^37 bases");
         } else if (sh.S) {
             b.aw = PlaneSet::word_of(plan->planes.add(b.a_off, b.m));
             b.bw = PlaneSet::word_of(plan->planes.add(b.b_off, b.n));
@@ -608,6 +615,26 @@ int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> 
     void *dh = nullptr;
     const int rc = bits_finish_plan(ctx, pool, head, jobs, maxC, sc, scores, score_cap, prefix, plan, &dh);
     plan->ba.tasks = (const BitsTask *)dh;
+    return rc;
+}
+
+void bits_release(nw_ctx *ctx, const std::string &prefix) {
+    free_prefix(ctx, prefix + "_plane");
+    free_prefix(ctx, prefix + "_bits");
+}
+
+int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> &tasks, const nw_scoring &sc,
+                 int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan) {
+    *plan = BitsPlan{};
+    if (tasks.empty()) return NW_OK;
+    const std::string before = ctx->msg;
+    bool own = false;
+    int rc = bits_prepare_slots(ctx, pool, tasks, sc, scores, score_cap, prefix, plan, false, &own);
+    if (rc == NW_ERR_OOM && own) {  // the sequences' own slots left too little for the rest
+        bits_release(ctx, prefix);
+        ctx->msg = before;
+        rc = bits_prepare_slots(ctx, pool, tasks, sc, scores, score_cap, prefix, plan, true, &own);
+    }
     return rc;
 }
 

@@ -210,6 +210,8 @@ bool bits_batch_ok(const nw_scoring &sc);
 // scores[out1]) receive each task's score.
 int bits_prepare(nw_ctx *ctx, const uint8_t *pool, const std::vector<BatchTask> &tasks, const nw_scoring &sc,
                  int32_t *scores, uint32_t score_cap, const std::string &prefix, BitsPlan *plan);
+// Hands a plan's scratch back (after a plan that did not fit).
+void bits_release(nw_ctx *ctx, const std::string &prefix);
 // The same for every pair of nseq sequences (the off-diagonal entries of the
 // nseq x nseq matrix `scores`).
 int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, const uint32_t *len, uint32_t nseq,

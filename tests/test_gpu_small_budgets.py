@@ -1,0 +1,45 @@
+"""Calls on contexts whose scratch budget leaves little beyond what the call
+cannot do without: the plan falls back to the form that fits instead of
+reporting NW_ERR_OOM, with the results of a context of any size.  Sequences are
+random bytes of a device pool (four bases each)."""
+import numpy as np
+import pytest
+
+import oracle
+import seqgen
+
+pytestmark = pytest.mark.gpu
+
+
+def _bases(pool, off, n):
+    b = pool[off:off + (n + 3) // 4]
+    return ((b[:, None] >> (2 * np.arange(4, dtype=np.uint8))) & 3).reshape(-1)[:n].astype(np.uint8)
+
+
+def _random_pool(seed, nbytes):
+    return np.random.default_rng(seed).integers(0, 256, nbytes, dtype=np.uint8)
+
+
+def _scores(nw, ctx, pool, a, m, b, n, sc):
+    import torch
+    out = torch.full((len(m),), -1, dtype=torch.int32, device="cuda")
+    nw.nw_align_batch(ctx, pool, a, m, b, n, sc, 0, scores=out)
+    ctx.sync()
+    return out.cpu().numpy()
+
+
+# few sequences far up in a large pool, read by many pairs: slots of the pairs'
+# own would take 3.9 MB (first) or, fitting by themselves, leave too little
+# for the row buffers (second)
+@pytest.mark.parametrize("m,n,pairs,budget", [(1500, 1500, 5000, 3 << 20), (60, 20000, 32, 1400 << 10)])
+def test_score_batch_of_few_sequences_in_a_large_pool(m, n, pairs, budget):
+    import torch
+    import paper_2412_21103_gb300 as nw
+    pool = _random_pool(5, 8 << 20)
+    at = pool.size - 8192
+    a = np.full(pairs, at, np.uint64)
+    b = np.full(pairs, at + 1024, np.uint64)
+    ml, nl = np.full(pairs, m, np.uint32), np.full(pairs, n, np.uint32)
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=budget) as ctx:
+        got = _scores(nw, ctx, torch.from_numpy(pool).cuda(), a, ml, b, nl, (1, -1, -1))
+    assert (got == oracle.score(_bases(pool, at, m), _bases(pool, at + 1024, n))).all()
