@@ -1045,10 +1045,22 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     if (!want || ctx->autotune) {
         // score-only: the bit-sliced kernel (rows per lane 32) where the
         // scoring fits two bit planes
-        const bool bits = score_bits;
+        bool bits = score_bits;
         const uint32_t cap = score_slots(tasks.data(), npairs);
         BitsPlan bp;
-        if (bits && (rc = bits_prepare(ctx, pool, tasks, sc, scores, cap, pre, &bp))) return rc;
+        if (bits) {
+            const std::string before = ctx->msg;
+            rc = bits_prepare(ctx, pool, tasks, sc, scores, cap, pre, &bp);
+            if (rc == NW_ERR_OOM && !bits_scoring_ok(sc)) {
+                // no room for the planes of a scoring that the scalar kernel
+                // takes as well: its rows grow with the GPU, not with the batch
+                bits_release(ctx, pre);
+                ctx->msg = before;
+                bits = false;
+            } else if (rc) {
+                return rc;
+            }
+        }
         std::vector<BatchTask> lpt;
         BatchArgs bs = ba;
         if (!bits || ctx->autotune) {  // the scalar kernel runs, or is timed

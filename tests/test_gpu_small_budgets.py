@@ -43,3 +43,22 @@ def test_score_batch_of_few_sequences_in_a_large_pool(m, n, pairs, budget):
     with nw.Context(0, torch.cuda.current_stream(), mem_budget=budget) as ctx:
         got = _scores(nw, ctx, torch.from_numpy(pool).cuda(), a, ml, b, nl, (1, -1, -1))
     assert (got == oracle.score(_bases(pool, at, m), _bases(pool, at + 1024, n))).all()
+
+
+def test_score_batch_in_units_without_room_for_its_planes():
+    """60,000 pairs of 1,000 bases scored +2/-1/-2: 45 MB on the bit planes, 24
+    MB on the scalar kernel."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    count, n = 60000, 1000
+    pool = _random_pool(6, 2 * count * 250)
+    off = np.arange(2 * count, dtype=np.uint64) * 250
+    ln = np.full(count, n, np.uint32)
+    dev = torch.from_numpy(pool).cuda()
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        want = _scores(nw, ctx, dev, off[0::2], ln, off[1::2], ln, (2, -1, -2))
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=30 << 20) as ctx:
+        got = _scores(nw, ctx, dev, off[0::2], ln, off[1::2], ln, (2, -1, -2))
+    assert (got == want).all()
+    for k in (0, 31, count - 1):
+        assert got[k] == oracle.score(_bases(pool, int(off[2 * k]), n), _bases(pool, int(off[2 * k + 1]), n), 2, -1, -2)
