@@ -599,6 +599,16 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
     if (want) {
         free_prefix(ctx, "batch_ptr");
         free_prefix(ctx, "ptr");
+        // the bit-sliced kernels' records too, where they hold more than a
+        // quarter of what is left (else the fallback finds its slots as it
+        // left them)
+        uint64_t held = 0;
+        for (const char *name : {"bgroup_rec", "bpair_rec"})
+            if (const auto it = ctx->bufs.find(name); it != ctx->bufs.end()) held += it->second.cap;
+        if (held > (ctx->budget - std::min(ctx->budget, ctx->used)) / 4) {
+            free_prefix(ctx, "bgroup_rec");
+            free_prefix(ctx, "bpair_rec");
+        }
     }
     // the paper's scoring (s' = 3 on a match, 1 on a mismatch) runs on the
     // bit-sliced window kernel, from a planar copy of the pool;

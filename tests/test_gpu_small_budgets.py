@@ -62,3 +62,60 @@ def test_score_batch_in_units_without_room_for_its_planes():
     assert (got == want).all()
     for k in (0, 31, count - 1):
         assert got[k] == oracle.score(_bases(pool, int(off[2 * k]), n), _bases(pool, int(off[2 * k + 1]), n), 2, -1, -2)
+
+
+def _similar(rs, n, subs):
+    """A sequence of n bases and a copy with `subs` substitutions."""
+    a = rs.bases(n)
+    b = a.copy()
+    at = rs.integers(0, n - 1, subs)
+    b[at] = (b[at] + 1 + rs.integers(0, 2, subs)) % 4
+    return a, b.astype(np.uint8)
+
+
+def _banded(nw, ctx, pairs, w):
+    """Banded alignments on device buffers: scores, CIGARs, pairs certified in a band."""
+    import torch
+    pool, off, ln = nw.pool_of([s for p in pairs for s in p])
+    co = np.concatenate([[0], np.cumsum([nw.nw_cigar_bound(a.size, b.size) for a, b in pairs])]).astype(np.uint64)
+    s = torch.full((len(pairs),), -1, dtype=torch.int32, device="cuda")
+    cp = torch.zeros(int(co[-1]), dtype=torch.uint8, device="cuda")
+    cl = torch.zeros(len(pairs), dtype=torch.int64, device="cuda")
+    before = sum(nw.nw_ctx_band_stats(ctx)["certified_round"])
+    nw.nw_align_batch_banded(ctx, torch.from_numpy(pool).cuda(), off[0::2], ln[0::2], off[1::2], ln[1::2],
+                             np.full(len(pairs), w, np.uint32), (1, -1, -1), nw.NW_CIGAR, s, cp, co, cl)
+    ctx.sync()
+    h, n = cp.cpu().numpy(), cl.cpu().numpy()
+    text = [bytes(h[int(co[k]):int(co[k]) + int(n[k])]).decode() for k in range(len(pairs))]
+    return s.cpu().numpy(), text, sum(nw.nw_ctx_band_stats(ctx)["certified_round"]) - before
+
+
+def _align(nw, ctx, pairs):
+    import torch
+    pool, off, ln = nw.pool_of([s for p in pairs for s in p])
+    co = np.concatenate([[0], np.cumsum([nw.nw_cigar_bound(a.size, b.size) for a, b in pairs])]).astype(np.uint64)
+    s = torch.full((len(pairs),), -1, dtype=torch.int32, device="cuda")
+    cp = torch.zeros(int(co[-1]), dtype=torch.uint8, device="cuda")
+    cl = torch.zeros(len(pairs), dtype=torch.int64, device="cuda")
+    nw.nw_align_batch(ctx, torch.from_numpy(pool).cuda(), off[0::2], ln[0::2], off[1::2], ln[1::2], (1, -1, -1),
+                      nw.NW_CIGAR, s, cp, co, cl)
+    ctx.sync()
+    h, n = cp.cpu().numpy(), cl.cpu().numpy()
+    return s.cpu().numpy(), [bytes(h[int(co[k]):int(co[k]) + int(n[k])]).decode() for k in range(len(pairs))]
+
+
+def test_band_after_a_batch_that_filled_the_scratch(monkeypatch):
+    """Alignments of 3 kb leave records of half the budget behind; the pairs of
+    the next call still run in their band."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    monkeypatch.setenv("NW_BAND_KEEP", "1")
+    rs = seqgen.Stream(91)
+    first = [_similar(rs, 3000, 90) for _ in range(200)]
+    pairs = [_similar(rs, 8000, 200) for _ in range(3)]
+    want = oracle.align_many(pairs)
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=16 << 20) as ctx:
+        _align(nw, ctx, first)
+        s, c, banded = _banded(nw, ctx, pairs, 900)
+    assert banded == len(pairs)
+    assert list(s) == [v for v, _ in want] and c == [oracle.rle(o) for _, o in want]
