@@ -430,6 +430,16 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
                       const nw_scoring &sc, uint32_t flags, int32_t *scores, char *cigar_pool,
                       const uint64_t *cigar_off, uint64_t *cigar_len);
 
+// Scratch of a wave of the window kernel: a third of what is left beside its own
+// slots, so that waves of other mixes of kept planes, moves and tables (slots
+// keep their largest size) and the stretches of the walks fit as well.
+static uint64_t bits_wave_budget(nw_ctx *ctx) {
+    uint64_t mine = 0;
+    for (const char *name : {"bband_ptr", "bband_moves"})
+        if (const auto it = ctx->bufs.find(name); it != ctx->bufs.end()) mine += it->second.cap;
+    return (ctx->budget - std::min(ctx->budget, ctx->used - mine)) / 3;
+}
+
 // One banded round on the bit-sliced window kernel (nw_bits_band.cu) for
 // the items (half-widths iw): pairs that would keep the GPU waiting on one
 // warp go to `rest` (the full kernels), the others run in waves bounded by
@@ -489,20 +499,21 @@ static int bits_round(nw_ctx *ctx, const uint8_t *pool, const PlaneSet &planes, 
     }
     if (round == 0) ctx->band_stats[0] += items.size();
     ht_prep.stop();
-    const uint64_t wave_budget = scratch_headroom(ctx, "bband_ptr") / 2;
+    const uint64_t wave_budget = bits_wave_budget(ctx);
     size_t k0 = 0;
     while (k0 < items.size()) {
         std::vector<BandBitsItem> wave;
         std::vector<uint32_t> ww;
-        uint64_t recs = 0;
+        uint64_t recs = 0, bytes = 0;
         size_t k = k0;
         for (; k < items.size(); ++k) {
             BandBitsItem it = items[k];
-            const uint64_t r = band_bits_kept(it.shape);
             if (want) {
-                if (!wave.empty() && (recs + r) * 16 > wave_budget) break;
+                const uint64_t more = band_bits_scratch(it.m, it.n, it.shape);
+                if (!wave.empty() && bytes + more > wave_budget) break;
+                bytes += more;
                 it.ptr_off = recs;
-                recs += r;
+                recs += band_bits_kept(it.shape);
             }
             ctx->band_stats[6] += band_bits_cells(it.shape);
             wave.push_back(it);

@@ -277,6 +277,9 @@ bool band_bits_shape(uint32_t m, uint32_t n, int32_t lo, int32_t hi, BandBitsSha
 bool band_bits_spread(BandBitsShape *s);
 uint64_t band_bits_cells(const BandBitsShape &s);  // cells of the pair's window, over all its chunks
 uint64_t band_bits_kept(const BandBitsShape &s);   // its kept planes (16-byte units)
+// Bytes an alignment takes there beside the planar copy: kept planes, moves and
+// its entries in the tables of fill and walk.
+uint64_t band_bits_scratch(uint32_t m, uint32_t n, const BandBitsShape &s);
 // The widest half-width whose band fits the window of an m x n pair.
 uint32_t band_bits_max_width(uint32_t m, uint32_t n);
 double band_bits_seconds(const BandBitsShape &s);    // estimated time of the pair on one warp

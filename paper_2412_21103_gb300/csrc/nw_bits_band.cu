@@ -961,6 +961,11 @@ uint64_t band_bits_kept(const BandBitsShape &s) {
     return (uint64_t)((s.nchunks + kBlockChunks - 1) / kBlockChunks) * s.g * s.Q;
 }
 
+uint64_t band_bits_scratch(uint32_t m, uint32_t n, const BandBitsShape &s) {
+    return band_bits_kept(s) * 16 + m + n + 16 + sizeof(BandBitsTask) + sizeof(BandBitsJob) + sizeof(BitsWalkTask) +
+           sizeof(TraceTask) + sizeof(uint64_t) + 4 + (s.nchunks / kStretch + 1) * sizeof(BitsWalker);
+}
+
 double band_bits_seconds(const BandBitsShape &s) {
     // 32 pairs of anti-diagonals per chunk, 20 instructions per word and 14
     // per lane each, 2.1 cycles apiece on a scheduler of its own, 2 GHz

@@ -119,3 +119,22 @@ def test_band_after_a_batch_that_filled_the_scratch(monkeypatch):
         s, c, banded = _banded(nw, ctx, pairs, 900)
     assert banded == len(pairs)
     assert list(s) == [v for v, _ in want] and c == [oracle.rle(o) for _, o in want]
+
+
+def test_band_waves_leave_room_for_the_moves(monkeypatch):
+    """Narrow bands keep fewer bytes of planes than their walks have moves: 600
+    pairs of 5 kb keep 1.5 MB and walk 6 MB, under a budget of 5."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    monkeypatch.setenv("NW_BAND_KEEP", "1")
+    rs = seqgen.Stream(93)
+    pairs = [_similar(rs, 5000, 10) for _ in range(600)]
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=5 << 20) as ctx:
+        s, c, banded = _banded(nw, ctx, pairs, 20)
+    assert banded == len(pairs)
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        s2, c2 = _align(nw, ctx, pairs)
+    assert (s == s2).all() and c == c2
+    for k in (0, 299, 599):
+        v, ops = oracle.align(*pairs[k])
+        assert s[k] == v and c[k] == oracle.rle(ops)
