@@ -648,6 +648,10 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
         std::vector<BatchTask> tasks;
         std::vector<uint32_t> tw;  // width used per task
         std::vector<uint32_t> next, nextw;  // rejected pairs and their next widths
+        // whether the scalar banded kernel's pointer words of a pair fit
+        const auto words_fit = [&](const BatchTask &t) {
+            return !want || band_cells(t, R) / 4 <= (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
+        };
         for (size_t q = 0; q < pending.size(); ++q) {
             const uint32_t id = pending[q];
             BatchTask t{};
@@ -665,8 +669,7 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
             band_task(t, R, w);
             // (a banded cell costs about what a full-grid cell costs, so the
             // band pays off up to ~85% of the grid)
-            if (band_cells(t, R) * 20 >= full_cells(t, R) * 17 ||
-                (want && band_cells(t, R) / 4 > (ctx->budget - std::min(ctx->budget, ctx->used)) / 2)) {
+            if (band_cells(t, R) * 20 >= full_cells(t, R) * 17 || (!use_bits && !words_fit(t))) {
                 rest.push_back(id);
                 continue;
             }
@@ -674,7 +677,7 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
             tw.push_back(width[q]);
         }
         if (use_bits && !tasks.empty()) {
-            // every pair whose band fits the window kernel (at most 8,192 rows)
+            // every pair whose band fits the window kernel (at most 4,096 rows)
             std::vector<BandBitsItem> items;
             std::vector<uint32_t> iw, keep_w;
             std::vector<BatchTask> keep;
@@ -698,12 +701,19 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
                     band_task(tb, R, wq);
                 }
                 if (band_bits_shape(tb.m, tb.n, tb.lo, tb.hi, &sh, max_q)) {
+                    // (a pair that even alone leaves its walk no scratch)
+                    if (want && band_bits_scratch(tb.m, tb.n, sh) > bits_wave_budget(ctx)) {
+                        rest.push_back(t.out0);
+                        continue;
+                    }
                     items.push_back(BandBitsItem{tb.a_off, tb.b_off, 0, bp.a_slot[tb.out0], bp.b_slot[tb.out0], tb.m,
                                                  tb.n, tb.out0, sh});
                     iw.push_back(wq);
-                } else {
+                } else if (words_fit(t)) {
                     keep.push_back(t);
                     keep_w.push_back(tw[q]);
+                } else {
+                    rest.push_back(t.out0);
                 }
             }
             tasks.swap(keep);

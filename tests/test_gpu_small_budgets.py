@@ -121,6 +121,19 @@ def test_band_after_a_batch_that_filled_the_scratch(monkeypatch):
     assert list(s) == [v for v, _ in want] and c == [oracle.rle(o) for _, o in want]
 
 
+def test_band_of_a_pair_whose_full_records_do_not_fit(monkeypatch):
+    """A band of 5.6 million cells under 2 MB: kept planes take 24 KB of it."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    monkeypatch.setenv("NW_BAND_KEEP", "1")
+    pairs = [_similar(seqgen.Stream(92), 6000, 180)]
+    want = oracle.align_many(pairs)
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=2 << 20) as ctx:
+        s, c, banded = _banded(nw, ctx, pairs, 200)
+    assert banded == 1
+    assert list(s) == [v for v, _ in want] and c == [oracle.rle(o) for _, o in want]
+
+
 def test_band_waves_leave_room_for_the_moves(monkeypatch):
     """Narrow bands keep fewer bytes of planes than their walks have moves: 600
     pairs of 5 kb keep 1.5 MB and walk 6 MB, under a budget of 5."""
