@@ -652,24 +652,28 @@ int affine_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const
         if ((rc = affine_jobs(ctx, all, R, aa))) return rc;
         return launch_affine(ctx, R, false, aa);
     }
-    // waves whose kept states and stripe rows fit half the free budget
-    const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
+    // Waves that fit a third of the free budget with all they take: kept states,
+    // stripe rows, and the moves and tables, which are most of it for short
+    // pairs.  A third, because the slots keep the largest size of every wave.
+    const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 3;
     const uint32_t state_units = (2u * (uint32_t)R + 4u) / 4u * 32u;  // 16-byte units of a kept state
     size_t k0 = 0;
     while (k0 < all.size()) {
         std::vector<AffTask> wave;
         std::vector<uint64_t> moff;
-        uint64_t units = 0, mbytes = 0, rbytes = 0;
+        uint64_t units = 0, mbytes = 0, bytes = 0;
         size_t k = k0;
         for (; k < all.size(); ++k) {
             AffTask t = all[k];
             const uint64_t S = (t.m + SH - 1) / SH;
             const uint64_t u = S * t.keep_n * state_units;
             const uint64_t rb = S > 1 ? (S - 1) * 8 * (((uint64_t)t.n + 31) / 32 * 32) : 0;
-            if (!wave.empty() && (units + u) * 16 + rbytes + rb > wave_budget) break;
+            const uint64_t more = u * 16 + rb + t.m + t.n + 16 + 2 * sizeof(uint64_t) + sizeof(TraceTask) +
+                                  sizeof(AffTask) + std::max<uint64_t>(S, 1) * (sizeof(AffJob) + 4);
+            if (!wave.empty() && bytes + more > wave_budget) break;
+            bytes += more;
             t.keep_off = units;
             units += u;
-            rbytes += rb;
             moff.push_back(mbytes);
             mbytes += (uint64_t)t.m + t.n + 16;
             wave.push_back(t);

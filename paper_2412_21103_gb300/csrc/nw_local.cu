@@ -678,15 +678,18 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     int rc;
     cudaError_t e0 = cudaMemsetAsync(scores, 0, (size_t)npairs * 4, ctx->stream);  // the stripes' maxima are merged
     if (e0 != cudaSuccess) return cuda_fail(ctx, e0, "local scores reset");
-    // waves whose stripe rows and kept states fit half the free budget
-    const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
+    // Waves that fit a third of the free budget with all they take: stripe rows,
+    // kept states, and the moves and tables, which are most of it for short
+    // pairs.  A third, because the slots keep the largest size of every wave.
+    const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 3;
+    const uint64_t per_job = sizeof(LocalJob) + 4 + (mode == kScore ? 0 : sizeof(LocalBest));
     const uint32_t state_units = ((uint32_t)R + 5u) / 4u * 32u;  // 16-byte units of a kept state
     size_t k0 = 0;
     while (k0 < all.size()) {
         std::vector<LocalTask> wave;
         std::vector<LocalJob> jobs;
         std::vector<uint64_t> moff;
-        uint64_t units = 0, rows = 0, mbytes = 0;
+        uint64_t units = 0, rows = 0, mbytes = 0, bytes = 0;
         bool turn = mode == kScore;  // rows: two in turn
         size_t k = k0;
         for (; k < all.size(); ++k) {
@@ -694,10 +697,14 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
             const uint32_t S = (t.m && t.n) ? (t.m + SH - 1) / SH : 1;
             const uint64_t u = (uint64_t)S * t.keep_n * state_units;
             uint64_t rw = (uint64_t)(mode == kScore ? std::min(S - 1, 2u) : S - 1) * t.nr;
-            if (!wave.empty() && ((turn && mode == kEnds) || (units + u) * 16 + (rows + rw) * 4 > wave_budget)) break;
+            const uint64_t tables = sizeof(LocalTask) + S * per_job +
+                                    (want ? t.m + t.n + 16 + 2 * sizeof(uint64_t) + sizeof(TraceTask) : 0);
+            const uint64_t more = u * 16 + rw * 4 + tables;
+            if (!wave.empty() && ((turn && mode == kEnds) || bytes + more > wave_budget)) break;
+            bytes += more;
             // a lone pair whose rows alone exceed the budget keeps two and
             // finds its end cell by sweeping the stripes above it again
-            if (mode == kEnds && wave.empty() && rw * 4 + (64u << 10) > scratch_headroom(ctx, "local_rows")) {
+            if (mode == kEnds && wave.empty() && rw * 4 + tables + (64u << 10) > scratch_headroom(ctx, "local_rows")) {
                 turn = true;
                 rw = (uint64_t)std::min(S - 1, 2u) * t.nr;
             }

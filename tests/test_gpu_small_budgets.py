@@ -151,3 +151,42 @@ def test_band_waves_leave_room_for_the_moves(monkeypatch):
     for k in (0, 299, 599):
         v, ops = oracle.align(*pairs[k])
         assert s[k] == v and c[k] == oracle.rle(ops)
+
+
+@pytest.mark.parametrize("kind", ["local", "affine"])
+def test_waves_of_short_pairs_count_their_moves_and_tables(kind):
+    """20,000 pairs of 90 bases keep no state between steps, but have 8 MB of
+    moves and tables, under a budget of 4."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    count, n = 20000, 90
+    pool = _random_pool(7, 2 * count * 23)
+    off = np.arange(2 * count, dtype=np.uint64) * 23
+    ln = np.full(count, n, np.uint32)
+    dev = torch.from_numpy(pool).cuda()
+    co = np.arange(count + 1, dtype=np.uint64) * nw.nw_cigar_bound(n, n)
+    got = []
+    for budget in (4 << 20, 0):
+        with nw.Context(0, torch.cuda.current_stream(), mem_budget=budget) as ctx:
+            s = torch.full((count,), -1, dtype=torch.int32, device="cuda")
+            e = torch.zeros((count, 4), dtype=torch.int32, device="cuda")
+            cp = torch.zeros(int(co[-1]), dtype=torch.uint8, device="cuda")
+            cl = torch.zeros(count, dtype=torch.int64, device="cuda")
+            if kind == "local":
+                nw.nw_local_align_batch(ctx, dev, off[0::2], ln, off[1::2], ln, (1, -1, -1), nw.NW_CIGAR, s, e, cp, co, cl)
+            else:
+                nw.nw_affine_align_batch(ctx, dev, off[0::2], ln, off[1::2], ln, (2, -3, -5, -2), nw.NW_CIGAR, s, cp, co, cl)
+            ctx.sync()
+            got.append([x.cpu().numpy() for x in (s, e, cl, cp)])
+    for x, y in zip(got[0][:3], got[1][:3]):
+        assert (x == y).all()
+    texts = [[bytes(g[3][int(co[k]):int(co[k]) + int(g[2][k])]) for k in range(count)] for g in got]
+    assert texts[0] == texts[1]
+    for k in (0, 7777, count - 1):
+        pair = (_bases(pool, int(off[2 * k]), n), _bases(pool, int(off[2 * k + 1]), n))
+        if kind == "local":
+            v, ends, ops = oracle.local_align_many([pair])[0]
+            assert tuple(int(x) for x in got[0][1][k]) == tuple(ends)
+        else:
+            v, ops = oracle.affine_align_many([pair], 2, -3, -5, -2)[0]
+        assert int(got[0][0][k]) == v and texts[0][k].decode() == oracle.rle(ops)
