@@ -47,12 +47,12 @@
 #include <vector>
 
 #include "nw_bits.cuh"
+#include "nw_bits_shape.h"
 #include "nw_order.h"
 
 namespace nw {
 
 constexpr int kPairWarps = 4;        // most warps per CTA (one per scheduler)
-constexpr uint32_t kPairRows = 31;   // rows per stripe (bits 0..30 of a word)
 // One pair of a launch (device array).
 struct PairDesc {
     int64_t Ag, Bg;             // slots of a (rows) and b (columns)
@@ -671,21 +671,6 @@ int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &job
 }
 
 namespace {
-// A pair on G lanes of a warp: its chunks, and its 16-byte record units.
-struct GroupGeom {
-    uint32_t S, C, period, K;
-    uint64_t rec;
-};
-GroupGeom group_geom(uint32_t m, uint32_t n, uint32_t G) {
-    GroupGeom g{};
-    if (!m || !n) return g;
-    g.S = (m + kPairRows - 1) / kPairRows;
-    g.C = (uint32_t)(((uint64_t)n + kPairRows - 1 + 31u) / 32u);
-    g.period = std::max(g.C, G + 2);
-    g.K = (g.S - 1) / G * g.period + g.C + (g.S - 1) % G;
-    g.rec = (uint64_t)g.K * 16u * G;
-    return g;
-}
 constexpr double kGroupStep = 45.0 / 2.07e9;  // a step of a warp, two per scheduler in flight
 }  // namespace
 
@@ -768,7 +753,7 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
         std::vector<uint64_t> keys(nt);
         for (size_t q = 0; q < nt; ++q) {
             const PairJob &j = pairs[wave[q]];
-            keys[q] = (uint64_t)lanes[wave[q]] << 32 | group_geom(j.m, j.n, lanes[wave[q]]).K;
+            keys[q] = (uint64_t)lanes[wave[q]] << 56 | group_geom(j.m, j.n, lanes[wave[q]]).K;
         }
         const std::vector<uint32_t> to = radix_order_desc(std::move(keys));
         std::vector<GroupTask> tasks(nt);
@@ -792,11 +777,11 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
             const PairJob &j = pairs[k];
             const GroupGeom g = group_geom(j.m, j.n, G);
             GroupTask &t = tasks[q];
-            t = GroupTask{ag[k], bg[k], j.m, j.n, g.S, g.C, g.period, g.K, g.S ? (j.m - 1) - kPairRows * (g.S - 1) : 0u,
+            t = GroupTask{ag[k], bg[k], j.m, j.n, g.S, g.C, g.period, (uint32_t)g.K, g.S ? (j.m - 1) - kPairRows * (g.S - 1) : 0u,
                           0u, (uint64_t)((const uint4 *)tts[w].ptr - (const uint4 *)rv), row_off, j.score};
             row_off += g.C;
             if (jobs.empty() || jobs.back().G != G || jobs.back().cnt == 32u / G) {
-                jobs.push_back(GroupJob{(uint32_t)q, 0, G, g.K});
+                jobs.push_back(GroupJob{(uint32_t)q, 0, G, (uint32_t)g.K});
                 jk.push_back(g.K);
             }
             ++jobs.back().cnt;

@@ -1,5 +1,6 @@
-// Shapes and counts of the bit-sliced score kernel (nw_bits.cu): plain
-// arithmetic, for the host plan and the kernel alike.
+// Shapes and counts of the bit-sliced score kernel (nw_bits.cu) and of the
+// groups of lanes (nw_bits_pair.cu): plain arithmetic, for the host plans and
+// the kernels alike.
 #pragma once
 
 #include <cstdint>
@@ -39,6 +40,26 @@ NW_HOST_DEVICE void bits_last_row_span(uint64_t c, uint64_t last, uint32_t n, in
     const int32_t e = (int32_t)(32 * (c - last));
     lo = e + 1 > (int32_t)n ? e + 1 - (int32_t)n : 0;
     hi = e < 31 ? e : 31;
+}
+
+// A pair on G lanes of a warp, stripes of 31 rows: its chunks (K in all, from one
+// pass of a lane to its next `period`), and its 16-byte record units.  A pair of
+// 1.3e14 cells has more than 2^32 chunks; those that a launch takes have records
+// that fit the scratch, so their K fits 32 bits.
+constexpr uint32_t kPairRows = 31;  // rows per stripe (bits 0..30 of a word)
+struct GroupGeom {
+    uint32_t S, C, period;
+    uint64_t K, rec;
+};
+inline GroupGeom group_geom(uint32_t m, uint32_t n, uint32_t G) {
+    GroupGeom g{};
+    if (!m || !n) return g;
+    g.S = (m + kPairRows - 1) / kPairRows;
+    g.C = (uint32_t)(((uint64_t)n + kPairRows - 1 + 31u) / 32u);
+    g.period = g.C > G + 2 ? g.C : G + 2;
+    g.K = (uint64_t)((g.S - 1) / G) * g.period + g.C + (g.S - 1) % G;
+    g.rec = g.K * 16u * G;
+    return g;
 }
 
 }  // namespace nw

@@ -1,7 +1,8 @@
-"""Shapes and column counts of the bit-sliced score kernel (nw_bits_shape.h),
-compiled for the host, against Python's integers: where the columns of the
-last stripe's bottom row leave, for sizes up to the accepted 2^30 bases, and
-that the chunks of a pair hand out each of its columns exactly once."""
+"""Shapes and column counts of the bit-sliced score kernel and of the groups of
+lanes (nw_bits_shape.h), compiled for the host, against Python's integers:
+where the columns of the last stripe's bottom row leave, for sizes up to the
+accepted 2^30 bases, that the chunks of a pair hand out each of its columns
+exactly once, and the chunks and records of a pair on a group."""
 import ctypes
 import os
 import shutil
@@ -18,6 +19,11 @@ void span(uint64_t c, uint32_t S, uint32_t C, uint32_t K, uint32_t n, int32_t *o
 }
 uint32_t period(uint32_t K, uint32_t S, uint32_t n) { return nw::BitsShape{K, S, 10 * K + 6}.period(n); }
 uint64_t chunks(uint32_t K, uint32_t S, uint32_t n) { return nw::BitsShape{K, S, 10 * K + 6}.chunks(n); }
+uint64_t group(uint32_t m, uint32_t n, uint32_t G, uint64_t *rec) {
+    const nw::GroupGeom g = nw::group_geom(m, n, G);
+    *rec = g.rec;
+    return g.K;
+}
 }
 """
 
@@ -31,7 +37,7 @@ def lib(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, str(d / "shape.cpp"), "-o", so], check=True)
     lib = ctypes.CDLL(so)
     lib.span.argtypes = [ctypes.c_uint64] + [ctypes.c_uint32] * 4 + [ctypes.POINTER(ctypes.c_int32)]
-    lib.period.restype, lib.chunks.restype = ctypes.c_uint32, ctypes.c_uint64
+    lib.period.restype, lib.chunks.restype, lib.group.restype = ctypes.c_uint32, ctypes.c_uint64, ctypes.c_uint64
     return lib
 
 
@@ -77,3 +83,13 @@ def test_every_column_once(lib, K):
                 lo, hi = _span(lib, c, S, C, K, n)
                 cols += [32 * (c - (S - 1) * C - K + 1) - b for b in range(lo, hi + 1)]
             assert sorted(cols) == list(range(n)), (S, n)
+
+
+def test_chunks_and_records_of_a_group(lib):
+    # the last pair: 127 passes of 2^25 chunks and one more, 2^32 in all
+    for m, n in SIZES + [(0, 5), (5, 0), (31, 1), (32, 2), (993, 1025), (31 * 4064 + 1, (1 << 30) - 61)]:
+        for G in (1, 4, 32):
+            S, C = -(-m // 31), (n + 61) // 32
+            K = (S - 1) // G * max(C, G + 2) + C + (S - 1) % G if m and n else 0
+            rec = ctypes.c_uint64()
+            assert lib.group(m, n, G, ctypes.byref(rec)) == K and rec.value == K * 16 * G, (m, n, G)
