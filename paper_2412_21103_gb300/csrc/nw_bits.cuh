@@ -142,6 +142,8 @@ class PlaneSet {
     // Slot (global base index of base 0) of the sequence at pool byte `off`
     // with `len` bases, added on first use.
     int64_t add(uint64_t off, uint32_t len);
+    // Scratch that a sequence of `len` bases takes: its words in both planes and its segment.
+    static uint64_t bytes_of(uint32_t len) { return ((uint64_t)(len + 31) / 32 + 2) * 8 + sizeof(PlaneSeg); }
     // First word of a slot that add() returned.
     static uint32_t word_of(int64_t slot) { return (uint32_t)((slot + kPlanePad) / 32); }
     // Room for `words` words of slots laid out by the caller from word 2 on.

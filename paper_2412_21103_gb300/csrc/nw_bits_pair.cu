@@ -689,18 +689,11 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
     HostTimer ht(ctx, "bits_groups");
     const bool gen = gen_of(sc);
     const size_t np = pairs.size();
-    PlaneSet ps;
-    ps.reserve(std::min<size_t>(2 * np, 1u << 16));
-    std::vector<int64_t> ag(np, 0), bg(np, 0);
     double work = 0;  // lane-chunks
     for (size_t k = 0; k < np; ++k) {
-        if (!pairs[k].m || !pairs[k].n) continue;
-        ag[k] = ps.add(pairs[k].a_off, pairs[k].m);
-        bg[k] = ps.add(pairs[k].b_off, pairs[k].n);
         const GroupGeom g = group_geom(pairs[k].m, pairs[k].n, 1);
         work += (double)g.S * g.C;
     }
-    if ((rc = ps.launch(ctx, pool, "bgroup"))) return rc;
     // Lanes per pair: the fewest (fewer lanes leave fewer idle while a pair
     // starts and ends) that bring the pair's own time under half of the time
     // the batch takes with every scheduler busy, at least four (records of 64
@@ -717,8 +710,6 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
     }
     const std::vector<uint32_t> order = radix_order_desc(std::move(by_moves));  // longest first, as the walks want them
     GroupLaunch L{};
-    L.pl0 = ps.pl0;
-    L.pl1 = ps.pl1;
     const BitsUnits units = bits_units(sc);
     L.unit = units.unit;
     L.gap = sc.gap;
@@ -728,21 +719,41 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kPairWarps * 32, 0);
     occ = std::max(1, std::min(occ, 2));
-    // waves of pairs whose records fit half of what their slot may grow to
-    const uint64_t room = scratch_headroom(ctx, "bgroup_rec") / 2 / 16;
+    // Waves of pairs that fit half of the scratch that is left beside these slots
+    // with all they take, the planar copies of their sequences too (of a whole
+    // batch of long pairs these alone would leave a small budget no room).
+    uint64_t mine = 0;
+    for (auto it = ctx->bufs.lower_bound("bgroup_"); it != ctx->bufs.end() && it->first.compare(0, 7, "bgroup_") == 0; ++it)
+        mine += it->second.cap;
+    const uint64_t room = (ctx->budget - std::min(ctx->budget, ctx->used - mine)) / 2;
+    std::vector<int64_t> ag(np, 0), bg(np, 0);
     for (size_t next = 0; next < np;) {
         std::vector<uint32_t> wave;
-        uint64_t rec = 0, rows = 0, moves = 0;
+        uint64_t rec = 0, rows = 0, moves = 0, bytes = 0;
         for (; next < np; ++next) {
             const PairJob &j = pairs[order[next]];
             const GroupGeom g = group_geom(j.m, j.n, lanes[order[next]]);
-            if (!wave.empty() && rec + g.rec > room) break;
+            const uint64_t more = g.rec * 16 + g.C * sizeof(uint2) + (uint64_t)j.m + j.n + 16 + sizeof(uint64_t) +
+                                  sizeof(GroupTask) + sizeof(GroupJob) + sizeof(TraceTask) +
+                                  PlaneSet::bytes_of(j.m) + PlaneSet::bytes_of(j.n);
+            if (!wave.empty() && bytes + more > room) break;
+            bytes += more;
             wave.push_back(order[next]);
             rec += g.rec;
             rows += g.C;
             moves += (uint64_t)j.m + j.n + 16;
         }
         const size_t nt = wave.size();
+        PlaneSet ps;
+        ps.reserve(std::min<size_t>(2 * nt, 1u << 16));
+        for (const uint32_t k : wave) {
+            if (!pairs[k].m || !pairs[k].n) continue;
+            ag[k] = ps.add(pairs[k].a_off, pairs[k].m);
+            bg[k] = ps.add(pairs[k].b_off, pairs[k].n);
+        }
+        if ((rc = ps.launch(ctx, pool, "bgroup"))) return rc;
+        L.pl0 = ps.pl0;
+        L.pl1 = ps.pl1;
         void *rv = nullptr, *wv = nullptr, *mv = nullptr, *nm = nullptr, *dv = nullptr;
         // (a walk may read up to 32 rows past a stripe's last)
         if ((rc = scratch(ctx, "bgroup_rec", (rec + 32u * 32u) * 16 + 16, &rv))) return rc;

@@ -190,3 +190,20 @@ def test_waves_of_short_pairs_count_their_moves_and_tables(kind):
         else:
             v, ops = oracle.affine_align_many([pair], 2, -3, -5, -2)[0]
         assert int(got[0][0][k]) == v and texts[0][k].decode() == oracle.rle(ops)
+
+
+def test_alignments_whose_planar_copies_alone_fill_the_budget():
+    """1,500 pairs of 1 kb: .8 MB of planar copies, .3 to .5 MB of records a pair,
+    under a budget of 1.2 MB."""
+    import torch
+    import paper_2412_21103_gb300 as nw
+    rs = seqgen.Stream(94)
+    pairs = [_similar(rs, 1000, 40) for _ in range(1500)]
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=1200 << 10) as ctx:
+        s, c = _align(nw, ctx, pairs)
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        s2, c2 = _align(nw, ctx, pairs)
+    assert (s == s2).all() and c == c2
+    for k in (0, 700, 1499):
+        v, ops = oracle.align(*pairs[k])
+        assert s[k] == v and c[k] == oracle.rle(ops)
