@@ -1206,7 +1206,7 @@ int band_bits_walk(nw_ctx *ctx, const PlaneSet &planes, const void *ptr, const s
         wa.own = at;
     }
     {
-        LaunchTimer t(ctx, "bband_walk");
+        LaunchTimer t(ctx, "bband_walk", split ? 7 : 1);  // peaks, stretches, joints, two rounds of link and lost
         // one warp per CTA; its 17 KB of records let 13 share an SM
         constexpr int smem = kSubPairs * kTileRecs * (int)sizeof(uint4);
         static_assert(smem <= 48 * 1024, "above the default limit of dynamic shared memory");
