@@ -71,14 +71,15 @@ __device__ __forceinline__ bool wait_geq(const uint32_t *flag, uint32_t target, 
 
 // Warp-uniform bounded wait until *flag >= target; `seen` holds what an
 // earlier call saw, so a producer far ahead costs no load.  Every lane
-// acquires, so its following loads see what the producer published.
+// acquires, so its following loads see what the producer published; later
+// calls go by the least that any lane saw, which all of them acquired.
 __device__ __forceinline__ bool warp_wait_geq(const uint32_t *flag, uint32_t target, uint32_t &seen, uint32_t *err,
                                               uint32_t where) {
     if (seen >= target) return true;
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = wait_geq(flag, target, err, where) ? 1 : 0;
     ok = __shfl_sync(kFull, ok, 0);
-    if (ok) seen = __shfl_sync(kFull, ld_acquire(flag), 0);
+    if (ok) seen = __reduce_min_sync(kFull, ld_acquire(flag));
     return ok != 0;
 }
 
