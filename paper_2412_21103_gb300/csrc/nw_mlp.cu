@@ -39,7 +39,7 @@ struct BandModel {
     float *master = nullptr;      // kNParams
     __nv_bfloat16 *wb = nullptr;  // BF16 copies of W1, W2, W3 (same offsets)
     float *adam_m = nullptr, *adam_v = nullptr;
-    float *grad = nullptr;        // kNParams
+    float *grad = nullptr;        // kNParams + 1 (gradients and loss)
     int64_t step = 0;
 };
 
@@ -425,7 +425,7 @@ static int model_of(nw_ctx *ctx, BandModel **out, bool create) {
         if (e == cudaSuccess) e = cudaMalloc(&bm->wb, kNParams * 2);
         if (e == cudaSuccess) e = cudaMalloc(&bm->adam_m, kNParams * 4);
         if (e == cudaSuccess) e = cudaMalloc(&bm->adam_v, kNParams * 4);
-        if (e == cudaSuccess) e = cudaMalloc(&bm->grad, kNParams * 4);
+        if (e == cudaSuccess) e = cudaMalloc(&bm->grad, (kNParams + 1) * 4);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(ctx, NW_ERR_OOM, "band model allocation failed");
@@ -484,10 +484,20 @@ static int forward(nw_ctx *ctx, BandModel *bm, const float *x, uint32_t n, float
 
 // Gradients into grad (kNParams) and the loss.
 static int gradients(nw_ctx *ctx, BandModel *bm, const float *x, const float *t, uint32_t nb, float *grad, float *loss) {
-    // shares of at least 32 samples
-    const uint32_t per = std::max<uint32_t>(32, (nb + 31) / 32), shares = (nb + per - 1) / per;
+    // Shares of at least 32 samples, as many as the scratch has room for (100 KB
+    // each beside the activations); one share's sums fit the model's own
+    // gradients.
+    const size_t acts = (size_t)nb * (4 * kH + 2) * 4 + 64, one = (size_t)(kNParams + 1) * 4;
+    const uint64_t room = scratch_headroom(ctx, "mlp_acts");
+    uint32_t per = std::max<uint32_t>(32, (nb + 31) / 32), shares = (nb + per - 1) / per;
+    if (acts + shares * one > room) {
+        shares = (uint32_t)std::max<uint64_t>(1, (room - std::min<uint64_t>(room, acts)) / one);
+        per = (nb + shares - 1) / shares;
+        shares = (nb + per - 1) / per;
+    }
+    const bool in_model = acts + shares * one > room;
     void *v = nullptr;
-    int rc = scratch(ctx, "mlp_acts", ((size_t)nb * (4 * kH + 2) + (size_t)shares * (kNParams + 1)) * 4 + 64, &v);
+    int rc = scratch(ctx, "mlp_acts", acts + (in_model ? 0 : shares * one), &v);
     if (rc) return rc;
     NetArgs a{};
     a.x = x;
@@ -501,7 +511,7 @@ static int gradients(nw_ctx *ctx, BandModel *bm, const float *x, const float *t,
     a.dh2 = a.dh1 + (size_t)nb * kH;
     a.dy = a.dh2 + (size_t)nb * kH;
     a.y = a.dy + nb;
-    float *part = a.y + nb;
+    float *part = in_model ? bm->grad : a.y + nb;
     {
         LaunchTimer lt(ctx, "mlp_forward", 1);
         if ((rc = launch_net(ctx, a, true))) return rc;
