@@ -740,7 +740,13 @@ int nw_band_model_forward(nw_ctx *ctx, const float *feat, uint32_t n, float *out
     BandModel *bm = nullptr;
     int rc = model_of(ctx, &bm, false);
     if (rc) return rc;
-    return forward(ctx, bm, feat, n, out);
+    // outputs that lie in the inputs (the kernel writes a tile's before others are read)
+    const uintptr_t f0 = (uintptr_t)feat, f1 = f0 + (size_t)n * kF * 4, o0 = (uintptr_t)out, o1 = o0 + (size_t)n * 4;
+    if (o0 >= f1 || f0 >= o1) return forward(ctx, bm, feat, n, out);
+    void *y = nullptr;
+    if ((rc = scratch(ctx, "mlp_acts", (size_t)n * 4, &y)) || (rc = forward(ctx, bm, feat, n, (float *)y))) return rc;
+    const cudaError_t e = cudaMemcpyAsync(out, y, (size_t)n * 4, cudaMemcpyDeviceToDevice, ctx->stream);
+    return e == cudaSuccess ? NW_OK : cuda_fail(ctx, e, "model forward");
 }
 
 int nw_band_model_grad(nw_ctx *ctx, const float *feat, const float *target, uint32_t n, float *grad, float *loss) {

@@ -42,3 +42,17 @@ def test_gradients_under_a_small_budget(n, budget):
     assert abs(l - lb) <= 1e-5 * l
     for lo, hi in zip(BLOCKS, BLOCKS[1:]):
         assert np.linalg.norm(g[lo:hi] - gb[lo:hi]) <= 1e-4 * np.linalg.norm(g[lo:hi]), (lo, hi)
+
+
+@pytest.mark.parametrize("at", [0, 20000 * F - 20000, 7 * F])
+def test_outputs_that_lie_in_the_inputs(at):
+    import torch
+    import paper_2412_21103_gb300 as nw
+    n = 20000
+    x, _ = _data(n)
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        nw.nw_band_model_init(ctx, 5)
+        want = nw.nw_band_model_forward(ctx, x).clone()
+        got = nw.nw_band_model_forward(ctx, x, x.view(-1)[at:at + n])
+        ctx.sync()
+        assert torch.equal(got, want)
