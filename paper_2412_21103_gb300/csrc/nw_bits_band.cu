@@ -527,6 +527,8 @@ struct BitsWalkArgs {
     BitsLink *links;           // per first stretch
     uint32_t last_round;       // lost pairs are walked to their end
     uint32_t half;             // 2^31
+    uint64_t moves_cap, own_cap, recs_cap;  // entries at moves, own, recs (checked build)
+    uint32_t ntasks;
     uint32_t *err;
 };
 
@@ -623,6 +625,7 @@ __global__ void k_bits_link(BitsWalkArgs p) {
         BitsLink l = p.links[h];
         if (tk.nblocks <= p.stretch || l.state > kLinkAt) continue;
         uint8_t *dst = p.moves + tk.moves_off;
+        const uint64_t dst_cap = min(cap_from(tk.moves_off, p.moves_cap), (uint64_t)tk.m + tk.n);
         if (l.state == kLinkNone) l = BitsLink{kLinkAt, h, 0u, (int32_t)tk.m, (int32_t)tk.n, 0u, 0ull};
         l.state = kLinkLost;  // unless the end is reached
         for (uint32_t w = l.w;; ++w) {
@@ -630,6 +633,7 @@ __global__ void k_bits_link(BitsWalkArgs p) {
             const BitsWalkEnd e = p.ends[w];
             l.w = kNoStretch;
             if (e.i < 0) break;
+            if (!in_range(l.moves + (e.k - l.from), dst_cap + 1, p.err, kSiteWalkMoves)) break;
             copy_bytes(dst + l.moves, p.own + wk.moves_off + l.from, e.k - l.from, lane, 32);
             l.moves += e.k - l.from;
             l.i = e.i;
@@ -640,6 +644,7 @@ __global__ void k_bits_link(BitsWalkArgs p) {
             }
             const BitsWalkEnd x = p.joints[w];
             if (x.i < 0) break;
+            if (!in_range(l.moves + x.k, dst_cap + 1, p.err, kSiteWalkMoves)) break;
             copy_bytes(dst + l.moves, p.own + wk.joint_off, x.k, lane, 32);
             l.moves += x.k;
             l.i = x.i;
@@ -653,8 +658,9 @@ __global__ void k_bits_link(BitsWalkArgs p) {
         }
         if (l.state == kLinkDone) {
             const uint32_t rest = (uint32_t)(max(l.i, 0) + max(l.j, 0));
-            for (uint32_t q = lane; q < rest; q += 32) dst[l.moves + q] = l.i > 0 ? 1 : 2;
-            if (lane == 0) p.nmoves[tk.slot] = l.moves + rest;
+            for (uint32_t q = lane; q < rest; q += 32)
+                if (in_range(l.moves + q, dst_cap, p.err, kSiteWalkMoves)) dst[l.moves + q] = l.i > 0 ? 1 : 2;
+            if (lane == 0 && in_range(tk.slot, p.ntasks, p.err, kSiteWalkEnds)) p.nmoves[tk.slot] = l.moves + rest;
         }
         if (lane == 0) p.links[h] = l;
     }
@@ -729,7 +735,11 @@ __global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
         const int32_t R = (tk.a_first - tk.hi - 1) >> 1;
         const BandBases bs{p.pl0, p.pl1, p.max_base, tk.a_slot, tk.b_slot};
         const uint32_t nzt = gl == 0 ? 0u : 1u, nzb = (int32_t)gl >= nw - 1 ? 0u : 1u;
-        uint8_t *mv = whole ? p.moves + tk.moves_off + link.moves : p.own + (MODE == kWalkJoints ? wk.joint_off : wk.moves_off);
+        const uint64_t own_at = MODE == kWalkJoints ? wk.joint_off : wk.moves_off;
+        uint8_t *mv = whole ? p.moves + tk.moves_off + link.moves : p.own + own_at;
+        // moves that fit there (checked build): the pair's, or a stretch's
+        const uint64_t mv_cap = whole ? min(cap_from(tk.moves_off + link.moves, p.moves_cap), (uint64_t)tk.m + tk.n - link.moves)
+                                      : min(cap_from(own_at, p.own_cap), Stretch::stretch_bytes(p.stretch));
         int32_t a_stop = tk.a_first + 64 * c_stop;  // cells before it are not this walk's
         int32_t i = mine ? cell.x : 0, j = mine ? cell.y : 0, joined = -1;
         uint32_t k = 0;
@@ -779,7 +789,8 @@ __global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
             }
             const int32_t cc = on ? (a - tk.a_first) >> 6 : 0, c0 = cc - cc % kBlockChunks;
             if constexpr (MODE == kWalkStretches) {
-                if (on && wk.c_start >= 0 && gl == 0)
+                if (on && wk.c_start >= 0 && gl == 0 &&
+                    in_range(tk.rec_off + (uint64_t)c0, p.recs_cap, p.err, kSiteWalkRecs))
                     p.recs[tk.rec_off + (uint64_t)c0] = make_uint4((uint32_t)i, (uint32_t)j, k, 1u);
             }
             if constexpr (MODE != kWalkStretches) {
@@ -881,13 +892,15 @@ __global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
                     const int32_t run = min(fr, min(i, j));
 #pragma unroll
                     for (int q = 0; q < kAhead; ++q)
-                        if ((int32_t)gl + kSubWords * q < run) mv[k + gl + kSubWords * q] = 0;
+                        if ((int32_t)gl + kSubWords * q < run &&
+                            in_range(k + gl + kSubWords * q, mv_cap, p.err, kSiteWalkMoves))
+                            mv[k + gl + kSubWords * q] = 0;
                     k += (uint32_t)run;
                     i -= run;
                     j -= run;
                     if (run == fr && fr < 16 && x - fr >= 0 && i > 0 && j > 0) {
                         const uint32_t mvc = ((hb >> fr) & 1u) ? 2u : 1u;
-                        if (gl == 0) mv[k] = (uint8_t)mvc;
+                        if (gl == 0 && in_range(k, mv_cap, p.err, kSiteWalkMoves)) mv[k] = (uint8_t)mvc;
                         ++k;
                         i -= mvc == 1u;
                         j -= mvc == 2u;
@@ -897,15 +910,16 @@ __global__ void __launch_bounds__(32) k_bits_walk(BitsWalkArgs p) {
             __syncwarp();
         }
         if (mine && !whole) {
-            if (gl == 0) (MODE == kWalkJoints ? p.joints : p.ends)[wi] = BitsWalkEnd{i, j, k, joined};
+            if (gl == 0 && in_range(wi, p.nwalkers, p.err, kSiteWalkEnds)) (MODE == kWalkJoints ? p.joints : p.ends)[wi] = BitsWalkEnd{i, j, k, joined};
         } else if (mine && joined >= 0) {
-            if (gl == 0) p.links[wi] = BitsLink{kLinkAt, next, (uint32_t)joined, i, j, 0u, link.moves + k};
+            if (gl == 0 && in_range(wi, p.nwalkers, p.err, kSiteWalkEnds)) p.links[wi] = BitsLink{kLinkAt, next, (uint32_t)joined, i, j, 0u, link.moves + k};
         } else if (mine) {
             // row 0 / column 0: only horizontal / vertical moves remain
             const uint32_t rest = (uint32_t)(max(i, 0) + max(j, 0));
             const uint8_t mvr = i > 0 ? 1 : 2;
-            for (uint32_t q = gl; q < rest; q += kSubWords) mv[k + q] = mvr;
-            if (gl == 0) p.nmoves[tk.slot] = link.moves + k + rest;
+            for (uint32_t q = gl; q < rest; q += kSubWords)
+                if (in_range(k + q, mv_cap, p.err, kSiteWalkMoves)) mv[k + q] = mvr;
+            if (gl == 0 && in_range(tk.slot, p.ntasks, p.err, kSiteWalkEnds)) p.nmoves[tk.slot] = link.moves + k + rest;
             if (MODE == kWalkLost && gl == 0) p.links[wi].state = kLinkDone;
         }
         __syncwarp();
@@ -1186,6 +1200,10 @@ int band_bits_walk(nw_ctx *ctx, const PlaneSet &planes, const void *ptr, const s
     wa.stretch = len;
     wa.moves = (uint8_t *)mv;
     wa.nmoves = (uint64_t *)nm;
+    wa.moves_cap = mbytes;
+    wa.own_cap = own;
+    wa.recs_cap = recs;
+    wa.ntasks = (uint32_t)wt.size();
     wa.half = 1u << 31;
     wa.err = ctx->d_err;
     if (split) {

@@ -356,6 +356,7 @@ struct GroupLaunch {
     uint4 *rec;
     uint64_t rec_cap;
     uint2 *rows;
+    uint64_t rows_cap;  // entries at rec, rows (checked build)
     int32_t unit, gap;
     BitsScoring g;
     uint32_t *err;
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_bits_group(GroupLaunch L) {
                 Fn0 = b_next(cn, L.pl0);
                 Fn1 = b_next(cn, L.pl1);
             }
-            const bool write = mine && k < t.K && in_range((uint64_t)(recp - L.rec) + 15u * G, L.rec_cap, L.err, kSiteBandBitsPtr);
+            const bool write = mine && k < t.K && in_range((uint64_t)(recp - L.rec) + 15u * G, L.rec_cap, L.err, kSiteGroupRec);
             if (__any_sync(kFull, act && c == 0)) {
                 const uint32_t rz = c == 0 ? 0u : ~0u;
                 pair_chunk<GEN, true, true>(st, A0, A1, Rc0, Rc1, Rn0, Rn1, nz, gmul, rz, L.g, recp, G, write);
@@ -457,7 +458,8 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_bits_group(GroupLaunch L) {
             Rc0 = Rn0;
             Rc1 = Rn1;
             // outgoing bits: bit b is column 32c + 2 - b of the stripe's bottom row
-            if (act && l == G - 1u && s + 1 < S) __stcg(row + c, make_uint2(st.Qo0, st.Qo1));
+            if (act && l == G - 1u && s + 1 < S && in_range(t.row_off + (uint32_t)c, L.rows_cap, L.err, kSiteGroupRow))
+                __stcg(row + c, make_uint2(st.Qo0, st.Qo1));
             if (act && last) {
                 const int32_t top = 32 * c + 32 - (int32_t)t.pm;
                 const int32_t lo = max(top - (int32_t)t.n, 0), hi = min(31, top - 1);
@@ -818,6 +820,7 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
         L.rec = (uint4 *)rv;
         L.rec_cap = rec;
         L.rows = (uint2 *)wv;
+        L.rows_cap = rows;
         {
             LaunchTimer t(ctx, "bgroup_fill_ptr");
             const uint32_t blocks = std::min<uint32_t>((L.njobs + kPairWarps - 1) / kPairWarps,

@@ -83,8 +83,8 @@ __device__ __forceinline__ bool warp_wait_geq(const uint32_t *flag, uint32_t tar
     return ok != 0;
 }
 
-// Checked build (compiled with -DNW_CHECKS): the kernels' global stores go
-// through in_range(), which compares the index with the buffer's capacity;
+// Checked build (compiled with -DNW_CHECKS): the global stores at the sites
+// below go through in_range(), which compares the index with the buffer's capacity;
 // out of range it records NW_ERR_BOUNDS in the error word (detail: the
 // store site in the top 8 bits, the low 24 bits of the index) and the store
 // is skipped.  In the normal build in_range() is constant true and costs
@@ -96,7 +96,8 @@ constexpr bool kChecks = false;
 #endif
 enum CheckSite : uint32_t {
     kSiteBatchPtr = 1, kSiteBatchRing, kSiteBatchScore, kSiteLocalPtr, kSiteLocalRing, kSiteLocalOut,
-    kSiteLocalMoves, kSiteAffPtr, kSiteAffRing, kSiteAffScore, kSiteAffMoves, kSiteMsaRow, kSiteMsaSlot, kSiteBandBitsPtr
+    kSiteLocalMoves, kSiteAffPtr, kSiteAffRing, kSiteAffScore, kSiteAffMoves, kSiteMsaRow, kSiteMsaSlot, kSiteBandBitsPtr,
+    kSiteWalkMoves, kSiteWalkRecs, kSiteWalkEnds, kSiteGroupRec, kSiteGroupRow
 };
 __device__ __forceinline__ bool in_range(uint64_t idx, uint64_t cap, uint32_t *err, uint32_t site) {
     if constexpr (kChecks) {
@@ -107,6 +108,9 @@ __device__ __forceinline__ bool in_range(uint64_t idx, uint64_t cap, uint32_t *e
     }
     return true;
 }
+
+// Capacity from position `at` of a buffer of `cap` entries on.
+__device__ __forceinline__ uint64_t cap_from(uint64_t at, uint64_t cap) { return at < cap ? cap - at : 0u; }
 
 // Byte permute: output byte 0 = byte (sel & 7) of {hi:lo}, etc. (PTX prmt).
 __device__ __forceinline__ uint32_t prmt(uint32_t lo, uint32_t hi, uint32_t sel) {
