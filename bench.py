@@ -1020,8 +1020,8 @@ def bits_roofline(kernel, workload, cells, kernel_ms, bits_peak, bits_cell_peak,
            "peak_source": "measured live: slowest of nw_peak_int kinds 8/10 (LOP3, funnel shift; independent "
                           "chains on every SM)"}
     cell = {"unit": "GCUPS", "value": bits_cell_peak, "kernel_gcups": gcups, "frac": gcups / bits_cell_peak,
-            "source": "measured live: nw_peak_int kind 11, one bit-sliced anti-diagonal step (32 cells) on "
-                      "independent chains on every SM"}
+            "source": "measured live: nw_peak_int kind 11, bit-sliced anti-diagonal steps of four words a "
+                      "lane (128 cells), every SM full"}
     scalar = {"ops_per_cell": OPS_PER_CELL, "achieved": gcups * OPS_PER_CELL, "peak": scalar_peak,
               "frac": gcups * OPS_PER_CELL / scalar_peak,
               "note": "the scalar unit (4 int32 ops per cell against the DPX/max/prmt peak): above 1 because one "

@@ -582,8 +582,8 @@ void nw_server_destroy(nw_server *srv);
  * 3 = 3-input add, 4 = byte permute (prmt), 5 = cell as prmt + add-max +
  * max, 6 = cell as prmt + add + 3-input max, 7 = cell as prmt + add + max +
  * max, 8 = 3-input logic op, 9 = integer multiply-add, 10 = funnel shift,
- * 11 = one anti-diagonal step of the bit-sliced difference update (32
- * cells).  Not in the paper. */
+ * 11 = anti-diagonal steps of the bit-sliced difference update, four words
+ * of 32 cells a lane.  Not in the paper. */
 int nw_peak_int(nw_ctx *ctx, int kind, uint64_t iters, double *gops);
 
 #ifdef __cplusplus

@@ -74,40 +74,52 @@ __global__ void __launch_bounds__(kPeakThreads) k_peak(uint64_t iters, int32_t s
     if (acc == 0x7f3a5c11) *sink = acc;  // practically never true; keeps the work live
 }
 
-// Kind 11: one anti-diagonal step of the bit-sliced difference update (the
-// step of nw_bits.cu: two window shifts, the match word, the two shifted
-// upper inputs, T, dV, dH and the boundary shift register; 32 cells) on
-// four independent lanes' words per thread.
-constexpr int kBitsChains = 4;
+// Kind 11: anti-diagonal steps of the bit-sliced difference update as the score
+// kernel runs them (bits_chunk in nw_bits.cu away from a stripe's start): rows
+// dealt out over four words a lane, so a step is the match word and eight
+// operations per word, two window shifts, two shifts of the upper inputs and two
+// of the boundary register; 128 cells.  The shifts of the entering columns
+// are multiplies, as there.  All the warps an SM holds, where the kernel
+// runs two per scheduler.
+constexpr int kBitsWords = 4, kBitsSteps = 4;
 __global__ void __launch_bounds__(kPeakThreads) k_peak_bits(uint64_t iters, uint32_t seed, int32_t *sink) {
-    uint32_t H0[kBitsChains], H1[kBitsChains], V0[kBitsChains], V1[kBitsChains], Q0[kBitsChains], Q1[kBitsChains];
-    const uint32_t A0 = seed * 0x9E3779B9u + threadIdx.x, A1 = A0 * 2654435761u;
-    uint32_t Rc0 = ~A0, Rc1 = A1 ^ 0x5bd1e995u, Rn0 = A0 ^ 0x27d4eb2fu, Rn1 = ~A1;
+    uint32_t H0[kBitsWords], H1[kBitsWords], V0[kBitsWords], V1[kBitsWords], B0[kBitsWords], B1[kBitsWords],
+        A0[kBitsWords], A1[kBitsWords];
+    uint32_t X0 = seed * 0x9E3779B9u + threadIdx.x, X1 = X0 * 2654435761u, Q0 = ~X0, Q1 = X1 ^ 0x5bd1e995u;
 #pragma unroll
-    for (int c = 0; c < kBitsChains; ++c) {
-        H0[c] = A0 >> c;
-        H1[c] = 0;
-        V0[c] = A1 >> c;
-        V1[c] = 0;
-        Q0[c] = Rc0 + c;
-        Q1[c] = Rn1 - c;
+    for (int w = 0; w < kBitsWords; ++w) {
+        A0[w] = X0 * (2u * w + 3u);
+        A1[w] = X1 * (2u * w + 5u);
+        B0[w] = ~A1[w];
+        B1[w] = A0[w] ^ 0x27d4eb2fu;
+        H0[w] = X0 >> w;
+        H1[w] = 0;
+        V0[w] = X1 >> w;
+        V1[w] = 0;
     }
     for (uint64_t it = 0; it < iters; ++it) {
 #pragma unroll
-        for (int c = 0; c < kBitsChains; ++c) {
-            const uint32_t bw0 = __funnelshift_l(Rn0, Rc0, c + 1), bw1 = __funnelshift_l(Rn1, Rc1, c + 1);
-            const uint32_t eq = lop3<kLutEq>(A0, bw0, A1 ^ bw1);
-            const uint32_t a0 = __funnelshift_l(Q0[c], H0[c], 1), a1 = __funnelshift_l(Q1[c], H1[c], 1);
-            bits_cell(eq, a0, a1, V0[c], V1[c], H0[c], H1[c], V0[c], V1[c]);
-            Q0[c] = __funnelshift_l(H0[c], Q0[c], 1);
-            Q1[c] = __funnelshift_l(H1[c], Q1[c], 1);
-        }
-        Rc0 = Rn0 ^ Rc0;  // keep the windows moving (two ops per step of 4 x 32 cells)
-        Rn1 = Rc1 + Rn1;
-    }
-    uint32_t acc = 0;
+        for (int u = 0; u < kBitsSteps; ++u) {
+            constexpr auto mod = [](int x) { return (x + kBitsWords) % kBitsWords; };
+            const int w0 = mod(u);
+            B0[w0] = __funnelshift_l(u ? mul(X0, 1u << u) : X0, B0[w0], 1);
+            B1[w0] = __funnelshift_l(u ? mul(X1, 1u << u) : X1, B1[w0], 1);
+            const uint32_t h0 = __funnelshift_l(Q0, H0[kBitsWords - 1], 1), h1 = __funnelshift_l(Q1, H1[kBitsWords - 1], 1);
 #pragma unroll
-    for (int c = 0; c < kBitsChains; ++c) acc ^= H0[c] ^ H1[c] ^ V0[c] ^ V1[c] ^ Q0[c] ^ Q1[c];
+            for (int w = kBitsWords - 1; w >= 0; --w) {
+                const uint32_t a0 = w ? H0[w ? w - 1 : 0] : h0, a1 = w ? H1[w ? w - 1 : 0] : h1;
+                const uint32_t eq = lop3<kLutEq>(A0[w], B0[mod(u - w)], A1[w] ^ B1[mod(u - w)]);
+                bits_cell(eq, a0, a1, V0[w], V1[w], H0[w], H1[w], V0[w], V1[w]);
+            }
+            Q0 = __funnelshift_l(H0[kBitsWords - 1], Q0, 1);
+            Q1 = __funnelshift_l(H1[kBitsWords - 1], Q1, 1);
+        }
+        X0 = muladd(X0, 16u, seed);  // (a constant entering: the windows keep moving)
+        X1 = muladd(X1, 16u, seed);
+    }
+    uint32_t acc = Q0 ^ Q1;
+#pragma unroll
+    for (int w = 0; w < kBitsWords; ++w) acc ^= H0[w] ^ H1[w] ^ V0[w] ^ V1[w];
     if (acc == 0x7f3a5c11u) *sink = (int32_t)acc;  // practically never true; keeps the work live
 }
 
@@ -163,9 +175,9 @@ extern "C" int nw_peak_int(nw_ctx *ctx, int kind, uint64_t iters, double *gops) 
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "peak kernel");
-    // kinds 5-7 count cells, kind 11 cells (32 per word step), the others
+    // kinds 5-7 count cells, kind 11 cells (32 per word and step), the others
     // instructions (per lane)
-    const double per = kind == 11 ? (double)kBitsChains * 32 : (double)kChains;
+    const double per = kind == 11 ? (double)kBitsWords * kBitsSteps * 32 : (double)kChains;
     const double ops = (double)ctx->sm_count * 8 * kPeakThreads * per * (double)iters;
     *gops = ms > 0 ? ops / (ms * 1e-3) / 1e9 : 0.0;
     return NW_OK;
