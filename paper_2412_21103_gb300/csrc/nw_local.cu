@@ -28,7 +28,8 @@
 // End cells and alignments.  The fill keeps no pointers and no positions: a
 // lane notes the first and the last chunk of 32 steps in which its rows reached
 // their largest H, and every kTileSteps steps the state of a stripe's lanes is
-// kept.  The trace finds the pair's best lane, recomputes those chunks for the
+// kept, with the largest H of the steps since the last one.  The trace finds the
+// pair's best lane, recomputes the tiles that reach its largest H for the
 // first cell in row-major order, and walks back from it tile by tile -- a tile
 // is one stripe and the steps between two kept states -- recomputing only the
 // tiles the path crosses (a warp each) with the two pointer bits in shared
@@ -47,6 +48,12 @@ constexpr int kLocalWarps = 8;
 constexpr uint32_t kLocalMinPeriod = 96;   // columns a stripe counts at least (the limit on a pair's size)
 constexpr uint32_t kTileSteps = 128;       // steps between a stripe's kept states
 constexpr int kTraceWarps = 3;             // tiles the trace replays at once
+// End cells without alignments: pairs of up to this many stripes keep states as
+// well.  Replaying a whole stripe on one warp takes about as long as the fill's
+// one stripe (1,000 pairs of 200 bases and 200 kb: 33 ms beside a fill of 22, with
+// states .25); from a dozen stripes on it is a quarter of the fill, and the
+// states would be most of the scratch.
+constexpr uint32_t kEndStripes = 4;
 constexpr uint32_t kPadProfile = 0x80808080u;  // rows past the end: s = -128, never above a real row
 
 struct LocalTask {
@@ -114,6 +121,7 @@ __device__ __forceinline__ uint32_t rows_codes(const uint8_t *s, uint32_t i0, ui
 template <int R>
 struct LocalLane {
     static constexpr uint32_t kParts = (R + 5) / 4;  // 16-byte parts of a kept state
+    static_assert(R % 4 == 0 && R + 2 < 4 * kParts, "the top is the third word of the last part");
     uint32_t prof[R];
     int32_t Hl[R], Gl[R];  // H of the column before, and with the gap's score added (in the fill)
     int32_t dtop;        // H of the row above the lane's first, one column back
@@ -149,12 +157,14 @@ struct LocalLane {
         dtop = 0;
         xout = 0;
     }
-    __device__ __forceinline__ void save(uint4 *k, uint64_t cap_left, uint32_t *err) const {
+    // top: the largest H of the lane's rows in the tile that ends here
+    __device__ __forceinline__ void save(uint4 *k, int32_t top, uint64_t cap_left, uint32_t *err) const {
         uint32_t v[4 * kParts] = {};
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = (uint32_t)Hl[r];
         v[R] = (uint32_t)dtop;
         v[R + 1] = xout;
+        v[R + 2] = (uint32_t)top;
 #pragma unroll
         for (uint32_t q = 0; q < kParts; ++q)
             if (in_range(q * 32u, cap_left, err, kSiteLocalPtr))
@@ -259,7 +269,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         if (jidx >= p.njobs) break;
         const LocalJob jb = p.jobs[jidx];
         const LocalTask tk = p.tasks[jb.task];
-        const uint32_t s = jb.stripe, m = tk.m, n = tk.n;
+        const uint32_t s = jb.stripe, m = tk.m, n = tk.n, keep_n = MODE == kKeep ? tk.keep_n : 0u;
         if (m == 0 || n == 0) {  // a single job: the score stays 0
             if (MODE != kScore && lane == 0) p.best[jidx] = LocalBest{0, 0u, 0u, 0u};
             continue;
@@ -282,6 +292,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         uint4 *keep = MODE == kKeep ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * LocalLane<R>::kParts * 32u + lane
                                     : nullptr;
         int32_t best = 0, cm = 0;    // the lane's largest H before and in this chunk of 32 steps
+        int32_t top = 0;             // ... in this tile
         uint32_t bt = 0, bl = 0;     // the first and the last chunk that reached it
         int32_t c = -lane;
         uint32_t seen = 0;
@@ -299,8 +310,9 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
             if (lane == 0) st_release(mine, min(t - 31u, n));
         };
         for (uint32_t t = 0; t < T && alive; t += 32) {
-            if (MODE == kKeep && t && t % kTileSteps == 0) {
-                ln.save(keep, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
+            if (MODE == kKeep && keep_n && t && t % kTileSteps == 0) {
+                ln.save(keep, top, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
+                top = 0;
                 keep += LocalLane<R>::kParts * 32u;
             }
             __syncwarp();
@@ -335,17 +347,18 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
                 if (cm > best) bt = t;
                 if (cm >= best) bl = t;
                 best = max(best, cm);
+                if (MODE == kKeep) top = max(top, cm);
                 cm = 0;
             }
         }
         if (!alive) return;   // a wait gave up (NW_ERR_TIMEOUT is raised): leave
         if (MODE == kScore) best = cm;
         // the stripe's largest H and its first lane
-        const int32_t top = __reduce_max_sync(kFull, best);
-        if (lane == 0 && top > 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) atomicMax(p.scores + tk.out, top);
+        const int32_t most = __reduce_max_sync(kFull, best);
+        if (lane == 0 && most > 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) atomicMax(p.scores + tk.out, most);
         if (MODE != kScore) {
-            const uint32_t first = (uint32_t)__ffs(__ballot_sync(kFull, best == top)) - 1u;
-            if ((uint32_t)lane == first) p.best[jidx] = LocalBest{top, first, bt, bl};
+            const uint32_t first = (uint32_t)__ffs(__ballot_sync(kFull, best == most)) - 1u;
+            if ((uint32_t)lane == first) p.best[jidx] = LocalBest{most, first, bt, bl};
         }
         __syncwarp();
     }
@@ -414,8 +427,14 @@ struct LocalReplay {
 // about 2.3 tiles of a stripe), then the first warp follows the path to the first cell whose H is 0;
 // moves in reverse order (0 diagonal, 1 vertical, 2 horizontal).  A run of
 // diagonal moves is taken at a time: lane q reads the cell q diagonal moves
-// on, and H there follows from the matches before it (a ballot).  Without
-// WALK no states are kept: a stripe is replayed from its start.
+// on, and H there follows from the matches before it (a ballot).  A pair without
+// kept states (of end cells alone, or of few columns) replays its stripe from
+// the start.
+//
+// Where the best lane reaches its largest H again far on -- a read against a long
+// reference, one stripe of many tiles -- only the tiles that do are replayed:
+// 1,000 pairs of 200 bases and 200 kb .18 ms of trace, with every step from the
+// first to the last of them 35.
 template <int R, bool WALK>
 __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(LocalArgs p, uint32_t ntasks,
                                                                               uint8_t *moves, const uint64_t *move_off,
@@ -424,6 +443,7 @@ __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(Lo
     constexpr uint32_t SH = 32u * R;
     extern __shared__ uint4 tiles_[];  // [tile][step][lane]
     __shared__ int32_t at[3];          // i, j, h between the warps
+    __shared__ uint32_t first_[R];
     typename Bits::Word *tiles = reinterpret_cast<typename Bits::Word *>(tiles_);
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     for (uint32_t q = blockIdx.x; q < ntasks; q += gridDim.x) {
@@ -442,13 +462,46 @@ __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(Lo
         }
         uint32_t i = 0, j = 0;
         LocalReplay<R> rp;
-        if (bv > 0 && warp == 0) {
+        if (bv > 0) {
             // the first cell in row-major order among the best lane's rows
             const LocalBest b = p.best[tk.job0 + bs];
             const uint32_t lo = b.t0, hi = min(b.t1 + 32u, n + 31u);
-            if (!WALK && p.turn) {
-                // the rows above were overwritten: sweep the stripes above again
-                for (uint32_t s = 0; s < bs; ++s) {
+            uint32_t first[R];  // by row, the first column found
+#pragma unroll
+            for (int r = 0; r < R; ++r) first[r] = ~0u;
+            const auto look = [&](uint32_t end) {
+                while (rp.t < end) {
+                    const uint32_t t = rp.t;
+                    const bool act = rp.template step<false>(p.gap, lane);
+                    if (act && t >= lo && lane == b.lane) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            if (rp.ln.Hl[r] == bv && first[r] == ~0u) first[r] = t - lane;
+                    }
+                }
+            };
+            if (threadIdx.x < (uint32_t)R) first_[threadIdx.x] = ~0u;
+            __syncthreads();
+            if (p.keep && tk.keep_n) {
+                // the tiles that reach the largest H, dealt out to the warps
+                constexpr uint32_t kParts = LocalLane<R>::kParts;
+                const uint4 *tops = p.keep + tk.keep_off + ((uint64_t)bs * tk.keep_n * kParts + kParts - 1u) * 32u + b.lane;
+                const uint32_t last = b.t1 / kTileSteps;
+                uint32_t turn = 0;
+                for (uint32_t k0 = lo / kTileSteps; k0 <= last; k0 += 32) {
+                    const uint32_t tl = k0 + lane;
+                    const bool has = tl == last || (tl < last && (int32_t)__ldcg(tops + (size_t)tl * (kParts * 32u)).z == bv);
+                    for (uint32_t todo = __ballot_sync(kFull, has); todo; todo &= todo - 1u)
+                        if (turn++ % (blockDim.x >> 5) == warp) {
+                            const uint32_t t0 = (k0 + (uint32_t)__ffs(todo) - 1u) * kTileSteps;
+                            rp.begin(p, tk, bs, t0, lane);
+                            look(min(t0 + kTileSteps, hi));
+                        }
+                }
+            } else {
+                // no states: the stripe from its start, and where only two rows
+                // are kept (the rows above were overwritten) the stripes above it
+                for (uint32_t s = 0; p.turn && s < bs; ++s) {
                     rp.begin(p, tk, s, 0u, lane);
                     uint32_t *out = p.rows + tk.row_off + (size_t)(s & 1u) * tk.nr;
                     while (rp.t < n + 31u) {
@@ -458,28 +511,21 @@ __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(Lo
                     __threadfence();
                     __syncwarp();
                 }
+                rp.begin(p, tk, bs, 0u, lane);
+                look(hi);
             }
-            rp.begin(p, tk, bs, WALK ? lo - lo % kTileSteps : 0u, lane);
-            uint32_t first[R];
+            if (lane == b.lane) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) first[r] = ~0u;
-            while (rp.t < hi) {
-                const uint32_t t = rp.t;
-                const bool act = rp.template step<false>(p.gap, lane);
-                if (act && t >= lo && lane == b.lane) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        if (rp.ln.Hl[r] == bv && first[r] == ~0u) first[r] = t - lane;
-                }
+                for (int r = 0; r < R; ++r)
+                    if (first[r] != ~0u) atomicMin(&first_[r], first[r]);
             }
+            __syncthreads();
 #pragma unroll
             for (int r = R - 1; r >= 0; --r)
-                if (first[r] != ~0u) {
-                    i = bs * SH + lane * R + (uint32_t)r + 1u;
-                    j = first[r] + 1u;
+                if (first_[r] != ~0u) {
+                    i = bs * SH + b.lane * R + (uint32_t)r + 1u;
+                    j = first_[r] + 1u;
                 }
-            i = __shfl_sync(kFull, i, b.lane);
-            j = __shfl_sync(kFull, j, b.lane);
         }
         if (threadIdx.x == 0 && in_range(tk.out, p.out_cap, p.err, kSiteLocalOut)) {
             p.ends[4 * (size_t)tk.out + 2] = i;
@@ -566,7 +612,7 @@ __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(Lo
 }
 
 template <int R, int MODE>
-int launch_local_R(nw_ctx *ctx, LocalArgs &la) {
+int launch_local_R(nw_ctx *ctx, const char *name, LocalArgs &la) {
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local<R, MODE>, kLocalWarps * 32, 0);
     if (occ < 1) occ = 1;
@@ -579,17 +625,17 @@ int launch_local_R(nw_ctx *ctx, LocalArgs &la) {
     if (rc) return rc;
     la.counter = (uint32_t *)v;
     cudaMemsetAsync(la.counter, 0, 4, ctx->stream);
-    LaunchTimer t(ctx, MODE == kKeep ? "local_fill_ptr" : (MODE == kEnds ? "local_score_pos" : "local_score"));
+    LaunchTimer t(ctx, name);
     k_local<R, MODE><<<blocks, kLocalWarps * 32, 0, ctx->stream>>>(la);
     return NW_OK;
 }
 
-int launch_local(nw_ctx *ctx, int R, LocalMode mode, LocalArgs &la) {
-#define NW_LOCAL_CASES(MODEV)                                    \
-    switch (R) {                                                 \
-        case 4: return launch_local_R<4, MODEV>(ctx, la);        \
-        case 16: return launch_local_R<16, MODEV>(ctx, la);      \
-        default: return launch_local_R<8, MODEV>(ctx, la);       \
+int launch_local(nw_ctx *ctx, int R, LocalMode mode, const char *name, LocalArgs &la) {
+#define NW_LOCAL_CASES(MODEV)                                         \
+    switch (R) {                                                      \
+        case 4: return launch_local_R<4, MODEV>(ctx, name, la);       \
+        case 16: return launch_local_R<16, MODEV>(ctx, name, la);     \
+        default: return launch_local_R<8, MODEV>(ctx, name, la);      \
     }
     if (mode == kKeep) NW_LOCAL_CASES(kKeep)
     if (mode == kEnds) NW_LOCAL_CASES(kEnds)
@@ -649,7 +695,7 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     int R = 8;
     if (const char *e = getenv("NW_LOCAL_R")) R = atoi(e) == 4 ? 4 : atoi(e) == 16 ? 16 : 8;
     const uint32_t SH = 32u * R;
-    const LocalMode mode = want ? kKeep : ends ? kEnds : kScore;
+    LocalMode mode = want ? kKeep : ends ? kEnds : kScore;
     LocalArgs la{};
     la.pool = pool;
     local_profile(sc, la.prof);
@@ -660,6 +706,12 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     la.ends = ends;
     la.err = ctx->d_err;
     la.out_cap = npairs;
+    // Waves that fit a third of the free budget with all they take: stripe rows,
+    // kept states, and the moves and tables, which are most of it for short
+    // pairs.  A third, because the slots keep the largest size of every wave.
+    const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 3;
+    const uint32_t state_units = ((uint32_t)R + 5u) / 4u * 32u;  // 16-byte units of a kept state
+    uint64_t kept = 0;
     std::vector<LocalTask> all(npairs);
     for (uint32_t k = 0; k < npairs; ++k) {
         LocalTask &t = all[k];
@@ -669,8 +721,15 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
             return fail(ctx, NW_ERR_UNSUPPORTED, "pair %u too large for one warp (m*n/%u >= 2^31)", k, SH);
         t.nr = (t.n + 31) / 32 * 32;
         // states before steps kTileSteps, 2 kTileSteps, .. of a stripe's n + 31
-        if (want && t.m && t.n) t.keep_n = (t.n + 30) / kTileSteps;
+        const uint32_t S = (t.m + SH - 1) / SH, states = t.m && t.n ? (t.n + 30) / kTileSteps : 0;
+        if (want || (ends && S <= kEndStripes)) t.keep_n = states;
+        kept += want ? 0 : (uint64_t)S * t.keep_n * state_units * 16;
     }
+    // End cells alone: the states of pairs of few stripes, where they fit.
+    if (mode == kEnds && kept > wave_budget / 2)
+        for (LocalTask &t : all) t.keep_n = 0;
+    else if (mode == kEnds && kept)
+        mode = kKeep;
     // longest first (the atomic queue then balances the tail)
     std::stable_sort(all.begin(), all.end(), [](const LocalTask &x, const LocalTask &y) {
         return (uint64_t)x.m * x.n > (uint64_t)y.m * y.n;
@@ -678,12 +737,8 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     int rc;
     cudaError_t e0 = cudaMemsetAsync(scores, 0, (size_t)npairs * 4, ctx->stream);  // the stripes' maxima are merged
     if (e0 != cudaSuccess) return cuda_fail(ctx, e0, "local scores reset");
-    // Waves that fit a third of the free budget with all they take: stripe rows,
-    // kept states, and the moves and tables, which are most of it for short
-    // pairs.  A third, because the slots keep the largest size of every wave.
-    const uint64_t wave_budget = (ctx->budget - std::min(ctx->budget, ctx->used)) / 3;
+    const bool ends_only = !want && mode != kScore;
     const uint64_t per_job = sizeof(LocalJob) + 4 + (mode == kScore ? 0 : sizeof(LocalBest));
-    const uint32_t state_units = ((uint32_t)R + 5u) / 4u * 32u;  // 16-byte units of a kept state
     size_t k0 = 0;
     while (k0 < all.size()) {
         std::vector<LocalTask> wave;
@@ -695,18 +750,20 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         for (; k < all.size(); ++k) {
             LocalTask t = all[k];
             const uint32_t S = (t.m && t.n) ? (t.m + SH - 1) / SH : 1;
-            const uint64_t u = (uint64_t)S * t.keep_n * state_units;
+            uint64_t u = (uint64_t)S * t.keep_n * state_units;
             uint64_t rw = (uint64_t)(mode == kScore ? std::min(S - 1, 2u) : S - 1) * t.nr;
             const uint64_t tables = sizeof(LocalTask) + S * per_job +
                                     (want ? t.m + t.n + 16 + 2 * sizeof(uint64_t) + sizeof(TraceTask) : 0);
             const uint64_t more = u * 16 + rw * 4 + tables;
-            if (!wave.empty() && ((turn && mode == kEnds) || bytes + more > wave_budget)) break;
+            if (!wave.empty() && ((turn && ends_only) || bytes + more > wave_budget)) break;
             bytes += more;
             // a lone pair whose rows alone exceed the budget keeps two and
             // finds its end cell by sweeping the stripes above it again
-            if (mode == kEnds && wave.empty() && rw * 4 + tables + (64u << 10) > scratch_headroom(ctx, "local_rows")) {
+            if (ends_only && wave.empty() && rw * 4 + tables + (64u << 10) > scratch_headroom(ctx, "local_rows")) {
                 turn = true;
                 rw = (uint64_t)std::min(S - 1, 2u) * t.nr;
+                t.keep_n = 0;  // (a replay from a state reads the row above, which may be overwritten)
+                u = 0;
             }
             t.keep_off = units;
             t.row_off = rows;
@@ -722,8 +779,8 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         if ((rc = scratch(ctx, "local_rows", rows * 4 + 16, &rv))) return rc;
         if ((rc = scratch(ctx, "local_progress", jobs.size() * 4 + 16, &pv))) return rc;
         if (mode != kScore && (rc = scratch(ctx, "local_best", jobs.size() * sizeof(LocalBest) + 16, &bv))) return rc;
+        if (mode == kKeep && (rc = scratch(ctx, "local_keep", units * 16 + 16, &kv))) return rc;
         if (want) {
-            if ((rc = scratch(ctx, "local_keep", units * 16 + 16, &kv))) return rc;
             if ((rc = scratch(ctx, "local_moves", mbytes + 16, &mv))) return rc;
             if ((rc = scratch(ctx, "local_nmoves", wave.size() * 8 + 16, &nm))) return rc;
         }
@@ -753,8 +810,9 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         la.keep_cap = units;
         const uint32_t nt = (uint32_t)wave.size();
         k0 = k;
-        if ((rc = launch_local(ctx, R, mode, la))) return rc;
-        if (mode == kEnds && (rc = launch_local_trace<false>(ctx, R, la, nt, nullptr, nullptr, nullptr))) return rc;
+        if ((rc = launch_local(ctx, R, mode, want ? "local_fill_ptr" : ends_only ? "local_score_pos" : "local_score", la)))
+            return rc;
+        if (ends_only && (rc = launch_local_trace<false>(ctx, R, la, nt, nullptr, nullptr, nullptr))) return rc;
         if (!want) continue;
         if ((rc = launch_local_trace<true>(ctx, R, la, nt, (uint8_t *)mv, dmoff, (uint64_t *)nm))) return rc;
         std::vector<TraceTask> tt(wave.size());
