@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "nw_internal.cuh"
+#include "nw_order.h"
 
 namespace nw {
 namespace {
@@ -667,16 +668,20 @@ int launch_local_trace(nw_ctx *ctx, int R, const LocalArgs &la, uint32_t ntasks,
     return launch_local_trace_R<8, WALK>(ctx, la, ntasks, moves, move_off, nmoves);
 }
 
+// (the caller waits for the copy: uploaded)
 template <typename T>
 int upload_vec(nw_ctx *ctx, const char *slot, const std::vector<T> &v, T **dev) {
     void *d = nullptr;
     int rc = to_device(ctx, v.data(), v.size() * sizeof(T), slot, &d);
     if (rc) return rc;
-    // the host vector may be freed right after: wait for the copy
-    cudaError_t e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "task upload sync");
     *dev = (T *)d;
     return NW_OK;
+}
+
+// Waits for the copies of host vectors that the caller is about to free.
+int uploaded(nw_ctx *ctx) {
+    const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+    return e == cudaSuccess ? NW_OK : cuda_fail(ctx, e, "task upload sync");
 }
 
 // Row profiles of the plain scores s (the global kernels use s - 2*gap).
@@ -731,9 +736,9 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
     else if (mode == kEnds && kept)
         mode = kKeep;
     // longest first (the atomic queue then balances the tail)
-    std::stable_sort(all.begin(), all.end(), [](const LocalTask &x, const LocalTask &y) {
-        return (uint64_t)x.m * x.n > (uint64_t)y.m * y.n;
-    });
+    std::vector<uint64_t> cells(npairs);
+    for (uint32_t q = 0; q < npairs; ++q) cells[q] = (uint64_t)all[q].m * all[q].n;
+    const std::vector<uint32_t> order = radix_order_desc(std::move(cells));
     int rc;
     cudaError_t e0 = cudaMemsetAsync(scores, 0, (size_t)npairs * 4, ctx->stream);  // the stripes' maxima are merged
     if (e0 != cudaSuccess) return cuda_fail(ctx, e0, "local scores reset");
@@ -747,8 +752,11 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         uint64_t units = 0, rows = 0, mbytes = 0, bytes = 0;
         bool turn = mode == kScore;  // rows: two in turn
         size_t k = k0;
+        wave.reserve(all.size() - k0);
+        jobs.reserve(all.size() - k0);
+        if (want) moff.reserve(all.size() - k0);
         for (; k < all.size(); ++k) {
-            LocalTask t = all[k];
+            LocalTask t = all[order[k]];
             const uint32_t S = (t.m && t.n) ? (t.m + SH - 1) / SH : 1;
             uint64_t u = (uint64_t)S * t.keep_n * state_units;
             uint64_t rw = (uint64_t)(mode == kScore ? std::min(S - 1, 2u) : S - 1) * t.nr;
@@ -771,7 +779,7 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
             for (uint32_t s = 0; s < S; ++s) jobs.push_back(LocalJob{(uint32_t)wave.size(), s});
             units += u;
             rows += rw;
-            moff.push_back(mbytes);
+            if (want) moff.push_back(mbytes);
             mbytes += (uint64_t)t.m + t.n + 16;
             wave.push_back(t);
         }
@@ -798,6 +806,7 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
         if ((rc = upload_vec(ctx, "local_tasks", wave, &dt))) return rc;
         if ((rc = upload_vec(ctx, "local_jobs", jobs, &dj))) return rc;
         if (want && (rc = upload_vec(ctx, "local_move_off", moff, &dmoff))) return rc;
+        if ((rc = uploaded(ctx))) return rc;
         la.tasks = dt;
         la.jobs = dj;
         la.njobs = (uint32_t)jobs.size();
@@ -832,7 +841,7 @@ int local_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const 
             tt[q] = x;
         }
         TraceTask *dtt = nullptr;
-        if ((rc = upload_vec(ctx, "local_trace_tasks", tt, &dtt))) return rc;
+        if ((rc = upload_vec(ctx, "local_trace_tasks", tt, &dtt)) || (rc = uploaded(ctx))) return rc;
         if ((rc = launch_finish(ctx, tt[0], dtt, (uint32_t)tt.size(), (flags & NW_CIGAR_M) ? 1u : 0u))) return rc;
     }
     cudaError_t e = cudaGetLastError();
