@@ -251,7 +251,7 @@ struct LocalAbove {
 // cells, and waits for the stripe above.  4,000 pairs of 2 to 10 kb: 9.8 ms;
 // with max, add and add-max per cell (3.5 operations) 12.4, with a prmt for
 // every row 10.7, for half of them 10.3.
-template <int R, int MODE>
+template <int R, int MODE, bool TAB>
 __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
     constexpr uint32_t SH = 32u * R;
     const int lane = threadIdx.x & 31;
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
     // a chunk's inputs of lane 0 and outputs of lane 31, per warp
     __shared__ uint32_t ins_[kLocalWarps][32], outs_[kLocalWarps][32];
     uint32_t *ins = ins_[threadIdx.x >> 5], *outs = outs_[threadIdx.x >> 5];
-    constexpr int kTab = 4 * LocalLane<R>::kTabRows / 4 * 32;  // a warp's scores, [base][four rows][lane]
+    constexpr int kTab = TAB ? 4 * LocalLane<R>::kTabRows / 4 * 32 : 0;  // a warp's scores, [base][four rows][lane]
     __shared__ int4 tabs_[kTab ? kLocalWarps * kTab : 1];
     int4 *tab = tabs_ + (kTab ? (threadIdx.x >> 5) * kTab + lane : 0);
 
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         LocalLane<R> ln;
         const uint32_t i0 = s * SH + (uint32_t)lane * R;
         ln.rows(p, p.pool + tk.a_off, i0, m);
-        ln.table(tab);
+        if constexpr (TAB) ln.table(tab);
         ln.start(p.gap);
         uint4 *keep = MODE == kKeep ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * LocalLane<R>::kParts * 32u + lane
                                     : nullptr;
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
                     uint32_t x = __shfl_up_sync(kFull, ln.xout, 1);
                     const uint32_t in = ins[uu];
                     if (lane == 0) x = in;
-                    ln.template column<false, true>(g, x, cm, tab);
+                    ln.template column<false, TAB>(g, x, cm, tab);
                     if (lane == 31) outs[uu] = ln.xout;
                 }
                 c += 32;
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
                     const uint32_t in = ins[uu];
                     if (lane == 0) x = in;
                     if (c >= 0 && c < (int32_t)n) {
-                        ln.template column<false, true>(g, x, cm, tab);
+                        ln.template column<false, TAB>(g, x, cm, tab);
                         if (lane == 31) outs[uu] = ln.xout;
                     }
                     ++c;
@@ -612,10 +612,10 @@ __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(Lo
     }
 }
 
-template <int R, int MODE>
+template <int R, int MODE, bool TAB>
 int launch_local_R(nw_ctx *ctx, const char *name, LocalArgs &la) {
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local<R, MODE>, kLocalWarps * 32, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_local<R, MODE, TAB>, kLocalWarps * 32, 0);
     if (occ < 1) occ = 1;
     // every CTA resident: a job's warp may wait on an earlier job's warp
     uint32_t blocks = (uint32_t)occ * (uint32_t)ctx->sm_count;
@@ -627,16 +627,23 @@ int launch_local_R(nw_ctx *ctx, const char *name, LocalArgs &la) {
     la.counter = (uint32_t *)v;
     cudaMemsetAsync(la.counter, 0, 4, ctx->stream);
     LaunchTimer t(ctx, name);
-    k_local<R, MODE><<<blocks, kLocalWarps * 32, 0, ctx->stream>>>(la);
+    k_local<R, MODE, TAB><<<blocks, kLocalWarps * 32, 0, ctx->stream>>>(la);
     return NW_OK;
 }
 
 int launch_local(nw_ctx *ctx, int R, LocalMode mode, const char *name, LocalArgs &la) {
-#define NW_LOCAL_CASES(MODEV)                                         \
-    switch (R) {                                                      \
-        case 4: return launch_local_R<4, MODEV>(ctx, name, la);       \
-        case 16: return launch_local_R<16, MODEV>(ctx, name, la);     \
-        default: return launch_local_R<8, MODEV>(ctx, name, la);      \
+    // Scores from shared memory (TAB) take 8 operations a column off the logic pipe
+    // and put a shared load into the column's chain: they pay from about three
+    // warps per scheduler on.  Pairs of 200 bases and 50 kb, table / permutes: 50 to
+    // 1,200 pairs 5.5 / 4.9 ms, 2,400 6.9 / 7.5, 4,800 12.9 / 14.3; 100 pairs of 3 kb
+    // (1,200 jobs) .87 / .83, 500 (6,000) 1.47 / 1.71.
+    const bool tab = la.njobs > 12u * (uint32_t)ctx->sm_count;
+#define NW_LOCAL_CASES(MODEV)                                                      \
+    switch (R) {                                                                   \
+        case 4: return launch_local_R<4, MODEV, false>(ctx, name, la);             \
+        case 16: return launch_local_R<16, MODEV, true>(ctx, name, la);            \
+        default: return tab ? launch_local_R<8, MODEV, true>(ctx, name, la)        \
+                            : launch_local_R<8, MODEV, false>(ctx, name, la);      \
     }
     if (mode == kKeep) NW_LOCAL_CASES(kKeep)
     if (mode == kEnds) NW_LOCAL_CASES(kEnds)
