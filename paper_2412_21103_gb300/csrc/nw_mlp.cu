@@ -34,6 +34,7 @@ constexpr int kNW1 = kH * kF, kNB1 = kH, kNW2 = kH * kH, kNB2 = kH, kNW3 = kH, k
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kNW1, kOffW2 = kOffB1 + kNB1, kOffB2 = kOffW2 + kNW2,
               kOffW3 = kOffB2 + kNB2, kOffB3 = kOffW3 + kNW3, kNParams = kOffB3 + kNB3;
 constexpr int kAnchors = 256, kBins = 64;
+constexpr int kShortWindow = 256;  // offsets of a window whose matches are counted one by one (k_features)
 
 struct BandModel {
     float *master = nullptr;      // kNParams
@@ -53,6 +54,11 @@ struct BandModel {
 // of them, its count a population count and one warp-wide sum, with no atomics
 // and no division per match.
 //
+// The flush of the 64 bins takes about as long as 8 words with a match at every
+// position, so a window of up to kShortWindow offsets (sequences under 1,024
+// bases) takes its matches one by one: 100,000 pairs of 50 to 150 bases .50 ms, with
+// the flush 1.52; byte by byte .47.
+//
 // One byte per position, compared four at a time, the matches taken out one by
 // one with a 64-bit division each and added by atomics: 2.37 ms for 10,000
 // pairs of 2 to 20 kb; this form 0.53 ms.
@@ -62,7 +68,8 @@ __device__ __forceinline__ void letter_words(const uint2 v, const uint32_t (&c0)
     for (int k = 0; k < 4; ++k) E[k] = ~((v.x ^ c0[k]) | (v.y ^ c1[k]));
 }
 
-__global__ void __launch_bounds__(kAnchors) k_features(const uint8_t *pool, const uint64_t *a_off,
+template <int CTAS>
+__global__ void __launch_bounds__(kAnchors, CTAS) k_features(const uint8_t *pool, const uint64_t *a_off,
                                                        const uint32_t *a_len, const uint64_t *b_off,
                                                        const uint32_t *b_len, uint32_t npairs, float *feat) {
     extern __shared__ uint2 bpl[];  // the bit planes of B, 32 bases an element
@@ -92,7 +99,9 @@ __global__ void __launch_bounds__(kAnchors) k_features(const uint8_t *pool, cons
         const uint32_t K = ok ? min((uint32_t)kAnchors, m - 3) : 0;
         if ((threadIdx.x & ~31u) < K) {  // a warp with an anchor
             const bool live = threadIdx.x < K;
-            const uint32_t i = live && K > 1 ? (uint32_t)(((uint64_t)threadIdx.x * (m - 4)) / (K - 1)) : 0u;
+            uint32_t i = 0;  // (in 32 bits where it fits: the division takes a third of the instructions)
+            if (live && K > 1)
+                i = m < (1u << 24) ? threadIdx.x * (m - 4) / (K - 1) : (uint32_t)(((uint64_t)threadIdx.x * (m - 4)) / (K - 1));
             uint32_t c0[4], c1[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -119,40 +128,60 @@ __global__ void __launch_bounds__(kAnchors) k_features(const uint8_t *pool, cons
                 return E[0] & __funnelshift_r(E[1], F[1], 1) & __funnelshift_r(E[2], F[2], 2) &
                        __funnelshift_r(E[3], F[3], 3) & valid;
             };
-            const int64_t D = 2 * (int64_t)W + 1;
-            uint32_t bin = (uint32_t)((int64_t)t * 32 * kBins / D);
-            const auto bin_end = [&](uint32_t b) { return (int32_t)(((int64_t)(b + 1) * D + kBins - 1) / kBins); };
-            int32_t end = bin_end(bin);  // the first d past the bin
-            uint32_t acc = 0, h0 = 0, h1 = 0;
-            const auto flush = [&] {
-                const uint32_t sum = __reduce_add_sync(~0u, acc);
-                if (lane == (bin & 31u)) (bin < 32u ? h0 : h1) = sum;
-            };
-            uint32_t E[4], F[4];
-            letter_words(planes(w), c0, c1, E);
-            letter_words(planes(w + 1), c0, c1, F);
-            uint32_t M = match(w, E, F);
-            for (; 32 * t <= dhi; ++t) {
-                ++w;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) E[k] = F[k];
+            // f(t, x): the match bits of offsets 32 t .. 32 t + 31
+            const auto words = [&](auto f) {
+                uint32_t E[4], F[4];
+                letter_words(planes(w), c0, c1, E);
                 letter_words(planes(w + 1), c0, c1, F);
-                const uint32_t N = match(w, E, F);
-                uint32_t x = __funnelshift_r(M, N, s);  // offsets 32 t .. 32 t + 31
-                M = N;
-                while (bin < (uint32_t)kBins && end <= 32 * t + 32) {
-                    const uint32_t in = ~0u >> (32 * t + 32 - end);  // end > 32 t
-                    acc += __popc(x & in);
-                    x &= ~in;
-                    flush();
-                    acc = 0;
-                    end = bin_end(++bin);
+                uint32_t M = match(w, E, F);
+                for (; 32 * t <= dhi; ++t) {
+                    ++w;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) E[k] = F[k];
+                    letter_words(planes(w + 1), c0, c1, F);
+                    const uint32_t N = match(w, E, F);
+                    f(t, __funnelshift_r(M, N, s));
+                    M = N;
                 }
-                acc += __popc(x);
+            };
+            if (2 * W + 1 <= kShortWindow) {
+                // A short window has fewer matches than bins: each is taken by
+                // itself.  Its bin is floor(64 d / D), from a multiply by 1 / D:
+                // 64 d + 0.5 keeps at least 0.5 / D = 2^-9 from the next whole number,
+                // the rounding is below 2^-17.
+                const uint32_t D = 2u * (uint32_t)W + 1u;
+                const float inv = 1.f / (float)D;
+                words([&](int32_t at, uint32_t x) {
+                    for (; x; x &= x - 1) {
+                        const uint32_t d = 32u * (uint32_t)at + (uint32_t)__ffs(x) - 1u;
+                        if (d < D) atomicAdd(&hist[(uint32_t)(((float)(d * kBins) + 0.5f) * inv)], 1u);
+                    }
+                });
+            } else {
+                const int64_t D = 2 * (int64_t)W + 1;
+                uint32_t bin = (uint32_t)((int64_t)t * 32 * kBins / D);
+                const auto bin_end = [&](uint32_t b) { return (int32_t)(((int64_t)(b + 1) * D + kBins - 1) / kBins); };
+                int32_t end = bin_end(bin);  // the first d past the bin
+                uint32_t acc = 0, h0 = 0, h1 = 0;
+                const auto flush = [&] {
+                    const uint32_t sum = __reduce_add_sync(~0u, acc);
+                    if (lane == (bin & 31u)) (bin < 32u ? h0 : h1) = sum;
+                };
+                words([&](int32_t at, uint32_t x) {
+                    while (bin < (uint32_t)kBins && end <= 32 * at + 32) {
+                        const uint32_t in = ~0u >> (32 * at + 32 - end);  // end > 32 t
+                        acc += __popc(x & in);
+                        x &= ~in;
+                        flush();
+                        acc = 0;
+                        end = bin_end(++bin);
+                    }
+                    acc += __popc(x);
+                });
+                if (bin < (uint32_t)kBins) flush();
+                if (h0) atomicAdd(&hist[lane], h0);
+                if (h1) atomicAdd(&hist[lane + 32], h1);
             }
-            if (bin < (uint32_t)kBins) flush();
-            if (h0) atomicAdd(&hist[lane], h0);
-            if (h1) atomicAdd(&hist[lane + 32], h1);
         }
         __syncthreads();
         if (threadIdx.x < kBins) {
@@ -539,13 +568,18 @@ static int launch_features(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_o
                            const uint64_t *b_off, const uint32_t *b_len, uint32_t npairs, uint32_t maxn, float *feat) {
     // (the default limit counts the kernel's static words too)
     if (feature_bytes(maxn) + kBins * sizeof(uint32_t) > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_features, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        const cudaError_t e = cudaFuncSetAttribute(k_features<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)feature_bytes(kFeatMaxB));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "feature kernel shared memory");
     }
     {
         LaunchTimer t(ctx, "features");
-        k_features<<<std::min<uint32_t>(npairs, (uint32_t)ctx->sm_count * 8), kAnchors, feature_bytes(maxn),
+        // Short pairs are a chain of loads and barriers, so an SM holds eight CTAs (32
+        // registers a thread, a few spilled); longer ones take the 48 registers.
+        // 100,000 pairs of 50 to 150 bases .50 ms against .71; 10,000 of 2 kb .38 against
+        // .37.
+        const auto kern = maxn < 1024 ? k_features<8> : k_features<1>;
+        kern<<<std::min<uint32_t>(npairs, (uint32_t)ctx->sm_count * 8), kAnchors, feature_bytes(maxn),
                      ctx->stream>>>(pool, a_off, a_len, b_off, b_len, npairs, feat);
     }
     const cudaError_t e = cudaGetLastError();
