@@ -610,17 +610,18 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
     if (want) {
         free_prefix(ctx, "batch_ptr");
         free_prefix(ctx, "ptr");
-        // the bit-sliced kernels' records too, where they hold more than a
-        // quarter of what is left (else the fallback finds its slots as it
-        // left them)
-        uint64_t held = 0;
-        for (const char *name : {"bgroup_rec", "bpair_rec"})
-            if (const auto it = ctx->bufs.find(name); it != ctx->bufs.end()) held += it->second.cap;
-        if (held > (ctx->budget - std::min(ctx->budget, ctx->used)) / 4) {
-            free_prefix(ctx, "bgroup_rec");
-            free_prefix(ctx, "bpair_rec");
-        }
     }
+    // The bit-sliced kernels' records only when a pair does not fit beside them:
+    // the fallback takes them again, and memory freed here and reused in smaller
+    // parts would have to be mapped anew for it, call after call (a server's
+    // workers, whose budgets are small: 5 to 15% of a burst).
+    bool handed_back = !want;
+    const auto hand_back = [&] {
+        if (handed_back) return false;
+        free_prefix(ctx, "bgroup_rec");
+        free_prefix(ctx, "bpair_rec");
+        return handed_back = true;
+    };
     // the paper's scoring (s' = 3 on a match, 1 on a mismatch) runs on the
     // bit-sliced window kernel, from a planar copy of the pool;
     // NW_BAND_SCALAR=1 keeps every round on the scalar banded kernel (for
@@ -669,7 +670,8 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
             band_task(t, R, w);
             // (a banded cell costs about what a full-grid cell costs, so the
             // band pays off up to ~85% of the grid)
-            if (band_cells(t, R) * 20 >= full_cells(t, R) * 17 || (!use_bits && !words_fit(t))) {
+            if (band_cells(t, R) * 20 >= full_cells(t, R) * 17 ||
+                (!use_bits && !words_fit(t) && !(hand_back() && words_fit(t)))) {
                 rest.push_back(id);
                 continue;
             }
@@ -682,6 +684,7 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
             std::vector<uint32_t> iw, keep_w;
             std::vector<BatchTask> keep;
             const int max_q = band_bits_max_q();
+            uint64_t wave_budget = bits_wave_budget(ctx);
             for (size_t q = 0; q < tasks.size(); ++q) {
                 const BatchTask &t = tasks[q];
                 BandBitsShape sh;
@@ -702,14 +705,18 @@ static int band_rounds(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, 
                 }
                 if (band_bits_shape(tb.m, tb.n, tb.lo, tb.hi, &sh, max_q)) {
                     // (a pair that even alone leaves its walk no scratch)
-                    if (want && band_bits_scratch(tb.m, tb.n, sh) > bits_wave_budget(ctx)) {
-                        rest.push_back(t.out0);
-                        continue;
+                    if (want) {
+                        const uint64_t need = band_bits_scratch(tb.m, tb.n, sh);
+                        if (need > wave_budget && hand_back()) wave_budget = bits_wave_budget(ctx);
+                        if (need > wave_budget) {
+                            rest.push_back(t.out0);
+                            continue;
+                        }
                     }
                     items.push_back(BandBitsItem{tb.a_off, tb.b_off, 0, bp.a_slot[tb.out0], bp.b_slot[tb.out0], tb.m,
                                                  tb.n, tb.out0, sh});
                     iw.push_back(wq);
-                } else if (words_fit(t)) {
+                } else if (words_fit(t) || (hand_back() && words_fit(t))) {
                     keep.push_back(t);
                     keep_w.push_back(tw[q]);
                 } else {

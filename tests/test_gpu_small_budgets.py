@@ -73,7 +73,7 @@ def _similar(rs, n, subs):
     return a, b.astype(np.uint8)
 
 
-def _banded(nw, ctx, pairs, w):
+def _banded(nw, ctx, pairs, w, sc=(1, -1, -1)):
     """Banded alignments on device buffers: scores, CIGARs, pairs certified in a band."""
     import torch
     pool, off, ln = nw.pool_of([s for p in pairs for s in p])
@@ -83,40 +83,42 @@ def _banded(nw, ctx, pairs, w):
     cl = torch.zeros(len(pairs), dtype=torch.int64, device="cuda")
     before = sum(nw.nw_ctx_band_stats(ctx)["certified_round"])
     nw.nw_align_batch_banded(ctx, torch.from_numpy(pool).cuda(), off[0::2], ln[0::2], off[1::2], ln[1::2],
-                             np.full(len(pairs), w, np.uint32), (1, -1, -1), nw.NW_CIGAR, s, cp, co, cl)
+                             np.full(len(pairs), w, np.uint32), sc, nw.NW_CIGAR, s, cp, co, cl)
     ctx.sync()
     h, n = cp.cpu().numpy(), cl.cpu().numpy()
     text = [bytes(h[int(co[k]):int(co[k]) + int(n[k])]).decode() for k in range(len(pairs))]
     return s.cpu().numpy(), text, sum(nw.nw_ctx_band_stats(ctx)["certified_round"]) - before
 
 
-def _align(nw, ctx, pairs):
+def _align(nw, ctx, pairs, sc=(1, -1, -1)):
     import torch
     pool, off, ln = nw.pool_of([s for p in pairs for s in p])
     co = np.concatenate([[0], np.cumsum([nw.nw_cigar_bound(a.size, b.size) for a, b in pairs])]).astype(np.uint64)
     s = torch.full((len(pairs),), -1, dtype=torch.int32, device="cuda")
     cp = torch.zeros(int(co[-1]), dtype=torch.uint8, device="cuda")
     cl = torch.zeros(len(pairs), dtype=torch.int64, device="cuda")
-    nw.nw_align_batch(ctx, torch.from_numpy(pool).cuda(), off[0::2], ln[0::2], off[1::2], ln[1::2], (1, -1, -1),
+    nw.nw_align_batch(ctx, torch.from_numpy(pool).cuda(), off[0::2], ln[0::2], off[1::2], ln[1::2], sc,
                       nw.NW_CIGAR, s, cp, co, cl)
     ctx.sync()
     h, n = cp.cpu().numpy(), cl.cpu().numpy()
     return s.cpu().numpy(), [bytes(h[int(co[k]):int(co[k]) + int(n[k])]).decode() for k in range(len(pairs))]
 
 
-def test_band_after_a_batch_that_filled_the_scratch(monkeypatch):
+@pytest.mark.parametrize("sc", [(1, -1, -1), (2, -1, -2)])
+def test_band_after_a_batch_that_filled_the_scratch(sc, monkeypatch):
     """Alignments of 3 kb leave records of half the budget behind; the pairs of
-    the next call still run in their band."""
+    the next call still run in their band (+2/-1/-2: on the scalar banded kernel,
+    whose pointer words fit only once the records are handed back)."""
     import torch
     import paper_2412_21103_gb300 as nw
     monkeypatch.setenv("NW_BAND_KEEP", "1")
     rs = seqgen.Stream(91)
     first = [_similar(rs, 3000, 90) for _ in range(200)]
     pairs = [_similar(rs, 8000, 200) for _ in range(3)]
-    want = oracle.align_many(pairs)
+    want = oracle.align_many(pairs, *sc)
     with nw.Context(0, torch.cuda.current_stream(), mem_budget=16 << 20) as ctx:
-        _align(nw, ctx, first)
-        s, c, banded = _banded(nw, ctx, pairs, 900)
+        _align(nw, ctx, first, sc)
+        s, c, banded = _banded(nw, ctx, pairs, 900, sc)
     assert banded == len(pairs)
     assert list(s) == [v for v, _ in want] and c == [oracle.rle(o) for _, o in want]
 
