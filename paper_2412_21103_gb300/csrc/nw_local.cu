@@ -26,7 +26,7 @@
 // ends.
 //
 // End cells and alignments.  The fill keeps no pointers and no positions: a
-// lane notes the first and the last chunk of 32 steps in which its rows reached
+// lane notes the first and the last chunk of steps in which its rows reached
 // their largest H, and every kTileSteps steps the state of a stripe's lanes is
 // kept, with the largest H of the steps since the last one.  The trace finds the
 // pair's best lane, recomputes the tiles that reach its largest H for the
@@ -73,7 +73,7 @@ struct LocalJob {
 };
 
 // The largest H of a stripe: the first lane that reached it, and the first
-// and the last chunk of 32 steps in which it did.
+// and the last chunk of 32 steps (in a fill that keeps states: tile) in which it did.
 struct LocalBest {
     int32_t v;
     uint32_t lane, t0, t1;
@@ -292,9 +292,9 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         ln.start(p.gap);
         uint4 *keep = MODE == kKeep ? p.keep + tk.keep_off + (uint64_t)s * tk.keep_n * LocalLane<R>::kParts * 32u + lane
                                     : nullptr;
-        int32_t best = 0, cm = 0;    // the lane's largest H before and in this chunk of 32 steps
-        int32_t top = 0;             // ... in this tile
-        uint32_t bt = 0, bl = 0;     // the first and the last chunk that reached it
+        int32_t best = 0, cm = 0;    // the lane's largest H before and in this chunk of 32 steps, or tile
+        int32_t top = 0;             // ... in the last tile
+        uint32_t bt = 0, bl = 0;     // the first and the last chunk or tile that reached it
         int32_t c = -lane;
         uint32_t seen = 0;
         bool alive = !s || warp_wait_geq(prev, min(32u, n), seen, p.err, jidx);
@@ -313,7 +313,6 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
         for (uint32_t t = 0; t < T && alive; t += 32) {
             if (MODE == kKeep && keep_n && t && t % kTileSteps == 0) {
                 ln.save(keep, top, p.keep_cap - (uint64_t)(keep - p.keep), p.err);
-                top = 0;
                 keep += LocalLane<R>::kParts * 32u;
             }
             __syncwarp();
@@ -344,11 +343,13 @@ __global__ void __launch_bounds__(kLocalWarps * 32) k_local(LocalArgs p) {
                 }
             }
             row_out(t + 32u);
-            if (MODE != kScore) {
-                if (cm > best) bt = t;
-                if (cm >= best) bl = t;
+            // (with states a tile at a time: once a chunk took 1% of the fill)
+            if (MODE == kEnds || (MODE == kKeep && ((t + 32) % kTileSteps == 0 || t + 32 >= T))) {
+                const uint32_t from = MODE == kKeep ? t - t % kTileSteps : t;
+                if (cm > best) bt = from;
+                if (cm >= best) bl = from;
                 best = max(best, cm);
-                if (MODE == kKeep) top = max(top, cm);
+                top = cm;
                 cm = 0;
             }
         }
@@ -466,7 +467,7 @@ __global__ void __launch_bounds__(WALK ? 32 * kTraceWarps : 32) k_local_trace(Lo
         if (bv > 0) {
             // the first cell in row-major order among the best lane's rows
             const LocalBest b = p.best[tk.job0 + bs];
-            const uint32_t lo = b.t0, hi = min(b.t1 + 32u, n + 31u);
+            const uint32_t lo = b.t0, hi = min(b.t1 + (p.keep ? kTileSteps : 32u), n + 31u);
             uint32_t first[R];  // by row, the first column found
 #pragma unroll
             for (int r = 0; r < R; ++r) first[r] = ~0u;
