@@ -62,7 +62,7 @@ BITS_CELL_KIND = 11          # nw_peak_int kind: one bit-sliced step, 32 cells (
 BITS_KERNELS = ("bits_score", "bband_fill_ptr", "bband_score", "bpair_fill_ptr")
 # The single-pair kernel (bpair_fill_ptr) keeps 31 rows per word (bit 31 is a
 # spare row) and runs one anti-diagonal step of a stripe after another: its
-# time is the wavefront's chain of m + n + m/31 steps, each 24 logic ops of
+# time is the wavefront's chain of m + n + m/31 steps, each 18 logic ops of
 # one warp (the 16-lane logic pipe of one scheduler: 2 cycles each).
 PAIR_ROWS = 31
 PAIR_ALU_OPS_PER_STEP = 18

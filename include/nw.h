@@ -302,9 +302,8 @@ int nw_align_batch(nw_ctx *ctx, const uint8_t *pool2b,
  * cigar_pool + cigar_off[k] as in nw_align_batch (capacity at least
  * nw_cigar_bound).  Pool, scores, ends and CIGAR buffers are device memory
  * unless NW_HOST_IO; metadata arrays are host arrays.  Scoring as nw_align,
- * with max(match, 0) * min(m, n) below 2^29; a pair whose one-warp sweep
- * would exceed 2^31 stripe steps (about m*n/256 >= 2^31) is
- * NW_ERR_UNSUPPORTED. */
+ * with max(match, 0) * min(m, n) below 2^29; a pair of 2^31 stripe steps or
+ * more (ceil(m/256) * max(n, 96)) is NW_ERR_UNSUPPORTED. */
 int nw_local_align_batch(nw_ctx *ctx, const uint8_t *pool2b, const uint64_t *a_off, const uint32_t *a_len,
                          const uint64_t *b_off, const uint32_t *b_len, uint32_t npairs, nw_scoring sc,
                          uint32_t flags, int32_t *scores, uint32_t *ends, char *cigar_pool,
@@ -325,9 +324,7 @@ int nw_local_align_batch(nw_ctx *ctx, const uint8_t *pool2b, const uint64_t *a_o
  * equals nw_align_batch with gap = gap_extend, move for move.  Memory and
  * arguments as nw_align_batch (NW_HOST_IO, NW_CIGAR, NW_CIGAR_M; kept
  * rows and states take about 0.11 byte per cell).  Scores in [-40, 40], both gap scores <=
- * 0, mismatch <= match, max(match - 2*gap_extend, 0) * min(m,n) below 2^29;
- * a pair whose one-warp sweep would exceed 2^31 stripe steps is
- * NW_ERR_UNSUPPORTED. */
+ * 0, mismatch <= match, max(match - 2*gap_extend, 0) * min(m,n) below 2^29. */
 int nw_affine_align_batch(nw_ctx *ctx, const uint8_t *pool2b, const uint64_t *a_off, const uint32_t *a_len,
                           const uint64_t *b_off, const uint32_t *b_len, uint32_t npairs, nw_affine_scoring sc,
                           uint32_t flags, int32_t *scores, char *cigar_pool, const uint64_t *cigar_off,

@@ -443,7 +443,7 @@ static uint64_t bits_wave_budget(nw_ctx *ctx) {
 // One banded round on the bit-sliced window kernel (nw_bits_band.cu) for
 // the items (half-widths iw): pairs that would keep the GPU waiting on one
 // warp go to `rest` (the full kernels), the others run in waves bounded by
-// pointer memory; each wave's certified pairs are walked into CIGARs, the
+// their scratch; each wave's certified pairs are walked into CIGARs, the
 // others return in next / nextw with their next widths.
 static int bits_round(nw_ctx *ctx, const uint8_t *pool, const PlaneSet &planes, std::vector<BandBitsItem> &items, std::vector<uint32_t> &iw, int round, const nw_scoring &sc,
                       uint32_t flags, int32_t *scores, uint32_t score_cap, char *cigar_pool, const uint64_t *cigar_off,

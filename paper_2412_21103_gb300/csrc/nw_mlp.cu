@@ -602,13 +602,13 @@ int learned_band_widths(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off,
     // The first round's width is 0.75x the predicted one: a round that fails
     // its certificate is followed by one at the smallest width the failed
     // score proves sufficient, so under-predicting costs one narrow pass
-    // while over-predicting widens every band.  Measured on GB300 (20,000
-    // pairs of 2-20 kb, same context and memory budget): 0.25 -> 6,526,
-    // 0.5 -> 6,100, 0.75 -> 5,691, 1 -> 5,285 effective GCUPS, against 6,962
-    // from the fixed start 64; 0.75 is kept because it is the smallest
-    // margin at which the network certifies more pairs in the first round
-    // than the fixed start on held-out pairs while sweeping fewer banded
-    // cells there.  NW_BAND_MARGIN and NW_BAND_PROBE_CAP for sweeps.
+    // while over-predicting widens every band.  Effective GCUPS on GB300 (20,000
+    // pairs of 2-20 kb): 0.25 -> 58,300, 0.5 -> 56,700, 0.75 -> 55,000, 1 -> 52,500,
+    // against 60,600 from the fixed start 64: the first round costs more than the
+    // second it saves.  0.75 is the smallest margin at which the network certifies
+    // more pairs in the first round than the fixed start on held-out pairs while
+    // sweeping fewer banded cells there.  NW_BAND_MARGIN and NW_BAND_PROBE_CAP for
+    // sweeps.
     double margin = 0.75;
     if (const char *e = getenv("NW_BAND_MARGIN")) margin = std::max(0.25, atof(e));
     int rc = model_of(ctx, &bm, false);
