@@ -615,10 +615,13 @@ int bits_pairs(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &job
         }
         L.pairs = (const PairDesc *)v;
         L.blocks = (const PairBlock *)((char *)v + dbytes);
+        const auto slot = ctx->bufs.find("bpair_ring");
+        const bool fresh = slot == ctx->bufs.end() || slot->second.cap < ring + 64;
         if ((rc = scratch(ctx, "bpair_ring", ring + 64, &v))) return rc;
-        if (v != ctx->bits_ring || ctx->bits_epoch == 0xffffffffu) {
-            // a new ring may hold anything, also tags of an earlier context:
-            // clear it and start the epochs again
+        if (fresh || v != ctx->bits_ring || ctx->bits_epoch == 0xffffffffu) {
+            // a new ring may hold anything, also tags of an earlier context, and
+            // may lie where the one before it lay: clear it and start the epochs
+            // again
             const cudaError_t e = cudaMemsetAsync(v, 0, ring + 64, ctx->stream);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "ring clear");
             ctx->bits_ring = v;
