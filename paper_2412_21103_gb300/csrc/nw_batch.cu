@@ -959,12 +959,21 @@ static int band_batch(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
     return NW_OK;
 }
 
+// Hands back the scratch of the full-grid alignment paths (idle between their
+// launches; in stream order).
+static void free_path_scratch(nw_ctx *ctx) {
+    for (const char *slots : {"bgroup_", "bpair_", "batch_", "tb_", "ckpt_", "pair_", "ptr", "moves", "nmoves"})
+        free_prefix(ctx, slots);
+}
+
 // Score-only or CIGAR batch on device buffers (the C entry point stages
-// host buffers around this).
-int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const uint32_t *a_len,
-                      const uint64_t *b_off, const uint32_t *b_len, const uint32_t *ids, uint32_t npairs,
-                      const nw_scoring &sc, uint32_t flags, int32_t *scores, char *cigar_pool,
-                      const uint64_t *cigar_off, uint64_t *cigar_len) {
+// host buffers around this); groups: alignments of scorings that fit two bit
+// planes run on the groups of lanes; tight (alignments): only pairs that do not
+// fit the batch kernel leave it, none for time, and one at a time.
+static int batch_device(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const uint32_t *a_len,
+                        const uint64_t *b_off, const uint32_t *b_len, const uint32_t *ids, uint32_t npairs,
+                        const nw_scoring &sc, uint32_t flags, int32_t *scores, char *cigar_pool,
+                        const uint64_t *cigar_off, uint64_t *cigar_len, bool groups, bool tight) {
     const Profile pf = make_profile(sc);
     const bool want = flags & NW_CIGAR;
     int rc;
@@ -1010,9 +1019,6 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
         max_n = std::max(max_n, t.n);
         tasks[q] = t;
     }
-    // alignments whose scoring fits two bit planes run on groups of lanes of
-    // the bit-sliced kernel, the others on the scalar batch kernel
-    const bool groups = want && bits_batch_ok(sc) && !getenv("NW_PAIR_SCALAR");
     const bool score_bits = !want && bits_scores_pay(ctx, tasks, sc);
     // pairs that would leave the GPU idle on one warp take the single-pair
     // kernel, and so do pairs whose pointer matrix alone exceeds half the
@@ -1041,7 +1047,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
         }
         // (no pair outlasts the batch: nothing to route)
         std::vector<size_t> strag;
-        if (longest / kWarpRate > total / rate) strag = pick_stragglers(wc, fc, ps, ctx->sm_count, rate);
+        if (!tight && longest / kWarpRate > total / rate) strag = pick_stragglers(wc, fc, ps, ctx->sm_count, rate);
         if (want) {
             const uint64_t room = (ctx->budget - std::min(ctx->budget, ctx->used)) / 2;
             std::vector<char> in(tasks.size(), 0);
@@ -1059,7 +1065,25 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
                 st.push_back(tasks[q]);
                 routed[q] = 1;
             }
-            if ((rc = run_stragglers(ctx, pool, st, sc, flags, scores, cigar_pool, cigar_off, cigar_len))) return rc;
+            if (!tight) {
+                rc = run_stragglers(ctx, pool, st, sc, flags, scores, cigar_pool, cigar_off, cigar_len);
+            } else {
+                // one at a time, each with the others' scratch if it needs it
+                for (const BatchTask &t : st) {
+                    const uint32_t id = t.out0;
+                    const auto single = [&] {
+                        return run_straggler(ctx, pool, t.a_off, t.m, t.b_off, t.n, sc, flags, scores + id,
+                                             cigar_pool + cigar_off[id], cigar_off[id + 1] - cigar_off[id], cigar_len + id);
+                    };
+                    if ((rc = single()) == NW_ERR_OOM) {
+                        free_path_scratch(ctx);
+                        rc = single();
+                    }
+                    if (rc) break;
+                }
+                free_path_scratch(ctx);
+            }
+            if (rc) return rc;
             std::vector<BatchTask> keep;
             for (size_t q = 0; q < tasks.size(); ++q)
                 if (!routed[q]) keep.push_back(tasks[q]);
@@ -1165,7 +1189,7 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
             wave.push_back(t);
             ids_w.push_back(t.out0);
         }
-        if (k < npairs || k0 > 0) {  // a true wave (not the whole batch): route its stragglers
+        if (!tight && (k < npairs || k0 > 0)) {  // a true wave (not the whole batch): route its stragglers
             std::vector<double> wc(wave.size());
             std::vector<PairCost> ps(wave.size());
             for (size_t q = 0; q < wave.size(); ++q) {
@@ -1226,6 +1250,29 @@ int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, c
         k0 = k;
     }
     return NW_OK;
+}
+
+int batch_device_impl(nw_ctx *ctx, const uint8_t *pool, const uint64_t *a_off, const uint32_t *a_len,
+                      const uint64_t *b_off, const uint32_t *b_len, const uint32_t *ids, uint32_t npairs,
+                      const nw_scoring &sc, uint32_t flags, int32_t *scores, char *cigar_pool,
+                      const uint64_t *cigar_off, uint64_t *cigar_len) {
+    // alignments whose scoring fits two bit planes run on groups of lanes of
+    // the bit-sliced kernel, the others on the scalar batch kernel
+    const bool groups = (flags & NW_CIGAR) && bits_batch_ok(sc) && !getenv("NW_PAIR_SCALAR");
+    const std::string before = ctx->msg;
+    const auto run = [&](bool g, bool tight) {
+        return batch_device(ctx, pool, a_off, a_len, b_off, b_len, ids, npairs, sc, flags, scores, cigar_pool, cigar_off,
+                            cigar_len, g, tight);
+    };
+    const int rc = run(groups, false);
+    if (!groups || rc != NW_ERR_OOM) return rc;
+    // A budget so small that a pair does not fit the groups or the single-pair
+    // kernel -- a whole warp's records, planar copies, tables -- may still hold it
+    // on the scalar batch kernel.
+    free_path_scratch(ctx);
+    const int again = run(false, true);
+    if (!again) ctx->msg = before;
+    return again;
 }
 
 // The CIGARs of a host-I/O batch, packed back to back (pair k's bytes at

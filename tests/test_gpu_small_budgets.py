@@ -209,3 +209,24 @@ def test_alignments_whose_planar_copies_alone_fill_the_budget():
     for k in (0, 700, 1499):
         v, ops = oracle.align(*pairs[k])
         assert s[k] == v and c[k] == oracle.rle(ops)
+
+
+# budgets that the scalar kernel fits, a warp's records and planar copies of some
+# pairs do not; twice, because the second call finds the first one's slots
+@pytest.mark.parametrize("rows,cols,count,budget", [((2000, 4000), (2000, 4000), 4, 1680000), ((300, 1500), (300, 1500), 200, 497000),
+                                                    ((100, 300), (5000, 20000), 50, 3780000),
+                                                    ((5000, 20000), (100, 300), 50, 1680000)])
+@pytest.mark.parametrize("sc", [(1, -1, -1), (2, -1, -2)])
+def test_alignments_that_fit_only_the_scalar_kernel(rows, cols, count, budget, sc):
+    import torch
+    import paper_2412_21103_gb300 as nw
+    rs = seqgen.Stream(96)
+    pairs = [(rs.bases(int(m)), rs.bases(int(n))) for m, n in zip(rs.integers(*rows, count), rs.integers(*cols, count))]
+    with nw.Context(0, torch.cuda.current_stream(), mem_budget=budget) as ctx:
+        got = [_align(nw, ctx, pairs, sc) for _ in range(2)]
+    with nw.Context(0, torch.cuda.current_stream()) as ctx:
+        s, c = _align(nw, ctx, pairs, sc)
+    for s2, c2 in got:
+        assert (s == s2).all() and c == c2
+    v, ops = oracle.align(*pairs[0], *sc)
+    assert s[0] == v and c[0] == oracle.rle(ops)
