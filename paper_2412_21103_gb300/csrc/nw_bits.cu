@@ -162,8 +162,9 @@ __device__ __forceinline__ void deal_rows(const uint32_t *pl, int64_t Ag, int32_
 }
 
 // W(m, n) of a lane's pair, in the steps of its job: job.T chunks, a stripe
-// every job.C.
-template <bool GEN, int K>
+// every job.C.  (Count: 64 bits only where T needs them, they cost a lone warp 3%
+// of its time.)
+template <bool GEN, int K, class Count = uint32_t>
 __device__ __forceinline__ int32_t bits_pairs_of(const BitsArgs &p, const BitsJob &job, uint32_t m, uint32_t n,
                                                  int64_t Ag, int64_t Bg, uint2 *rows) {
     constexpr int32_t SH = 32 * K;
@@ -184,8 +185,8 @@ __device__ __forceinline__ int32_t bits_pairs_of(const BitsArgs &p, const BitsJo
     int32_t W = 0;
     uint32_t stripe = 0, cl = 0;   // of the stripe's row 0
     uint32_t started = 0, lift = 0;  // chunks since a stripe began; all ones once it is not the first
-    const uint64_t last = bits_last_row(S, C, K);
-    for (uint64_t c = 0; c < job.T; ++c) {
+    const Count last = bits_last_row<Count>(S, C, K), T = (Count)job.T;
+    for (Count c = 0; c < T; ++c) {
         if (cl == 0 && stripe < S) {
             started = 0;
             lift = stripe ? ~0u : 0u;
@@ -221,8 +222,8 @@ __device__ __forceinline__ int32_t bits_pairs_of(const BitsArgs &p, const BitsJo
         // outgoing bits: bit b is column 32 (c - K + 1) - b of the bottom row, from the stripe's first chunk on
         if (S > 1 && c <= last) __stcg(rows + (size_t)cl * 32u, make_uint2(Q0, Q1));
         int32_t lo, hi;
-        bits_last_row_span(c, last, n, lo, hi);
-        if (lo <= hi) {
+        bits_last_row_span((uint32_t)(c - last), n, lo, hi);
+        if (c >= last && lo <= hi) {
             const uint32_t mk = (hi == 31 ? ~0u : ((2u << hi) - 1u)) & (~0u << lo);
             W += __popc(Q0 & mk) + 2 * __popc(Q1 & mk);
         }
@@ -253,8 +254,9 @@ __device__ __forceinline__ void class_pair(const BitsClass &k, uint32_t q, uint3
     r = c + 1u + (uint32_t)(t - x * (b - x) / 2ull);
 }
 
-template <bool GEN>
-__global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
+// The warps of a launch take its jobs.  WIDE: jobs of 2^32 chunks or more.
+template <bool GEN, bool WIDE>
+__device__ __forceinline__ void bits_jobs(const BitsArgs &p) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     uint2 *rows = p.rows + (size_t)gw * p.rows_chunks * 32u + lane;
@@ -288,7 +290,8 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
         int32_t W = 0;
         const int64_t Ag = (int64_t)aw * 32 - kPlanePad, Bg = (int64_t)bw * 32 - kPlanePad;  // planar slots
         if (job.S) {
-            if (job.K == 4) W = bits_pairs_of<GEN, 4>(p, job, m, n, Ag, Bg, rows);
+            if constexpr (WIDE) W = bits_pairs_of<GEN, 1, uint64_t>(p, job, m, n, Ag, Bg, rows);
+            else if (job.K == 4) W = bits_pairs_of<GEN, 4>(p, job, m, n, Ag, Bg, rows);
             else if (job.K == 2) W = bits_pairs_of<GEN, 2>(p, job, m, n, Ag, Bg, rows);
             else W = bits_pairs_of<GEN, 1>(p, job, m, n, Ag, Bg, rows);
         }
@@ -298,6 +301,16 @@ __global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
             if (out1 != ~0u && in_range(out1, p.score_cap, p.err, kSiteBatchScore)) p.scores[out1] = sc;
         }
     }
+}
+
+template <bool GEN>
+__global__ void __launch_bounds__(kBitsWarps * 32) k_bits_score(BitsArgs p) {
+    bits_jobs<GEN, false>(p);
+}
+// (a kernel of its own: the second count in the first one's code cost a lone warp 5%)
+template <bool GEN>
+__global__ void __launch_bounds__(kBitsWarps * 32) k_bits_wide(BitsArgs p) {
+    bits_jobs<GEN, true>(p);
 }
 
 // Planar copy of a sequence by a warp: word w of its slot holds bit k of the
@@ -461,10 +474,13 @@ class BitsShapes {
             }
         }
     }
-    BitsShape of(uint32_t m) const {  // m = 0: no stripes
+    // m = 0: no stripes.  Rows that with n columns come to 2^32 chunks or more run
+    // one word a lane, the form that counts in 64 bits.
+    BitsShape of(uint32_t m, uint32_t n) const {
         const uint32_t w = (m + 31) / 32;
         if (w <= kWords) return by_words_[w];
-        return shape(w, by_words_[kWords].K / 2);
+        const BitsShape s = shape(w, by_words_[kWords].K / 2);
+        return s.chunks(n) >> 32 ? shape(w, 0) : s;
     }
 
   private:
@@ -488,7 +504,9 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
     // longest jobs first, ties in job order
     std::vector<uint64_t> keys(jobs.size());
     for (size_t q = 0; q < jobs.size(); ++q) keys[q] = jobs[q].T * (10 * jobs[q].K + 6);
-    const std::vector<uint32_t> jo = radix_order_desc(std::move(keys));
+    std::vector<uint32_t> jo = radix_order_desc(std::move(keys));
+    // jobs of 2^32 chunks or more lead: they have a launch of their own
+    plan->wide = (uint32_t)(std::stable_partition(jo.begin(), jo.end(), [&](uint32_t q) { return jobs[q].T >> 32; }) - jo.begin());
     const size_t jobs_at = (head.size() + 15) / 16 * 16;
     head.resize(jobs_at + jobs.size() * sizeof(BitsJob));
     BitsJob *hj = reinterpret_cast<BitsJob *>(head.data() + jobs_at);
@@ -558,9 +576,9 @@ static int bits_prepare_slots(nw_ctx *ctx, const uint8_t *pool, const std::vecto
             keys[k] = std::max(t.m, t.n);  // no stripes
             continue;
         }
-        BitsShape sh = shapes.of(t.m);
+        BitsShape sh = shapes.of(t.m, t.n);
         if ((t.m + 31) / 32 != (t.n + 31) / 32) {
-            const BitsShape sn = shapes.of(t.n);
+            const BitsShape sn = shapes.of(t.n, t.m);
             turned[k] = sn.work(t.m) < sh.work(t.n);
             if (turned[k]) sh = sn;
         }
@@ -593,7 +611,7 @@ static int bits_prepare_slots(nw_ctx *ctx, const uint8_t *pool, const std::vecto
             std::swap(b.a_off, b.b_off);
             std::swap(b.m, b.n);
         }
-        const BitsShape sh = shapes.of(b.n ? b.m : 0);
+        const BitsShape sh = shapes.of(b.n ? b.m : 0, b.n);
         if (sh.S && own) {
             b.aw = (uint32_t)words;
             b.bw = b.aw + (b.m + 31) / 32 + 2;
@@ -656,11 +674,12 @@ int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, cons
     std::vector<BitsClass> classes;
     std::vector<BitsJob> jobs;
     uint32_t maxC = 1;
+    const uint32_t widest = nseq ? seqs[0].len : 0u;
     for (uint32_t r0 = 0; r0 < nseq;) {
-        const BitsShape sh = shapes.of(seqs[r0].len);
+        const BitsShape sh = shapes.of(seqs[r0].len, widest);
         uint32_t r1 = r0 + 1;
         for (; r1 < nseq; ++r1)
-            if (const BitsShape x = shapes.of(seqs[r1].len); x.S != sh.S || x.K != sh.K) break;
+            if (const BitsShape x = shapes.of(seqs[r1].len, widest); x.S != sh.S || x.K != sh.K) break;
         const uint32_t rows = r1 - r0, pairs = r0 * rows + rows * (rows - 1) / 2;
         // the pairs run through the columns in order: a job's first column is its widest
         uint32_t c = 0;
@@ -689,7 +708,7 @@ int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, cons
 
 int bits_launch(nw_ctx *ctx, const BitsPlan &plan) {
     if (plan.ba.njobs == 0) return NW_OK;
-    cudaMemsetAsync(plan.ba.counter, 0, 4, ctx->stream);
+    cudaMemsetAsync(plan.ba.counter, 0, 8, ctx->stream);
     if (plan.ntasks) {
         LaunchTimer t(ctx, "planes");
         const uint32_t blocks = std::min<uint32_t>((plan.ntasks + 3) / 4, 4096);
@@ -698,10 +717,21 @@ int bits_launch(nw_ctx *ctx, const BitsPlan &plan) {
     } else if (int rc = plan.planes.enqueue(ctx, plan.pool)) {
         return rc;
     }
-    {
+    BitsArgs ba = plan.ba;
+    if (plan.wide) {
+        LaunchTimer t(ctx, "bits_wide");
+        ba.njobs = plan.wide;
+        ++ba.counter;
+        if (plan.gen) k_bits_wide<true><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(ba);
+        else k_bits_wide<false><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(ba);
+        ba = plan.ba;
+        ba.jobs += plan.wide;
+        ba.njobs -= plan.wide;
+    }
+    if (ba.njobs) {
         LaunchTimer t(ctx, "bits_score");
-        if (plan.gen) k_bits_score<true><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(plan.ba);
-        else k_bits_score<false><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(plan.ba);
+        if (plan.gen) k_bits_score<true><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(ba);
+        else k_bits_score<false><<<plan.blocks, kBitsWarps * 32, 0, ctx->stream>>>(ba);
     }
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? NW_OK : cuda_fail(ctx, e, "bit-sliced launch");

@@ -183,6 +183,7 @@ class PlaneSet {
 struct BitsPlan {
     BitsArgs ba{};
     uint32_t blocks = 0;
+    uint32_t wide = 0;        // leading jobs of 2^32 chunks or more
     const uint8_t *pool = nullptr;
     uint32_t ntasks = 0;      // tasks whose sequences have slots of their own
     PlaneSet planes;          // or the distinct sequences

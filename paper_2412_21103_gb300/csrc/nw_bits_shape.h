@@ -27,22 +27,22 @@ struct BitsShape {
 };
 
 // The chunk from which on the last stripe's bottom row leaves: its bit 0 is
-// column 0 there, and column 32 d - b is bit b of the d-th chunk after it.
-NW_HOST_DEVICE uint64_t bits_last_row(uint32_t S, uint32_t C, uint32_t K) { return (uint64_t)(S - 1) * C + K - 1; }
+// column 0 there, and column 32 d - b is bit b of the d-th chunk after it.  Count:
+// uint32_t for pairs of fewer than 2^32 chunks, else uint64_t.
+template <class Count>
+NW_HOST_DEVICE Count bits_last_row(uint32_t S, uint32_t C, uint32_t K) {
+    return (Count)(S - 1) * C + K - 1;
+}
 
-// The bits [lo, hi] of chunk c that are columns 0 .. n-1 of that row (lo > hi:
-// none).  Chunks of earlier stripes hold none: the difference is formed only
-// from `last` on, where it is small.
-NW_HOST_DEVICE void bits_last_row_span(uint64_t c, uint64_t last, uint32_t n, int32_t &lo, int32_t &hi) {
-    lo = 1;
-    hi = 0;
-    if (c < last) return;
-    const int32_t e = (int32_t)(32 * (c - last));
-    lo = e + 1 > (int32_t)n ? e + 1 - (int32_t)n : 0;
+// The bits [lo, hi] of the d-th chunk from there on that are columns 0 .. n-1 of
+// that row (lo > hi: none).  Of chunks before it the difference means nothing.
+NW_HOST_DEVICE void bits_last_row_span(uint32_t d, uint32_t n, int32_t &lo, int32_t &hi) {
+    const int32_t e = (int32_t)(32u * d), from = (int32_t)(32u * d + 1u - n);
+    lo = from > 0 ? from : 0;
     hi = e < 31 ? e : 31;
 }
 
-// A pair on G lanes of a warp, stripes of 31 rows: its chunks (K in all, from one
+// A pair on G lanes of a warp stripes of 31 rows: its chunks (K in all, from one
 // pass of a lane to its next `period`), and its 16-byte record units.  A pair of
 // 1.3e14 cells has more than 2^32 chunks; those that a launch takes have records
 // that fit the scratch, so their K fits 32 bits.

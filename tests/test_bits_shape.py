@@ -13,10 +13,15 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2412_21103_gb300", "csrc")
 SOURCE = r"""
 #include "nw_bits_shape.h"
-extern "C" {
-void span(uint64_t c, uint32_t S, uint32_t C, uint32_t K, uint32_t n, int32_t *out) {
-    nw::bits_last_row_span(c, nw::bits_last_row(S, C, K), n, out[0], out[1]);
+template <class Count>
+void span_of(Count c, uint32_t S, uint32_t C, uint32_t K, uint32_t n, int32_t *out) {
+    const Count last = nw::bits_last_row<Count>(S, C, K);
+    nw::bits_last_row_span((uint32_t)(c - last), n, out[0], out[1]);
+    if (c < last) out[0] = 1, out[1] = 0;
 }
+extern "C" {
+void span(uint64_t c, uint32_t S, uint32_t C, uint32_t K, uint32_t n, int32_t *out) { span_of<uint64_t>(c, S, C, K, n, out); }
+void span32(uint32_t c, uint32_t S, uint32_t C, uint32_t K, uint32_t n, int32_t *out) { span_of<uint32_t>(c, S, C, K, n, out); }
 uint32_t period(uint32_t K, uint32_t S, uint32_t n) { return nw::BitsShape{K, S, 10 * K + 6}.period(n); }
 uint64_t chunks(uint32_t K, uint32_t S, uint32_t n) { return nw::BitsShape{K, S, 10 * K + 6}.chunks(n); }
 uint64_t group(uint32_t m, uint32_t n, uint32_t G, uint64_t *rec) {
@@ -37,13 +42,17 @@ def lib(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, str(d / "shape.cpp"), "-o", so], check=True)
     lib = ctypes.CDLL(so)
     lib.span.argtypes = [ctypes.c_uint64] + [ctypes.c_uint32] * 4 + [ctypes.POINTER(ctypes.c_int32)]
+    lib.span32.argtypes = [ctypes.c_uint32] * 5 + [ctypes.POINTER(ctypes.c_int32)]
     lib.period.restype, lib.chunks.restype, lib.group.restype = ctypes.c_uint32, ctypes.c_uint64, ctypes.c_uint64
     return lib
 
 
 def _span(lib, c, S, C, K, n):
-    out = (ctypes.c_int32 * 2)()
+    out, out32 = (ctypes.c_int32 * 2)(), (ctypes.c_int32 * 2)()
     lib.span(c, S, C, K, n, out)
+    if lib.chunks(K, S, n) < 1 << 32:  # the form the kernel takes then
+        lib.span32(c, S, C, K, n, out32)
+        assert (out32[0], out32[1]) == (out[0], out[1]) or (out32[0] > out32[1] and out[0] > out[1])
     return out[0], out[1]
 
 
