@@ -751,7 +751,8 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
         const size_t nt = wave.size();
         PlaneSet ps;
         ps.reserve(std::min<size_t>(2 * nt, 1u << 16));
-        for (const uint32_t k : wave) {
+        for (size_t q = 0; q < nt; ++q) {
+            const size_t k = nt == np ? q : wave[q];  // (the whole batch: in the caller's order, by address)
             if (!pairs[k].m || !pairs[k].n) continue;
             ag[k] = ps.add(pairs[k].a_off, pairs[k].m);
             bg[k] = ps.add(pairs[k].b_off, pairs[k].n);

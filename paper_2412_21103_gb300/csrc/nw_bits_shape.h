@@ -42,7 +42,7 @@ NW_HOST_DEVICE void bits_last_row_span(uint32_t d, uint32_t n, int32_t &lo, int3
     hi = e < 31 ? e : 31;
 }
 
-// A pair on G lanes of a warp stripes of 31 rows: its chunks (K in all, from one
+// A pair on G lanes of a warp (a power of two), stripes of 31 rows: its chunks (K in all, from one
 // pass of a lane to its next `period`), and its 16-byte record units.  A pair of
 // 1.3e14 cells has more than 2^32 chunks; those that a launch takes have records
 // that fit the scratch, so their K fits 32 bits.
@@ -57,7 +57,8 @@ inline GroupGeom group_geom(uint32_t m, uint32_t n, uint32_t G) {
     g.S = (m + kPairRows - 1) / kPairRows;
     g.C = (uint32_t)(((uint64_t)n + kPairRows - 1 + 31u) / 32u);
     g.period = g.C > G + 2 ? g.C : G + 2;
-    g.K = (uint64_t)((g.S - 1) / G) * g.period + g.C + (g.S - 1) % G;
+    const uint32_t passes = (g.S - 1) >> __builtin_ctz(G);  // (a division, ten times a pair, showed in small batches)
+    g.K = (uint64_t)passes * g.period + g.C + ((g.S - 1) & (G - 1));
     g.rec = g.K * 16u * G;
     return g;
 }
