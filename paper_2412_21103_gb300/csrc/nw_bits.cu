@@ -503,10 +503,16 @@ static int bits_finish_plan(nw_ctx *ctx, const uint8_t *pool, std::vector<uint8_
     int rc;
     // longest jobs first, ties in job order
     std::vector<uint64_t> keys(jobs.size());
-    for (size_t q = 0; q < jobs.size(); ++q) keys[q] = jobs[q].T * (10 * jobs[q].K + 6);
+    uint64_t most = 0;
+    for (size_t q = 0; q < jobs.size(); ++q) {
+        keys[q] = jobs[q].T * (10 * jobs[q].K + 6);
+        most = std::max(most, jobs[q].T);
+    }
     std::vector<uint32_t> jo = radix_order_desc(std::move(keys));
     // jobs of 2^32 chunks or more lead: they have a launch of their own
-    plan->wide = (uint32_t)(std::stable_partition(jo.begin(), jo.end(), [&](uint32_t q) { return jobs[q].T >> 32; }) - jo.begin());
+    plan->wide = 0;
+    if (most >> 32)
+        plan->wide = (uint32_t)(std::stable_partition(jo.begin(), jo.end(), [&](uint32_t q) { return jobs[q].T >> 32; }) - jo.begin());
     const size_t jobs_at = (head.size() + 15) / 16 * 16;
     head.resize(jobs_at + jobs.size() * sizeof(BitsJob));
     BitsJob *hj = reinterpret_cast<BitsJob *>(head.data() + jobs_at);
@@ -673,6 +679,7 @@ int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, cons
     const BitsShapes shapes;
     std::vector<BitsClass> classes;
     std::vector<BitsJob> jobs;
+    jobs.reserve((uint64_t)nseq * nseq / 64 + 64);  // 32 pairs a job, and a class's last
     uint32_t maxC = 1;
     const uint32_t widest = nseq ? seqs[0].len : 0u;
     for (uint32_t r0 = 0; r0 < nseq;) {
@@ -682,15 +689,22 @@ int bits_prepare_all(nw_ctx *ctx, const uint8_t *pool, const uint64_t *off, cons
             if (const BitsShape x = shapes.of(seqs[r1].len, widest); x.S != sh.S || x.K != sh.K) break;
         const uint32_t rows = r1 - r0, pairs = r0 * rows + rows * (rows - 1) / 2;
         // the pairs run through the columns in order: a job's first column is its widest
-        uint32_t c = 0;
+        uint32_t c = ~0u, end = 0;
+        BitsJob j{};
         auto end_of = [&](uint32_t col) {  // pairs of the columns up to col
             const uint32_t x = col < r0 ? 0u : col - r0 + 1u;
             return col < r0 ? (col + 1u) * rows : r0 * rows + (uint32_t)((uint64_t)x * (2ull * rows - x - 1u) / 2u);
         };
         for (uint32_t q = 0; q < pairs; q += 32) {
-            while (end_of(c) <= q) ++c;
-            jobs.push_back(job_of(sh, seqs[c].len, q, std::min(32u, pairs - q), (uint32_t)classes.size()));
-            maxC = std::max(maxC, jobs.back().C);
+            if (end <= q) {
+                do end = end_of(++c);
+                while (end <= q);
+                j = job_of(sh, seqs[c].len, 0, 0, (uint32_t)classes.size());
+                maxC = std::max(maxC, j.C);
+            }
+            j.t0 = q;
+            j.cnt = std::min(32u, pairs - q);
+            jobs.push_back(j);
         }
         classes.push_back(BitsClass{r0, r1});
         r0 = r1;
