@@ -705,14 +705,11 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
     // bytes per store) where the pair has that many stripes.
     const double half = 0.5 * work / (4.0 * ctx->sm_count);  // in chunks of a warp at 32 lanes .. of one lane
     std::vector<uint8_t> lanes(np);
-    std::vector<GroupGeom> geom(np);
     std::vector<uint64_t> by_moves(np);
     for (size_t k = 0; k < np; ++k) {
         uint32_t G = 1;
         const uint32_t S = (pairs[k].m + kPairRows - 1) / kPairRows;
-        while (G < 4 && G < S) G *= 2;
-        geom[k] = group_geom(pairs[k].m, pairs[k].n, G);
-        while (G < 32 && G < S && (double)geom[k].K > half / 32.0) geom[k] = group_geom(pairs[k].m, pairs[k].n, G *= 2);
+        while (G < 32 && G < S && (G < 4 || (double)group_geom(pairs[k].m, pairs[k].n, G).K > half / 32.0)) G *= 2;
         lanes[k] = (uint8_t)G;
         by_moves[k] = (uint64_t)pairs[k].m + pairs[k].n;
     }
@@ -737,16 +734,20 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
     std::vector<int64_t> ag(np, 0), bg(np, 0);
     for (size_t next = 0; next < np;) {
         std::vector<uint32_t> wave;
+        std::vector<uint64_t> keys;  // tasks by lanes, then chunks
+        wave.reserve(np - next);
+        keys.reserve(np - next);
         uint64_t rec = 0, rows = 0, moves = 0, bytes = 0;
         for (; next < np; ++next) {
             const PairJob &j = pairs[order[next]];
-            const GroupGeom &g = geom[order[next]];
+            const GroupGeom g = group_geom(j.m, j.n, lanes[order[next]]);
             const uint64_t more = g.rec * 16 + g.C * sizeof(uint2) + (uint64_t)j.m + j.n + 16 + sizeof(uint64_t) +
                                   sizeof(GroupTask) + sizeof(GroupJob) + sizeof(TraceTask) +
                                   PlaneSet::bytes_of(j.m) + PlaneSet::bytes_of(j.n);
             if (!wave.empty() && bytes + more > room) break;
             bytes += more;
             wave.push_back(order[next]);
+            keys.push_back((uint64_t)lanes[order[next]] << 56 | g.K);
             rec += g.rec;
             rows += g.C;
             moves += (uint64_t)j.m + j.n + 16;
@@ -769,9 +770,7 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
         if ((rc = scratch(ctx, "bgroup_rows", rows * sizeof(uint2) + 16, &wv))) return rc;
         if ((rc = scratch(ctx, "bgroup_moves", moves + 16, &mv))) return rc;
         if ((rc = scratch(ctx, "bgroup_nmoves", nt * 8 + 16, &nm))) return rc;
-        // tasks by lanes, then chunks; jobs of 32 / G of them, longest first
-        std::vector<uint64_t> keys(nt);
-        for (size_t q = 0; q < nt; ++q) keys[q] = (uint64_t)lanes[wave[q]] << 56 | geom[wave[q]].K;
+        // jobs of 32 / G tasks, longest first
         const std::vector<uint32_t> to = radix_order_desc(std::move(keys));
         std::vector<GroupTask> tasks(nt);
         std::vector<TraceTask> tts(nt);
@@ -781,7 +780,7 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
         for (size_t q = 0; q < nt; ++q) {  // records in the walks' order
             const PairJob &j = pairs[wave[q]];
             const uint32_t G = lanes[wave[q]];
-            const GroupGeom &g = geom[wave[q]];
+            const GroupGeom g = group_geom(j.m, j.n, G);
             const uint8_t *a = pool ? pool + j.a_off : (const uint8_t *)(uintptr_t)j.a_off;
             const uint8_t *b = pool ? pool + j.b_off : (const uint8_t *)(uintptr_t)j.b_off;
             tts[q] = TraceTask{(const uint32_t *)((uint4 *)rv + rec_off), 16u * g.period, j.m, j.n, (uint8_t *)mv + moff,
@@ -792,7 +791,7 @@ int bits_groups(nw_ctx *ctx, const uint8_t *pool, const std::vector<PairJob> &pa
         for (size_t q = 0; q < nt; ++q) {
             const uint32_t w = to[q], k = wave[w], G = lanes[k];
             const PairJob &j = pairs[k];
-            const GroupGeom &g = geom[k];
+            const GroupGeom g = group_geom(j.m, j.n, G);
             GroupTask &t = tasks[q];
             t = GroupTask{ag[k], bg[k], j.m, j.n, g.S, g.C, g.period, (uint32_t)g.K, g.S ? (j.m - 1) - kPairRows * (g.S - 1) : 0u,
                           0u, (uint64_t)((const uint4 *)tts[w].ptr - (const uint4 *)rv), row_off, j.score};
